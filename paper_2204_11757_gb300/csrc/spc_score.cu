@@ -813,18 +813,29 @@ k_score_staged(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restr
 // S3, packed schedule for binary32 rows: the normalise kernel stores every entry as one 8-byte
 // (column, p) pair, so a row is one contiguous run of bytes.  A warp takes 32 consecutive
 // edges (one lane each): the tile's rows a, one contiguous slice, are copied by the whole warp,
-// and every lane copies its own row b into the warp's area, the rows packed one after the other
-// (a prefix sum of their lengths places them), all with 16-byte asynchronous copies.  A copy
+// and the 32 rows b by groups of kPkLanes lanes, packed one after the other in the warp's area (a
+// prefix sum of their lengths places them), all with 16-byte asynchronous copies.  A copy
 // keeps each entry's position modulo two entries, so both of its ends are 16-byte aligned; a
 // row that starts or ends inside a 16-byte chunk brings its neighbour along, never read.  Then
 // every lane walks its edge's union from shared memory, one 8-byte load per step, with the
 // uniform step of k_score_edges (the same bits).  Rows that do not fit are walked in place.
 // Binary32 inputs have their symmetry checked by the fingerprint of the normalise kernel, so
 // the walk carries no mirror check (and no arithmetic count, which serves binary64 only).
+//
+// What bounds it: on a graph in random node order the rows b are random reads, 13.9 GB for the
+// 49.9 M edges of the 2^23-point random geometric graph.  With every lane copying its own row a
+// warp instruction asked for 32 unrelated 16-byte pieces, two requests for each sector; with
+// four lanes to a row neighbouring lanes share sectors and lines.  First level, ms (one lane per
+// row / 8 lanes / 4 / 2): 2^23 points 5.83 / 2.31 / 2.34 / 3.94, 2^21 points 0.559 / 0.548 /
+// 0.505 / 0.512, 2048^2 mesh 0.301 / 0.350 / 0.301 / 0.295, 129^3 mesh 0.659 / 0.596 / 0.585 /
+// 0.598: eight lanes idle on rows of six entries, two ask twice as often.  The next tile's edge
+// ends are read at the top of a tile and its row pointers just before the walk, which hides two
+// of a tile's three dependent reads: 2^21 points 0.503 -> 0.487, 2048^2 mesh 0.301 -> 0.281.
 constexpr int kPkWarps = 8;
 constexpr int kPkA = 192;  // entries of the tile's row-a slice staged per warp
 constexpr int kPkB = 576;  // entries of the tile's 32 rows b staged per warp
 constexpr int kPkRegion = kPkA + kPkB;
+constexpr int kPkLanes = 4;  // lanes that copy one row b together
 constexpr size_t kPkSmem = (size_t)kPkWarps * kPkRegion * sizeof(uint2);
 
 // L2 eviction priority (createpolicy, sm_80 and later): the row pointers, read at random once
@@ -859,18 +870,26 @@ k_score_packed(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restr
     constexpr int32_t kEnd = 0x7fffffff;  // the end marker's column
     const uint64_t keep = l2_policy_evict_last();
     const int64_t step_e = (int64_t)gridDim.x * kPkWarps * 32;
-    for (int64_t e0 = ((int64_t)blockIdx.x * kPkWarps + wib) * 32; e0 < m; e0 += step_e) {
+    int32_t a = 0, b = 0;
+    int64_t ra = 0, re = 0, rb = 0, rbe = 0;
+    const int64_t first = ((int64_t)blockIdx.x * kPkWarps + wib) * 32;
+    if (first + lane < m) {
+        a = eu[first + lane];
+        b = ev[first + lane];
+        ra = ld_l2hint(rowptr + a, keep);
+        re = ld_l2hint(rowptr + a + 1, keep);
+        rb = ld_l2hint(rowptr + b, keep);
+        rbe = ld_l2hint(rowptr + b + 1, keep);
+    }
+    for (int64_t e0 = first; e0 < m; e0 += step_e) {
         const int64_t e = e0 + lane;
         const bool act = e < m;
-        int32_t a = 0, b = 0;
-        int64_t ra = 0, da = 0, rb = 0, db = 0;
-        if (act) {
-            a = eu[e];
-            b = ev[e];
-            ra = ld_l2hint(rowptr + a, keep);
-            da = ld_l2hint(rowptr + a + 1, keep) - ra;
-            rb = ld_l2hint(rowptr + b, keep);
-            db = ld_l2hint(rowptr + b + 1, keep) - rb;
+        const int64_t da = re - ra, db = rbe - rb;
+        int32_t a1 = 0, b1 = 0;
+        const bool act1 = e + step_e < m;
+        if (act1) {
+            a1 = eu[e + step_e];
+            b1 = ev[e + step_e];
         }
         const bool hub = act && (da > kLongRow || db > kLongRow);
         // packed positions: row x's pairs start at rowptr[x] + x, its end marker follows them
@@ -884,9 +903,9 @@ k_score_packed(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restr
         if (a_staged)
             for (int64_t q = ac0 + lane; q < ac1; q += 32)
                 cp_async_16(sa + 2 * (q - ac0), pk16 + q);
-        // this lane's row b: its pairs, chunks [pb0 / 2, (pb0 + db + 1) / 2), placed after the
-        // other lanes'; its end marker is written in shared memory (a random row fetches no
-        // more than its pairs), in one more chunk of room when the pairs fill their last one
+        // the row b of this lane's edge: its pairs, chunks [pb0 / 2, (pb0 + db + 1) / 2), placed
+        // after the other lanes'; its end marker is written in shared memory (a random row fetches
+        // no more than its pairs), in one more chunk of room when the pairs fill their last one
         const int64_t bc0 = pb0 >> 1;
         const int nch = (act && !hub) ? (int)(((pb0 + db + 1) >> 1) - bc0) : 0;
         const int nroom = nch + ((act && !hub && (pb0 & 1) + db == 2 * nch) ? 1 : 0);
@@ -898,13 +917,31 @@ k_score_packed(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restr
         }
         choff -= nroom;
         const bool b_staged = 2 * (choff + nroom) <= kPkB;
-        const int maxch = __reduce_max_sync(0xffffffffu, b_staged ? nch : 0);
-        for (int k = 0; k < maxch; ++k)
-            if (b_staged && k < nch) cp_async_16(sb + 2 * (choff + k), pk16 + bc0 + k);
+        const uint32_t bc32 = (uint32_t)bc0;  // below 2^32: fewer than 2^33 pairs
+        const int nst = b_staged ? nch : 0;
+#pragma unroll
+        for (int g = 0; g < kPkLanes; ++g) {
+            const int r = g * (32 / kPkLanes) + lane / kPkLanes;
+            const int64_t c0 = __shfl_sync(0xffffffffu, bc32, r);
+            const int cn = __shfl_sync(0xffffffffu, nst, r);
+            const int co = __shfl_sync(0xffffffffu, choff, r);
+            for (int k = lane % kPkLanes; k < cn; k += kPkLanes)
+                cp_async_16(sb + 2 * (co + k), pk16 + c0 + k);
+        }
         cp_async_wait_all();
         if (b_staged && act && !hub)
             sb[2 * choff + (pb0 & 1) + db] = make_uint2((uint32_t)kEnd, 0u);
         __syncwarp();
+        // the next tile's row pointers, in flight during the walk
+        ra = re = rb = rbe = 0;
+        if (act1) {
+            ra = ld_l2hint(rowptr + a1, keep);
+            re = ld_l2hint(rowptr + a1 + 1, keep);
+            rb = ld_l2hint(rowptr + b1, keep);
+            rbe = ld_l2hint(rowptr + b1 + 1, keep);
+        }
+        a = a1;
+        b = b1;
         if (act && !hub) {
             // both rows end in their marker: the walk advances without bounds
             const uint2* A = a_staged ? sa + (pa0 - 2 * ac0) : pk + pa0;
@@ -915,9 +952,9 @@ k_score_packed(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restr
                 const int32_t ca = (int32_t)xa.x, cb = (int32_t)xb.x;
                 if (ca == kEnd && cb == kEnd) break;
                 const bool ta = ca <= cb, tb = cb <= ca;
-                const float pa = ta ? __uint_as_float(xa.y) : 0.f;
-                const float pb = tb ? __uint_as_float(xb.y) : 0.f;
-                s = p_add(s, p_absdiff(pa, pb));
+                const float fa = ta ? __uint_as_float(xa.y) : 0.f;
+                const float fb = tb ? __uint_as_float(xb.y) : 0.f;
+                s = p_add(s, p_absdiff(fa, fb));
                 if (ta) xa = *++A;
                 if (tb) xb = *++B;
             }
