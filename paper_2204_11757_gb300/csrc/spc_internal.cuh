@@ -111,7 +111,7 @@ struct Work {
     Buf sort_hist, scan_tmp;                                    // sort / scan temporaries
     Buf stage_rowptr, stage_col, stage_w, stage_lift, stage_gptr;  // host staging
     Buf pool_key, pool_val, pool_key2, pool_val2, pool_cnt, pool_off;  // feature pooling
-    Buf pool_nch, pool_choff, pool_owner, pool_part;
+    Buf pool_nch, pool_choff, pool_owner, pool_part, pool_stats;
     // the same temporaries for work running on the second stream (SideBranch)
     Buf sort_hist_side, scan_tmp_side, long_segs_side;
     Buf seg_base_side, seg_len_side, seg_idx_side, seg_terms_side;

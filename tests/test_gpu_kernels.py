@@ -35,3 +35,30 @@ def test_binary32_scores_packed_and_in_place(ctx, n, p):
     for schedule in (1, 3):
         ctx.coarsen(csr, g.n, levels=1, schedule=schedule)
         assert np.array_equal(_bits(ctx.level(0).score.cpu().numpy()), _bits(ref))
+
+
+# super-nodes of up to 256 members are gathered in one pass, larger ones (or too much ranking)
+# go through the sort and the tree; features around the 16-byte accesses and the lanes of a row
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("F", [1, 2, 4, 31, 64, 132])
+@pytest.mark.parametrize("sizes", [[1], [256], [257, 1, 0, 3], [0, 5, 256, 255, 2, 1, 33, 0] * 3,
+                                   [7, 9] * 200, [65, 64, 63] * 30, [256] * 40])
+def test_pooling_routes(ctx, dtype, F, sizes):
+    rng = np.random.default_rng(F)
+    lift = rng.permutation(np.repeat(np.arange(len(sizes)), sizes)).astype(np.int32)
+    n, n_c = lift.shape[0], len(sizes)
+    x = (rng.standard_normal((n, F)) * 10.0 ** rng.integers(-3, 4, size=(n, 1))).astype(dtype)
+    g = rng.standard_normal((n_c, F)).astype(dtype)
+    lt = torch.from_numpy(lift).cuda()
+
+    def put(a, shift):  # a tensor whose data starts `shift` elements into its storage
+        t = torch.zeros(a.size + shift, dtype=torch.from_numpy(a).dtype, device="cuda")
+        t[shift:] = torch.from_numpy(a.ravel()).cuda()
+        return t[shift:].view(a.shape)
+
+    ref, ref_g = O.pool_features(lift, n_c, x), O.pool_backward(lift, n_c, g)
+    for shift in (0, 1):
+        xc = ctx.pool_features(lt, n_c, put(x, shift)).cpu().numpy()
+        assert np.array_equal(_bits(xc), _bits(ref))
+        gx = ctx.pool_features_backward(lt, n_c, put(g, shift)).cpu().numpy()
+        assert np.array_equal(_bits(gx), _bits(ref_g))
