@@ -106,6 +106,46 @@ constexpr int kBlockSortThreads = 512;
 static_assert((kBlockSortThreads / 32) * kWarpBucket <= kBlockBucket,
               "the warps' stages share the CTA's");
 
+// Statistics of a block's scanned values, K sides of (sum of squares, maximum), added into
+// stats[2 k] and stats[2 k + 1]: by shuffles inside the warps, then one thread per statistic over
+// the warps' results.  Every thread of the block (up to 1024) calls it once.  (Shared-memory
+// atomics of every thread on one 64-bit word made the one-CTA scan of 16,384 buckets 75 us long,
+// 20 without them.)
+template <int K>
+__device__ __forceinline__ void block_stats(const unsigned long long* sq,
+                                            const unsigned long long* mx,
+                                            unsigned long long* stats) {
+    __shared__ unsigned long long sh[2 * K][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        unsigned long long s = sq[k], m = mx[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
+            m = t > m ? t : m;
+        }
+        if (lane == 0) {
+            sh[2 * k][warp] = s;
+            sh[2 * k + 1][warp] = m;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * K) {
+        unsigned long long v = 0ull;
+        const bool is_max = threadIdx.x & 1;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            const unsigned long long t = sh[threadIdx.x][w];
+            v = is_max ? (t > v ? t : v) : v + t;
+        }
+        if (v) {
+            if (is_max) atomicMax(stats + threadIdx.x, v);
+            else atomicAdd(stats + threadIdx.x, v);
+        }
+    }
+}
+
 // scan storer of the two packed bucket sizes (spc_scan.cuh PairLd: inter, intra): both
 // exclusive prefixes and totals, and per side the ranking statistics -- sum of squared sizes in
 // stats[0] / stats[2], largest size in stats[1] / stats[3] -- and the list of buckets longer
@@ -136,18 +176,7 @@ struct BucketOffSt {
         }
     }
     __device__ void finish(Local& L) const {
-        __shared__ unsigned long long sh[4];
-        if (threadIdx.x < 4) sh[threadIdx.x] = 0ull;
-        __syncthreads();
-        for (int side = 0; side < 2; ++side) {
-            if (L.sq[side]) atomicAdd(&sh[2 * side], L.sq[side]);
-            if (L.mx[side]) atomicMax(&sh[2 * side + 1], L.mx[side]);
-        }
-        __syncthreads();
-        if (threadIdx.x < 4 && sh[threadIdx.x]) {
-            if (threadIdx.x & 1) atomicMax(stats + threadIdx.x, sh[threadIdx.x]);
-            else atomicAdd(stats + threadIdx.x, sh[threadIdx.x]);
-        }
+        block_stats<2>(L.sq, L.mx, stats);
     }
     __device__ void total(unsigned long long tot) const {
         off_c[n] = (int32_t)(tot >> 31);
@@ -180,14 +209,7 @@ struct RowPtrSt {
         L.mx = low > L.mx ? low : L.mx;
     }
     __device__ void finish(Local& L) const {
-        __shared__ unsigned long long sh[2];
-        if (threadIdx.x < 2) sh[threadIdx.x] = 0ull;
-        __syncthreads();
-        if (L.sq) atomicAdd(&sh[0], L.sq);
-        if (L.mx) atomicMax(&sh[1], L.mx);
-        __syncthreads();
-        if (threadIdx.x == 0 && sh[0]) atomicAdd(stats, sh[0]);
-        if (threadIdx.x == 1 && sh[1]) atomicMax(stats + 1, sh[1]);
+        block_stats<1>(&L.sq, &L.mx, stats);
     }
     __device__ void total(unsigned long long tot) const {
         const int32_t u = (int32_t)(tot >> 31), l = (int32_t)(tot & 0x7fffffffull);

@@ -158,10 +158,12 @@ constexpr uint32_t kFlagInc = 2u << 30;
 constexpr uint32_t kValMask = (1u << 30) - 1u;
 constexpr int kMaxPasses = 8;
 
+// The last block to finish (ticket) also turns every pass's bins into its 256 output bases, a
+// warp per pass (a launch of its own, one thread walking 256 bins per pass, took 6-12 us).
 template <class K>
 __global__ void __launch_bounds__(RT) k_os_hist(const K* __restrict__ keys, int64_t count,
-                                                int npass, int end_bit,
-                                                uint32_t* __restrict__ hist) {
+                                                int npass, int end_bit, uint32_t* hist,
+                                                uint32_t* __restrict__ base, uint32_t* ticket) {
     spc::pdl_wait();
     constexpr int kCopies = 2;  // two copies (warps 0-3, 4-7) halve the contention on a bin
     __shared__ uint32_t h[kCopies][kMaxPasses][RADIX];
@@ -183,26 +185,34 @@ __global__ void __launch_bounds__(RT) k_os_hist(const K* __restrict__ keys, int6
         for (int w = 0; w < kCopies; ++w) s += h[w][i / RADIX][i % RADIX];
         if (s) atomicAdd(hist + i, s);
     }
-}
-
-// exclusive scan of every pass's 256 bins (one block, one thread per bin)
-__global__ void k_os_bases(int npass, const uint32_t* __restrict__ hist, uint32_t* __restrict__ base) {
-    spc::pdl_wait();
-    __shared__ uint32_t sh[RADIX];
-    for (int p = 0; p < npass; ++p) {
-        sh[threadIdx.x] = hist[p * RADIX + threadIdx.x];
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t run = 0;
-            for (int d = 0; d < RADIX; ++d) {
-                const uint32_t c = sh[d];
-                sh[d] = run;
-                run += c;
-            }
-        }
-        __syncthreads();
-        base[p * RADIX + threadIdx.x] = sh[threadIdx.x];
-        __syncthreads();
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+    static_assert(RT / 32 >= kMaxPasses, "a warp per pass");
+    if (p >= npass) return;
+    constexpr int kPer = RADIX / 32;
+    uint32_t c[kPer], run = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        c[j] = __ldcg(hist + p * RADIX + lane * kPer + j);
+        run += c[j];
+    }
+    uint32_t incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    uint32_t at = incl - run;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        base[p * RADIX + lane * kPer + j] = at;
+        at += c[j];
     }
 }
 
@@ -346,7 +356,7 @@ spc_status radix_sort_impl(spc_context* ctx, K* keys, uint32_t* vals, K* keys_al
     const int64_t tiles = (count + RTILE - 1) / RTILE;
     const int npass = (end_bit + 7) / 8;
     if (npass > kMaxPasses || count >= (int64_t)kValMask) return SPC_ERR_TOO_LARGE;
-    // hist [npass][256] | base [npass][256] | tile counters [npass] | status [npass][tiles][256]
+    // hist [npass][256] | base [npass][256] | tile counters [npass], [16] a ticket | status [npass][tiles][256]
     const size_t words = (size_t)npass * RADIX * 2 + 32 + (size_t)npass * tiles * RADIX;
     Buf& hbuf = on_side(ctx) ? ctx->work.sort_hist_side : ctx->work.sort_hist;
     SPC_TRY(ensure(ctx, hbuf, words * 4));
@@ -365,8 +375,7 @@ spc_status radix_sort_impl(spc_context* ctx, K* keys, uint32_t* vals, K* keys_al
     }
     note_bytes(ctx, (double)count * sizeof(K));  // every key read once
     SPC_LAUNCH(ctx, k_os_hist<K>, grid_for(count, RT, ctx->num_sms * 4), RT, 0, keys, count,
-               npass, end_bit, hist);
-    SPC_LAUNCH(ctx, k_os_bases, 1, RADIX, 0, npass, hist, base);
+               npass, end_bit, hist, base, tctr + 16);
     K* ka = keys;
     uint32_t* va = vals;
     K* kb = keys_alt;
