@@ -846,7 +846,14 @@ static spc_status drive(spc_context* ctx, const GraphView& v, const Schedule& S,
         if (R.exec) {
             bool mismatch = false;
             const spc_status st = replay_graph(ctx, &mismatch);
-            if (st < 0) return st;
+            if (st < 0) {
+                // a replay that stopped in between leaves counters that the graph takes as zero
+                drop_graph(R);
+                R.recorded = false;
+                ctx->work.sel_dirty = true;
+                ctx->work.b_dirty = true;
+                return st;
+            }
             if (!mismatch) {
                 ctx->replayed_last = 1;
                 const int L = (int)R.metas.size();

@@ -98,6 +98,8 @@ struct Work {
     Buf parent, best_k[2], best_e[2], wl_e[2], wl_u[2], wl_v[2], msf;   // S5 MSF
     Buf counters, key_hist;                                     // small device ints
     Buf sel_key, sel_val, sel_key2, sel_val2, node_graph, seg_start, k_graph;  // selection
+    Buf sel_blk;                                                // roots per CTA
+    bool sel_dirty = true;       // the selection's counters and score histogram may not be zero
     Buf g_need, g_tau, g_lo, g_short;                           // per-graph prefixes (batch)
     Buf parent2, flag, ids;                                     // S6
     Buf c_key, c_val, c_key2, c_val2, c_flag, c_pos, c_head, cU, cV;    // S7
@@ -358,6 +360,35 @@ cudaError_t launch_pdl(cudaStream_t stream, dim3 grid, dim3 block, size_t smem,
         spc::before_launch((ctx), #kernel);                                              \
         cudaError_t le_ = spc::launch_pdl((ctx)->stream, dim3(grid), dim3(block), (smem), \
                                           kernel, __VA_ARGS__);                          \
+        if (le_ == cudaSuccess) le_ = cudaGetLastError();                                \
+        spc::after_launch((ctx), #kernel);                                               \
+        if (le_ != cudaSuccess) {                                                        \
+            spc::set_last_cuda_error(le_, #kernel, __FILE__, __LINE__);                  \
+            return SPC_ERR_CUDA;                                                         \
+        }                                                                                \
+    } while (0)
+
+// A cooperative launch (every CTA resident at once, so the CTAs may wait on one another in bounded
+// grid barriers); it starts when its predecessor has finished.
+template <typename Param, typename Arg>
+cudaError_t launch_coop(cudaStream_t stream, dim3 grid, dim3 block, void (*kernel)(Param),
+                        const Arg& arg) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, arg);
+}
+
+#define SPC_LAUNCH_COOP(ctx, kernel, grid, block, arg)                                    \
+    do {                                                                                 \
+        spc::before_launch((ctx), #kernel);                                              \
+        cudaError_t le_ = spc::launch_coop((ctx)->stream, dim3(grid), dim3(block), kernel, arg); \
         if (le_ == cudaSuccess) le_ = cudaGetLastError();                                \
         spc::after_launch((ctx), #kernel);                                               \
         if (le_ != cudaSuccess) {                                                        \

@@ -15,11 +15,11 @@
 //      histogram to hold about 1.5 (n - n_c) edges (on very large graphs the slab's edges are
 //      first compacted into the work list); if that prefix's forest has fewer than n - n_c
 //      edges, the rounds resume on the next slab, the forest found so far kept.
-//   2. The forest edges are compacted in eid order.  For one graph an exact radix select on
+//   2. For one graph the forest edges are listed as they are picked, an exact radix select on
 //      11-bit digits of (score, eid) finds the (n - n_c)-th lightest and every forest edge up to
-//      it is united in a second union-find; for batches the forest edges are radix-sorted by
-//      score and then by graph (stable, so ties stay in eid order) and the first
-//      n_b - target_b of each graph are united.
+//      it is united in a second union-find; for batches the forest edges are compacted in eid
+//      order, radix-sorted by score and then by graph (stable, so ties stay in eid order) and the
+//      first n_b - target_b of each graph are united.
 //   3. Relabel: root = smallest member; flag roots, exclusive scan, id = scan[root] (Definition
 //      1's super-nodes, numbered by smallest member).
 // Every retry loop is bounded (spin_limit: kSpinLimit unless the context lowered it); giving up
@@ -45,23 +45,71 @@ __device__ __forceinline__ int32_t uf_find(int32_t* parent, int32_t x, uint32_t*
         int32_t p = ld_parent(parent, x);
         if (p == x) return x;
         int32_t gp = ld_parent(parent, p);
-        if (gp != p) parent[x] = gp;
+        if (gp == p) return p;
+        parent[x] = gp;
         x = gp;
     }
     atomicOr(status, DEV_TIMEOUT);
     return x;
 }
 
+// uf_find of several nodes at once (those whose bit of `live` is set): every step's loads are in
+// flight together.  kStatic: no set is united while the walks run (a phase or kernel of its
+// own), so a parent held by L1 is at worst an older ancestor and the walks read through L1
+// (Boruvka's first phase over a further slab, 1 M nodes: 149 -> 48 us).
+template <int N, bool kStatic>
+__device__ __forceinline__ void uf_find_n(int32_t* parent, int32_t (&x)[N], unsigned live,
+                                          uint32_t* status) {
+    if (!live) return;
+    const uint32_t lim = spin_limit(status);
+    for (uint32_t it = 0; it < lim; ++it) {
+        int32_t p[N], gp[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            p[i] = x[i];
+            if (live >> i & 1u) p[i] = kStatic ? parent[x[i]] : ld_parent(parent, x[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (p[i] == x[i]) live &= ~(1u << i);
+        if (!live) return;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            gp[i] = p[i];
+            if (live >> i & 1u) gp[i] = kStatic ? parent[p[i]] : ld_parent(parent, p[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            if (!(live >> i & 1u)) continue;
+            if (gp[i] == p[i]) live &= ~(1u << i);
+            else parent[x[i]] = gp[i];
+            x[i] = gp[i];
+        }
+        if (!live) return;
+    }
+    atomicOr(status, DEV_TIMEOUT);
+}
+
 // atomicMin of v into a[idx] by every active lane of the warp (all 32 lanes call it).  When
 // neighbouring lanes target the same slot -- the edges of a hub component -- the lanes of each
 // slot first take their minimum together and one lane issues the atomic.
+// `hot` (may be null): one slot, hot->idx, whose minimum the block keeps in shared memory.
+struct HotMin {
+    int32_t idx;
+    unsigned long long v;
+};
+
 __device__ __forceinline__ void warp_atomic_min_u64(unsigned long long* a, int32_t idx,
-                                                    unsigned long long v, bool act) {
+                                                    unsigned long long v, bool act,
+                                                    HotMin* hot = nullptr) {
     const int lane = threadIdx.x & 31;
     const int32_t key = act ? idx : -1;
     const int32_t prev = __shfl_up_sync(0xffffffffu, key, 1);
     if (!__any_sync(0xffffffffu, act && lane > 0 && prev == key)) {
-        if (act) atomicMin(a + idx, v);
+        if (act) {
+            if (hot && idx == hot->idx) atomicMin(&hot->v, v);
+            else atomicMin(a + idx, v);
+        }
         return;
     }
     const unsigned peers = __match_any_sync(0xffffffffu, key);
@@ -69,7 +117,11 @@ __device__ __forceinline__ void warp_atomic_min_u64(unsigned long long* a, int32
     const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
     const unsigned hmin = __reduce_min_sync(peers, hi);
     const unsigned lmin = __reduce_min_sync(peers, hi == hmin ? lo : 0xffffffffu);
-    if (lane == __ffs(peers) - 1) atomicMin(a + idx, ((unsigned long long)hmin << 32) | lmin);
+    if (lane == __ffs(peers) - 1) {
+        const unsigned long long w = ((unsigned long long)hmin << 32) | lmin;
+        if (hot && idx == hot->idx) atomicMin(&hot->v, w);
+        else atomicMin(a + idx, w);
+    }
 }
 
 __device__ __forceinline__ void warp_atomic_min_i32(int32_t* a, int32_t idx, int32_t v,
@@ -92,13 +144,13 @@ __device__ __forceinline__ void warp_atomic_min_i32(int32_t* a, int32_t idx, int
 __device__ __forceinline__ bool uf_unite(int32_t* parent, int32_t a, int32_t b,
                                          uint32_t* status) {
     const uint32_t lim = spin_limit(status);
+    int32_t x[2] = {a, b};
     for (uint32_t it = 0; it < lim; ++it) {
-        a = uf_find(parent, a, status);
-        b = uf_find(parent, b, status);
-        if (a == b) return false;
-        if (a > b) { int32_t t = a; a = b; b = t; }
-        int32_t old = atomicCAS(parent + b, b, a);
-        if (old == b) return true;
+        uf_find_n<2, false>(parent, x, 3u, status);
+        if (x[0] == x[1]) return false;
+        if (x[0] > x[1]) { int32_t t = x[0]; x[0] = x[1]; x[1] = t; }
+        int32_t old = atomicCAS(parent + x[1], x[1], x[0]);
+        if (old == x[1]) return true;
     }
     atomicOr(status, DEV_TIMEOUT);
     return false;
@@ -192,107 +244,21 @@ __global__ void k_bv_reinit(int64_t n, unsigned long long* __restrict__ bk0,
     if (t0 < 2) counts[t0] = 0;
 }
 
-// the slab just done becomes the lower bound of the next
-__global__ void k_bump_slab(const uint32_t* __restrict__ tau_top, uint32_t* __restrict__ tau_lo) {
-    spc::pdl_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *tau_lo = *tau_top;
-}
-
-// The edges of the current score slab as the first Boruvka work list: every edge whose key
-// lies in the slab is written as (e, eu[e], ev[e]).  A streaming pass: each thread takes
-// kSlItems consecutive edges (their keys in 16-byte loads; key 16-byte aligned), the ends are
-// read only for the slab's edges, and one global atomic per kThreads * kSlItems edges places
-// a block's survivors, so the list is in edge order within each block's chunk (the next
-// rounds' parent and flag accesses stay close together); the forest does not depend on the
-// order (every component's lightest edge is unique).
-constexpr int kSlItems = 16;
+constexpr int kSlItems = 16;  // consecutive edges a thread takes when it lists a slab's edges
 constexpr int64_t kSlabListMin = int64_t{1} << 25;
-
-template <class KT>
-__global__ void __launch_bounds__(kThreads)
-k_slab_list(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-            const KT* __restrict__ key, int tau_shift, const uint32_t* __restrict__ tau_top,
-            const uint32_t* __restrict__ tau_lo, int32_t* __restrict__ wo_e,
-            int32_t* __restrict__ wo_u, int32_t* __restrict__ wo_v,
-            int32_t* __restrict__ out_count) {
-    static_assert(kSlItems * sizeof(KT) % 16 == 0, "whole 16-byte loads");
-    constexpr int kVec = (int)(kSlItems * sizeof(KT) / 16);
-    spc::pdl_wait();
-    __shared__ int32_t sh_wsum[kThreads / 32];
-    __shared__ int32_t sh_base;
-    const uint32_t top = tau_top ? *tau_top : 0xffffffffu;
-    const uint32_t lo = tau_lo ? *tau_lo : kNoSlab;
-    const int64_t per = (int64_t)kThreads * kSlItems;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t base = (int64_t)blockIdx.x * per; base < m; base += (int64_t)gridDim.x * per) {
-        const int64_t i0 = base + (int64_t)threadIdx.x * kSlItems;
-        KT k[kSlItems];
-        if (i0 + kSlItems <= m) {
-            const uint4* p = reinterpret_cast<const uint4*>(key + i0);
-            uint4 q[kVec];
-#pragma unroll
-            for (int j = 0; j < kVec; ++j) q[j] = p[j];
-            memcpy(k, q, sizeof(k));
-        } else {
-#pragma unroll
-            for (int it = 0; it < kSlItems; ++it) k[it] = i0 + it < m ? key[i0 + it] : KT(0);
-        }
-        unsigned keep = 0;  // bit it: edge i0 + it lies in the slab
-#pragma unroll
-        for (int it = 0; it < kSlItems; ++it) {
-            const uint32_t bin = (uint32_t)(k[it] >> tau_shift);
-            const bool in = i0 + it < m && bin <= top && (lo == kNoSlab || bin > lo);
-            keep |= in ? 1u << it : 0u;
-        }
-        const int32_t nkeep = __popc(keep);
-        int32_t incl = nkeep;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) sh_wsum[warp] = incl;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int32_t tot = 0;
-            for (int w = 0; w < kThreads / 32; ++w) {
-                const int32_t t = sh_wsum[w];
-                sh_wsum[w] = tot;
-                tot += t;
-            }
-            sh_base = tot ? atomicAdd(out_count, tot) : 0;
-        }
-        __syncthreads();
-        int32_t slot = sh_base + sh_wsum[warp] + incl - nkeep;
-        while (keep) {
-            const int it = __ffs(keep) - 1;
-            keep &= keep - 1;
-            const int64_t i = i0 + it;
-            wo_e[slot] = (int32_t)i;
-            wo_u[slot] = eu[i];
-            wo_v[slot] = ev[i];
-            ++slot;
-        }
-        __syncthreads();
-    }
-}
 
 template <class KT>
 __global__ void __launch_bounds__(kThreads)
 k_bv_minkey(int round0, int direct, int64_t m, const int32_t* __restrict__ in_count,
             const int32_t* __restrict__ wi_e, const int32_t* __restrict__ wi_u,
             const int32_t* __restrict__ wi_v, const int32_t* __restrict__ eu,
-            const int32_t* __restrict__ ev, const KT* __restrict__ key, int tau_shift,
-            const uint32_t* __restrict__ tau_top, const uint32_t* __restrict__ tau_lo,
-            GraphSlab<KT> gs, int32_t* parent, unsigned long long* best_k, int32_t* wo_e,
-            int32_t* wo_u, int32_t* wo_v, int32_t* out_count, uint32_t* status) {
+            const int32_t* __restrict__ ev, const KT* __restrict__ key, GraphSlab<KT> gs,
+            int32_t* parent, unsigned long long* best_k, int32_t* wo_e, int32_t* wo_u,
+            int32_t* wo_v, int32_t* out_count, uint32_t* status) {
     spc::pdl_wait();
     __shared__ int32_t sh_wsum[kThreads / 32];
     __shared__ int32_t sh_base;
     const int64_t cnt = round0 ? m : (int64_t)*in_count;
-    const uint32_t top = tau_top ? *tau_top : 0xffffffffu;
-    // a first round over the next slab of scores skips the slabs already done
-    const uint32_t lo = tau_lo ? *tau_lo : kNoSlab;
     const int64_t per = (int64_t)blockDim.x * kMkItems;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t base = (int64_t)blockIdx.x * per; base < cnt; base += (int64_t)gridDim.x * per) {
@@ -312,19 +278,24 @@ k_bv_minkey(int round0, int direct, int64_t m, const int32_t* __restrict__ in_co
 #pragma unroll
         for (int it = 0; it < kMkItems; ++it) {
             k[it] = in[it] ? key[e[it]] : KT(0);
-            if (round0 && in[it]) {
-                const uint32_t bin = (uint32_t)(k[it] >> tau_shift);
-                if (bin > top || (lo != kNoSlab && bin <= lo)) in[it] = false;
-                if (gs.node_graph && gs.outside(u[it], k[it])) in[it] = false;
-            }
+            if (round0 && in[it] && gs.node_graph && gs.outside(u[it], k[it])) in[it] = false;
         }
+        // direct: the selection's first round, every node still its own component
+        int32_t rt[2 * kMkItems];
+        unsigned live = 0;
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            rt[2 * it] = in[it] ? u[it] : 0;
+            rt[2 * it + 1] = in[it] ? v[it] : 0;
+            if (in[it]) live |= 3u << (2 * it);
+        }
+        if (!direct) uf_find_n<2 * kMkItems, true>(parent, rt, live, status);
         int32_t ru[kMkItems], rv[kMkItems];
         int32_t nkeep = 0;
 #pragma unroll
         for (int it = 0; it < kMkItems; ++it) {
-            // direct: the selection's first round, every node still its own component
-            ru[it] = in[it] ? (direct ? u[it] : uf_find(parent, u[it], status)) : 0;
-            rv[it] = in[it] ? (direct ? v[it] : uf_find(parent, v[it], status)) : 0;
+            ru[it] = rt[2 * it];
+            rv[it] = rt[2 * it + 1];
             in[it] = in[it] && ru[it] != rv[it];
             const unsigned long long pk = MinKey<KT>::pack(k[it], e[it]);
             warp_atomic_min_u64(best_k, ru[it], pk, in[it]);
@@ -382,14 +353,10 @@ __global__ void __launch_bounds__(kFinishThreads, 1)
 k_bv_finish(int round0, int par0, int64_t m, int32_t* count_in, int32_t* li_e, int32_t* li_u,
             int32_t* li_v, int32_t* lo_e, int32_t* lo_u, int32_t* lo_v,
             const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-            const KT* __restrict__ key, int tau_shift, const uint32_t* __restrict__ tau_top,
-            const uint32_t* __restrict__ tau_lo, GraphSlab<KT> gs, int32_t* parent,
-            unsigned long long* bk0, unsigned long long* bk1, int32_t* be0, int32_t* be1,
+            const KT* __restrict__ key, GraphSlab<KT> gs, int32_t* parent, unsigned long long* bk0, unsigned long long* bk1, int32_t* be0, int32_t* be1,
             uint8_t* msf, uint32_t* status) {
     spc::pdl_wait();
     __shared__ int32_t sh_cnt[2];
-    const uint32_t top = tau_top ? *tau_top : 0xffffffffu;
-    const uint32_t slab_lo = tau_lo ? *tau_lo : kNoSlab;
     int64_t cnt = round0 ? m : (int64_t)*count_in;
     int par = par0;
     int32_t *ie = li_e, *iu = li_u, *iv = li_v, *oe = lo_e, *ou = lo_u, *ov = lo_v;
@@ -410,11 +377,7 @@ k_bv_finish(int round0, int par0, int64_t m, int32_t* count_in, int32_t* li_e, i
             if (round0 && r == 0) { e = (int32_t)i; u = eu[i]; v = ev[i]; }
             else { e = ie[i]; u = iu[i]; v = iv[i]; }
             const KT k = key[e];
-            if (round0 && r == 0) {
-                const uint32_t bin = (uint32_t)(k >> tau_shift);
-                if (bin > top || (slab_lo != kNoSlab && bin <= slab_lo)) continue;
-                if (gs.node_graph && gs.outside(u, k)) continue;
-            }
+            if (round0 && r == 0 && gs.node_graph && gs.outside(u, k)) continue;
             const int32_t ru = uf_find(parent, u, status), rv = uf_find(parent, v, status);
             if (ru == rv) continue;
             const unsigned long long pk = MinKey<KT>::pack(k, e);
@@ -516,60 +479,6 @@ __device__ __forceinline__ unsigned long long block_incl_scan(unsigned long long
     const unsigned long long r = x + (w ? ws[w - 1] : 0ull);
     __syncthreads();
     return r;
-}
-
-// smallest bin whose cumulative count reaches `need` (all bins when need >= m); the histogram
-// stays for a later attempt of the same selection.  Each thread holds 32 consecutive bins in registers; the
-// block scan of the thread totals is two rounds of warp shuffles.
-__global__ void __launch_bounds__(1024)
-k_pick_tau(uint32_t* __restrict__ hist, int64_t need, uint32_t* __restrict__ tau_top) {
-    spc::pdl_wait();
-    constexpr int kPer = 32768 / 1024;
-    __shared__ unsigned long long wsum[32];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    uint4* h4 = reinterpret_cast<uint4*>(hist) + (int64_t)t * (kPer / 4);
-    uint32_t v[kPer];
-    unsigned long long loc = 0;
-#pragma unroll
-    for (int j = 0; j < kPer / 4; ++j) {
-        const uint4 q = h4[j];
-        v[4 * j] = q.x;
-        v[4 * j + 1] = q.y;
-        v[4 * j + 2] = q.z;
-        v[4 * j + 3] = q.w;
-        loc += (unsigned long long)q.x + q.y + q.z + q.w;
-    }
-    unsigned long long x = loc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[w] = x;
-    if (t == 0) *tau_top = 32767u;
-    __syncthreads();
-    if (w == 0) {
-        unsigned long long y = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long z = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) y += z;
-        }
-        wsum[lane] = y;
-    }
-    __syncthreads();
-    const unsigned long long incl = x + (w ? wsum[w - 1] : 0ull);
-    unsigned long long run = incl - loc;
-    if (run < (unsigned long long)need && incl >= (unsigned long long)need) {
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            run += v[j];
-            if (run >= (unsigned long long)need) {
-                *tau_top = (uint32_t)(t * kPer + j);
-                break;
-            }
-        }
-    }
 }
 
 // Boruvka phase B (64-bit scores only): among the edges whose score equals the component
@@ -866,20 +775,14 @@ __global__ void k_graph_segments(int64_t B, const int64_t* __restrict__ graph_pt
 __global__ void __launch_bounds__(kThreads)
 k_select_unite(const int32_t* __restrict__ count, const uint32_t* __restrict__ eids,
                const uint32_t* __restrict__ gkey, const int32_t* __restrict__ seg_start,
-               const int32_t* __restrict__ k_graph, int64_t k_single,
-               const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, int32_t* parent,
+               const int32_t* __restrict__ k_graph, const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, int32_t* parent,
                uint8_t* merged, uint32_t* status) {
     spc::pdl_wait();
     const int64_t cnt = *count;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
          i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t rank = i, k = k_single;
-        if (gkey) {
-            const uint32_t b = gkey[i];
-            rank = i - seg_start[b];
-            k = k_graph[b];
-        }
-        if (rank < k) {
+        const uint32_t b = gkey[i];
+        if (i - seg_start[b] < k_graph[b]) {
             const int32_t e = (int32_t)eids[i];
             uf_unite(parent, eu[e], ev[e], status);
             if (merged) merged[e] = 1;
@@ -917,230 +820,15 @@ __device__ __forceinline__ uint32_t sel_digit(KT hi, uint32_t lo, int r) {
     return (lo >> lowb) & ((1u << (top - lowb)) - 1u);
 }
 
-struct SelState {
-    unsigned long long need;     // rank (1-based) still to find among the matching items
-    uint32_t dig[16];
-    uint32_t ticket[16];
-};
-
-// One select round: histogram of digit r over the items whose digits 0..r-1 are the ones
-// picked so far; the last block to finish picks digit r.  n_dev, when given, holds the item
-// count (a candidate list compacted on the device).
-template <class KT>
+// root flags (a root is its set's smallest member and its own parent)
 __global__ void __launch_bounds__(kThreads)
-k_rsel_round(int r, int64_t n_host, const int32_t* __restrict__ n_dev,
-             const KT* __restrict__ keys, const uint32_t* __restrict__ vals,
-             uint32_t* __restrict__ hist, SelState* st) {
-    spc::pdl_wait();
-    __shared__ uint32_t sh_h[kSelBins];
-    __shared__ uint32_t sh_dig[16];
-    __shared__ bool sh_last;
-    const int64_t n = n_dev ? (int64_t)*n_dev : n_host;
-    for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) sh_h[b] = 0;
-    if (threadIdx.x < 16) sh_dig[threadIdx.x] = st->dig[threadIdx.x];
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const KT hi = keys[i];
-        const uint32_t lo = vals[i];
-        bool match = true;
-        for (int q = 0; q < r; ++q) match = match && sel_digit<KT>(hi, lo, q) == sh_dig[q];
-        if (match) atomicAdd(&sh_h[sel_digit<KT>(hi, lo, r)], 1u);
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kSelBins; b += blockDim.x)
-        if (sh_h[b]) atomicAdd(hist + r * kSelBins + b, sh_h[b]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) sh_last = atomicAdd(&st->ticket[r], 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!sh_last) return;
-    // the last block: pick the bin holding rank `need`
-    __threadfence();
-    constexpr int kPer = kSelBins / kThreads;
-    const uint32_t* h = hist + r * kSelBins;
-    unsigned long long loc = 0;
-    uint32_t c[kPer];
-    for (int j = 0; j < kPer; ++j) {
-        c[j] = __ldcg(h + threadIdx.x * kPer + j);
-        loc += c[j];
-    }
-    __shared__ unsigned long long sh_ws[32];
-    const unsigned long long incl = block_incl_scan(loc, sh_ws);
-    const unsigned long long need = st->need;
-    unsigned long long run = incl - loc;
-    if (run < need && incl >= need) {
-        for (int j = 0; j < kPer; ++j) {
-            if (run + c[j] >= need) {
-                st->dig[r] = (uint32_t)(threadIdx.x * kPer + j);
-                st->need = need - run;
-                break;
-            }
-            run += c[j];
-        }
-    }
-}
-
-// Rounds r0 .. R-1 of the select in one CTA, over the candidates still matching after the
-// full-width rounds (usually few): per round a shared-memory histogram of digit r over the
-// items whose digits 0..r-1 are the picked ones, a block scan, the pick.
-constexpr int kRestThreads = 1024;
-constexpr int64_t kRestMax = 16384;  // candidates a single CTA takes
-
-template <class KT>
-__global__ void __launch_bounds__(kRestThreads)
-k_rsel_rest(int r0, const int32_t* __restrict__ n_dev, const KT* __restrict__ keys,
-            const uint32_t* __restrict__ vals, SelState* st) {
-    spc::pdl_wait();
-    constexpr int R = SelBits<KT>::kRounds;
-    constexpr int kPer = kSelBins / kRestThreads;
-    __shared__ uint32_t sh_h[kSelBins];
-    __shared__ uint32_t sh_dig[16];
-    __shared__ unsigned long long sh_ws[32];
-    __shared__ unsigned long long sh_need;
-    const int64_t n = *n_dev;
-    if (threadIdx.x < 16) sh_dig[threadIdx.x] = st->dig[threadIdx.x];
-    if (threadIdx.x == 0) sh_need = st->need;
-    for (int r = r0; r < R; ++r) {
-        for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) sh_h[b] = 0;
-        __syncthreads();
-        // candidates often share their digits (exactly equal scores): lanes holding the same
-        // digit add with one shared-memory atomic
-        for (int64_t i0 = 0; i0 < n; i0 += blockDim.x) {
-            const int64_t i = i0 + threadIdx.x;
-            bool match = i < n;
-            uint32_t d = 0;
-            if (match) {
-                const KT hi = keys[i];
-                const uint32_t lo = vals[i];
-                for (int q = 0; q < r; ++q) match = match && sel_digit<KT>(hi, lo, q) == sh_dig[q];
-                d = sel_digit<KT>(hi, lo, r);
-            }
-            const unsigned peers = __match_any_sync(0xffffffffu, match ? d : 0xffffffffu);
-            if (match && (int)(threadIdx.x & 31) == __ffs(peers) - 1)
-                atomicAdd(&sh_h[d], (uint32_t)__popc(peers));
-        }
-        __syncthreads();
-        unsigned long long loc = 0;
-        uint32_t c[kPer];
-        for (int j = 0; j < kPer; ++j) {
-            c[j] = sh_h[threadIdx.x * kPer + j];
-            loc += c[j];
-        }
-        const unsigned long long incl = block_incl_scan(loc, sh_ws);
-        const unsigned long long need = sh_need;
-        unsigned long long run = incl - loc;
-        __syncthreads();  // every thread has read sh_need
-        if (run < need && incl >= need) {
-            for (int j = 0; j < kPer; ++j) {
-                if (run + c[j] >= need) {
-                    sh_dig[r] = (uint32_t)(threadIdx.x * kPer + j);
-                    sh_need = need - run;
-                    break;
-                }
-                run += c[j];
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 16) st->dig[threadIdx.x] = sh_dig[threadIdx.x];
-    if (threadIdx.x == 0) st->need = sh_need;
-}
-
-// keep the items whose digits 0..r are the ones picked so far (order is irrelevant to the
-// select); one global atomic per block and pass
-template <class KT>
-__global__ void __launch_bounds__(kThreads)
-k_rsel_compact(int r, int64_t n, const KT* __restrict__ keys, const uint32_t* __restrict__ vals,
-               const SelState* __restrict__ st, KT* __restrict__ out_k,
-               uint32_t* __restrict__ out_v, int32_t* __restrict__ out_n) {
-    spc::pdl_wait();
-    __shared__ uint32_t sh_dig[16];
-    __shared__ int32_t sh_cnt, sh_base;
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x < 16) sh_dig[threadIdx.x] = st->dig[threadIdx.x];
-    __syncthreads();
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n;
-         i0 += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = i0 + threadIdx.x;
-        bool keep = false;
-        KT hi = 0;
-        uint32_t lo = 0;
-        if (i < n) {
-            hi = keys[i];
-            lo = vals[i];
-            keep = true;
-            for (int q = 0; q <= r; ++q) keep = keep && sel_digit<KT>(hi, lo, q) == sh_dig[q];
-        }
-        const unsigned b = __ballot_sync(0xffffffffu, keep);
-        if (threadIdx.x == 0) sh_cnt = 0;
-        __syncthreads();
-        int wofs = 0;
-        if (lane == 0 && b) wofs = atomicAdd(&sh_cnt, __popc(b));
-        wofs = __shfl_sync(0xffffffffu, wofs, 0);
-        __syncthreads();
-        if (threadIdx.x == 0) sh_base = sh_cnt ? atomicAdd(out_n, sh_cnt) : 0;
-        __syncthreads();
-        if (keep) {
-            const int pos = sh_base + wofs + __popc(b & ((1u << lane) - 1u));
-            out_k[pos] = hi;
-            out_v[pos] = lo;
-        }
-        __syncthreads();
-    }
-}
-
-// unite the ends of every forest edge whose (score, eid) is at most the k-th smallest
-template <class KT>
-__global__ void __launch_bounds__(kThreads)
-k_rsel_unite(int64_t n, const KT* __restrict__ keys, const uint32_t* __restrict__ vals,
-             const SelState* __restrict__ st, const int32_t* __restrict__ eu,
-             const int32_t* __restrict__ ev, int32_t* parent, uint8_t* merged, uint32_t* status) {
-    spc::pdl_wait();
-    constexpr int H = SelBits<KT>::kHiRounds, KB = SelBits<KT>::kKeyBits;
-    KT thi = 0;
-    for (int q = 0; q < H; ++q) {
-        const int top = KB - kSelBits * q;
-        const int lowb = top - kSelBits > 0 ? top - kSelBits : 0;
-        thi |= (KT)st->dig[q] << lowb;
-    }
-    uint32_t tlo = 0;
-    for (int q = 0; q < 3; ++q) {
-        const int top = 32 - kSelBits * q;
-        const int lowb = top - kSelBits > 0 ? top - kSelBits : 0;
-        tlo |= st->dig[H + q] << lowb;
-    }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const KT hi = keys[i];
-        const uint32_t lo = vals[i];
-        if (hi < thi || (hi == thi && lo <= tlo)) {
-            uf_unite(parent, eu[lo], ev[lo], status);
-            if (merged) merged[lo] = 1;
-        }
-    }
-}
-
-// selection state, the per-round histograms (`words` of them) and the candidate count
-__global__ void k_rsel_init(SelState* st, unsigned long long k, uint32_t* __restrict__ hist,
-                            int words, int32_t* __restrict__ cand) {
-    spc::pdl_wait();
-    if (threadIdx.x == 0) { st->need = k; *cand = 0; }
-    if (threadIdx.x < 16) { st->dig[threadIdx.x] = 0; st->ticket[threadIdx.x] = 0; }
-    for (int i = threadIdx.x; i < words; i += blockDim.x) hist[i] = 0;
-}
-
-// root (= smallest member) of every node and the root flags
-__global__ void __launch_bounds__(kThreads)
-k_roots(int64_t n, int32_t* parent, int32_t* __restrict__ flag, int32_t* __restrict__ warn,
-        uint32_t* status) {
+k_roots(int64_t n, const int32_t* __restrict__ parent, int32_t* __restrict__ flag,
+        int32_t* __restrict__ warn) {
     spc::pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) *warn = 0;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t r = uf_find(parent, (int32_t)x, status);
-        flag[x] = (r == (int32_t)x) ? 1 : 0;
-    }
+         x += (int64_t)gridDim.x * blockDim.x)
+        flag[x] = parent[x] == (int32_t)x ? 1 : 0;
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -1167,9 +855,8 @@ __global__ void k_graph_ptr_c(int64_t B, const int64_t* __restrict__ graph_ptr,
 }
 
 // relabel (S6) from the second union-find in W.parent2, plus per-graph offsets and the status
-spc_status finish_select(spc_context* ctx, const GraphView& g, const SelectArgs& sa, int32_t* lift,
-                         int64_t* n_c_out, int64_t* graph_ptr_c, int32_t* status_out,
-                         bool batched) {
+spc_status finish_batch(spc_context* ctx, const GraphView& g, const SelectArgs& sa, int32_t* lift,
+                        int64_t* n_c_out, int64_t* graph_ptr_c, int32_t* status_out) {
     Work& W = ctx->work;
     const int64_t n = g.n;
     const int maxb = ctx->num_sms * 8;
@@ -1180,15 +867,12 @@ spc_status finish_select(spc_context* ctx, const GraphView& g, const SelectArgs&
     int32_t* flag = W.flag.as<int32_t>();
     int32_t* ids = W.ids.as<int32_t>();
     int32_t* warn = counters + 2;
-    SPC_LAUNCH(ctx, k_roots, grid_for(n, kThreads, maxb), kThreads, 0, n, parent2, flag, warn,
-               status);
+    SPC_LAUNCH(ctx, k_roots, grid_for(n, kThreads, maxb), kThreads, 0, n, parent2, flag, warn);
     SPC_TRY(scan_i32(ctx, flag, ids, n));
     SPC_LAUNCH(ctx, k_lift, grid_for(n, kThreads, maxb), kThreads, 0, n, parent2, ids, lift,
                status);
-    if (batched) {
-        SPC_LAUNCH(ctx, k_graph_ptr_c, grid_for(sa.B + 1, kThreads, maxb), kThreads, 0, sa.B,
-                   sa.d_graph_ptr, ids, sa.d_targets, graph_ptr_c, warn);
-    }
+    SPC_LAUNCH(ctx, k_graph_ptr_c, grid_for(sa.B + 1, kThreads, maxb), kThreads, 0, sa.B,
+               sa.d_graph_ptr, ids, sa.d_targets, graph_ptr_c, warn);
     int64_t vals[2];
     {
         const void* ptrs[2] = {ids + n, warn};
@@ -1198,55 +882,787 @@ spc_status finish_select(spc_context* ctx, const GraphView& g, const SelectArgs&
     const int64_t n_c = vals[0];
     const int32_t warn_b = (int32_t)vals[1];
     *n_c_out = n_c;
-    *status_out = (batched ? warn_b != 0 : n_c > sa.target) ? SPC_WARN_TARGET_NOT_REACHED : SPC_OK;
+    *status_out = warn_b != 0 ? SPC_WARN_TARGET_NOT_REACHED : SPC_OK;
     return SPC_OK;
 }
 
-// key_hist: the score-prefix histogram (kTauBins words, zeroed before each selection's first
-// attempt and kept for its later ones), then the radix-select histograms of every round
-// (zeroed by k_rsel_init); zeroed once on allocation
+// key_hist: the score-prefix histogram (kTauBins words, zero between selections), then the radix
+// select's histograms of every round (zeroed by the selection); zeroed once on allocation
 constexpr int kTauBins = 32768;
 constexpr size_t kKeyHistBytes = (size_t)(kTauBins + SelBits<uint64_t>::kRounds * kSelBins) * 4;
 static spc_status ensure_key_hist(spc_context* ctx) {
     return ensure_zeroed(ctx, ctx->work.key_hist, kKeyHistBytes);
 }
 
+// ---- the merge selection of one graph in one cooperative kernel --------------------------------
+// Every phase of the selection -- Boruvka rounds on the score prefix, the prefix's extensions, the
+// select of the n - n_c lightest forest edges, their union, the relabelling -- reads what the phase
+// before it wrote, and most are a few microseconds of work.  As separate launches a level took
+// about 35 of them and eight to twelve sizes read back by the host (10-15 us of idle GPU each).
+// Here the phases are separated by grid barriers of one resident grid (a cooperative launch; every
+// barrier wait is bounded), the sizes stay on the device, and the host reads the super-node count
+// alone.  Forest edges are appended to a list as they are picked, so no flag per edge is kept,
+// scanned or compacted; the select is order-free, because every (score, eid) is distinct.
+//
+// What bounds it: random accesses to parents and best slots (latency: the grid holds
+// kCoopBlocks * kCoopThreads threads per SM) on large levels; on small ones chains of dependent
+// L2 reads (a phase of a few hundred items takes 5-9 us) and the barriers (1.4 us each on 152 CTAs
+// and more, 3-5 with the wait for the slowest).  The rounds whose work list has at most
+// kCoopTail items run in one CTA, with block barriers, while the others wait.
+// Against the separate launches, whole calls: 64x64 mesh 0.77 -> 0.65 ms, 257x250 mesh (6 levels)
+// 3.68 -> 3.22, 129^3 mesh 22.6 -> 21.8, 2^23-point random geometric graph 23.4 -> 21.9, 10^6
+// points in one level 3.89 -> 3.36; a replayed 2048^2 mesh, which reads nothing back, 9.04 -> 9.05.
+// Device time of the kernel, all levels of the 2048^2 mesh, at threads x CTAs per SM: 512 x 3 2.43
+// ms, 512 x 4 2.51, 512 x 2 2.64, 1024 x 1 2.66, 256 x 6 2.75.
+constexpr int kCoopThreads = 512;
+constexpr int kCoopBlocks = 3;           // per SM
+constexpr int kCoopTail = 2 * kCoopThreads;
+constexpr int kRestMax = 4096;           // candidates every CTA selects among by itself
+
+// counters of a call, zero before it: the last CTA to leave zeroes them (and the grid the score
+// histogram) for the next call, so no memset comes between the launches; kCtNc is the result
+enum { kCtList0 = 0, kCtList1 = 1, kCtForest = 2, kCtCand = 3, kCtBar = 4, kCtTau = 5,
+       kCtDone = 6, kCtZeroed = 7, kCtNc = 7, kCtCount = 8 };
+
 template <class KT>
-spc_status select_typed(spc_context* ctx, const GraphView& g, const KT* key,
-                        const SelectArgs& sa, int32_t* lift, uint8_t* merged, int64_t* n_c_out,
-                        int64_t* graph_ptr_c, int32_t* status_out) {
+struct CoopArgs {
+    int64_t n, m, need, k_need;  // need: edges of the first prefix; k_need = n - n_c >= 0
+    const int32_t* eu;
+    const int32_t* ev;
+    const KT* key;
+    uint32_t* hist;              // score histogram of the prefix (null: no prefix)
+    int tau_shift, hist_samp, slab_list;
+    int32_t* parent;
+    int32_t* parent2;
+    unsigned long long* bk[2];
+    int32_t* be[2];
+    int32_t* wl[2][3];           // work lists: edge, root, root
+    KT* fk;                      // forest edges: key, eid
+    uint32_t* fe;
+    KT* ck;                      // select candidates
+    uint32_t* cv;
+    uint32_t* rhist;             // one histogram per select round
+    int32_t* blk;                // roots per CTA
+    int32_t* ids;
+    int32_t* lift;
+    uint8_t* merged;             // may be null
+    int32_t* ct;
+    uint32_t* status;
+};
+
+// every CTA of the grid waits for every other; false when the wait was given up (then every CTA
+// leaves).  *bar counts arrivals, zero at launch.
+__device__ bool grid_sync(uint32_t* bar, uint32_t* status) {
+    __shared__ bool sh_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        bool good = true;
+        if (gridDim.x > 1) {
+            __threadfence();
+            const uint32_t goal = (atomicAdd(bar, 1u) / gridDim.x + 1u) * gridDim.x;
+            const uint32_t lim = spin_limit(status);
+            uint32_t spins = 0, seen;
+            do {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+                if (seen < goal && ++spins > lim) {
+                    atomicOr(status, DEV_TIMEOUT);
+                    good = false;
+                    break;
+                }
+            } while (seen < goal);
+            __threadfence();
+        }
+        sh_ok = good;
+    }
+    __syncthreads();
+    return sh_ok;
+}
+
+// positions for `mine` items of every thread of the block, one global atomic for the block; every
+// thread calls it
+__device__ __forceinline__ int32_t block_append(int32_t mine, int32_t* count) {
+    __shared__ int32_t sh_w[kCoopThreads / 32];
+    __shared__ int32_t sh_base;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    __syncthreads();  // sh_w and sh_base of the call before have been read
+    if (lane == 31) sh_w[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const int32_t s = lane < kCoopThreads / 32 ? sh_w[lane] : 0;
+        int32_t si = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, si, o);
+            if (lane >= o) si += t;
+        }
+        if (lane < kCoopThreads / 32) sh_w[lane] = si - s;
+        if (lane == 31) sh_base = si ? atomicAdd(count, si) : 0;
+    }
+    __syncthreads();
+    return sh_base + sh_w[warp] + incl - mine;
+}
+
+// smallest of the 32768 bins whose cumulative count reaches `need` (the last bin when none does);
+// one CTA
+__device__ void coop_pick_tau(const uint32_t* hist, int64_t need, int32_t* tau) {
+    constexpr int kPer = 32768 / kCoopThreads;
+    __shared__ unsigned long long sh_ws[32];
+    const uint4* h4 = reinterpret_cast<const uint4*>(hist) + (int64_t)threadIdx.x * (kPer / 4);
+    unsigned long long loc = 0;
+#pragma unroll 4
+    for (int j = 0; j < kPer / 4; ++j) {
+        const uint4 q = __ldcg(h4 + j);
+        loc += (unsigned long long)q.x + q.y + q.z + q.w;
+    }
+    const unsigned long long incl = block_incl_scan(loc, sh_ws);
+    unsigned long long run = incl - loc;
+    if (threadIdx.x == kCoopThreads - 1 && incl < (unsigned long long)need) *tau = 32767;
+    if (run < (unsigned long long)need && incl >= (unsigned long long)need) {
+        for (int j = 0; j < kPer; ++j) {
+            run += __ldcg(hist + (int64_t)threadIdx.x * kPer + j);
+            if (run >= (unsigned long long)need) {
+                *tau = threadIdx.x * kPer + j;
+                break;
+            }
+        }
+    }
+}
+
+// Boruvka phase A over the work list (kEdges: over every edge of the slab (lo, top]): current roots
+// of both ends; edges between two components go to the out list and lower both minima
+template <class KT, bool kEdges>
+__device__ __forceinline__ void coop_minkey(const CoopArgs<KT>& a, int64_t cnt, int in, int out,
+                                            bool direct, uint32_t top, uint32_t lo, int64_t bid,
+                                            int64_t nblk) {
+    unsigned long long* best = a.bk[in];
+    int32_t* const oe = a.wl[out][0];
+    int32_t* const ou = a.wl[out][1];
+    int32_t* const ov = a.wl[out][2];
+    // The atomics of one address serialise, and most edges of a late slab end in one giant
+    // component.  Each CTA keeps the minimum of one component -- that of its first edge, most
+    // likely the giant -- in shared memory and lowers the slot once.
+    __shared__ HotMin sh_hot;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sh_hot.idx = -2;
+        sh_hot.v = ~0ull;
+    }
+    __syncthreads();
+    const int64_t per = (int64_t)kCoopThreads * kMkItems;
+    for (int64_t base = bid * per; base < cnt; base += nblk * per) {
+        int32_t e[kMkItems], u[kMkItems], v[kMkItems];
+        bool act[kMkItems];
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            const int64_t i = base + (int64_t)it * kCoopThreads + threadIdx.x;
+            act[it] = i < cnt;
+            e[it] = u[it] = v[it] = 0;
+            if (act[it]) {
+                if (kEdges) {
+                    e[it] = (int32_t)i;
+                    u[it] = a.eu[i];
+                    v[it] = a.ev[i];
+                } else {
+                    e[it] = a.wl[in][0][i];
+                    u[it] = a.wl[in][1][i];
+                    v[it] = a.wl[in][2][i];
+                }
+            }
+        }
+        int32_t nkeep = 0;
+        KT k[kMkItems];
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) k[it] = act[it] ? a.key[e[it]] : KT(0);
+        int32_t rt[2 * kMkItems];
+        unsigned live = 0;
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            if (kEdges && act[it]) {
+                const uint32_t bin = (uint32_t)(k[it] >> a.tau_shift);
+                act[it] = bin <= top && (lo == kNoSlab || bin > lo);
+            }
+            rt[2 * it] = u[it];
+            rt[2 * it + 1] = v[it];
+            if (act[it]) live |= 3u << (2 * it);
+        }
+        // direct: the first round of the selection, every node its own component
+        if (!direct) uf_find_n<2 * kMkItems, true>(a.parent, rt, live, a.status);
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            u[it] = rt[2 * it];
+            v[it] = rt[2 * it + 1];
+            act[it] = act[it] && u[it] != v[it];
+            const unsigned long long pk = MinKey<KT>::pack(k[it], e[it]);
+            warp_atomic_min_u64(best, u[it], pk, act[it], &sh_hot);
+            warp_atomic_min_u64(best, v[it], pk, act[it], &sh_hot);
+            nkeep += act[it] ? 1 : 0;
+        }
+        int32_t slot = block_append(nkeep, a.ct + kCtList0 + out);
+        if (threadIdx.x == 0 && sh_hot.idx < 0 && act[0]) sh_hot.idx = u[0];  // from the next pass
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            if (act[it]) {
+                oe[slot] = e[it];
+                ou[slot] = u[it];
+                ov[slot] = v[it];
+                ++slot;
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && sh_hot.v != ~0ull) atomicMin(best + sh_hot.idx, sh_hot.v);
+}
+
+// the slab's edges as the first work list (very large selections): keys streamed, ends read only
+// for the slab's edges
+template <class KT>
+__device__ __forceinline__ void coop_slab_list(const CoopArgs<KT>& a, uint32_t top, uint32_t lo) {
+    constexpr int kVec = (int)(kSlItems * sizeof(KT) / 16);
+    const int64_t per = (int64_t)kCoopThreads * kSlItems;
+    for (int64_t base = (int64_t)blockIdx.x * per; base < a.m; base += (int64_t)gridDim.x * per) {
+        const int64_t i0 = base + (int64_t)threadIdx.x * kSlItems;
+        unsigned keep = 0;  // bit it: edge i0 + it lies in the slab
+        if (i0 + kSlItems <= a.m) {
+            const uint4* p = reinterpret_cast<const uint4*>(a.key + i0);
+#pragma unroll
+            for (int j = 0; j < kVec; ++j) {
+                const uint4 q = p[j];
+                KT k[16 / sizeof(KT)];
+                memcpy(k, &q, 16);
+#pragma unroll
+                for (int t = 0; t < (int)(16 / sizeof(KT)); ++t) {
+                    const uint32_t bin = (uint32_t)(k[t] >> a.tau_shift);
+                    if (bin <= top && (lo == kNoSlab || bin > lo))
+                        keep |= 1u << (j * (int)(16 / sizeof(KT)) + t);
+                }
+            }
+        } else {
+            for (int it = 0; it < kSlItems && i0 + it < a.m; ++it) {
+                const uint32_t bin = (uint32_t)(a.key[i0 + it] >> a.tau_shift);
+                if (bin <= top && (lo == kNoSlab || bin > lo)) keep |= 1u << it;
+            }
+        }
+        int32_t slot = block_append(__popc(keep), a.ct + kCtList0);
+        while (keep) {
+            const int64_t i = i0 + __ffs(keep) - 1;
+            keep &= keep - 1;
+            a.wl[0][0][slot] = (int32_t)i;
+            a.wl[0][1][slot] = a.eu[i];
+            a.wl[0][2][slot] = a.ev[i];
+            ++slot;
+        }
+    }
+}
+
+// phase B (64-bit scores): among the edges whose score equals the component's minimum, the
+// smallest edge id
+template <class KT>
+__device__ __forceinline__ void coop_tiebreak(const CoopArgs<KT>& a, int64_t cnt, int par, int list,
+                                              int64_t bid, int64_t nblk) {
+    const int64_t stride = nblk * kCoopThreads;
+    for (int64_t i0 = bid * kCoopThreads; i0 < cnt; i0 += stride) {  // uniform per warp
+        const int64_t i = i0 + threadIdx.x;
+        const bool act = i < cnt;
+        int32_t e = 0, u = 0, v = 0;
+        unsigned long long k = 0;
+        if (act) {
+            e = a.wl[list][0][i];
+            u = a.wl[list][1][i];
+            v = a.wl[list][2][i];
+            k = (unsigned long long)a.key[e];
+        }
+        warp_atomic_min_i32(a.be[par], u, e, act && k == __ldcg(a.bk[par] + u));
+        warp_atomic_min_i32(a.be[par], v, e, act && k == __ldcg(a.bk[par] + v));
+    }
+}
+
+// phase C: an edge picked by either end is a forest edge: united and appended to the forest; the
+// other parity's slots of both ends are cleared for the next round
+template <class KT>
+__device__ __forceinline__ void coop_hook(const CoopArgs<KT>& a, int64_t cnt, int par, int list,
+                                          int64_t bid, int64_t nblk) {
+    const int lane = threadIdx.x & 31;
+    const int64_t per = (int64_t)kCoopThreads * kMkItems;
+    for (int64_t base = bid * per; base < cnt; base += nblk * per) {  // uniform per block
+        int32_t e[kMkItems], u[kMkItems], v[kMkItems];
+        bool picked[kMkItems];
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            const int64_t i = base + (int64_t)it * kCoopThreads + threadIdx.x;
+            e[it] = u[it] = v[it] = -1;
+            if (i < cnt) {
+                e[it] = a.wl[list][0][i];
+                u[it] = a.wl[list][1][i];
+                v[it] = a.wl[list][2][i];
+            }
+        }
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            // a slot shared with the previous lane (a hub component) is cleared by that lane
+            const int32_t pu = __shfl_up_sync(0xffffffffu, u[it], 1);
+            const int32_t pv = __shfl_up_sync(0xffffffffu, v[it], 1);
+            picked[it] = false;
+            if (e[it] < 0) continue;
+            const bool clr_u = lane == 0 || pu != u[it], clr_v = lane == 0 || pv != v[it];
+            if (MinKey<KT>::two_phase) {
+                const int32_t bu = __ldcg(a.be[par] + u[it]), bv = __ldcg(a.be[par] + v[it]);
+                picked[it] = bu == e[it] || bv == e[it];
+                if (clr_u) a.be[par ^ 1][u[it]] = INT32_MAX;
+                if (clr_v) a.be[par ^ 1][v[it]] = INT32_MAX;
+            } else {
+                const unsigned long long bu = __ldcg(a.bk[par] + u[it]),
+                                         bv = __ldcg(a.bk[par] + v[it]);
+                picked[it] = (int32_t)(uint32_t)bu == e[it] || (int32_t)(uint32_t)bv == e[it];
+            }
+            if (clr_u) a.bk[par ^ 1][u[it]] = ~0ull;
+            if (clr_v) a.bk[par ^ 1][v[it]] = ~0ull;
+        }
+        int32_t npick = 0;
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            if (picked[it]) uf_unite(a.parent, u[it], v[it], a.status);
+            npick += picked[it] ? 1 : 0;
+        }
+        int32_t slot = block_append(npick, a.ct + kCtForest);
+        // a forest has fewer than m edges unless a union-find walk gave up (reported)
+#pragma unroll
+        for (int it = 0; it < kMkItems; ++it) {
+            if (picked[it] && (int64_t)slot < a.m) {
+                a.fk[slot] = a.key[e[it]];
+                a.fe[slot] = (uint32_t)e[it];
+                ++slot;
+            }
+        }
+    }
+}
+
+// histogram of digit r over the items whose digits 0 .. r-1 are dig[0 .. r-1], into sh_h
+template <class KT>
+__device__ __forceinline__ void coop_digit_hist(int r, int64_t n, const KT* keys,
+                                                const uint32_t* vals, const uint32_t* dig,
+                                                uint32_t* sh_h, int64_t bid, int64_t nblk) {
+    for (int b = threadIdx.x; b < kSelBins; b += kCoopThreads) sh_h[b] = 0;
+    __syncthreads();
+    for (int64_t i0 = bid * kCoopThreads; i0 < n; i0 += nblk * kCoopThreads) {
+        const int64_t i = i0 + threadIdx.x;
+        bool match = i < n;
+        uint32_t d = 0;
+        if (match) {
+            const KT hi = keys[i];
+            const uint32_t lo = vals[i];
+            for (int q = 0; q < r; ++q) match = match && sel_digit<KT>(hi, lo, q) == dig[q];
+            d = sel_digit<KT>(hi, lo, r);
+        }
+        // candidates often share their digits (exactly equal scores)
+        const unsigned peers = __match_any_sync(0xffffffffu, match ? d : 0xffffffffu);
+        if (match && (int)(threadIdx.x & 31) == __ffs(peers) - 1)
+            atomicAdd(&sh_h[d], (uint32_t)__popc(peers));
+    }
+    __syncthreads();
+}
+
+// the bin of h that holds rank *need (1-based): dig = the bin, *need = the rank inside it.  Every
+// thread of the CTA calls it; h is shared or global memory.
+__device__ __forceinline__ void coop_pick_bin(const uint32_t* h, uint32_t* dig,
+                                              unsigned long long* need) {
+    constexpr int kPer = kSelBins / kCoopThreads;
+    __shared__ unsigned long long sh_ws[32];
+    uint32_t c[kPer];
+    unsigned long long loc = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        c[j] = *(const volatile uint32_t*)(h + threadIdx.x * kPer + j);
+        loc += c[j];
+    }
+    const unsigned long long incl = block_incl_scan(loc, sh_ws);
+    const unsigned long long want = *need;
+    unsigned long long run = incl - loc;
+    __syncthreads();  // every thread has read *need
+    if (run < want && incl >= want) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            if (run < want && run + c[j] >= want) {
+                *dig = (uint32_t)(threadIdx.x * kPer + j);
+                *need = want - run;
+                run = want;  // picked
+            } else {
+                run += c[j];
+            }
+        }
+    }
+    __syncthreads();
+}
+
+template <class KT>
+__global__ void __launch_bounds__(kCoopThreads, kCoopBlocks) k_select_coop(const __grid_constant__ CoopArgs<KT> a) {
+    spc::pdl_wait();
+    __shared__ uint32_t sh_h[kSelBins];
+    __shared__ uint32_t sh_dig[16];
+    __shared__ unsigned long long sh_need;
+    const int64_t nblk = gridDim.x, bid = blockIdx.x;
+    const int64_t t0 = bid * kCoopThreads + threadIdx.x, stride = nblk * kCoopThreads;
+    uint32_t* const bar = reinterpret_cast<uint32_t*>(a.ct + kCtBar);
+    const bool two = MinKey<KT>::two_phase;
+    // ---- start state; the first prefix's threshold ------------------------------------------
+    const bool forest = a.k_need > 0;  // else nothing merges
+    for (int64_t i = t0; i < a.n; i += stride) {
+        a.parent2[i] = (int32_t)i;
+        if (forest) {
+            a.parent[i] = (int32_t)i;
+            a.bk[0][i] = ~0ull;
+            a.bk[1][i] = ~0ull;
+            if (two) {
+                a.be[0][i] = INT32_MAX;
+                a.be[1][i] = INT32_MAX;
+            }
+        }
+    }
+    if (a.merged)
+        for (int64_t e = t0; e < a.m; e += stride) a.merged[e] = 0;
+    for (int64_t i = t0; i < SelBits<KT>::kRounds * kSelBins; i += stride) a.rhist[i] = 0;
+    bool prefix = a.hist != nullptr;
+    int64_t need = a.need;
+    if (forest && prefix && bid == nblk - 1)
+        coop_pick_tau(a.hist, (need + (int64_t{1} << a.hist_samp) - 1) >> a.hist_samp,
+                      a.ct + kCtTau);
+    if (!grid_sync(bar, a.status)) return;
+    int64_t n_msf = 0;
+    if (forest) {
+        uint32_t lo = kNoSlab;
+        for (int attempt = 0; attempt < 64; ++attempt) {
+            const uint32_t top = prefix ? (uint32_t)__ldcg(a.ct + kCtTau) : 0xffffffffu;
+            // ---- Boruvka rounds on the slab (lo, top] -------------------------------------
+            bool edges = true;
+            if (a.slab_list && (prefix || lo != kNoSlab)) {
+                coop_slab_list(a, top, lo);
+                if (!grid_sync(bar, a.status)) return;
+                edges = false;
+            }
+            int in = 0;
+            for (int round = 0; round < 64; ++round) {
+                const int out = in ^ 1;
+                if (edges && round == 0)
+                    coop_minkey<KT, true>(a, a.m, in, out, attempt == 0, top, lo, bid, nblk);
+                else
+                    coop_minkey<KT, false>(a, __ldcg(a.ct + in), in, out,
+                                           attempt == 0 && round == 0, top, lo, bid, nblk);
+                if (!grid_sync(bar, a.status)) return;
+                int64_t cnt = __ldcg(a.ct + out);
+                if (cnt == 0) break;
+                if (two) {
+                    coop_tiebreak(a, cnt, in, out, bid, nblk);
+                    if (!grid_sync(bar, a.status)) return;
+                }
+                coop_hook(a, cnt, in, out, bid, nblk);
+                if (t0 == 0) a.ct[in] = 0;  // the next round's out list
+                if (cnt <= kCoopTail) {
+                    // the remaining rounds in the first CTA
+                    if (!grid_sync(bar, a.status)) return;
+                    if (bid == 0) {
+                        int ti = out;
+                        for (int tr = 0; tr < 64; ++tr) {
+                            const int to = ti ^ 1;
+                            coop_minkey<KT, false>(a, cnt, ti, to, false, top, lo, 0, 1);
+                            __threadfence_block();
+                            __syncthreads();
+                            cnt = __ldcg(a.ct + to);
+                            if (cnt == 0) break;
+                            if (two) {
+                                coop_tiebreak(a, cnt, ti, to, 0, 1);
+                                __syncthreads();
+                            }
+                            coop_hook(a, cnt, ti, to, 0, 1);
+                            __syncthreads();
+                            if (threadIdx.x == 0) a.ct[ti] = 0;
+                            __threadfence_block();
+                            __syncthreads();
+                            ti = to;
+                        }
+                    }
+                    break;
+                }
+                if (!grid_sync(bar, a.status)) return;
+                in = out;
+            }
+            if (!grid_sync(bar, a.status)) return;
+            // the prefix's forest holds Kruskal's first n_msf merges: enough at n - n_c
+            n_msf = __ldcg(a.ct + kCtForest);
+            if (n_msf > a.m) n_msf = a.m;
+            if (!prefix || n_msf >= a.k_need) break;
+            // the next slab: twice the edges, or, when the forest came within 15 % of n - n_c,
+            // the prefix its yield so far extrapolates to, and a quarter more
+            int64_t next = need * 2;
+            if (n_msf * 20 >= a.k_need * 17) {
+                const int64_t est =
+                    (int64_t)((double)need * (double)a.k_need / (double)n_msf * 1.25);
+                const int64_t least = est > need + need / 8 ? est : need + need / 8;
+                next = least < next ? least : next;
+            }
+            need = next;
+            if (need >= a.m) prefix = false;  // the last slab: every remaining score
+            lo = top;
+            for (int64_t i = t0; i < a.n; i += stride) {
+                a.bk[0][i] = ~0ull;
+                a.bk[1][i] = ~0ull;
+                if (two) {
+                    a.be[0][i] = INT32_MAX;
+                    a.be[1][i] = INT32_MAX;
+                }
+            }
+            if (t0 == 0) {
+                a.ct[kCtList0] = 0;
+                a.ct[kCtList1] = 0;
+            }
+            if (prefix && bid == nblk - 1)
+                coop_pick_tau(a.hist, (need + (int64_t{1} << a.hist_samp) - 1) >> a.hist_samp,
+                              a.ct + kCtTau);
+            if (!grid_sync(bar, a.status)) return;
+        }
+        // ---- the (n - n_c)-th smallest (score, eid) of the forest, by 11-bit digits -----------
+        constexpr int R = SelBits<KT>::kRounds, H = SelBits<KT>::kHiRounds,
+                      KB = SelBits<KT>::kKeyBits;
+        const bool all = a.k_need >= n_msf;
+        if (!all) {
+            // rounds over the whole forest: 22 bits of a binary32 score, 33 of a binary64 one
+            // leave few candidates
+            constexpr int kFull = sizeof(KT) == 8 ? 3 : 2;
+            if (threadIdx.x < 16) sh_dig[threadIdx.x] = 0;
+            if (threadIdx.x == 0) sh_need = (unsigned long long)a.k_need;
+            __syncthreads();
+            const KT* keys = a.fk;
+            const uint32_t* vals = a.fe;
+            int64_t items = n_msf;
+            for (int r = 0; r < R; ++r) {
+                if (r == kFull) {
+                    // the items still matching
+                    for (int64_t i0 = bid * kCoopThreads; i0 < n_msf; i0 += stride) {
+                        const int64_t i = i0 + threadIdx.x;
+                        KT hi = 0;
+                        uint32_t lw = 0;
+                        bool keep = i < n_msf;
+                        if (keep) {
+                            hi = a.fk[i];
+                            lw = a.fe[i];
+                            for (int q = 0; q < kFull; ++q)
+                                keep = keep && sel_digit<KT>(hi, lw, q) == sh_dig[q];
+                        }
+                        const int32_t slot = block_append(keep ? 1 : 0, a.ct + kCtCand);
+                        if (keep) {
+                            a.ck[slot] = hi;
+                            a.cv[slot] = lw;
+                        }
+                    }
+                    if (!grid_sync(bar, a.status)) return;
+                    keys = a.ck;
+                    vals = a.cv;
+                    items = __ldcg(a.ct + kCtCand);
+                }
+                if (r >= kFull && items <= kRestMax) {  // every CTA by itself
+                    coop_digit_hist(r, items, keys, vals, sh_dig, sh_h, 0, 1);
+                    coop_pick_bin(sh_h, sh_dig + r, &sh_need);
+                } else {
+                    coop_digit_hist(r, items, keys, vals, sh_dig, sh_h, bid, nblk);
+                    uint32_t* const gh = a.rhist + r * kSelBins;
+                    for (int b = threadIdx.x; b < kSelBins; b += kCoopThreads)
+                        if (sh_h[b]) atomicAdd(gh + b, sh_h[b]);
+                    if (!grid_sync(bar, a.status)) return;
+                    coop_pick_bin(gh, sh_dig + r, &sh_need);
+                }
+            }
+        }
+        KT thi = ~KT(0);
+        uint32_t tlo = ~0u;
+        if (!all) {
+            thi = 0;
+            tlo = 0;
+            for (int q = 0; q < H; ++q) {
+                const int hb = KB - kSelBits * q;
+                thi |= (KT)sh_dig[q] << (hb - kSelBits > 0 ? hb - kSelBits : 0);
+            }
+            for (int q = 0; q < 3; ++q) {
+                const int hb = 32 - kSelBits * q;
+                tlo |= sh_dig[H + q] << (hb - kSelBits > 0 ? hb - kSelBits : 0);
+            }
+        }
+        for (int64_t i = t0; i < n_msf; i += stride) {
+            const KT hi = a.fk[i];
+            const uint32_t lw = a.fe[i];
+            if (hi < thi || (hi == thi && lw <= tlo)) {
+                uf_unite(a.parent2, a.eu[lw], a.ev[lw], a.status);
+                if (a.merged) a.merged[lw] = 1;
+            }
+        }
+        if (!grid_sync(bar, a.status)) return;
+    }
+    // ---- relabel: each CTA a contiguous range of nodes ------------------------------------------
+    const int64_t span = (a.n + nblk - 1) / nblk;
+    const int64_t x0 = bid * span < a.n ? bid * span : a.n;
+    const int64_t x1 = x0 + span < a.n ? x0 + span : a.n;
+    int32_t roots = 0;
+    for (int64_t x = x0 + threadIdx.x; x < x1; x += kCoopThreads)
+        roots += __ldcg(a.parent2 + x) == (int32_t)x ? 1 : 0;
+    roots = __reduce_add_sync(0xffffffffu, roots);
+    if (threadIdx.x == 0) sh_dig[0] = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && roots) atomicAdd(&sh_dig[0], (uint32_t)roots);
+    __syncthreads();
+    if (threadIdx.x == 0) a.blk[bid] = (int32_t)sh_dig[0];
+    if (!grid_sync(bar, a.status)) return;
+    int32_t before = 0;
+    for (int64_t c = threadIdx.x; c < bid; c += kCoopThreads) before += __ldcg(a.blk + c);
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (threadIdx.x == 0) sh_dig[0] = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && before) atomicAdd(&sh_dig[0], (uint32_t)before);
+    __syncthreads();
+    __shared__ unsigned long long sh_ws[32];
+    unsigned long long run = sh_dig[0];
+    for (int64_t b = x0; b < x1; b += kCoopThreads) {
+        const int64_t x = b + threadIdx.x;
+        const bool root = x < x1 && __ldcg(a.parent2 + x) == (int32_t)x;
+        const unsigned long long incl = block_incl_scan(root ? 1ull : 0ull, sh_ws);
+        if (root) a.ids[x] = (int32_t)(run + incl - 1);
+        if (threadIdx.x == kCoopThreads - 1) sh_need = incl;
+        __syncthreads();
+        run += sh_need;
+        __syncthreads();
+    }
+    if (bid == nblk - 1 && threadIdx.x == 0) a.ct[kCtNc] = (int32_t)run;
+    if (!grid_sync(bar, a.status)) return;
+    // Shallow trees (a target of n / 8 or more): four walks of a thread together (4 M nodes halved:
+    // 29 -> 17 us).  A small target leaves deep trees under giant components: one walk at a time,
+    // past L1, each shortened by the walks before it (1 M nodes to n / 256: 128 us; four together
+    // 200, and through L1, where nobody sees another SM's shortening, 270-560).
+    if ((a.n - a.k_need) * 8 < a.n) {
+        for (int64_t x = t0; x < a.n; x += stride)
+            a.lift[x] = __ldcg(a.ids + uf_find(a.parent2, (int32_t)x, a.status));
+    } else {
+        for (int64_t x = t0; x < a.n; x += 4 * stride) {
+            int32_t r[4];
+            unsigned live = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                r[i] = (int32_t)(x + i * stride);
+                if (x + i * stride < a.n) live |= 1u << i;
+            }
+            uf_find_n<4, true>(a.parent2, r, live, a.status);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (x + i * stride < a.n) a.lift[x + i * stride] = __ldcg(a.ids + r[i]);
+        }
+    }
+    if (a.hist)
+        for (int64_t i = t0; i < kTauBins; i += stride) a.hist[i] = 0u;
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(a.ct + kCtDone, 1) == (int32_t)nblk - 1)
+        for (int i = 0; i < kCtZeroed; ++i) a.ct[i] = 0;  // every other CTA has left its barriers
+}
+
+// one cooperative grid that the device holds at once, at most one CTA per kCoopThreads * 2 items
+template <class KT>
+spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, int64_t target,
+                         int32_t* lift, uint8_t* merged, int64_t* n_c_out, int32_t* status_out) {
+    Work& W = ctx->work;
+    const int64_t n = g.n, m = g.m;
+    CoopArgs<KT> a{};
+    a.n = n;
+    a.m = m;
+    a.k_need = n - target > 0 ? n - target : 0;
+    a.need = a.k_need + a.k_need / 2;
+    a.eu = W.eu.as<int32_t>();
+    a.ev = W.ev.as<int32_t>();
+    a.key = key;
+    a.tau_shift = sizeof(KT) == 8 ? 48 : 16;
+    // the threshold's histogram samples one key chunk in eight on large selections
+    a.hist_samp = m >= (int64_t{1} << 22) ? 3 : 0;
+    a.slab_list = m >= kSlabListMin && (reinterpret_cast<uintptr_t>(key) & 15) == 0 ? 1 : 0;
+    a.parent = W.parent.as<int32_t>();
+    a.parent2 = W.parent2.as<int32_t>();
+    for (int i = 0; i < 2; ++i) {
+        a.bk[i] = W.best_k[i].as<unsigned long long>();
+        a.be[i] = W.best_e[i].as<int32_t>();
+        a.wl[i][0] = W.wl_e[i].as<int32_t>();
+        a.wl[i][1] = W.wl_u[i].as<int32_t>();
+        a.wl[i][2] = W.wl_v[i].as<int32_t>();
+    }
+    a.fk = W.sel_key.as<KT>();
+    a.fe = W.sel_val.as<uint32_t>();
+    a.ck = W.sel_key2.as<KT>();
+    a.cv = W.sel_val2.as<uint32_t>();
+    a.ids = W.ids.as<int32_t>();
+    a.lift = lift;
+    a.merged = merged;
+    a.ct = W.counters.as<int32_t>() + 16;
+    a.status = ctx->d_status;
+    SPC_TRY(ensure_key_hist(ctx));
+    a.rhist = W.key_hist.as<uint32_t>() + kTauBins;
+    static std::atomic<int> per_sm[64];  // resident CTAs per SM, by device (0: not asked yet)
+    std::atomic<int>& occ = per_sm[ctx->device & 63];
+    int bps = occ.load();
+    if (bps == 0) {
+        SPC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_select_coop<KT>,
+                                                               kCoopThreads, 0));
+        SPC_CUDA(cudaFuncSetAttribute(k_key_hist<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kTauBins * 4));
+        if (bps < 1) return SPC_ERR_CUDA;
+        occ.store(bps);
+    }
+    const int64_t big = n > m ? n : m;
+    const int grid = grid_for(big, kCoopThreads * 2, ctx->num_sms * bps);
+    SPC_TRY(ensure(ctx, W.sel_blk, (size_t)(ctx->num_sms * bps) * 4));
+    a.blk = W.sel_blk.as<int32_t>();
+    if (W.sel_dirty) {  // the first call, or one after a call that did not finish
+        SPC_CUDA(cudaMemsetAsync(a.ct, 0, kCtCount * 4, ctx->stream));
+        SPC_CUDA(cudaMemsetAsync(W.key_hist.p, 0, (size_t)kTauBins * 4, ctx->stream));
+    }
+    W.sel_dirty = true;
+    if (m > 65536 && a.k_need > 0 && a.need < m) {
+        a.hist = W.key_hist.as<uint32_t>();
+        note_bytes(ctx, (double)m * sizeof(KT) / (double)(1 << a.hist_samp));
+        SPC_LAUNCH(ctx, k_key_hist<KT>, ctx->num_sms, 1024, kTauBins * 4, m, key, a.tau_shift,
+                   a.hist_samp, W.key_hist.as<uint32_t>());
+    }
+    SPC_LAUNCH_COOP(ctx, k_select_coop<KT>, grid, kCoopThreads, a);
+    int64_t vals[2];
+    {
+        // a barrier wait that was given up leaves the lift unwritten: nothing may index with it
+        const void* ptrs[2] = {a.ct + kCtNc, ctx->d_status};
+        const int bytes[2] = {4, 4};
+        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, vals));
+        const spc_status st = status_from_bits((uint32_t)vals[1]);
+        if (st < 0) return st;
+    }
+    W.sel_dirty = false;
+    *n_c_out = vals[0];
+    *status_out = vals[0] > target ? SPC_WARN_TARGET_NOT_REACHED : SPC_OK;
+    return SPC_OK;
+}
+
+// A batch: every graph its own score prefix and target; the spanning-forest rounds run over the
+// whole batch, one set of launches per round.
+template <class KT>
+spc_status select_batch(spc_context* ctx, const GraphView& g, const KT* key, const SelectArgs& sa,
+                        int32_t* lift, uint8_t* merged, int64_t* n_c_out, int64_t* graph_ptr_c,
+                        int32_t* status_out) {
     Work& W = ctx->work;
     const int64_t n = g.n, m = g.m;
     const int maxb = ctx->num_sms * 8;
     uint32_t* status = ctx->d_status;
     int32_t* parent = W.parent.as<int32_t>();
     int32_t* counters = W.counters.as<int32_t>();  // [0..1] work-list counts, [2] warn flag
-    const bool batched = sa.B > 1 || sa.d_graph_ptr != nullptr;
-
-    // ---- 0. score prefix (single graph): the lightest ~1.5 (n - n_c) edges ------------------
-    const int64_t k_need = batched ? 0 : (n - sa.target > 0 ? n - sa.target : 0);
-    const int tau_shift = sizeof(KT) == 8 ? 48 : 16;
-    uint32_t* tau_top = reinterpret_cast<uint32_t*>(counters + 12);
-    // Kruskal's first n - n_c merges are the lightest n - n_c edges of the minimum spanning
-    // forest of any score prefix whose forest has that many edges; the forest of a longer
-    // prefix is the shorter prefix's forest plus Boruvka over the next slab of scores between
-    // its components.  So the selection starts with about 1.5 (n - n_c) edges and, when their
-    // forest falls short, extends it slab by slab (twice the edges each time) instead of
-    // starting over.
-    int64_t need = k_need + k_need / 2;
-    bool use_prefix = !batched && m > 65536 && k_need > 0 && need < m;
-    // the threshold's histogram samples one key chunk in eight on large selections
-    const int hist_samp = m >= (int64_t{1} << 22) ? 3 : 0;
-    uint32_t* tau_lo = reinterpret_cast<uint32_t*>(counters + 14);
+    constexpr bool two = MinKey<KT>::two_phase;
     int32_t* pos = W.c_pos.as<int32_t>();
     int64_t n_msf = 0;
-    // a batch: every graph its own prefix (k_graph_prefix), which needs the graph of every node
     int32_t* node_graph = W.node_graph.as<int32_t>();
-    if (batched) {
-        SPC_LAUNCH(ctx, k_node_graph, grid_for(n, kThreads, maxb), kThreads, 0, n, sa.B,
-                   sa.d_graph_ptr, node_graph);
-    }
-    const bool use_gprefix = batched && m > 65536 && sa.d_graph_ptr && sa.d_targets;
+    SPC_LAUNCH(ctx, k_node_graph, grid_for(n, kThreads, maxb), kThreads, 0, n, sa.B,
+               sa.d_graph_ptr, node_graph);
+    const bool use_gprefix = m > 65536 && sa.d_graph_ptr && sa.d_targets;
     GraphSlab<KT> gs{nullptr, nullptr, nullptr};
     int64_t* g_need = nullptr;
     KT* g_tau = nullptr;
@@ -1265,43 +1681,10 @@ spc_status select_typed(spc_context* ctx, const GraphView& g, const KT* key,
         gs = GraphSlab<KT>{node_graph, g_tau, g_lo};
     }
     for (int attempt = 0;; ++attempt) {
-        const bool two = MinKey<KT>::two_phase;
-        if (use_gprefix) {
-            if (attempt == 0)
-                SPC_LAUNCH(ctx, k_graph_prefix<KT>, g_grid, kGpThreads, 0, sa.B, 0,
-                           sa.d_graph_ptr, W.up_ptr.as<int32_t>(), sa.d_targets, key,
-                           W.msf.as<uint8_t>(), g_need, g_tau, g_lo, g_short);
-        } else if (use_prefix) {
-            SPC_TRY(ensure_key_hist(ctx));
-            static std::atomic<unsigned long long> attr_devs{0};  // devices already set up
-            const unsigned long long bit = 1ull << (ctx->device & 63);
-            if (!(attr_devs.load() & bit)) {
-                SPC_CUDA(cudaFuncSetAttribute(k_key_hist<KT>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              32768 * 4));
-                attr_devs.fetch_or(bit);
-            }
-            if (attempt > 0) {
-                // the histogram is still there: only the threshold moves up
-                SPC_LAUNCH(ctx, k_bump_slab, 1, 32, 0, tau_top, tau_lo);
-            } else {
-                SPC_CUDA(cudaMemsetAsync(W.key_hist.p, 0, (size_t)kTauBins * 4, ctx->stream));
-                note_bytes(ctx, (double)m * sizeof(KT) / (double)(1 << hist_samp));
-                SPC_LAUNCH(ctx, k_key_hist<KT>, ctx->num_sms, 1024, 32768 * 4, m, key,
-                           tau_shift, hist_samp, W.key_hist.as<uint32_t>());
-            }
-            // the histogram counts one key in 2^hist_samp
-            const int64_t need_s = (need + (int64_t{1} << hist_samp) - 1) >> hist_samp;
-            SPC_LAUNCH(ctx, k_pick_tau, 1, 1024, 0, W.key_hist.as<uint32_t>(), need_s, tau_top);
-        } else if (attempt > 0) {
-            SPC_LAUNCH(ctx, k_bump_slab, 1, 32, 0, tau_top, tau_lo);
-        }
-        const uint32_t* slab_lo = (attempt > 0 && !use_gprefix) ? tau_lo : nullptr;
-        // the slab of a very large single-graph selection: its edges become the first work
-        // list, so the first round does not sweep every edge.  Below kSlabListMin edges, and
-        // for a batch's per-graph slabs, the extra pass costs more than the sweep it replaces.
-        const bool slab_list = !batched && m >= kSlabListMin && (use_prefix || slab_lo) &&
-                               (reinterpret_cast<uintptr_t>(key) & 15) == 0;
+        if (use_gprefix && attempt == 0)
+            SPC_LAUNCH(ctx, k_graph_prefix<KT>, g_grid, kGpThreads, 0, sa.B, 0, sa.d_graph_ptr,
+                       W.up_ptr.as<int32_t>(), sa.d_targets, key, W.msf.as<uint8_t>(), g_need,
+                       g_tau, g_lo, g_short);
         if (attempt == 0) {
             SPC_LAUNCH(ctx, k_bv_init, grid_for(n > m ? n : m + 1, kThreads, maxb), kThreads, 0,
                        n, m, parent, W.best_k[0].as<unsigned long long>(),
@@ -1316,56 +1699,42 @@ spc_status select_typed(spc_context* ctx, const GraphView& g, const KT* key,
                        two ? W.best_e[0].as<int32_t>() : nullptr,
                        two ? W.best_e[1].as<int32_t>() : nullptr, counters);
         }
-        if (slab_list) {
-            note_bytes(ctx, (double)m * sizeof(KT) + (double)std::min<int64_t>(need, m) * 20);
-            SPC_LAUNCH(ctx, k_slab_list<KT>, grid_for(m, kThreads * kSlItems, maxb), kThreads,
-                       0, m, W.eu.as<int32_t>(), W.ev.as<int32_t>(), key, tau_shift,
-                       use_prefix ? tau_top : nullptr, slab_lo, W.wl_e[0].as<int32_t>(),
-                       W.wl_u[0].as<int32_t>(), W.wl_v[0].as<int32_t>(), counters);
-        }
-        // ---- 1. Boruvka minimum spanning forest (of the prefix) ---------------------------
-        // the first round reads the edges themselves (filtered by the slab) unless the slab
-        // list holds them; its count is then known on the device only
-        const bool scan0 = !slab_list;
+        // ---- 1. Boruvka minimum spanning forest (of the prefixes) ------------------------
         int64_t cur = m;
         for (int round = 0; cur > 0; ++round) {
             const int in = round & 1, out = in ^ 1;
             const int par = round & 1;
-            const int first = (round == 0 && scan0) ? 1 : 0;
+            const int first = round == 0 ? 1 : 0;  // reads the edges themselves
             const int direct = (round == 0 && attempt == 0) ? 1 : 0;
-            if (cur <= kFinishMax && (round > 0 || scan0)) {  // the remaining rounds in one CTA
+            if (cur <= kFinishMax) {  // the remaining rounds in one CTA
                 note_bytes(ctx, first ? (double)m * (8 + sizeof(KT))
                                       : (double)cur * (12 + sizeof(KT) + 8 + 32 + 12));
                 SPC_LAUNCH(ctx, k_bv_finish<KT>, 1, kFinishThreads, 0, first, par,
                            m, counters + in, W.wl_e[in].as<int32_t>(), W.wl_u[in].as<int32_t>(),
                            W.wl_v[in].as<int32_t>(), W.wl_e[out].as<int32_t>(),
                            W.wl_u[out].as<int32_t>(), W.wl_v[out].as<int32_t>(),
-                           W.eu.as<int32_t>(), W.ev.as<int32_t>(), key, tau_shift,
-                           use_prefix ? tau_top : nullptr, slab_lo, gs, parent,
+                           W.eu.as<int32_t>(), W.ev.as<int32_t>(), key, gs, parent,
                            W.best_k[0].as<unsigned long long>(),
                            W.best_k[1].as<unsigned long long>(),
-                           MinKey<KT>::two_phase ? W.best_e[0].as<int32_t>() : nullptr,
-                           MinKey<KT>::two_phase ? W.best_e[1].as<int32_t>() : nullptr,
-                           W.msf.as<uint8_t>(), status);
+                           two ? W.best_e[0].as<int32_t>() : nullptr,
+                           two ? W.best_e[1].as<int32_t>() : nullptr, W.msf.as<uint8_t>(),
+                           status);
                 break;
             }
             // algorithmic bytes: the first round reads every edge's ends and key; a later one
             // reads each work-list item (e, u, v) and key, walks two parents, lowers two best
             // slots (read and write) and writes the item back
-            // (a first round over the slab list: about `need` items)
-            const double items = round > 0 ? (double)cur : (double)std::min<int64_t>(need, m);
             note_bytes(ctx, first ? (double)m * (8 + sizeof(KT))
-                                  : items * (12 + sizeof(KT) + 8 + 32 + 12));
+                                  : (double)cur * (12 + sizeof(KT) + 8 + 32 + 12));
             SPC_LAUNCH(ctx, k_bv_minkey<KT>,
                        grid_for(cur, kThreads * kMkItems, maxb), kThreads, 0,
                        first, direct, m, counters + in,
                        W.wl_e[in].as<int32_t>(), W.wl_u[in].as<int32_t>(),
-                       W.wl_v[in].as<int32_t>(), W.eu.as<int32_t>(), W.ev.as<int32_t>(), key,
-                       tau_shift, use_prefix ? tau_top : nullptr, slab_lo, gs, parent,
-                       W.best_k[par].as<unsigned long long>(), W.wl_e[out].as<int32_t>(),
+                       W.wl_v[in].as<int32_t>(), W.eu.as<int32_t>(), W.ev.as<int32_t>(), key, gs,
+                       parent, W.best_k[par].as<unsigned long long>(), W.wl_e[out].as<int32_t>(),
                        W.wl_u[out].as<int32_t>(), W.wl_v[out].as<int32_t>(), counters + out,
                        status);
-            if (MinKey<KT>::two_phase) {
+            if (two) {
                 note_bytes(ctx, (double)cur * (12 + 8 + 16 + 8));
                 SPC_LAUNCH(ctx, k_bv_tiebreak, grid_for(cur, kThreads, maxb), kThreads, 0,
                            counters + out, W.wl_e[out].as<int32_t>(), W.wl_u[out].as<int32_t>(),
@@ -1389,29 +1758,16 @@ spc_status select_typed(spc_context* ctx, const GraphView& g, const KT* key,
         }
         SPC_TRY(scan_flags_u8(ctx, W.msf.as<uint8_t>(), pos, m));
         SPC_TRY(read_i32(ctx, pos + m, &n_msf));
-        if (use_gprefix) {
-            // graphs whose forest falls short take their next slab; done when none does
-            SPC_CUDA(cudaMemsetAsync(g_short, 0, sizeof(int32_t), ctx->stream));
-            SPC_LAUNCH(ctx, k_graph_prefix<KT>, g_grid, kGpThreads, 0, sa.B, attempt + 1,
-                       sa.d_graph_ptr, W.up_ptr.as<int32_t>(), sa.d_targets, key,
-                       W.msf.as<uint8_t>(), g_need, g_tau, g_lo, g_short);
-            int64_t n_short = 0;
-            SPC_TRY(read_i32(ctx, g_short, &n_short));
-            if (n_short == 0) break;
-            if (attempt > 64) return SPC_ERR_TIMEOUT;  // each slab doubles: never reached
-            continue;
-        }
-        // the prefix's forest holds Kruskal's first n_msf merges; enough when >= n - n_c
-        if (!use_prefix || n_msf >= k_need) break;
-        // the next slab: twice the edges, or, when the forest came within 15 % of n - n_c,
-        // the prefix its yield so far extrapolates to, and a quarter more
-        int64_t next = need * 2;
-        if (n_msf * 20 >= k_need * 17) {
-            const int64_t est = (int64_t)((double)need * (double)k_need / (double)n_msf * 1.25);
-            next = std::min(next, std::max(est, need + need / 8));
-        }
-        need = next;
-        if (need >= m) use_prefix = false;  // the last slab: every remaining score
+        if (!use_gprefix) break;
+        // graphs whose forest falls short take their next slab; done when none does
+        SPC_CUDA(cudaMemsetAsync(g_short, 0, sizeof(int32_t), ctx->stream));
+        SPC_LAUNCH(ctx, k_graph_prefix<KT>, g_grid, kGpThreads, 0, sa.B, attempt + 1,
+                   sa.d_graph_ptr, W.up_ptr.as<int32_t>(), sa.d_targets, key,
+                   W.msf.as<uint8_t>(), g_need, g_tau, g_lo, g_short);
+        int64_t n_short = 0;
+        SPC_TRY(read_i32(ctx, g_short, &n_short));
+        if (n_short == 0) break;
+        if (attempt > 64) return SPC_ERR_TIMEOUT;  // each slab doubles: never reached
     }
     // ---- 2. lightest forest edges per graph ---------------------------------------------
     KT* sk = W.sel_key.as<KT>();
@@ -1419,44 +1775,6 @@ spc_status select_typed(spc_context* ctx, const GraphView& g, const KT* key,
     SPC_LAUNCH(ctx, k_compact_msf<KT>, grid_for(m, kThreads, maxb), kThreads, 0, m,
                W.msf.as<uint8_t>(), pos, key, sk, sv);
     const int key_bits = sizeof(KT) == 8 ? 63 : 31;  // scores are >= +0: sign bit clear
-    const int64_t k_single_sel = batched ? 0 : (n - sa.target > 0 ? n - sa.target : 0);
-    if (!batched && k_single_sel > 0 && k_single_sel < n_msf) {
-        // single graph, proper subset: exact radix select of the k lightest, no sort
-        constexpr int R = SelBits<KT>::kRounds;
-        SPC_TRY(ensure_key_hist(ctx));
-        uint32_t* hist = W.key_hist.as<uint32_t>() + kTauBins;
-        SelState* sst = reinterpret_cast<SelState*>(counters + 16);
-        int32_t* cn = counters + 52;
-        SPC_LAUNCH(ctx, k_rsel_init, 1, 1024, 0, sst, (unsigned long long)k_single_sel, hist,
-                   R * kSelBins, cn);
-        const int gsel = grid_for(n_msf, kThreads, ctx->num_sms * 2);
-        // two rounds over the whole forest, then the rest over the items still matching
-        constexpr int kFull = 2;
-        KT* ck = W.sel_key2.as<KT>();
-        uint32_t* cv = W.sel_val2.as<uint32_t>();
-        for (int r = 0; r < kFull; ++r) {
-            SPC_LAUNCH(ctx, k_rsel_round<KT>, gsel, kThreads, 0, r, n_msf, nullptr, sk, sv,
-                       hist, sst);
-        }
-        SPC_LAUNCH(ctx, k_rsel_compact<KT>, grid_for(n_msf, kThreads, maxb), kThreads, 0,
-                   kFull - 1, n_msf, sk, sv, sst, ck, cv, cn);
-        // few candidates (the usual case): the remaining rounds in one CTA; many (a level
-        // where a large share of the forest has exactly equal scores): a launch per round
-        int64_t ncand = 0;
-        SPC_TRY(read_i32(ctx, cn, &ncand));
-        if (ncand <= kRestMax) {
-            SPC_LAUNCH(ctx, k_rsel_rest<KT>, 1, kRestThreads, 0, kFull, cn, ck, cv, sst);
-        } else {
-            for (int r = kFull; r < R; ++r)
-                SPC_LAUNCH(ctx, k_rsel_round<KT>, grid_for(ncand, kThreads, ctx->num_sms * 2),
-                           kThreads, 0, r, 0, cn, ck, cv, hist, sst);
-        }
-        int32_t* parent2 = W.parent2.as<int32_t>();
-        SPC_LAUNCH(ctx, k_iota, grid_for(n, kThreads, maxb), kThreads, 0, parent2, n);
-        SPC_LAUNCH(ctx, k_rsel_unite<KT>, grid_for(n_msf, kThreads, maxb), kThreads, 0, n_msf, sk,
-                   sv, sst, W.eu.as<int32_t>(), W.ev.as<int32_t>(), parent2, merged, status);
-        return finish_select(ctx, g, sa, lift, n_c_out, graph_ptr_c, status_out, batched);
-    }
     if (sizeof(KT) == 8) {
         SPC_TRY(radix_sort_u64(ctx, reinterpret_cast<uint64_t*>(sk), sv,
                                W.sel_key2.as<uint64_t>(), W.sel_val2.as<uint32_t>(), n_msf,
@@ -1466,49 +1784,50 @@ spc_status select_typed(spc_context* ctx, const GraphView& g, const KT* key,
                                W.sel_key2.as<uint32_t>(), W.sel_val2.as<uint32_t>(), n_msf,
                                key_bits));
     }
-    uint32_t* gkey = nullptr;
-    int32_t* seg_start = nullptr;
-    int32_t* k_graph = nullptr;
     int32_t* cnt_dev = counters + 3;
     SPC_CUDA(cudaMemcpyAsync(cnt_dev, pos + m, sizeof(int32_t), cudaMemcpyDeviceToDevice,
                              ctx->stream));
-    if (batched) {
-        gkey = W.sel_key2.as<uint32_t>();  // reuse: free after the score sort
-        uint32_t* gval = sv;
-        SPC_LAUNCH(ctx, k_graph_keys, grid_for(n_msf, kThreads, maxb), kThreads, 0, cnt_dev,
-                   gval, W.eu.as<int32_t>(), node_graph, gkey);
-        int gbits = 1;
-        while ((1ll << gbits) < sa.B) ++gbits;
-        // stable sort by graph id keeps the score order inside every graph
-        SPC_TRY(radix_sort_u32(ctx, gkey, gval, W.t_key.as<uint32_t>(), W.t_val.as<uint32_t>(),
-                               n_msf, gbits));
-        seg_start = W.seg_start.as<int32_t>();
-        k_graph = W.k_graph.as<int32_t>();
-        SPC_LAUNCH(ctx, k_graph_segments, grid_for(sa.B, kThreads, maxb), kThreads, 0, sa.B,
-                   sa.d_graph_ptr, sa.d_targets, W.up_ptr.as<int32_t>(), pos, seg_start,
-                   k_graph);
-    }
+    uint32_t* gkey = W.sel_key2.as<uint32_t>();  // reuse: free after the score sort
+    SPC_LAUNCH(ctx, k_graph_keys, grid_for(n_msf, kThreads, maxb), kThreads, 0, cnt_dev, sv,
+               W.eu.as<int32_t>(), node_graph, gkey);
+    int gbits = 1;
+    while ((1ll << gbits) < sa.B) ++gbits;
+    // stable sort by graph id keeps the score order inside every graph
+    SPC_TRY(radix_sort_u32(ctx, gkey, sv, W.t_key.as<uint32_t>(), W.t_val.as<uint32_t>(), n_msf,
+                           gbits));
+    int32_t* seg_start = W.seg_start.as<int32_t>();
+    int32_t* k_graph = W.k_graph.as<int32_t>();
+    SPC_LAUNCH(ctx, k_graph_segments, grid_for(sa.B, kThreads, maxb), kThreads, 0, sa.B,
+               sa.d_graph_ptr, sa.d_targets, W.up_ptr.as<int32_t>(), pos, seg_start, k_graph);
     int32_t* parent2 = W.parent2.as<int32_t>();
     SPC_LAUNCH(ctx, k_iota, grid_for(n, kThreads, maxb), kThreads, 0, parent2, n);
-    const int64_t k_single = batched ? 0 : (n - sa.target > 0 ? n - sa.target : 0);
     if (n_msf > 0) {
-        SPC_LAUNCH(ctx, k_select_unite, grid_for(n_msf, kThreads, maxb), kThreads, 0, cnt_dev,
-                   sv, gkey, seg_start, k_graph, k_single, W.eu.as<int32_t>(),
-                   W.ev.as<int32_t>(), parent2, merged, status);
+        SPC_LAUNCH(ctx, k_select_unite, grid_for(n_msf, kThreads, maxb), kThreads, 0, cnt_dev, sv,
+                   gkey, seg_start, k_graph, W.eu.as<int32_t>(), W.ev.as<int32_t>(), parent2,
+                   merged, status);
     }
-    return finish_select(ctx, g, sa, lift, n_c_out, graph_ptr_c, status_out, batched);
+    return finish_batch(ctx, g, sa, lift, n_c_out, graph_ptr_c, status_out);
 }
 
 }  // namespace
+
+template <class KT>
+static spc_status select_any(spc_context* ctx, const GraphView& g, const void* score,
+                             const SelectArgs& sa, int32_t* lift, uint8_t* merged, int64_t* n_c,
+                             int64_t* graph_ptr_c, int32_t* status) {
+    const KT* key = static_cast<const KT*>(score);
+    if (sa.B > 1 || sa.d_graph_ptr != nullptr)
+        return select_batch<KT>(ctx, g, key, sa, lift, merged, n_c, graph_ptr_c, status);
+    return select_single<KT>(ctx, g, key, sa.target, lift, merged, n_c, status);
+}
 
 spc_status run_select(spc_context* ctx, const GraphView& g, const void* score,
                       const SelectArgs& sa, int32_t* lift, uint8_t* merged, int64_t* n_c,
                       int64_t* graph_ptr_c, int32_t* status) {
     if (score_is_f32(g.wtype))
-        return select_typed<unsigned int>(ctx, g, static_cast<const unsigned int*>(score), sa,
-                                          lift, merged, n_c, graph_ptr_c, status);
-    return select_typed<unsigned long long>(ctx, g, static_cast<const unsigned long long*>(score),
-                                            sa, lift, merged, n_c, graph_ptr_c, status);
+        return select_any<unsigned int>(ctx, g, score, sa, lift, merged, n_c, graph_ptr_c, status);
+    return select_any<unsigned long long>(ctx, g, score, sa, lift, merged, n_c, graph_ptr_c,
+                                          status);
 }
 
 }  // namespace spc

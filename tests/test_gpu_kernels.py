@@ -62,3 +62,28 @@ def test_pooling_routes(ctx, dtype, F, sizes):
         assert np.array_equal(_bits(xc), _bits(ref))
         gx = ctx.pool_features_backward(lt, n_c, put(g, shift)).cpu().numpy()
         assert np.array_equal(_bits(gx), _bits(ref_g))
+
+
+# the one-kernel merge selection: one CTA and many, the tail's item count, the score prefix's edge
+# count (65,536), one target per relabelling rule (n / 8), nothing to merge, everything to merge, a
+# disconnected graph (the target is not reached), equal scores (the edge id decides)
+@pytest.mark.parametrize("dtype", [np.float32, np.float64, np.int32])
+@pytest.mark.parametrize("n,p", [(2, 1.0), (40, 0.2), (513, 0.01), (1025, 0.004), (3000, 0.002),
+                                 (6000, 0.0036), (6000, 0.0038), (20000, 0.0006)])
+def test_selection_at_the_edges_of_its_phases(ctx, n, p, dtype):
+    from paper_2204_11757_gb300 import api
+    weight = "unit" if dtype == np.int32 else "float"
+    g = I.random_graph(n, p, seed=n, weight=weight, dtype=dtype, connected=n != 6000)
+    csr = api.CSR.from_graph(g)
+    for target in sorted({1, max(1, n // 256), max(1, n // 8 - 1), max(1, n // 8), max(1, n // 2),
+                          max(1, n - 1), n}):
+        ref = O.coarsen_level(g, target)
+        lift, n_c, st = ctx.coarsen(csr, target, levels=1)
+        assert n_c == ref.n_c and st == (1 if ref.n_c > target else 0)
+        assert np.array_equal(lift.cpu().numpy(), ref.lift)
+    f = ctx.score(csr)
+    target = max(1, n // 3)
+    ref = O.coarsen_level(g, target)
+    lift, merged, n_c, st = ctx.select_merges(csr, f, target)
+    assert n_c == ref.n_c and int(merged.sum()) == n - n_c
+    assert np.array_equal(lift.cpu().numpy(), ref.lift)
