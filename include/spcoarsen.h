@@ -256,6 +256,11 @@ SPC_API void spc_result_free(spc_context* ctx, spc_result* r);
  * host or device memory; used to read retained results into caller buffers. */
 SPC_API spc_status spc_copy(spc_context* ctx, void* dst, const void* src, size_t bytes);
 
+/* `count` copies as by spc_copy (bytes[i] from src[i] to dst[i]) with one wait for all of them.
+ * An entry of 0 bytes is skipped. */
+SPC_API spc_status spc_copy_many(spc_context* ctx, int32_t count, void* const* dst,
+                                 const void* const* src, const size_t* bytes);
+
 /* ---- single steps (the same kernels spc_coarsen runs) ------------------------------------- */
 
 /* S0-S3: validate g, weighted degrees, normalised rows, and the score of every undirected

@@ -157,13 +157,17 @@ class Context:
             raise TypeError(f"unsupported weight dtype {g.w.dtype}")
         return N.spc_csr(g.n, g.nnz, _ptr(g.rowptr), _ptr(g.col), _ptr(g.w), _DT[g.w.dtype])
 
-    def _copy_from(self, ptr, count: int, dtype, device=None) -> torch.Tensor:
-        t = torch.empty(max(count, 0), dtype=dtype, device=device or self.device)
-        if count > 0:
-            nbytes = count * t.element_size()
-            N.check(self.lib.spc_copy(self._handle, _ptr(t), ctypes.c_void_p(ptr), nbytes),
-                    "spc_copy")
-        return t
+    def _copy_many(self, parts) -> List[torch.Tensor]:
+        """Tensors copied from (pointer, count, dtype) parts, with one wait for all copies."""
+        out = [torch.empty(max(count, 0), dtype=dtype, device=self.device)
+               for _, count, dtype in parts]
+        k = len(parts)
+        N.check(self.lib.spc_copy_many(
+            self._handle, k, (N.P * k)(*[t.data_ptr() for t in out]),
+            (N.P * k)(*[p for p, _, _ in parts]),
+            (ctypes.c_size_t * k)(*[t.numel() * t.element_size() for t in out])),
+            "spc_copy_many")
+        return out
 
     @staticmethod
     def _score_dtype(w: torch.Tensor):
@@ -267,25 +271,36 @@ class Context:
         N.check(self.lib.spc_get_level(self._handle, l, ctypes.byref(info)), "spc_get_level")
         return info
 
-    def level(self, l: int, batched_B: Optional[int] = None) -> Level:
-        i = self.level_info(l)
+    def _level_parts(self, i: N.spc_level, batched_B: Optional[int]):
+        """(pointer, count, dtype) of every array of one level, by the names of Level."""
         wt = _TD[i.wtype]
         st = _TD[i.scoretype]
         acc = torch.int64 if i.wtype == N.SPC_I32 else wt
-        cp = self._copy_from
-        return Level(
-            n=i.n, m=i.m, n_c=i.n_c, m_c=i.m_c, m_inter=i.m_inter, status=i.status, ms=i.ms,
-            score=cp(i.score, i.m, st), lift=cp(i.lift, i.n, torch.int32),
-            emap=cp(i.emap, i.m, torch.int32), self_mass=cp(i.self_mass, i.n_c, acc),
-            a_und=cp(i.a_und, i.m_c, wt), rowptr_c=cp(i.rowptr_c, i.n_c + 1, torch.int64),
-            col_c=cp(i.col_c, 2 * i.m_c, torch.int32), w_c=cp(i.w_c, 2 * i.m_c, wt),
-            perm=cp(i.perm, i.m_inter, torch.int32), seg=cp(i.seg, i.m_c + 1, torch.int32),
-            graph_ptr_c=(cp(i.graph_ptr_c, batched_B + 1, torch.int64)
-                         if batched_B is not None else None),
-            mass=cp(i.mass, i.n_c, acc) if i.mass else None)
+        parts = dict(
+            score=(i.score, i.m, st), lift=(i.lift, i.n, torch.int32),
+            emap=(i.emap, i.m, torch.int32), self_mass=(i.self_mass, i.n_c, acc),
+            a_und=(i.a_und, i.m_c, wt), rowptr_c=(i.rowptr_c, i.n_c + 1, torch.int64),
+            col_c=(i.col_c, 2 * i.m_c, torch.int32), w_c=(i.w_c, 2 * i.m_c, wt),
+            perm=(i.perm, i.m_inter, torch.int32), seg=(i.seg, i.m_c + 1, torch.int32))
+        if batched_B is not None:
+            parts["graph_ptr_c"] = (i.graph_ptr_c, batched_B + 1, torch.int64)
+        if i.mass:
+            parts["mass"] = (i.mass, i.n_c, acc)
+        return parts
+
+    def _copy_levels(self, which, batched_B: Optional[int]) -> List[Level]:
+        infos = [self.level_info(l) for l in which]
+        parts = [self._level_parts(i, batched_B) for i in infos]
+        copies = iter(self._copy_many([v for p in parts for v in p.values()]))
+        return [Level(n=i.n, m=i.m, n_c=i.n_c, m_c=i.m_c, m_inter=i.m_inter, status=i.status,
+                      ms=i.ms, **{name: next(copies) for name in p})
+                for i, p in zip(infos, parts)]
+
+    def level(self, l: int, batched_B: Optional[int] = None) -> Level:
+        return self._copy_levels([l], batched_B)[0]
 
     def levels(self, batched_B: Optional[int] = None) -> List[Level]:
-        return [self.level(l, batched_B) for l in range(self.level_count())]
+        return self._copy_levels(range(self.level_count()), batched_B)
 
     def compose_emap(self) -> torch.Tensor:
         m = self.level_info(0).m
@@ -378,13 +393,16 @@ class Result:
 
     def tensors(self) -> dict:
         """Copies of every buffer as tensors on the context's device."""
-        r, cp = self._r, self.context._copy_from
+        r = self._r
         acc = torch.int64 if self.wtype == torch.int32 else self.wtype
-        out = {"lift": cp(r.lift, self.n, torch.int32), "emap": cp(r.emap, self.m, torch.int32),
-               "rowptr_c": cp(r.rowptr_c, self.n_c + 1, torch.int64),
-               "col_c": cp(r.col_c, 2 * self.m_c, torch.int32),
-               "w_c": cp(r.w_c, 2 * self.m_c, self.wtype)}
-        out["mass"] = cp(r.mass, self.n_c, acc) if r.mass else None
+        parts = {"lift": (r.lift, self.n, torch.int32), "emap": (r.emap, self.m, torch.int32),
+                 "rowptr_c": (r.rowptr_c, self.n_c + 1, torch.int64),
+                 "col_c": (r.col_c, 2 * self.m_c, torch.int32),
+                 "w_c": (r.w_c, 2 * self.m_c, self.wtype)}
+        if r.mass:
+            parts["mass"] = (r.mass, self.n_c, acc)
+        out = dict(zip(parts, self.context._copy_many(list(parts.values()))))
+        out.setdefault("mass", None)
         return out
 
     def free(self):

@@ -801,10 +801,12 @@ k_backward(int64_t m, const int32_t* __restrict__ emap, const WT* __restrict__ g
 }
 
 // Sums of the segments that k_segsum_short left to the long list: integer weights by CTA
-// reductions, floating point by per-binade tables (exact left-to-right sums).
+// reductions, floating point by per-binade tables (exact left-to-right sums).  nlong: their number
+// when the host knows it.
 template <class WT, class Out>
 spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint32_t* idx,
-                             const uint32_t* key, const WT* w_und, Out* out) {
+                             const uint32_t* key, const WT* w_und, Out* out,
+                             int64_t nlong = -1) {
     Work& W = ctx->work;
     const bool side = on_side(ctx);
     int32_t* long_list = (side ? W.long_segs_side : W.long_segs).as<int32_t>();
@@ -814,8 +816,7 @@ spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint3
                    w_und, out, long_list, long_cnt, ctx->d_status);
         return SPC_OK;
     } else {
-        int64_t nlong = 0;
-        SPC_TRY(read_i32(ctx, long_cnt, &nlong));
+        if (nlong < 0) SPC_TRY(read_i32(ctx, long_cnt, &nlong));
         if (nlong == 0) return SPC_OK;
         int64_t* len = (side ? W.seg_len_side : W.seg_len).as<int64_t>();
         int64_t* base = (side ? W.seg_base_side : W.seg_base).as<int64_t>();
@@ -926,6 +927,9 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
     const int64_t long_c = bv[6], long_i = bv[7];  // buckets longer than kSmallBucket
     const int64_t m_inter = bv[0];
     const int64_t m_intra = bv[1];
+    // no segment is longer than its bucket: without a long bucket no list of long segments is read
+    const bool long_inter = bv[3] > kLongRow, long_intra = bv[5] > kLongRow;
+    lv.max_intra = bv[5];
     const bool buckets = bv[3] <= kBlockBucket && bv[5] <= kBlockBucket;
     if (buckets) {
         if (m > 0) {
@@ -976,8 +980,9 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         SPC_LAUNCH(ctx, (k_segsum_short<WT, Acc>), grid_for(n_c, kThreads, maxb), kThreads, 0,
                    n_c, off_i, ival2, nullptr, W.w_und.as<WT>(), self_mass,
                    W.long_segs_side.as<int32_t>(), W.counters.as<int32_t>() + 11, status);
-        SPC_TRY((long_segment_sums<WT, Acc>(ctx, off_i, ival2, nullptr, W.w_und.as<WT>(),
-                                             self_mass)));
+        if (long_intra)
+            SPC_TRY((long_segment_sums<WT, Acc>(ctx, off_i, ival2, nullptr, W.w_und.as<WT>(),
+                                                 self_mass)));
     } else {
         // self-mass: runs of equal super-node ids after a stable sort, summed in eid order
         SPC_TRY(radix_sort_u32(ctx, ikey, ival, W.i_key2.as<uint32_t>(),
@@ -997,8 +1002,9 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
             SPC_LAUNCH(ctx, (k_segsum_short<WT, Acc>), grid_for(n_runs, kThreads, maxb),
                        kThreads, 0, n_runs, istart, ival, ikey, W.w_und.as<WT>(), self_mass,
                        long_list, long_cnt, status);
-            SPC_TRY((long_segment_sums<WT, Acc>(ctx, istart, ival, ikey, W.w_und.as<WT>(),
-                                                 self_mass)));
+            if (long_intra)
+                SPC_TRY((long_segment_sums<WT, Acc>(ctx, istart, ival, ikey, W.w_und.as<WT>(),
+                                                     self_mass)));
         }
     }
     side->leave();
@@ -1063,8 +1069,9 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(m_c, kThreads, maxb), kThreads, 0,
                    m_c, seg, reinterpret_cast<const uint32_t*>(perm), nullptr, W.w_und.as<WT>(),
                    a_und, long_list, long_cnt, status);
-        SPC_TRY((long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm),
-                                            nullptr, W.w_und.as<WT>(), a_und)));
+        if (long_inter)
+            SPC_TRY((long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm),
+                                                nullptr, W.w_und.as<WT>(), a_und)));
     }
     if (m_c > 0) {
         const int gc = grid_for(m_c, kThreads, maxb);
@@ -1100,7 +1107,7 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
 template <class WT>
 spc_status forward_typed(spc_context* ctx, const int32_t* perm, const int32_t* seg, int64_t m_c,
                          const WT* w_und, WT* a_und) {
-    if (m_c <= 0) return SPC_OK;
+    if (m_c <= 0) return sync_status(ctx);
     Work& W = ctx->work;
     const size_t M = (size_t)m_c + 1;
     SPC_TRY(ensure(ctx, W.long_segs, M * 4));
@@ -1114,8 +1121,17 @@ spc_status forward_typed(spc_context* ctx, const int32_t* perm, const int32_t* s
     SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(m_c, kThreads, ctx->num_sms * 8), kThreads,
                0, m_c, seg, reinterpret_cast<const uint32_t*>(perm), nullptr, w_und, a_und,
                long_list, long_cnt, ctx->d_status);
-    return long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm), nullptr,
-                                     w_und, a_und);
+    int64_t vals[2];
+    {
+        const void* ptrs[2] = {long_cnt, ctx->d_status};
+        const int bytes[2] = {4, 4};
+        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, vals));
+        const spc_status st = status_from_bits((uint32_t)vals[1]);
+        if (st < 0 || vals[0] == 0) return st;
+    }
+    SPC_TRY((long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm), nullptr,
+                                       w_und, a_und, vals[0])));
+    return sync_status(ctx);
 }
 
 // ---- the self-mass reading of the multilevel driver ----------------------------------------
@@ -1276,7 +1292,8 @@ k_diag_place(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __res
 
 template <class WT>
 spc_status carry_mass_typed(spc_context* ctx, int64_t n, const int32_t* lift, int64_t n_c,
-                            const void* prev_mass, const void* self_mass, Buf& mass_out) {
+                            const void* prev_mass, const void* self_mass, int64_t max_intra,
+                            Buf& mass_out) {
     using Acc = typename CT<WT>::Acc;
     Work& W = ctx->work;
     const int maxb = ctx->num_sms * 8;
@@ -1307,7 +1324,9 @@ spc_status carry_mass_typed(spc_context* ctx, int64_t n, const int32_t* lift, in
         SPC_LAUNCH(ctx, k_set_i32, 1, 32, 0, long_cnt, 0);
         SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(n_c, kThreads, maxb), kThreads, 0,
                    n_c, start, val, nullptr, prev, out, long_list, long_cnt, ctx->d_status);
-        SPC_TRY((long_segment_sums<WT, WT>(ctx, start, val, nullptr, prev, out)));
+        // a super-node is connected by its intra edges: at most max_intra + 1 members
+        if (max_intra >= kLongRow)
+            SPC_TRY((long_segment_sums<WT, WT>(ctx, start, val, nullptr, prev, out)));
         SPC_LAUNCH(ctx, k_mass_add_self<WT>, grid_for(n_c, kThreads, maxb), kThreads, 0, n_c,
                    self, out);
         return SPC_OK;
@@ -1399,16 +1418,19 @@ namespace spc {
 
 spc_status run_carry_mass(spc_context* ctx, int64_t n, const int32_t* lift, int64_t n_c,
                           const void* prev_mass, const void* self_mass, spc_dtype wt,
-                          Buf& mass_out, const void** mass_ptr) {
+                          int64_t max_intra, Buf& mass_out, const void** mass_ptr) {
     if (!prev_mass) {  // nothing carried in: (0 + 0 + ...) + self = self, bit for bit
         *mass_ptr = self_mass;
         return SPC_OK;
     }
     spc_status st = SPC_ERR_INVALID_ARG;
     switch (wt) {
-        case SPC_I32: st = carry_mass_typed<int32_t>(ctx, n, lift, n_c, prev_mass, self_mass, mass_out); break;
-        case SPC_F32: st = carry_mass_typed<float>(ctx, n, lift, n_c, prev_mass, self_mass, mass_out); break;
-        case SPC_F64: st = carry_mass_typed<double>(ctx, n, lift, n_c, prev_mass, self_mass, mass_out); break;
+        case SPC_I32: st = carry_mass_typed<int32_t>(ctx, n, lift, n_c, prev_mass, self_mass, max_intra,
+                                                mass_out); break;
+        case SPC_F32: st = carry_mass_typed<float>(ctx, n, lift, n_c, prev_mass, self_mass, max_intra,
+                                                mass_out); break;
+        case SPC_F64: st = carry_mass_typed<double>(ctx, n, lift, n_c, prev_mass, self_mass, max_intra,
+                                                mass_out); break;
     }
     *mass_ptr = st == SPC_OK ? mass_out.p : nullptr;
     return st;

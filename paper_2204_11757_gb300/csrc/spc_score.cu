@@ -1408,12 +1408,14 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
                W.lr_base.as<int64_t>(), W.lr_len.as<int64_t>(), W.lr_idx.as<int64_t>(),
                heavy_count);
     SPC_TRY(scan_i32(ctx, W.up_cnt.as<int32_t>(), W.up_ptr.as<int32_t>(), n));
-    // the edge count and the number of long rows
-    int64_t sizes[2];
+    // the edge count, the number of long rows, and the verdict of the row checks
+    int64_t sizes[3];
     {
-        const void* ptrs[2] = {W.up_ptr.as<int32_t>() + n, long_count};
-        const int bytes[2] = {4, 4};
-        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, sizes));
+        const void* ptrs[3] = {W.up_ptr.as<int32_t>() + n, long_count, status};
+        const int bytes[3] = {4, 4, 4};
+        SPC_TRY(read_vals(ctx, 3, ptrs, bytes, sizes));
+        const spc_status st = status_from_bits((uint32_t)sizes[2]);
+        if (st < 0) return st;
     }
     const int64_t m = sizes[0];
     const int64_t n_long = sizes[1];
@@ -1422,9 +1424,8 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
         SPC_LAUNCH(ctx, k_long_rows_flat<WT>, maxb, kThreads, 0, n, g.rowptr, g.col,
                    static_cast<const WT*>(g.w), validate ? 1 : 0, long_rows, long_count,
                    W.lr_eoff.as<int64_t>(), W.deg.as<Acc>(), status);
+        if (validate) SPC_TRY(check_status(ctx));  // the long rows' checks
     }
-    // every input check of every row so far
-    SPC_TRY(check_status(ctx));
     if (2 * m + g.ndiag != nnz) return SPC_ERR_NOT_SYMMETRIC;
     g.m = m;
     // rowptr, columns, weights, degrees and row counts read once; p and the undirected edge

@@ -85,6 +85,8 @@ SIGNATURES = {
     "spc_level_count": (ctypes.c_int32, [P]),
     "spc_get_level": (ctypes.c_int, [P, ctypes.c_int32, ctypes.POINTER(spc_level)]),
     "spc_copy": (ctypes.c_int, [P, P, P, ctypes.c_size_t]),
+    "spc_copy_many": (ctypes.c_int, [P, ctypes.c_int32, ctypes.POINTER(P), ctypes.POINTER(P),
+                                     ctypes.POINTER(ctypes.c_size_t)]),
     "spc_take_result": (ctypes.c_int, [P, ctypes.POINTER(spc_result)]),
     "spc_result_free": (None, [P, ctypes.POINTER(spc_result)]),
     "spc_score": (ctypes.c_int, [P, ctypes.POINTER(spc_csr), P, PI64]),

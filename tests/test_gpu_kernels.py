@@ -87,3 +87,32 @@ def test_selection_at_the_edges_of_its_phases(ctx, n, p, dtype):
     lift, merged, n_c, st = ctx.select_merges(csr, f, target)
     assert n_c == ref.n_c and int(merged.sum()) == n - n_c
     assert np.array_equal(lift.cpu().numpy(), ref.lift)
+
+
+# segments and super-nodes around the 256 terms from which the tables of the long sums take over:
+# the contraction and the carried mass decide from the bucket sizes whether to look for them
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("leaves", [255, 256, 257, 258])
+def test_long_segments_found_from_bucket_sizes(ctx, dtype, leaves):
+    from paper_2204_11757_gb300 import api
+    # two hubs with a fan of light leaves each, a chain between the leaves of both: merging leaves
+    # one coarse edge of `leaves` fine edges and, a level later, super-nodes of about that many
+    rng = np.random.default_rng(leaves)
+    a, b = 0, leaves + 1
+    eu = np.concatenate([np.full(leaves, a), np.full(leaves, b), 1 + np.arange(leaves), [a]])
+    ev = np.concatenate([1 + np.arange(leaves), b + 1 + np.arange(leaves),
+                         b + 1 + np.arange(leaves), [b]])
+    g = I.csr_from_edges(2 * leaves + 2, eu, ev, rng.uniform(0.5, 2, eu.shape[0]).astype(dtype))
+    for ratio in (4, 32):
+        ref, total = O.coarsen(g, ratio, "halving")
+        lift, n_c, _ = ctx.coarsen(api.CSR.from_graph(g), ref[-1].target, levels=len(ref))
+        assert np.array_equal(lift.cpu().numpy(), total)
+        for lv, r in zip(ctx.levels(), ref):
+            assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(r.coarse.graph.w))
+            assert np.array_equal(_bits(lv.self_mass.cpu().numpy()), _bits(r.coarse.self_mass))
+            assert np.array_equal(_bits(lv.score.cpu().numpy()), _bits(r.f))
+    lift = np.repeat(np.int32([0, 1]), leaves + 1)
+    lv = ctx.contract(api.CSR.from_graph(g), torch.from_numpy(lift).cuda(), 2)
+    c = O.contract(g, lift, 2)
+    assert np.array_equal(_bits(lv.a_und.cpu().numpy()), _bits(c.a_und))
+    assert np.array_equal(_bits(lv.self_mass.cpu().numpy()), _bits(c.self_mass))
