@@ -561,6 +561,11 @@ k_run_starts(int64_t cnt, const uint8_t* __restrict__ head, const int32_t* __res
 // Segment sums: out[slot(r)] = sum of w_und[idx[j]] for j in [start[r], start[r+1]), left to
 // right.  slot(r) = r, or key[start[r]] when `key` is given (self-mass by super-node).  Short
 // segments: one thread each; segments longer than kLongRow go to a list for k_segsum_long.
+// terms in flight; device time over all launches of a call at 4 / 6 / 8 (before): 2048^2 mesh 690 /
+// 699 / 707 us (802), 129^3 mesh 1051 / 847 / 832 (1089), 2^23 points 932 / 971 / 1121 (1003), 2,500
+// meshes 868 / 850 / 1240 (975)
+constexpr int kSegFlight = 6;
+
 template <class WT, class Out>
 __global__ void __launch_bounds__(kThreads)
 k_segsum_short(int64_t nseg, const int32_t* __restrict__ start, const uint32_t* __restrict__ idx,
@@ -576,21 +581,20 @@ k_segsum_short(int64_t nseg, const int32_t* __restrict__ start, const uint32_t* 
             continue;
         }
         typename CT<WT>::Acc s = 0;
-        if (j1 - j0 <= 4) {
-            // short segment: every index and term in flight before the left-to-right sum
-            uint32_t ix[4];
-            WT t[4];
+        // kSegFlight indices, then their terms, in flight before the left-to-right additions (one
+        // term at a time, every term of a segment of more than four was a wait of its own)
+        for (int32_t j = j0; j < j1; j += kSegFlight) {
+            uint32_t ix[kSegFlight];
+            WT t[kSegFlight];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (j0 + q < j1) ix[q] = idx[j0 + q];
+            for (int q = 0; q < kSegFlight; ++q)
+                if (j + q < j1) ix[q] = idx[j + q];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (j0 + q < j1) t[q] = w_und[ix[q]];
+            for (int q = 0; q < kSegFlight; ++q)
+                if (j + q < j1) t[q] = w_und[ix[q]];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (j0 + q < j1) s = CT<WT>::add(s, t[q]);
-        } else {
-            for (int32_t j = j0; j < j1; ++j) s = CT<WT>::add(s, w_und[idx[j]]);
+            for (int q = 0; q < kSegFlight; ++q)
+                if (j + q < j1) s = CT<WT>::add(s, t[q]);
         }
         if constexpr (std::is_same<WT, int32_t>::value && sizeof(Out) == 4) {
             if (s > 2147483647ll) atomicOr(status, DEV_OVERFLOW);
