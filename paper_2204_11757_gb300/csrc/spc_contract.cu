@@ -560,7 +560,8 @@ k_run_starts(int64_t cnt, const uint8_t* __restrict__ head, const int32_t* __res
 
 // Segment sums: out[slot(r)] = sum of w_und[idx[j]] for j in [start[r], start[r+1]), left to
 // right.  slot(r) = r, or key[start[r]] when `key` is given (self-mass by super-node).  Short
-// segments: one thread each; segments longer than kLongRow go to a list for k_segsum_long.
+// segments: one thread each; segments longer than kLongRow go to a list (long_segment_sums), the
+// largest length to *longest (may be null).
 // terms in flight; device time over all launches of a call at 4 / 6 / 8 (before): 2048^2 mesh 690 /
 // 699 / 707 us (802), 129^3 mesh 1051 / 847 / 832 (1089), 2^23 points 932 / 971 / 1121 (1003), 2,500
 // meshes 868 / 850 / 1240 (975)
@@ -570,7 +571,7 @@ template <class WT, class Out>
 __global__ void __launch_bounds__(kThreads)
 k_segsum_short(int64_t nseg, const int32_t* __restrict__ start, const uint32_t* __restrict__ idx,
                const uint32_t* __restrict__ key, const WT* __restrict__ w_und, Out* __restrict__ out,
-               int32_t* __restrict__ long_list, int32_t* __restrict__ long_count,
+               int32_t* __restrict__ long_list, int32_t* long_count, int32_t* longest,
                uint32_t* status) {
     spc::pdl_wait();
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nseg;
@@ -578,6 +579,7 @@ k_segsum_short(int64_t nseg, const int32_t* __restrict__ start, const uint32_t* 
         const int32_t j0 = start[r], j1 = start[r + 1];
         if (j1 - j0 > kLongRow) {
             long_list[atomicAdd(long_count, 1)] = (int32_t)r;
+            if (longest) atomicMax(longest, j1 - j0);
             continue;
         }
         typename CT<WT>::Acc s = 0;
@@ -804,12 +806,12 @@ k_backward(int64_t m, const int32_t* __restrict__ emap, const WT* __restrict__ g
     }
 }
 
-// Sums of the segments that k_segsum_short left to the long list: integer weights by CTA
-// reductions, floating point by per-binade tables (exact left-to-right sums).  nlong: their number
-// when the host knows it.
+// Sums of the segments that k_segsum_short left to the long list, none longer than `bound`: integer
+// weights by CTA reductions, floating point exactly left to right, streamed or by per-binade tables.
+// nlong: their number when the host knows it.
 template <class WT, class Out>
 spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint32_t* idx,
-                             const uint32_t* key, const WT* w_und, Out* out,
+                             const uint32_t* key, const WT* w_und, Out* out, int64_t bound,
                              int64_t nlong = -1) {
     Work& W = ctx->work;
     const bool side = on_side(ctx);
@@ -820,6 +822,9 @@ spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint3
                    w_und, out, long_list, long_cnt, ctx->d_status);
         return SPC_OK;
     } else {
+        if (bound <= kStreamMax)
+            return stream_segments(ctx, std::is_same<WT, float>::value, long_cnt, long_list, start,
+                                   idx, key, w_und, out);
         if (nlong < 0) SPC_TRY(read_i32(ctx, long_cnt, &nlong));
         if (nlong == 0) return SPC_OK;
         int64_t* len = (side ? W.seg_len_side : W.seg_len).as<int64_t>();
@@ -983,10 +988,10 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         }
         SPC_LAUNCH(ctx, (k_segsum_short<WT, Acc>), grid_for(n_c, kThreads, maxb), kThreads, 0,
                    n_c, off_i, ival2, nullptr, W.w_und.as<WT>(), self_mass,
-                   W.long_segs_side.as<int32_t>(), W.counters.as<int32_t>() + 11, status);
+                   W.long_segs_side.as<int32_t>(), W.counters.as<int32_t>() + 11, nullptr, status);
         if (long_intra)
             SPC_TRY((long_segment_sums<WT, Acc>(ctx, off_i, ival2, nullptr, W.w_und.as<WT>(),
-                                                 self_mass)));
+                                                 self_mass, bv[5])));
     } else {
         // self-mass: runs of equal super-node ids after a stable sort, summed in eid order
         SPC_TRY(radix_sort_u32(ctx, ikey, ival, W.i_key2.as<uint32_t>(),
@@ -1005,10 +1010,10 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
             SPC_TRY(read_i32(ctx, ihpos + m_intra, &n_runs));
             SPC_LAUNCH(ctx, (k_segsum_short<WT, Acc>), grid_for(n_runs, kThreads, maxb),
                        kThreads, 0, n_runs, istart, ival, ikey, W.w_und.as<WT>(), self_mass,
-                       long_list, long_cnt, status);
+                       long_list, long_cnt, nullptr, status);
             if (long_intra)
                 SPC_TRY((long_segment_sums<WT, Acc>(ctx, istart, ival, ikey, W.w_und.as<WT>(),
-                                                     self_mass)));
+                                                     self_mass, bv[5])));
         }
     }
     side->leave();
@@ -1072,10 +1077,10 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
     if (m_c > 0) {
         SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(m_c, kThreads, maxb), kThreads, 0,
                    m_c, seg, reinterpret_cast<const uint32_t*>(perm), nullptr, W.w_und.as<WT>(),
-                   a_und, long_list, long_cnt, status);
+                   a_und, long_list, long_cnt, nullptr, status);
         if (long_inter)
             SPC_TRY((long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm),
-                                                nullptr, W.w_und.as<WT>(), a_und)));
+                                                nullptr, W.w_und.as<WT>(), a_und, bv[3])));
     }
     if (m_c > 0) {
         const int gc = grid_for(m_c, kThreads, maxb);
@@ -1121,20 +1126,21 @@ spc_status forward_typed(spc_context* ctx, const int32_t* perm, const int32_t* s
     SPC_TRY(ensure(ctx, W.seg_idx, M * 8));
     int32_t* long_list = W.long_segs.as<int32_t>();
     int32_t* long_cnt = W.counters.as<int32_t>() + 9;
-    SPC_CUDA(cudaMemsetAsync(long_cnt, 0, sizeof(int32_t), ctx->stream));
+    int32_t* longest = long_cnt + 1;
+    SPC_CUDA(cudaMemsetAsync(long_cnt, 0, 2 * sizeof(int32_t), ctx->stream));
     SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(m_c, kThreads, ctx->num_sms * 8), kThreads,
                0, m_c, seg, reinterpret_cast<const uint32_t*>(perm), nullptr, w_und, a_und,
-               long_list, long_cnt, ctx->d_status);
-    int64_t vals[2];
+               long_list, long_cnt, longest, ctx->d_status);
+    int64_t vals[3];
     {
-        const void* ptrs[2] = {long_cnt, ctx->d_status};
-        const int bytes[2] = {4, 4};
-        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, vals));
+        const void* ptrs[3] = {long_cnt, ctx->d_status, longest};
+        const int bytes[3] = {4, 4, 4};
+        SPC_TRY(read_vals(ctx, 3, ptrs, bytes, vals));
         const spc_status st = status_from_bits((uint32_t)vals[1]);
         if (st < 0 || vals[0] == 0) return st;
     }
     SPC_TRY((long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm), nullptr,
-                                       w_und, a_und, vals[0])));
+                                       w_und, a_und, vals[2], vals[0])));
     return sync_status(ctx);
 }
 
@@ -1327,10 +1333,11 @@ spc_status carry_mass_typed(spc_context* ctx, int64_t n, const int32_t* lift, in
         int32_t* long_cnt = W.counters.as<int32_t>() + 9;
         SPC_LAUNCH(ctx, k_set_i32, 1, 32, 0, long_cnt, 0);
         SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(n_c, kThreads, maxb), kThreads, 0,
-                   n_c, start, val, nullptr, prev, out, long_list, long_cnt, ctx->d_status);
+                   n_c, start, val, nullptr, prev, out, long_list, long_cnt, nullptr, ctx->d_status);
         // a super-node is connected by its intra edges: at most max_intra + 1 members
         if (max_intra >= kLongRow)
-            SPC_TRY((long_segment_sums<WT, WT>(ctx, start, val, nullptr, prev, out)));
+            SPC_TRY((long_segment_sums<WT, WT>(ctx, start, val, nullptr, prev, out,
+                                               max_intra + 1)));
         SPC_LAUNCH(ctx, k_mass_add_self<WT>, grid_for(n_c, kThreads, maxb), kThreads, 0, n_c,
                    self, out);
         return SPC_OK;

@@ -438,6 +438,16 @@ spc_status seqtab_full(spc_context* ctx, const void* terms, bool f32, int64_t ns
                        const int64_t* base, const int64_t* len, const int64_t* out_idx, void* out,
                        SeqTabBufs& tb);
 
+// The same full sums, one CTA per sequence and no tables, for sequences of at most kStreamMax terms:
+// rows w[base[q] .. + len[q]) into out[slot[q]], and segments list[q] of gathered terms (as
+// k_segsum_short sums them) into out[r] or out[key[start[r]]].  *count (device): the sequences.
+constexpr int64_t kStreamMax = 65536;
+spc_status stream_rows(spc_context* ctx, const void* w, bool f32, const int32_t* count,
+                       const int64_t* base, const int64_t* len, const int64_t* slot, void* out);
+spc_status stream_segments(spc_context* ctx, bool f32, const int32_t* count, const int32_t* list,
+                           const int32_t* start, const uint32_t* idx, const uint32_t* key,
+                           const void* w, void* out);
+
 // ---- steps (spc_score.cu, spc_merge.cu, spc_contract.cu) ----------------------------------
 
 struct GraphView {

@@ -146,7 +146,7 @@ k_long_rows_meta(const int64_t* __restrict__ rowptr, const int32_t* __restrict__
                  typename Tr<WT>::Acc* __restrict__ deg, int32_t* __restrict__ up_cnt,
                  int32_t* __restrict__ nlow_out, int64_t* __restrict__ lr_base,
                  int64_t* __restrict__ lr_len, int64_t* __restrict__ lr_idx,
-                 int32_t* __restrict__ heavy_count) {
+                 int32_t* __restrict__ heavy_count, int32_t* longest) {
     spc::pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) *heavy_count = 0;  // for k_score_hub
     const int32_t cnt = *long_count;
@@ -175,6 +175,7 @@ k_long_rows_meta(const int64_t* __restrict__ rowptr, const int32_t* __restrict__
             up_cnt[x] = (int32_t)(r1 - r0) - nl;
             lr_base[i] = r0;
             lr_len[i] = r1 - r0;
+            atomicMax(longest, (int32_t)(r1 - r0 < INT32_MAX ? r1 - r0 : INT32_MAX));
             lr_idx[i] = x;
             if constexpr (std::is_same<WT, int32_t>::value) deg[x] = 0;
         }
@@ -1397,7 +1398,8 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
     int32_t* long_rows = W.long_rows.as<int32_t>();
     const int gb = grid_for(n, kThreads, maxb);
     const double s_w = sizeof(WT), s_p = sizeof(P), s_acc = sizeof(Acc), s_key = sizeof(Key);
-    SPC_CUDA(cudaMemsetAsync(long_count, 0, sizeof(int32_t), ctx->stream));
+    int32_t* longest = long_count + 1;  // entries of the longest row
+    SPC_CUDA(cudaMemsetAsync(long_count, 0, 2 * sizeof(int32_t), ctx->stream));
     // rowptr, columns and weights read once; degree and the two per-row counts written once
     note_bytes(ctx, 8.0 * (n + 1) + nnz * (4 + s_w) + n * (s_acc + 8));
     SPC_LAUNCH(ctx, k_rows_degree<WT>, gb, kThreads, 0, n, nnz, g.rowptr, g.col,
@@ -1406,14 +1408,14 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
     SPC_LAUNCH(ctx, k_long_rows_meta<WT>, persist, kThreads, 0, g.rowptr, g.col, long_rows,
                long_count, W.deg.as<Acc>(), W.up_cnt.as<int32_t>(), W.first_up.as<int32_t>(),
                W.lr_base.as<int64_t>(), W.lr_len.as<int64_t>(), W.lr_idx.as<int64_t>(),
-               heavy_count);
+               heavy_count, longest);
     SPC_TRY(scan_i32(ctx, W.up_cnt.as<int32_t>(), W.up_ptr.as<int32_t>(), n));
     // the edge count, the number of long rows, and the verdict of the row checks
-    int64_t sizes[3];
+    int64_t sizes[4];
     {
-        const void* ptrs[3] = {W.up_ptr.as<int32_t>() + n, long_count, status};
-        const int bytes[3] = {4, 4, 4};
-        SPC_TRY(read_vals(ctx, 3, ptrs, bytes, sizes));
+        const void* ptrs[4] = {W.up_ptr.as<int32_t>() + n, long_count, status, longest};
+        const int bytes[4] = {4, 4, 4, 4};
+        SPC_TRY(read_vals(ctx, 4, ptrs, bytes, sizes));
         const spc_status st = status_from_bits((uint32_t)sizes[2]);
         if (st < 0) return st;
     }
@@ -1463,7 +1465,11 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
         if (n_long > 0) {
             side.reset(new SideBranch(ctx));
             SPC_TRY(side->status());
-            if (fp) {
+            if (fp && sizes[3] <= kStreamMax) {
+                SPC_TRY(stream_rows(ctx, g.w, std::is_same<WT, float>::value, long_count,
+                                    W.lr_base.as<int64_t>(), W.lr_len.as<int64_t>(),
+                                    W.lr_idx.as<int64_t>(), W.deg.p));
+            } else if (fp) {
                 SPC_TRY(seqtab_full(ctx, g.w, std::is_same<WT, float>::value, n_long,
                                     W.lr_base.as<int64_t>(), W.lr_len.as<int64_t>(),
                                     W.lr_idx.as<int64_t>(), W.deg.p, W.tab_w));

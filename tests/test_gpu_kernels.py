@@ -116,3 +116,47 @@ def test_long_segments_found_from_bucket_sizes(ctx, dtype, leaves):
     c = O.contract(g, lift, 2)
     assert np.array_equal(_bits(lv.a_und.cpu().numpy()), _bits(c.a_und))
     assert np.array_equal(_bits(lv.self_mass.cpu().numpy()), _bits(c.self_mass))
+
+
+# long sums (rows' degrees, coarse weights, self-masses) streamed by one CTA: lengths around the first
+# 32 terms and the blocks of 1,024 after them, the limit of 65,536 terms, terms over 60 binades, exact
+# half-grid ties, and leading zeros (the masses carried into a giant super-node)
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("L", [257, 1055, 1056, 1057, 2080, 4100, 65535, 65536, 65537])
+def test_streamed_long_sums(ctx, dtype, L):
+    from paper_2204_11757_gb300 import api
+    rng = np.random.default_rng(L)
+    ties = I.star_ties(12, dtype).w_und  # 1 + eps, 1 - eps in turn
+    for w in (rng.uniform(0.5, 2.0, L), np.exp2(rng.uniform(-40, 20, L)),
+              np.resize(np.asarray(ties), L), np.full(L, 0.1)):
+        w = w.astype(dtype)
+        g = I.csr_from_edges(L + 1, np.zeros(L, np.int64), 1 + np.arange(L), w)
+        if L < 5000:  # the hub's degree is in every score (the oracle's time grows with L^2)
+            f = ctx.score(api.CSR.from_graph(g)).cpu().numpy()
+            assert np.array_equal(_bits(f), _bits(O.score(g)))
+        lift = np.r_[np.int32(0), np.ones(L, np.int32)]
+        for lt, n_c in ((lift, 2), (np.zeros(L + 1, np.int32), 1)):
+            lv = ctx.contract(api.CSR.from_graph(g), torch.from_numpy(lt).cuda(), n_c)
+            c = O.contract(g, lt, n_c)
+            assert np.array_equal(_bits(lv.a_und.cpu().numpy()), _bits(c.a_und))
+            assert np.array_equal(_bits(lv.self_mass.cpu().numpy()), _bits(c.self_mass))
+            if n_c == 2:
+                a = ctx.contract_forward(lv.perm, lv.seg, lv.m_c, torch.from_numpy(w).cuda())
+                assert np.array_equal(_bits(a.cpu().numpy()), _bits(c.a_und))
+
+
+# one giant super-node per level whose members mostly carry no mass yet
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_streamed_masses_of_a_giant(ctx, dtype):
+    from paper_2204_11757_gb300 import api
+    rng = np.random.default_rng(3)
+    n = 3000
+    eu = np.r_[np.zeros(n - 1, np.int64), 1 + np.arange(n - 2)]
+    ev = np.r_[1 + np.arange(n - 1), 2 + np.arange(n - 2)]
+    g = I.csr_from_edges(n, eu, ev, rng.uniform(0.5, 2.0, eu.shape[0]).astype(dtype))
+    ref, total = O.coarsen(g, 64, "halving")
+    lift, n_c, _ = ctx.coarsen(api.CSR.from_graph(g), ref[-1].target, levels=len(ref))
+    assert np.array_equal(lift.cpu().numpy(), total)
+    for lv, r in zip(ctx.levels(), ref):
+        assert np.array_equal(_bits(lv.score.cpu().numpy()), _bits(r.f))
+        assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(r.coarse.graph.w))
