@@ -206,9 +206,8 @@ template <> struct MinKey<unsigned int> {
 
 // Boruvka phase A: current roots of both ends; keep inter-component edges; lower the
 // component minima.  The first Boruvka pass reads every edge directly and keeps only the
-// score prefix (key >> tau_shift <= *tau_top).  Each thread takes kMkItems edges per pass
-// (their loads overlap), and the survivors are appended with one global atomic per block
-// and pass.
+// score prefix.  Each thread takes kMkItems edges per pass (their loads overlap), and the
+// survivors are appended with one global atomic per block and pass.
 constexpr int kMkItems = 2;
 constexpr uint32_t kNoSlab = 0xffffffffu;  // no lower bound on the score slab
 
@@ -420,29 +419,45 @@ k_bv_finish(int round0, int par0, int64_t m, int32_t* count_in, int32_t* li_e, i
     }
 }
 
-// histogram of the top 15 bits of the scores (bits below the sign), per block in shared memory,
-// over a sample of the keys: one chunk of kHistChunk consecutive keys in every 2^samp (samp 0:
-// every key).  The threshold it gives only sizes the score prefix, never changes a result.
+// The score prefix's bins: 512 to a binade, 64 binades up to 2, the largest score there is (smaller
+// scores share bin 0, larger ones -- a caller's own -- the last bin).  The 15 highest bits of a
+// binary64 score gave 16 bins to a binade, and a level's scores lie within one or two: the first
+// prefix of the 129^3 mesh held 5.5 M edges instead of the 1.6 M asked for, its selection took 2.1
+// ms instead of 0.8 and the seven levels 19.8 instead of 18.4.
+constexpr int kTauBins = 32768;
+
+template <class KT>
+__device__ __forceinline__ uint32_t tau_bin(KT k) {
+    constexpr int kShift = sizeof(KT) == 8 ? 43 : 14;
+    constexpr KT kTwo = sizeof(KT) == 8 ? (KT)0x4000000000000000ull : (KT)0x40000000u;
+    constexpr KT kBase = (kTwo >> kShift) - (kTauBins - 1);
+    const KT b = k >> kShift;
+    return b <= kBase ? 0u : b - kBase >= (KT)kTauBins ? kTauBins - 1 : (uint32_t)(b - kBase);
+}
+
+// histogram of the scores' bins, per block in shared memory, over a sample of the keys: one chunk
+// of kHistChunk consecutive keys in every 2^samp (samp 0: every key).  The threshold it gives only
+// sizes the score prefix, never changes a result.
 constexpr int kHistChunk = 256;
 
 template <class KT>
 __global__ void __launch_bounds__(1024)
-k_key_hist(int64_t m, const KT* __restrict__ key, int shift, int samp,
+k_key_hist(int64_t m, const KT* __restrict__ key, int samp,
            uint32_t* __restrict__ hist) {
     spc::pdl_wait();
     extern __shared__ uint32_t sh_hist[];
-    for (int b = threadIdx.x; b < 32768; b += blockDim.x) sh_hist[b] = 0;
+    for (int b = threadIdx.x; b < kTauBins; b += blockDim.x) sh_hist[b] = 0;
     __syncthreads();
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = ((v / kHistChunk) << samp) * kHistChunk + v % kHistChunk;
         if (i >= m) break;  // i grows with v
-        const uint32_t b = (uint32_t)(key[i] >> shift) & 32767u;
+        const uint32_t b = tau_bin(key[i]);
         const unsigned peers = __match_any_sync(__activemask(), b);
         if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&sh_hist[b], __popc(peers));
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < 32768; b += blockDim.x)
+    for (int b = threadIdx.x; b < kTauBins; b += blockDim.x)
         if (sh_hist[b]) atomicAdd(hist + b, sh_hist[b]);
 }
 
@@ -882,7 +897,6 @@ spc_status finish_batch(spc_context* ctx, const GraphView& g, const SelectArgs& 
 
 // key_hist: the score-prefix histogram (kTauBins words, zero between selections), then the radix
 // select's histograms of every round (zeroed by the selection); zeroed once on allocation
-constexpr int kTauBins = 32768;
 constexpr size_t kKeyHistBytes = (size_t)(kTauBins + SelBits<uint64_t>::kRounds * kSelBins) * 4;
 static spc_status ensure_key_hist(spc_context* ctx) {
     return ensure_zeroed(ctx, ctx->work.key_hist, kKeyHistBytes);
@@ -925,7 +939,7 @@ struct CoopArgs {
     const int32_t* ev;
     const KT* key;
     uint32_t* hist;              // score histogram of the prefix (null: no prefix)
-    int tau_shift, hist_samp, slab_list;
+    int hist_samp, slab_list;
     int32_t* parent;
     int32_t* parent2;
     unsigned long long* bk[2];
@@ -1081,7 +1095,7 @@ __device__ __forceinline__ void coop_minkey(const CoopArgs<KT>& a, int64_t cnt, 
 #pragma unroll
         for (int it = 0; it < kMkItems; ++it) {
             if (kEdges && act[it]) {
-                const uint32_t bin = (uint32_t)(k[it] >> a.tau_shift);
+                const uint32_t bin = tau_bin(k[it]);
                 act[it] = bin <= top && (lo == kNoSlab || bin > lo);
             }
             rt[2 * it] = u[it];
@@ -1134,14 +1148,14 @@ __device__ __forceinline__ void coop_slab_list(const CoopArgs<KT>& a, uint32_t t
                 memcpy(k, &q, 16);
 #pragma unroll
                 for (int t = 0; t < (int)(16 / sizeof(KT)); ++t) {
-                    const uint32_t bin = (uint32_t)(k[t] >> a.tau_shift);
+                    const uint32_t bin = tau_bin(k[t]);
                     if (bin <= top && (lo == kNoSlab || bin > lo))
                         keep |= 1u << (j * (int)(16 / sizeof(KT)) + t);
                 }
             }
         } else {
             for (int it = 0; it < kSlItems && i0 + it < a.m; ++it) {
-                const uint32_t bin = (uint32_t)(a.key[i0 + it] >> a.tau_shift);
+                const uint32_t bin = tau_bin(a.key[i0 + it]);
                 if (bin <= top && (lo == kNoSlab || bin > lo)) keep |= 1u << it;
             }
         }
@@ -1576,7 +1590,6 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
     a.eu = W.eu.as<int32_t>();
     a.ev = W.ev.as<int32_t>();
     a.key = key;
-    a.tau_shift = sizeof(KT) == 8 ? 48 : 16;
     // the threshold's histogram samples one key chunk in eight on large selections
     a.hist_samp = m >= (int64_t{1} << 22) ? 3 : 0;
     a.slab_list = m >= kSlabListMin && (reinterpret_cast<uintptr_t>(key) & 15) == 0 ? 1 : 0;
@@ -1623,8 +1636,8 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
     if (m > 65536 && a.k_need > 0 && a.need < m) {
         a.hist = W.key_hist.as<uint32_t>();
         note_bytes(ctx, (double)m * sizeof(KT) / (double)(1 << a.hist_samp));
-        SPC_LAUNCH(ctx, k_key_hist<KT>, ctx->num_sms, 1024, kTauBins * 4, m, key, a.tau_shift,
-                   a.hist_samp, W.key_hist.as<uint32_t>());
+        SPC_LAUNCH(ctx, k_key_hist<KT>, ctx->num_sms, 1024, kTauBins * 4, m, key, a.hist_samp,
+                   W.key_hist.as<uint32_t>());
     }
     SPC_LAUNCH_COOP(ctx, k_select_coop<KT>, grid, kCoopThreads, a);
     int64_t vals[2];
