@@ -187,6 +187,23 @@ __global__ void k_expect(Expect x, int32_t* mismatch) {
     if (got != x.want[i]) *mismatch = 1;
 }
 
+// the values a read takes, written to pinned host memory by one launch (a copy per value was 1.5-2
+// us each on the stream, and a contraction reads eight)
+constexpr int kReadMax = 8;
+struct ReadVals {
+    const void* dev[kReadMax];
+    int bytes[kReadMax];
+    int count;
+};
+
+__global__ void k_read_vals(ReadVals x, int64_t* host) {
+    spc::pdl_wait();
+    const int i = threadIdx.x;
+    if (i >= x.count) return;
+    host[i] = x.bytes[i] == 8 ? *static_cast<const int64_t*>(x.dev[i])
+                              : (int64_t)*static_cast<const int32_t*>(x.dev[i]);
+}
+
 spc_status read_vals(spc_context* ctx, int count, const void* const* dev, const int* bytes,
                      int64_t* out) {
     Replay& R = ctx->replay;
@@ -205,14 +222,17 @@ spc_status read_vals(spc_context* ctx, int count, const void* const* dev, const 
         }
         return SPC_OK;
     }
+    if (count > kReadMax) return SPC_ERR_INVALID_ARG;
+    ReadVals x{};
+    x.count = count;
     for (int i = 0; i < count; ++i) {
-        SPC_CUDA(cudaMemcpyAsync(ctx->h_scalars + 16 + i, dev[i], bytes[i], cudaMemcpyDeviceToHost,
-                                 ctx->stream));
+        x.dev[i] = dev[i];
+        x.bytes[i] = bytes[i];
     }
+    SPC_LAUNCH(ctx, k_read_vals, 1, 32, 0, x, ctx->h_scalars + 16);
     SPC_CUDA(cudaStreamSynchronize(ctx->stream));
     for (int i = 0; i < count; ++i) {
-        out[i] = bytes[i] == 8 ? ctx->h_scalars[16 + i]
-                               : (int64_t)*reinterpret_cast<int32_t*>(ctx->h_scalars + 16 + i);
+        out[i] = ctx->h_scalars[16 + i];
         if (R.mode == Replay::kRecord) R.log.push_back(out[i]);
     }
     return SPC_OK;
