@@ -306,38 +306,51 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-// The rows of a tile of consecutive CSR entries [base, end), for kernels that run flat over the
-// stored entries: every thread of the block calls it (it synchronises the block).  Two searches
-// find the first row r_lo and the last row of the tile; one thread per row then marks the row
-// of each of its entries, s_row[j - base] = row - r_lo, or -2 - (row - r_lo) for a row of
-// more than `long_row` entries (long_row < 0: no limit).  Returns r_lo.  Rows spanned by a tile are
-// visited by that tile alone (neighbouring tiles share at most one row), so the marking is
-// O(rows + entries) over the whole array.
-__device__ __forceinline__ int64_t csr_last_row_at(const int64_t* __restrict__ rowptr, int64_t lo,
-                                                   int64_t hi, int64_t j) {
-    while (lo < hi) {  // the last row x in [lo, hi] with rowptr[x] <= j
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (rowptr[mid] <= j) lo = mid; else hi = mid - 1;
+// The rows of tiles of consecutive CSR entries, for kernels that run flat over the stored entries.
+// A block takes a contiguous range of tiles: csr_row_of finds the row of its first entry, and
+// tile_rows marches on from there (a search for every tile -- 23 dependent reads over 2^23 rows
+// while the block waits -- was most of such a kernel's time).
+//
+// csr_row_of: the last row x with rowptr[x] <= j, for an entry j < rowptr[n]; every lane of a warp
+// calls it (32 probes a step).
+__device__ __forceinline__ int64_t csr_row_of(const int64_t* __restrict__ rowptr, int64_t n,
+                                              int64_t j) {
+    const int lane = threadIdx.x & 31;
+    int64_t lo = 0, hi = n - 1;  // rowptr[lo] <= j; the answer lies in [lo, hi]
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t at = lo + (lane + 1) * step;
+        const bool below = at <= hi && rowptr[at] <= j;
+        const int k = __popc(__ballot_sync(0xffffffffu, below));  // row pointers ascend
+        const int64_t cap = lo + (k + 1) * step - 1;
+        lo += k * step;
+        hi = cap < hi ? cap : hi;
     }
     return lo;
 }
 
-__device__ __forceinline__ int64_t tile_rows(const int64_t* __restrict__ rowptr, int64_t n,
-                                             int64_t base, int64_t end, int64_t long_row,
-                                             int32_t* s_row, int64_t* s_rows) {
-    if (threadIdx.x < 2)
-        s_rows[threadIdx.x] = csr_last_row_at(rowptr, 0, n - 1, threadIdx.x ? end - 1 : base);
-    __syncthreads();
-    const int64_t r_lo = s_rows[0], r_hi = s_rows[1];
-    for (int64_t x = r_lo + threadIdx.x; x <= r_hi; x += blockDim.x) {
-        const int64_t r0 = rowptr[x], r1 = rowptr[x + 1];
+// tile_rows: for the tile [base, end) whose first entry lies in row r_lo, s_row[j - base] = row of
+// entry j minus r_lo, or -2 - that for a row of more than `long_row` entries (long_row < 0: no
+// limit), and fn(x, x - r_lo, r0, r1) once for every row x = [r0, r1) of the tile; *s_next = the row
+// of entry `end` (when there is one).  Every thread of the block calls it; the caller synchronises
+// the block before s_row, s_next and what fn wrote are read.
+template <class Fn>
+__device__ __forceinline__ void tile_rows(const int64_t* __restrict__ rowptr, int64_t n,
+                                          int64_t base, int64_t end, int64_t r_lo,
+                                          int64_t long_row, int32_t* s_row, int64_t* s_next,
+                                          const Fn& fn) {
+    for (int64_t x = r_lo + threadIdx.x; x < n; x += blockDim.x) {
+        const int64_t r0 = rowptr[x];
+        if (r0 > end) break;
+        const int64_t r1 = rowptr[x + 1];
+        if (r1 > end) *s_next = x;  // r0 <= end < r1: one row
+        if (r0 == end) continue;
         const int32_t rel = (int32_t)(x - r_lo);
         const int32_t mark = (long_row >= 0 && r1 - r0 > long_row) ? -2 - rel : rel;
         for (int64_t j = r0 > base ? r0 : base; j < (r1 < end ? r1 : end); ++j)
             s_row[j - base] = mark;
+        fn(x, rel, r0, r1);
     }
-    __syncthreads();
-    return r_lo;
 }
 
 template <typename... Params, typename... Args>

@@ -282,60 +282,6 @@ k_long_rows_edges(const int64_t* __restrict__ rowptr, const int32_t* __restrict_
     }
 }
 
-// S2 (+ the edge list): one thread per row.  p[j] = w[j] / d[x]; for the entries above the
-// diagonal writes the undirected edge (x, y) at its edge id; when `validate` (set only when no
-// score kernel follows: those check every upper entry's mirror on their walks), looks up the
-// mirror entry (y, x) by binary search and compares the weight bits.
-template <class WT>
-__global__ void __launch_bounds__(kThreads)
-k_rows_edges(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-             const WT* __restrict__ w, int validate, const typename Tr<WT>::Acc* __restrict__ deg,
-             const int32_t* __restrict__ nlow, const int32_t* __restrict__ up_ptr,
-             typename Tr<WT>::P* __restrict__ p, int32_t* __restrict__ eu,
-             int32_t* __restrict__ ev, WT* __restrict__ w_und, uint32_t* __restrict__ status) {
-    spc::pdl_wait();
-    if (*status) return;  // invalid input: nothing below may index with it
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) {
-        const int64_t r0 = rowptr[x], r1 = rowptr[x + 1];
-        if (r1 - r0 > kLongRow) continue;  // k_long_rows_edges
-        const typename Tr<WT>::Acc d = deg[x];
-        const int64_t ubase = (int64_t)up_ptr[x] - (r0 + nlow[x]);
-        // binary64 rows: one correctly rounded reciprocal per row, Markstein per entry
-        double dd = 0.0, rcp = 0.0;
-        bool d_mid = false;
-        if constexpr (!std::is_same<WT, float>::value) {
-            dd = (double)d;
-            d_mid = mid_range(dd);
-            rcp = d_mid ? __drcp_rn(dd) : 0.0;
-        }
-        uint32_t bits = 0;
-        for (int64_t j = r0; j < r1; ++j) {
-            const int32_t y = col[j];
-            const WT wj = w[j];
-            if constexpr (std::is_same<WT, float>::value) p[j] = Tr<WT>::div(wj, d);
-            else p[j] = div_row((double)wj, dd, rcp, d_mid);
-            if (validate) {
-                int64_t lo = rowptr[y], hi = rowptr[y + 1];
-                while (lo < hi) {
-                    int64_t mid = (lo + hi) >> 1;
-                    if ((int64_t)col[mid] < x) lo = mid + 1; else hi = mid;
-                }
-                if (lo >= rowptr[y + 1] || (int64_t)col[lo] != x ||
-                    Tr<WT>::bits(w[lo]) != Tr<WT>::bits(wj))
-                    bits |= DEV_NOT_SYMMETRIC;
-            }
-            if ((int64_t)y > x) {
-                const int64_t e = ubase + j;
-                eu[e] = (int32_t)x;
-                ev[e] = y;
-                w_und[e] = wj;
-            }
-        }
-        if (bits) atomicOr(status, bits);
-    }
-}
-
 // Symmetry fingerprint (S0) of a binary32 graph: every stored entry (x, y, w) off the diagonal
 // adds +H(min, max, bits of w) when x < y and -H(...) when x > y, modulo 2^64.  A symmetric
 // graph pairs every upper entry with a lower one of the same (min, max, w), so the sum is 0
@@ -356,49 +302,142 @@ __device__ __forceinline__ uint64_t sym_term(int64_t x, int32_t y, uint32_t wbit
     return (int64_t)y > x ? h : (uint64_t)0 - h;
 }
 
-// S2 (+ the edge list) for binary32 weights, flat over the stored entries: each block takes
-// kFlatTile consecutive entries and marks the row of each in shared memory (tile_rows), so the
-// columns, weights and p values of a warp are consecutive (the row-per-thread kernel reads 32
-// rows at once).  p = w / d is one IEEE division per entry, exactly as k_rows_edges computes
-// it.  `p` (may be null) receives p alone, `pk` the (column, p) pair of every entry.  Rows
-// longer than kLongRow are left to k_long_rows_edges.  With `sym` (input validation), every
-// entry of every row, long ones included, also adds its symmetry fingerprint term into *sym.
-constexpr int64_t kFlatTile = 2048;
+// raw bits of entry j of a weight array of wsize-byte elements (int32, binary32 or binary64)
+__device__ __forceinline__ uint64_t weight_bits(const void* w, int wsize, int64_t j) {
+    return wsize == 8 ? static_cast<const unsigned long long*>(w)[j]
+                      : (uint64_t)static_cast<const unsigned int*>(w)[j];
+}
 
+// true if row [j0, j1) (sorted) holds column a with weight bits wb: the mirror of entry (a, .)
+__device__ __forceinline__ bool has_mirror(const int32_t* __restrict__ col, const void* w,
+                                           int wsize, int64_t j0, int64_t j1, int64_t a,
+                                           uint64_t wb) {
+    int64_t lo = j0, hi = j1;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if ((int64_t)col[mid] < a) lo = mid + 1; else hi = mid;
+    }
+    return lo < j1 && (int64_t)col[lo] == a && weight_bits(w, wsize, lo) == wb;
+}
+
+// S2 (+ the edge list), flat over the stored entries: each block takes kFlatTile consecutive entries,
+// marks the row of each in shared memory (tile_rows) and keeps the rows' degrees, reciprocals and
+// edge-id bases there, so a warp's columns, weights and p values are consecutive (a thread per row
+// reads 32 rows at once).  p = w / d is the correctly rounded quotient: binary32 by the IEEE division, binary64
+// and integer weights by one reciprocal per row and Markstein's steps per entry.  Entries above the
+// diagonal write the undirected edge (x, y) at its edge id.  `p` receives p alone,
+// `pk` (binary32; both may be null, and without scores both are) the (column, p) pair of every entry and the end marker of every row.  Rows longer
+// than kLongRow are left to k_long_rows_edges.  With `sym` (input validation of binary32 rows), every
+// entry of every row, long ones included, also adds its symmetry fingerprint term into *sym.
+// Bound by the entries' traffic and, binary64, by that pipe (three operations an entry).  All
+// launches of a call, a thread per row or a search per tile before: 129^3 mesh 1.37 -> 0.67 ms, 2048^2
+// mesh 0.81 -> 0.66, 2^23 points 1.55 -> 1.22, 2,500 meshes 1.57 -> 1.30.  Tiles of 4,096 entries: 0.69,
+// 0.67, 1.42, 1.52 (fewer CTAs); four entries in flight instead of two slowed the searching version by
+// a quarter on binary32.
+constexpr int64_t kFlatTile = 2048;
+constexpr int kFlatRows = 768;  // rows of a tile kept in shared memory (more: read where used)
+constexpr int kFlatItems = 2;   // entries of a thread in flight
+
+// what an entry needs of its row: the degree, its reciprocal (0: divide), and the edge id of
+// entry j as ubase + j
+template <class P>
+struct FlatRow {
+    P d, rcp;
+    int64_t ubase;
+};
+
+template <class WT>
+__device__ __forceinline__ FlatRow<typename Tr<WT>::P> flat_row(
+    int64_t x, const int64_t* __restrict__ rowptr, const typename Tr<WT>::Acc* __restrict__ deg,
+    const int32_t* __restrict__ nlow, const int32_t* __restrict__ up_ptr) {
+    using P = typename Tr<WT>::P;
+    FlatRow<P> r;
+    r.d = (P)deg[x];
+    r.rcp = P(0);
+    if constexpr (std::is_same<P, double>::value)
+        if (mid_range(r.d)) r.rcp = __drcp_rn(r.d);
+    r.ubase = (int64_t)up_ptr[x] - (rowptr[x] + nlow[x]);
+    return r;
+}
+
+template <class WT>
 __global__ void __launch_bounds__(kThreads)
 k_rows_edges_flat(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
-                  const int32_t* __restrict__ col, const float* __restrict__ w,
-                  const float* __restrict__ deg, const int32_t* __restrict__ nlow,
-                  const int32_t* __restrict__ up_ptr, float* __restrict__ p,
+                  const int32_t* __restrict__ col, const WT* __restrict__ w,
+                  const typename Tr<WT>::Acc* __restrict__ deg, const int32_t* __restrict__ nlow,
+                  const int32_t* __restrict__ up_ptr, typename Tr<WT>::P* __restrict__ p,
                   uint2* __restrict__ pk, int32_t* __restrict__ eu, int32_t* __restrict__ ev,
-                  float* __restrict__ w_und, unsigned long long* sym, uint64_t k0, uint64_t k1,
+                  WT* __restrict__ w_und, unsigned long long* sym, uint64_t k0, uint64_t k1,
                   const uint32_t* status) {
     spc::pdl_wait();
     if (*status) return;  // invalid input: nothing below may index with it
-    __shared__ int64_t s_rows[2];
+    using P = typename Tr<WT>::P;
+    constexpr bool kF32 = std::is_same<WT, float>::value;
+    __shared__ int64_t s_next;            // the row of the next tile's first entry
     __shared__ int32_t s_row[kFlatTile];  // row of each entry of the tile minus the first row
+    __shared__ FlatRow<P> s_data[kFlatRows];
     uint64_t fp = 0;                      // this thread's fingerprint terms
-    for (int64_t base = (int64_t)blockIdx.x * kFlatTile; base < nnz;
-         base += (int64_t)gridDim.x * kFlatTile) {
+    // a contiguous range of tiles per block
+    const int64_t tiles = (nnz + kFlatTile - 1) / kFlatTile;
+    const int64_t per = (tiles + gridDim.x - 1) / gridDim.x * kFlatTile;
+    const int64_t begin = (int64_t)blockIdx.x * per;
+    const int64_t stop = begin + per < nnz ? begin + per : nnz;
+    if (begin < stop && threadIdx.x < 32) {
+        const int64_t x = csr_row_of(rowptr, n, begin);
+        if (threadIdx.x == 0) s_next = x;
+    }
+    __syncthreads();
+    for (int64_t base = begin; base < stop; base += kFlatTile) {
         const int64_t end = base + kFlatTile < nnz ? base + kFlatTile : nnz;
-        const int64_t r_lo = tile_rows(rowptr, n, base, end, kLongRow, s_row, s_rows);
-        for (int64_t j = base + threadIdx.x; j < end; j += blockDim.x) {
-            const int32_t rel = s_row[j - base];
-            const int64_t x = r_lo + (rel >= 0 ? rel : -2 - rel);
-            const int32_t y = col[j];
-            const float wj = w[j];
-            if (sym && (int64_t)y != x) fp += sym_term(x, y, __float_as_uint(wj), k0, k1);
-            if (rel < 0) continue;  // long row: k_long_rows_edges
-            const float pj = __fdiv_rn(wj, deg[x]);
-            if (p) p[j] = pj;
-            // row x's pairs at pk[rowptr[x] + x ..], then its end marker
-            pk[j + x] = make_uint2((uint32_t)y, __float_as_uint(pj));
-            if (j + 1 == rowptr[x + 1]) pk[j + x + 1] = make_uint2(0x7fffffffu, 0u);
-            if ((int64_t)y > x) {
-                const int64_t e = (int64_t)up_ptr[x] + (j - (rowptr[x] + nlow[x]));
-                eu[e] = (int32_t)x;
-                ev[e] = y;
-                w_und[e] = wj;
+        const int64_t r_lo = s_next;
+        __syncthreads();  // every thread has read s_next
+        tile_rows(rowptr, n, base, end, r_lo, kLongRow, s_row, &s_next,
+                  [&](int64_t x, int32_t rel, int64_t, int64_t r1) {
+                      if (rel < kFlatRows)
+                          s_data[rel] = flat_row<WT>(x, rowptr, deg, nlow, up_ptr);
+                      if constexpr (kF32)  // the row's end marker, by the tile of its last entry
+                          if (pk && r1 <= end) pk[r1 + x] = make_uint2(0x7fffffffu, 0u);
+                  });
+        __syncthreads();
+        for (int64_t j0 = base + threadIdx.x; j0 < end; j0 += kFlatItems * kThreads) {
+            int32_t y[kFlatItems];
+            WT wj[kFlatItems];
+#pragma unroll
+            for (int q = 0; q < kFlatItems; ++q) {
+                const int64_t j = j0 + q * kThreads;
+                if (j < end) {
+                    y[q] = col[j];
+                    wj[q] = w[j];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kFlatItems; ++q) {
+                const int64_t j = j0 + q * kThreads;
+                if (j >= end) break;
+                const int32_t rel = s_row[j - base];
+                const int64_t x = r_lo + (rel >= 0 ? rel : -2 - rel);
+                if constexpr (kF32)
+                    if (sym && (int64_t)y[q] != x)
+                        fp += sym_term(x, y[q], __float_as_uint(wj[q]), k0, k1);
+                if (rel < 0) continue;  // long row: k_long_rows_edges
+                const FlatRow<P> r = rel < kFlatRows
+                                         ? s_data[rel]
+                                         : flat_row<WT>(x, rowptr, deg, nlow, up_ptr);
+                if constexpr (kF32) {
+                    if (p || pk) {
+                        const float pj = __fdiv_rn(wj[q], r.d);
+                        if (p) p[j] = pj;
+                        if (pk) pk[j + x] = make_uint2((uint32_t)y[q], __float_as_uint(pj));
+                    }
+                } else {
+                    if (p) p[j] = div_row((double)wj[q], r.d, r.rcp, r.rcp != 0.0);
+                }
+                if ((int64_t)y[q] > x) {
+                    const int64_t e = r.ubase + j;
+                    eu[e] = (int32_t)x;
+                    ev[e] = y[q];
+                    w_und[e] = wj[q];
+                }
             }
         }
         __syncthreads();
@@ -407,6 +446,28 @@ k_rows_edges_flat(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
         for (int o = 16; o > 0; o >>= 1) fp += __shfl_xor_sync(0xffffffffu, fp, o);
         if ((threadIdx.x & 31) == 0 && fp) atomicAdd(sym, (unsigned long long)fp);
     }
+}
+
+// S0's symmetry where no score walk follows to check it: every undirected edge's mirror entry is
+// looked up by binary search in row v and its weight bits compared; equal counts of upper and lower
+// entries (2 m = nnz) make that symmetry.  A kernel of its own, a thread per edge: the probes live
+// on L1, which the normalise kernel's tiles leave little of (97^3 mesh: searches inside the normalise
+// kernel 0.24 ms, the two kernels 0.085 + 0.064).
+__global__ void __launch_bounds__(kThreads)
+k_mirror_edges(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
+               const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+               const void* __restrict__ w, const void* __restrict__ w_und, int wsize,
+               uint32_t* status) {
+    spc::pdl_wait();
+    if (*status) return;
+    bool asym = false;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t v = ev[e];
+        asym = asym || !has_mirror(col, w, wsize, rowptr[v], rowptr[v + 1], eu[e],
+                                   weight_bits(w_und, wsize, e));
+    }
+    if (asym) atomicOr(status, DEV_NOT_SYMMETRIC);
 }
 
 // the verdict of the symmetry fingerprint: a nonzero sum is an asymmetric input (unless a row
@@ -428,24 +489,6 @@ __device__ __forceinline__ void count_ops(unsigned long long* ops, uint32_t n_ad
         atomicAdd(ops, (unsigned long long)a);
         atomicAdd(ops + 1, (unsigned long long)b);
     }
-}
-
-// raw bits of entry j of a weight array of wsize-byte elements (int32, binary32 or binary64)
-__device__ __forceinline__ uint64_t weight_bits(const void* w, int wsize, int64_t j) {
-    return wsize == 8 ? static_cast<const unsigned long long*>(w)[j]
-                      : (uint64_t)static_cast<const unsigned int*>(w)[j];
-}
-
-// true if row [j0, j1) (sorted) holds column a with weight bits wb: the mirror of entry (a, .)
-__device__ __forceinline__ bool has_mirror(const int32_t* __restrict__ col, const void* w,
-                                           int wsize, int64_t j0, int64_t j1, int64_t a,
-                                           uint64_t wb) {
-    int64_t lo = j0, hi = j1;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)col[mid] < a) lo = mid + 1; else hi = mid;
-    }
-    return lo < j1 && (int64_t)col[lo] == a && weight_bits(w, wsize, lo) == wb;
 }
 
 // S3, edge-tile schedule: one thread per undirected edge; consecutive threads take consecutive
@@ -1436,11 +1479,11 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
         note_bytes(ctx, 8.0 * (n + 1) + nnz * (4 + s_w) + n * (s_acc + 8) + nnz * s_p +
                             m * (8 + s_w));
     // the symmetry of rows up to kLongRow is checked by the score kernels' walks when scores
-    // are computed; without scores, here
+    // are computed; without scores, by k_mirror_edges
     const int wsize = (int)sizeof(WT);
     const bool mirror_here = validate && (score == nullptr || m == 0);
     // binary32 levels that are scored check symmetry by the fingerprint of the flat normalise
-    // kernel; the others by the score walks (or, without scores, by k_rows_edges' searches)
+    // kernel; the others by the score walks
     const bool fingerprint = std::is_same<WT, float>::value && validate && !mirror_here && n > 0;
     const int vflag = validate && !fingerprint ? 1 : 0;
     // the score schedule: forced, or autotuned once per shape bucket (every schedule computes
@@ -1457,7 +1500,8 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
     }
     // binary32 rows: the packed schedule reads only the (column, p) pairs; p alone serves the
     // other schedules (and the autotuner, which times them) and the hub kernels
-    const bool need_p = score == nullptr || n_long > 0 || schedule != 3;
+    constexpr bool f32 = std::is_same<WT, float>::value;
+    const bool need_p = score != nullptr && (!f32 || n_long > 0 || schedule != 3);
     {
         // long rows (exact degrees from per-binade tables, then p and their edges) on the
         // second stream while the short rows run here
@@ -1481,33 +1525,25 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
                        W.ev.as<int32_t>(), W.w_und.as<WT>(), status);
             side->leave();
         }
-        if constexpr (std::is_same<WT, float>::value) {
-            if (!mirror_here && n > 0) {
-                unsigned long long* sym = nullptr;
-                if (fingerprint) {
-                    sym = W.sym.as<unsigned long long>();
-                    SPC_CUDA(cudaMemsetAsync(sym, 0, 8, ctx->stream));
-                }
-                SPC_LAUNCH(ctx, k_rows_edges_flat, grid_for(nnz, (int)kFlatTile, maxb), kThreads,
-                           0, n, nnz, g.rowptr, g.col, static_cast<const float*>(g.w),
-                           W.deg.as<float>(), W.first_up.as<int32_t>(), W.up_ptr.as<int32_t>(),
-                           need_p ? W.p.as<float>() : nullptr, W.pk.as<uint2>(),
-                           W.eu.as<int32_t>(), W.ev.as<int32_t>(), W.w_und.as<float>(), sym,
-                           ctx->sym_key[0], ctx->sym_key[1], status);
-                if (fingerprint) SPC_LAUNCH(ctx, k_sym_check, 1, 32, 0, sym, status);
-            } else {
-                SPC_LAUNCH(ctx, k_rows_edges<WT>, gb, kThreads, 0, n, g.rowptr, g.col,
-                           static_cast<const WT*>(g.w), mirror_here ? 1 : 0, W.deg.as<Acc>(),
-                           W.first_up.as<int32_t>(), W.up_ptr.as<int32_t>(), W.p.as<P>(),
-                           W.eu.as<int32_t>(), W.ev.as<int32_t>(), W.w_und.as<WT>(), status);
-            }
-        } else {
-            SPC_LAUNCH(ctx, k_rows_edges<WT>, gb, kThreads, 0, n, g.rowptr, g.col,
-                       static_cast<const WT*>(g.w), mirror_here ? 1 : 0, W.deg.as<Acc>(),
-                       W.first_up.as<int32_t>(), W.up_ptr.as<int32_t>(), W.p.as<P>(),
-                       W.eu.as<int32_t>(), W.ev.as<int32_t>(), W.w_und.as<WT>(), status);
+        unsigned long long* sym = nullptr;
+        if (fingerprint) {
+            sym = W.sym.as<unsigned long long>();
+            SPC_CUDA(cudaMemsetAsync(sym, 0, 8, ctx->stream));
         }
+        SPC_LAUNCH(ctx, k_rows_edges_flat<WT>, grid_for(nnz, (int)kFlatTile, maxb), kThreads, 0, n,
+                   nnz, g.rowptr, g.col, static_cast<const WT*>(g.w), W.deg.as<Acc>(),
+                   W.first_up.as<int32_t>(), W.up_ptr.as<int32_t>(),
+                   need_p ? W.p.as<P>() : nullptr,
+                   f32 && score != nullptr ? W.pk.as<uint2>() : nullptr, W.eu.as<int32_t>(),
+                   W.ev.as<int32_t>(), W.w_und.as<WT>(), sym, ctx->sym_key[0], ctx->sym_key[1],
+                   status);
+        if (fingerprint) SPC_LAUNCH(ctx, k_sym_check, 1, 32, 0, sym, status);
     }  // the main stream waits for the long rows here
+    if (mirror_here && m > 0) {
+        SPC_LAUNCH(ctx, k_mirror_edges, grid_for(m, kThreads, maxb), kThreads, 0, m,
+                   W.eu.as<int32_t>(), W.ev.as<int32_t>(), g.rowptr, g.col, g.w, W.w_und.p, wsize,
+                   status);
+    }
     if (score == nullptr || m == 0) {
         if (validate) SPC_TRY(check_status(ctx));
         return SPC_OK;

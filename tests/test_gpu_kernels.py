@@ -160,3 +160,46 @@ def test_streamed_masses_of_a_giant(ctx, dtype):
     for lv, r in zip(ctx.levels(), ref):
         assert np.array_equal(_bits(lv.score.cpu().numpy()), _bits(r.f))
         assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(r.coarse.graph.w))
+
+
+# the flat normalise and diagonal kernels march over tiles of 2,048 and 1,024 stored entries: entry
+# counts around a tile, rows longer than a tile's share, more rows in a tile than shared memory
+# holds (a path: 1,024), runs of empty rows longer than a block, long rows between short ones
+def _flat_graphs(dtype):
+    rng = np.random.default_rng(5)
+    out = []
+    for m in (511, 512, 513, 1023, 1024, 1025, 5000):  # paths: 2 m entries
+        out.append((m + 1, np.arange(m), 1 + np.arange(m)))
+    gaps = np.cumsum(rng.integers(1, 900, 60))         # a path over a few nodes of many
+    out.append((int(gaps[-1]) + 700, gaps[:-1], gaps[1:]))
+    u = np.r_[np.zeros(2500, np.int64), np.full(300, 2000), 1 + np.arange(2400)]
+    v = np.r_[1 + np.arange(2500), 2101 + np.arange(300), 2 + np.arange(2400)]
+    key = np.unique(np.minimum(u, v) * 4000 + np.maximum(u, v))
+    out.append((3000, key // 4000, key % 4000))
+    for n, eu, ev in out:
+        w = np.ones(eu.shape[0]) if dtype == np.int32 else rng.uniform(0.1, 2.0, eu.shape[0])
+        yield I.csr_from_edges(n, eu, ev, w.astype(dtype))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64, np.int32])
+def test_flat_kernels_at_tile_edges(ctx, dtype):
+    from paper_2204_11757_gb300 import api, native as N
+    for g in _flat_graphs(dtype):
+        csr = api.CSR.from_graph(g)
+        assert np.array_equal(_bits(ctx.score(csr).cpu().numpy()), _bits(O.score(g)))
+        ref, total = O.coarsen(g, 4, "halving")
+        lift, n_c, _ = ctx.coarsen(csr, ref[-1].target, levels=len(ref))
+        assert np.array_equal(lift.cpu().numpy(), total)
+        for lv, r in zip(ctx.levels(), ref):
+            assert np.array_equal(_bits(lv.score.cpu().numpy()), _bits(r.f))
+            assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(r.coarse.graph.w))
+        # without scores the mirrors are looked up edge by edge: one weight changed on one side
+        lt = torch.from_numpy(ref[0].lift).cuda()
+        assert ctx.contract(csr, lt, ref[0].n_c).m_c == ref[0].coarse.m_c
+        for j in (0, g.col.shape[0] - 1):
+            w = g.w.copy()
+            w[j] = w[j] + 1
+            bad = api.CSR.from_numpy(g.rowptr, g.col, w)
+            with pytest.raises(N.SpcError) as e:
+                ctx.contract(bad, lt, ref[0].n_c)
+            assert e.value.status == -2  # SPC_ERR_NOT_SYMMETRIC
