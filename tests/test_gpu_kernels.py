@@ -203,3 +203,16 @@ def test_flat_kernels_at_tile_edges(ctx, dtype):
             with pytest.raises(N.SpcError) as e:
                 ctx.contract(bad, lt, ref[0].n_c)
             assert e.value.status == -2  # SPC_ERR_NOT_SYMMETRIC
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n", [2, 31, 33, 4095, 4096, 4097, 4096 * 5 + 1, 4096 * 40 - 1])
+@pytest.mark.parametrize("values", [1, 3, 40, 0])
+def test_sort_ranks_and_look_back(ctx, dtype, n, values):
+    """Equal keys keep their order whether a warp's 32 share one digit, a few or none, in partial
+    tiles and over more tiles than a look-back window."""
+    rng = np.random.default_rng(n + values)
+    f = rng.random(n) if values == 0 else rng.integers(0, values, n) * 0.37
+    f = f.astype(dtype)
+    order = ctx.sort_fitness(torch.from_numpy(f).cuda()).cpu().numpy()
+    assert np.array_equal(order, np.argsort(f, kind="stable").astype(np.int32))
