@@ -216,3 +216,27 @@ def test_sort_ranks_and_look_back(ctx, dtype, n, values):
     f = f.astype(dtype)
     order = ctx.sort_fitness(torch.from_numpy(f).cuda()).cpu().numpy()
     assert np.array_equal(order, np.argsort(f, kind="stable").astype(np.int32))
+
+
+@pytest.mark.parametrize("dtype", [np.int32, np.float32, np.float64])
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 97, 1000])
+@pytest.mark.parametrize("shape", ["stars", "cliques"])
+def test_lower_rows_over_groups_of_32(ctx, dtype, n, shape):
+    """Coarse rows' lower entries, rows pooled 32 to a warp: empty rows, rows on both sides of 32
+    entries next to one another, a last group that is not full."""
+    from paper_2204_11757_gb300 import api
+    rng = np.random.default_rng(n)
+    if shape == "stars":  # every 13th row holds many lower entries, the others none
+        e = [(u, v) for v in range(12, n, 13) for u in range(max(0, v - 70), v)]
+        e = e or [(0, 1)]
+    else:
+        e = [(u, v) for v in range(n) for u in range(max(0, v - int(rng.integers(0, 40))), v)]
+        e = e or [(0, 1)]
+    eu, ev = (np.array(x, dtype=np.int32) for x in zip(*e))
+    w = rng.integers(1, 9, eu.shape[0]) if dtype == np.int32 else rng.random(eu.shape[0]) + 0.1
+    g = I.csr_from_edges(n, eu, ev, w.astype(dtype))
+    lift = np.arange(n, dtype=np.int32)  # nothing merged: the coarse graph is the graph itself
+    lv = ctx.contract(api.CSR.from_graph(g), torch.from_numpy(lift).cuda(), n)
+    assert np.array_equal(lv.rowptr_c.cpu().numpy(), g.rowptr)
+    assert np.array_equal(lv.col_c.cpu().numpy(), g.col)
+    assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(g.w))
