@@ -443,10 +443,11 @@ static spc_status reserve_work(spc_context* ctx, int64_t n, int64_t m, int64_t B
     SPC_TRY(ensure(ctx, W.b_off, 2 * N * 4));
     SPC_TRY(ensure_zeroed(ctx, W.b_stats, 8 * 8));
     SPC_TRY(ensure(ctx, W.b_list, (2 * (M / 64 + 1) + 16) * 4));  // long-bucket lists
-    // scan of up to max(n, m, 256 * tiles) items -> tile sums; radix histograms
+    // tile statuses: scans of up to max(n, m, 256 * tiles) items, the ranking's tiles of 1,024
+    // edges; radix histograms
     const size_t big = (N > M ? N : M) + 256 * ((M + 4095) / 4096) + 4096;
     // the scans keep their statuses zero between calls; a new block starts zeroed
-    SPC_TRY(ensure_zeroed(ctx, W.scan_tmp, (big / 4096 + 4) * 8 + 256));
+    SPC_TRY(ensure_zeroed(ctx, W.scan_tmp, (big / 1024 + 4) * 8 + 256));
     // one-sweep sort: 8 passes x (tiles x 256) look-back words + histograms (sorts of up to
     // max(n, m) items: the super-node members of the self-mass reading sort n)
     const size_t NM = N > M ? N : M;

@@ -320,13 +320,11 @@ k_bucket_scatter(int64_t m, const int32_t* __restrict__ eu, const int32_t* __res
 // item's rank is the number of smaller keys of the bucket (all distinct: they hold the eid).
 // Each lane keeps its items (lane, lane + 32, ...) in registers and every key is read once per
 // warp (a broadcast) and compared with all of them; the items then move to their ranks in the
-// stage and leave it in order, with the head flag of every coarse edge's first item.
+// stage and leave it in order.
 template <bool kInter, int kPer>
 __device__ __forceinline__ void warp_sort_bucket(unsigned long long* sk, int s, int lane,
-                                                 int32_t bkt, int32_t lo, int nb,
-                                                 uint64_t* __restrict__ key2,
-                                                 uint32_t* __restrict__ val2,
-                                                 uint8_t* __restrict__ head) {
+                                                 int32_t bkt, int32_t lo, uint4* citem,
+                                                 uint32_t* __restrict__ val2) {
     unsigned long long k[kPer];
     int r[kPer];
 #pragma unroll
@@ -347,27 +345,23 @@ __device__ __forceinline__ void warp_sort_bucket(unsigned long long* sk, int s, 
     __syncwarp();
     for (int i = lane; i < s; i += 32) {
         const unsigned long long x = sk[i];
-        if constexpr (kInter) {
-            key2[lo + i] = ((uint64_t)bkt << nb) | (x >> 32);
+        if constexpr (kInter)
+            citem[lo + i] = make_uint4((uint32_t)bkt, (uint32_t)(x >> 32), (uint32_t)x, 0u);
+        else
             val2[lo + i] = (uint32_t)x;
-            head[lo + i] = (i == 0 || (sk[i - 1] >> 32) != (x >> 32)) ? 1 : 0;
-        } else {
-            val2[lo + i] = (uint32_t)x;
-        }
     }
 }
 
 // Step 3, long buckets (listed by the scan of the sizes), sorted by one 64-bit key -- (b << 32)
-// | eid for inter edges (a is the bucket), the eid for intra edges -- and written back in
-// order: inter edges as (key, eid) with their head flags, intra edges as eids.  Buckets of more
+// | eid for inter edges (a is the bucket), the eid for intra edges -- and written in order: inter
+// edges back to their bucket (read into the stage first), intra edges as eids.  Buckets of more
 // than kWarpBucket items: one CTA each, a bitonic network over the next power of two (padding
 // keys all ones) in shared memory.  The others: one warp each (warp_sort_bucket).
 template <bool kInter>
 __global__ void __launch_bounds__(kBlockSortThreads, 3)
 k_bucket_sort_long(const int32_t* __restrict__ list, const unsigned long long* __restrict__ list_cnt,
-                   const int32_t* __restrict__ off, int nb, const uint4* __restrict__ citem,
-                   const uint2* __restrict__ iitem, uint64_t* __restrict__ key2,
-                   uint32_t* __restrict__ val2, uint8_t* __restrict__ head) {
+                   const int32_t* __restrict__ off, uint4* citem,
+                   const uint2* __restrict__ iitem, uint32_t* __restrict__ val2) {
     spc::pdl_wait();
     extern __shared__ unsigned long long sk[];  // kBlockBucket keys
     const int64_t cnt = (int64_t)*list_cnt;
@@ -407,14 +401,10 @@ k_bucket_sort_long(const int32_t* __restrict__ list, const unsigned long long* _
         }
         for (int i = threadIdx.x; i < s; i += blockDim.x) {
             const unsigned long long k = sk[i];
-            if constexpr (kInter) {
-                const uint64_t b = k >> 32;
-                key2[lo + i] = ((uint64_t)bkt << nb) | b;
+            if constexpr (kInter)
+                citem[lo + i] = make_uint4((uint32_t)bkt, (uint32_t)(k >> 32), (uint32_t)k, 0u);
+            else
                 val2[lo + i] = (uint32_t)k;
-                head[lo + i] = (i == 0 || (sk[i - 1] >> 32) != b) ? 1 : 0;
-            } else {
-                val2[lo + i] = (uint32_t)k;
-            }
         }
         __syncthreads();
     }
@@ -437,42 +427,142 @@ k_bucket_sort_long(const int32_t* __restrict__ list, const unsigned long long* _
         }
         __syncwarp();
         if (s <= 128)
-            warp_sort_bucket<kInter, 4>(wk, s, lane, bkt, lo, nb, key2, val2, head);
+            warp_sort_bucket<kInter, 4>(wk, s, lane, bkt, lo, citem, val2);
         else
-            warp_sort_bucket<kInter, 8>(wk, s, lane, bkt, lo, nb, key2, val2, head);
+            warp_sort_bucket<kInter, 8>(wk, s, lane, bkt, lo, citem, val2);
         __syncwarp();  // the next bucket overwrites the stage
     }
 }
 
-// Step 3, inter edges in short buckets: the item at p goes to its rank by (key, eid) within
-// its bucket [off_c[a], off_c[a + 1]); head marks the first item (smallest eid) of every
-// coarse edge.  Runs after k_bucket_sort_long, whose list it then empties.
-__global__ void __launch_bounds__(kThreads)
-k_bucket_rank_inter(int64_t cnt, int nb, const int32_t* __restrict__ off_c,
-                    const uint4* __restrict__ citem, uint64_t* __restrict__ key2,
-                    uint32_t* __restrict__ val2, uint8_t* __restrict__ head,
-                    unsigned long long* __restrict__ list_cnt) {
+// Step 3, inter edges: a CTA orders the items of kRankTile consecutive positions and emits them.
+// Every item of a short bucket [off_c[a], off_c[a + 1]) goes to its rank by (b, eid) in the bucket,
+// among the keys in shared memory; the items within a bucket's length of the tile are loaded too, for
+// the buckets that cross its edges.  Long buckets are in order already (k_bucket_sort_long, whose
+// list this empties).  The tile's positions are then in (a, b, eid) order, each new (a, b) starts a
+// coarse edge, and its id is a prefix sum over the tiles by look-back: emap, perm, the segment starts
+// and end points and the coarse degrees go out with no sorted copy, head flags or positions in
+// memory.  Ranked, scanned and emitted by three kernels, the items were written and read again: all
+// levels of a random geometric graph of 2^23 nodes 2,250 -> 1,380 us, 2,500 graphs 1,450 -> 775, a
+// triangle grid of 2048^2 510 -> 420.  Loads and the emission's scattered stores bound it, so many
+// CTAs take turns: tiles of 2,048 items 1,498, 874 and 464, with 128 threads 2,193, 1,018 and 569.
+constexpr int kRankTile = 1024;
+constexpr int kRankThreads = 256;
+constexpr int kRankHalo = kSmallBucket;
+constexpr int kRankStage = kRankTile + 2 * kRankHalo;
+constexpr int kRankItems = (kRankStage + kRankThreads - 1) / kRankThreads;
+constexpr int kRankRows = kRankTile / kRankThreads;  // positions of a thread when it emits
+constexpr int kRankGroups = kRankTile / 1024;        // groups of 32 positions per lane of the scan
+static_assert(kRankTile % 1024 == 0 && kRankTile % kRankThreads == 0, "whole groups and rows");
+
+__global__ void __launch_bounds__(kRankThreads, 8)
+k_bucket_rank_inter(int64_t cnt, const int32_t* __restrict__ off_c,
+                    const uint4* __restrict__ citem, int32_t* __restrict__ emap,
+                    int32_t* __restrict__ perm, int32_t* __restrict__ seg,
+                    int32_t* __restrict__ cU, int32_t* __restrict__ cV, int32_t* up_deg,
+                    int32_t* low_deg, int32_t* __restrict__ total,
+                    unsigned long long* __restrict__ list_cnt, unsigned long long* status,
+                    uint32_t* tile_ctr, int64_t nt, uint32_t* err) {
     spc::pdl_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *list_cnt = 0ull;  // long buckets are sorted
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < cnt;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const uint4 it = citem[p];
-        const uint32_t b = it.y, v = it.z;
-        const int32_t lo = off_c[it.x], hi = off_c[it.x + 1];
-        if (hi - lo > kSmallBucket) continue;
-        int32_t r = 0;
-        bool first = true;
-#pragma unroll 4
-        for (int32_t j = lo; j < hi; ++j) {
-            const uint4 jt = citem[j];
-            const bool same_before = jt.y == b && jt.z < v;
-            r += (jt.y < b || same_before) ? 1 : 0;
-            first = first && !same_before;
+    __shared__ unsigned long long s_in[kRankStage];      // (b << 32) | eid, as the items came
+    __shared__ unsigned long long s_key[kRankTile + 1];  // in order, from position base - 1
+    __shared__ int32_t s_a[kRankTile + 1];
+    __shared__ int32_t s_cnt[kRankTile / 32];
+    __shared__ uint32_t sh_tile;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) sh_tile = atomicAdd(tile_ctr, 1u);
+    __syncthreads();
+    const int64_t tile = sh_tile;
+    const int64_t base = tile * kRankTile;
+    const int64_t first = base - kRankHalo;
+    const int64_t end = base + kRankTile < cnt ? base + kRankTile : cnt;
+    if (tile == 0 && threadIdx.x == 0) *list_cnt = 0ull;
+    int32_t a[kRankItems];
+#pragma unroll
+    for (int k = 0; k < kRankItems; ++k) {
+        const int i = k * kRankThreads + threadIdx.x;
+        const int64_t p = first + i;
+        a[k] = -1;
+        if (i < kRankStage && p >= 0 && p < cnt) {
+            const uint4 it = citem[p];
+            a[k] = (int32_t)it.x;
+            s_in[i] = ((unsigned long long)it.y << 32) | it.z;
         }
-        key2[lo + r] = ((uint64_t)it.x << nb) | b;
-        val2[lo + r] = v;
-        head[lo + r] = first ? 1 : 0;
     }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kRankItems; ++k) {
+        if (a[k] < 0) continue;
+        const int i = k * kRankThreads + threadIdx.x;
+        const int64_t lo = off_c[a[k]], hi = off_c[a[k] + 1];
+        const unsigned long long x = s_in[i];
+        int64_t at = first + i;
+        if (hi - lo <= kSmallBucket) {
+            if (hi < base || lo >= end) continue;  // reaches no position from base - 1 to end - 1
+            const int j1 = (int)(hi - first);      // in the stage: hi - lo <= kRankHalo
+            int r = 0;
+#pragma unroll 4
+            for (int j = (int)(lo - first); j < j1; ++j) r += s_in[j] < x ? 1 : 0;
+            at = lo + r;
+        }
+        if (at >= base - 1 && at < end) {
+            s_key[at - base + 1] = x;
+            s_a[at - base + 1] = a[k];
+        }
+    }
+    __syncthreads();
+    unsigned heads[kRankRows];  // of the warp's 32 positions
+#pragma unroll
+    for (int k = 0; k < kRankRows; ++k) {
+        const int i = k * kRankThreads + threadIdx.x;
+        const bool h = base + i < end && (base + i == 0 || s_a[i] != s_a[i + 1] ||
+                                          (s_key[i] >> 32) != (s_key[i + 1] >> 32));
+        heads[k] = __ballot_sync(0xffffffffu, h);
+        if (lane == 0) s_cnt[k * (kRankThreads / 32) + warp] = __popc(heads[k]);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int32_t c[kRankGroups], mine = 0;
+#pragma unroll
+        for (int g = 0; g < kRankGroups; ++g) {
+            c[g] = s_cnt[lane * kRankGroups + g];
+            mine += c[g];
+        }
+        const int32_t incl = scanf::warp_incl_scan(mine);
+        const int32_t tot = __shfl_sync(0xffffffffu, incl, 31);
+        const int32_t before = (int32_t)scanf::look_back(status, tile, (uint32_t)tot, err);
+        int32_t run = before + incl - mine;
+#pragma unroll
+        for (int g = 0; g < kRankGroups; ++g) {
+            s_cnt[lane * kRankGroups + g] = run;
+            run += c[g];
+        }
+        if (lane == 0 && tile == nt - 1) *total = before + tot;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kRankRows; ++k) {
+        const int i = k * kRankThreads + threadIdx.x;
+        const int64_t p = base + i;
+        const bool h = (heads[k] >> lane) & 1u;
+        int32_t U = 0, V = 0;
+        if (p < end) {
+            const unsigned long long x = s_key[i + 1];
+            const int32_t ce = s_cnt[k * (kRankThreads / 32) + warp] - 1 +
+                               __popc(heads[k] & (0xffffffffu >> (31 - lane)));
+            emap[(uint32_t)x] = ce;
+            perm[p] = (int32_t)(uint32_t)x;
+            if (h) {
+                U = s_a[i + 1];
+                V = (int32_t)(x >> 32);
+                seg[ce] = (int32_t)p;
+                cU[ce] = U;
+                cV[ce] = V;
+            }
+        }
+        warp_count(up_deg, U, h);
+        warp_count(low_deg, V, h);
+    }
+    scanf::reset_when_last(status, tile_ctr, nt);
 }
 
 // Step 3, intra edges in short buckets: the eid at p goes to its rank within its super-node's
@@ -881,8 +971,7 @@ constexpr int64_t kRankWork = 48;
 // one CTA per long bucket, each with kBlockBucket keys of shared memory
 static spc_status sort_long_buckets(spc_context* ctx, bool inter, const int32_t* list,
                                     const unsigned long long* list_cnt, const int32_t* off,
-                                    int nb, const uint4* citem, const uint2* iitem,
-                                    uint64_t* key2, uint32_t* val2, uint8_t* head) {
+                                    uint4* citem, const uint2* iitem, uint32_t* val2) {
     constexpr int smem = kBlockBucket * 8;
     static std::atomic<unsigned long long> attr_devs{0};  // devices already set up
     const unsigned long long bit = 1ull << (ctx->device & 63);
@@ -896,10 +985,10 @@ static spc_status sort_long_buckets(spc_context* ctx, bool inter, const int32_t*
     const int grid = ctx->num_sms * 3;
     if (inter) {
         SPC_LAUNCH(ctx, k_bucket_sort_long<true>, grid, kBlockSortThreads, smem, list, list_cnt,
-                   off, nb, citem, iitem, key2, val2, head);
+                   off, citem, iitem, val2);
     } else {
         SPC_LAUNCH(ctx, k_bucket_sort_long<false>, grid, kBlockSortThreads, smem, list, list_cnt,
-                   off, nb, citem, iitem, key2, val2, head);
+                   off, citem, iitem, val2);
     }
     return SPC_OK;
 }
@@ -1005,8 +1094,8 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         uint32_t* ival2 = W.i_val2.as<uint32_t>();
         if (m_intra > 0) {
             if (long_i > 0)
-                SPC_TRY(sort_long_buckets(ctx, false, list_i, bstats + 7, off_i, nb, nullptr,
-                                          iitem, nullptr, ival2, nullptr));
+                SPC_TRY(sort_long_buckets(ctx, false, list_i, bstats + 7, off_i, nullptr, iitem,
+                                          ival2));
             SPC_LAUNCH(ctx, k_bucket_rank_intra, grid_for(m_intra, kThreads, maxb), kThreads, 0,
                        m_intra, off_i, iitem, ival2, bstats + 7);
         }
@@ -1041,43 +1130,34 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         }
     }
     side->leave();
-    // coarse edges: the inter edges in (a, b, eid) order with a head flag per coarse edge
+    // coarse edges: the inter edges in (a, b, eid) order
     int32_t* long_list = W.long_segs.as<int32_t>();
     int32_t* long_cnt = W.counters.as<int32_t>() + 9;
     uint8_t* head = W.c_flag.as<uint8_t>();  // flags are consumed; reuse as heads
     int32_t* hpos = W.c_pos.as<int32_t>();
-    const uint64_t* skey = ckey;
-    const uint32_t* sval = cval;
-    if (buckets) {
-        if (m_inter > 0) {
-            if (long_c > 0)
-                SPC_TRY(sort_long_buckets(ctx, true, list_c, bstats + 6, off_c, nb, citem,
-                                          nullptr, W.c_key2.as<uint64_t>(),
-                                          W.c_val2.as<uint32_t>(), head));
-            SPC_LAUNCH(ctx, k_bucket_rank_inter, grid_for(m_inter, kThreads, maxb), kThreads, 0,
-                       m_inter, nb, off_c, citem, W.c_key2.as<uint64_t>(),
-                       W.c_val2.as<uint32_t>(), head, bstats + 6);
-        }
-        skey = W.c_key2.as<uint64_t>();
-        sval = W.c_val2.as<uint32_t>();
-    } else {
-        SPC_TRY(radix_sort_u64(ctx, ckey, cval, W.c_key2.as<uint64_t>(), W.c_val2.as<uint32_t>(),
-                               m_inter, 2 * nb));
-        if (m_inter > 0) {
-            SPC_LAUNCH(ctx, k_heads<uint64_t>, grid_for(m_inter, kThreads, maxb), kThreads, 0,
-                       m_inter, ckey, head);
-        }
-    }
     int32_t* seg = lv.seg.as<int32_t>();
     int32_t* perm = lv.perm.as<int32_t>();
     int32_t* cU = W.cU.as<int32_t>();
     int32_t* cV = W.cV.as<int32_t>();
     int64_t m_c = 0;
     bool lower_buckets = true;
-    if (m_inter > 0) {
+    if (m_inter > 0 && buckets) {
+        if (long_c > 0)
+            SPC_TRY(sort_long_buckets(ctx, true, list_c, bstats + 6, off_c, citem, nullptr, nullptr));
+        const int64_t nt = (m_inter + kRankTile - 1) / kRankTile;
+        unsigned long long* tile_status;
+        uint32_t* tile_ctr;
+        SPC_TRY(scan_tiles(ctx, nt, &tile_status, &tile_ctr));
+        SPC_LAUNCH(ctx, k_bucket_rank_inter, (unsigned)nt, kRankThreads, 0, m_inter, off_c, citem, emap,
+                   perm, seg, cU, cV, up_deg, low_deg, hpos + m_inter, bstats + 6, tile_status,
+                   tile_ctr, nt, status);
+    } else if (m_inter > 0) {
         const int gi = grid_for(m_inter, kThreads, maxb);
+        SPC_TRY(radix_sort_u64(ctx, ckey, cval, W.c_key2.as<uint64_t>(), W.c_val2.as<uint32_t>(),
+                               m_inter, 2 * nb));
+        SPC_LAUNCH(ctx, k_heads<uint64_t>, gi, kThreads, 0, m_inter, ckey, head);
         SPC_TRY(scan_flags_u8(ctx, head, hpos, m_inter));
-        SPC_LAUNCH(ctx, k_emit_segments, gi, kThreads, 0, m_inter, nb, skey, sval, head, hpos,
+        SPC_LAUNCH(ctx, k_emit_segments, gi, kThreads, 0, m_inter, nb, ckey, cval, head, hpos,
                    emap, perm, seg, cU, cV, up_deg, low_deg);
     }
     // coarse CSR: row U holds its lower entries (coarse edges (U', U), ascending U') and then

@@ -68,6 +68,66 @@ __device__ __forceinline__ T block_excl_scan(T v, T* total) {
     return before + incl - v;
 }
 
+// A tile's look-back, by one warp: publishes the tile's own sum, adds up its predecessors' and
+// publishes the inclusive prefix; every lane returns the exclusive one.
+__device__ __forceinline__ unsigned long long look_back(unsigned long long* status, int64_t tile,
+                                                        unsigned long long tot, uint32_t* err) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long prefix = 0;
+    if (tile > 0) {
+        if (lane == 0) atomicExch(status + tile, kScanAgg | tot);
+        int64_t top = tile - 1;
+        bool done = false;
+        while (!done) {
+            const int64_t idx = top - lane;
+            unsigned long long w = kScanInc;  // before tile 0: an inclusive zero
+            if (idx >= 0) w = *reinterpret_cast<volatile unsigned long long*>(status + idx);
+            uint32_t spins = 0;
+            while (__any_sync(0xffffffffu, (w >> 62) == 0ull)) {
+                if ((w >> 62) == 0ull)
+                    w = *reinterpret_cast<volatile unsigned long long*>(status + idx);
+                if (++spins > spin_limit(err)) {
+                    if (lane == 0) atomicOr(err, DEV_TIMEOUT);
+                    w = kScanInc;  // give up; the call reports the timeout
+                }
+            }
+            const unsigned inc = __ballot_sync(0xffffffffu, (w >> 62) == 2ull);
+            const int stop = inc ? __ffs(inc) - 1 : 31;
+            unsigned long long part = (lane <= stop) ? (w & kScanVal) : 0ull;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+            prefix += part;
+            done = inc != 0u;
+            top -= 32;
+        }
+    }
+    if (lane == 0) atomicExch(status + tile, kScanInc | (prefix + tot));
+    return prefix;
+}
+
+// The tile that finishes last resets the statuses and counters for the next scan: every other
+// tile has counted itself done after its look-back, so none reads them again.  Every thread of
+// the block calls it.
+__device__ __forceinline__ void reset_when_last(unsigned long long* status, uint32_t* tile_ctr,
+                                                int64_t nt) {
+    __shared__ bool sh_last;
+    uint32_t* done_ctr = tile_ctr + 1;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        sh_last = atomicAdd(done_ctr, 1u) == (uint32_t)(nt - 1);
+    }
+    __syncthreads();
+    if (sh_last) {
+        __threadfence();
+        for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) status[t] = 0ull;
+        if (threadIdx.x == 0) {
+            *tile_ctr = 0u;
+            *done_ctr = 0u;
+        }
+    }
+}
+
 // One pass over nt tiles.  Tiles take ids in launch order from *tile_ctr, so every tile a
 // tile waits for has already started.  A tile reads all of its items before it stores any.
 template <class T, class Ld, class St>
@@ -79,8 +139,6 @@ __global__ void __launch_bounds__(ST) k_scan_fused(Ld ld, St st, int64_t n,
     __shared__ T buf[STILE + STILE / 32];
     __shared__ uint32_t sh_tile;
     __shared__ T sh_prefix;
-    __shared__ bool sh_last;
-    uint32_t* done_ctr = tile_ctr + 1;
     if (threadIdx.x == 0) sh_tile = atomicAdd(tile_ctr, 1u);
     __syncthreads();
     const int64_t tile = sh_tile;
@@ -109,38 +167,8 @@ __global__ void __launch_bounds__(ST) k_scan_fused(Ld ld, St st, int64_t n,
     T tot;
     const T pre = block_excl_scan<T>(run, &tot);
     if (warp == 0) {
-        unsigned long long prefix = 0;
-        if (tile > 0) {
-            if (lane == 0) atomicExch(status + tile, kScanAgg | (unsigned long long)tot);
-            int64_t top = tile - 1;
-            bool done = false;
-            while (!done) {
-                const int64_t idx = top - lane;
-                unsigned long long w = kScanInc;  // before tile 0: an inclusive zero
-                if (idx >= 0) w = *reinterpret_cast<volatile unsigned long long*>(status + idx);
-                uint32_t spins = 0;
-                while (__any_sync(0xffffffffu, (w >> 62) == 0ull)) {
-                    if ((w >> 62) == 0ull)
-                        w = *reinterpret_cast<volatile unsigned long long*>(status + idx);
-                    if (++spins > spin_limit(err)) {
-                        if (lane == 0) atomicOr(err, DEV_TIMEOUT);
-                        w = kScanInc;  // give up; the call reports the timeout
-                    }
-                }
-                const unsigned inc = __ballot_sync(0xffffffffu, (w >> 62) == 2ull);
-                const int stop = inc ? __ffs(inc) - 1 : 31;
-                unsigned long long part = (lane <= stop) ? (w & kScanVal) : 0ull;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-                prefix += part;
-                done = inc != 0u;
-                top -= 32;
-            }
-        }
-        if (lane == 0) {
-            atomicExch(status + tile, kScanInc | (prefix + (unsigned long long)tot));
-            sh_prefix = (T)prefix;
-        }
+        const unsigned long long prefix = look_back(status, tile, (unsigned long long)tot, err);
+        if (lane == 0) sh_prefix = (T)prefix;
     }
     __syncthreads();
     const T off = sh_prefix + pre;
@@ -159,22 +187,7 @@ __global__ void __launch_bounds__(ST) k_scan_fused(Ld ld, St st, int64_t n,
     }
     st.finish(sl);
     if (tile == nt - 1 && threadIdx.x == 0) st.total(sh_prefix + tot);
-    // The tile that finishes last resets the statuses and counters for the next scan: every
-    // other tile has counted itself done after its look-back, so none reads them again.
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        sh_last = atomicAdd(done_ctr, 1u) == (uint32_t)(nt - 1);
-    }
-    __syncthreads();
-    if (sh_last) {
-        __threadfence();
-        for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) status[t] = 0ull;
-        if (threadIdx.x == 0) {
-            *tile_ctr = 0u;
-            *done_ctr = 0u;
-        }
-    }
+    reset_when_last(status, tile_ctr, nt);
 }
 
 // small inputs: one CTA scans everything in chunks of 4 items per thread with a carry
@@ -215,6 +228,16 @@ __global__ void __launch_bounds__(kSmallThreads) k_scan_small_fused(Ld ld, St st
 
 }  // namespace scanf
 
+// statuses [nt] | tile counter, done counter: zero between scans, zeroed when allocated
+inline spc_status scan_tiles(spc_context* ctx, int64_t nt, unsigned long long** status,
+                             uint32_t** tile_ctr) {
+    Buf& tmp = on_side(ctx) ? ctx->work.scan_tmp_side : ctx->work.scan_tmp;
+    SPC_TRY(ensure_zeroed(ctx, tmp, (size_t)(nt + 1) * 8));
+    *status = tmp.as<unsigned long long>();
+    *tile_ctr = reinterpret_cast<uint32_t*>(*status + nt);
+    return SPC_OK;
+}
+
 // Scan of n items from `ld` into `st` on the context's current stream; `bytes`: the
 // operation's algorithmic DRAM bytes for the kernel profile (0: no model).
 template <class T, class Ld, class St>
@@ -225,11 +248,9 @@ spc_status scan_fused(spc_context* ctx, int64_t n, const Ld& ld, const St& st, d
         return SPC_OK;
     }
     const int64_t nt = (n + STILE - 1) / STILE;
-    // statuses [nt] | tile counter, done counter: zero between scans, zeroed when allocated
-    Buf& tmp = on_side(ctx) ? ctx->work.scan_tmp_side : ctx->work.scan_tmp;
-    SPC_TRY(ensure_zeroed(ctx, tmp, (size_t)(nt + 1) * 8));
-    unsigned long long* status = tmp.as<unsigned long long>();
-    uint32_t* tile_ctr = reinterpret_cast<uint32_t*>(status + nt);
+    unsigned long long* status;
+    uint32_t* tile_ctr;
+    SPC_TRY(scan_tiles(ctx, nt, &status, &tile_ctr));
     if (bytes > 0) note_bytes(ctx, bytes);
     SPC_LAUNCH(ctx, (k_scan_fused<T, Ld, St>), (unsigned)nt, ST, 0, ld, st, n, status, tile_ctr,
                nt, ctx->d_status);

@@ -240,3 +240,35 @@ def test_lower_rows_over_groups_of_32(ctx, dtype, n, shape):
     assert np.array_equal(lv.rowptr_c.cpu().numpy(), g.rowptr)
     assert np.array_equal(lv.col_c.cpu().numpy(), g.col)
     assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(g.w))
+
+
+@pytest.mark.parametrize("dtype", [np.int32, np.float64])
+@pytest.mark.parametrize("size", [1, 9, 63, 64, 65, 200, 300])
+def test_buckets_across_the_ranking_tiles(ctx, dtype, size):
+    """Coarse edges from buckets around the 64 items that are ranked in a tile, and longer ones, with
+    several fine edges to most of them, over a few tiles of 1,024 positions."""
+    from paper_2204_11757_gb300 import api
+    rng = np.random.default_rng(size)
+    n_c, per = max(8, 5000 // size), 24
+    n = n_c * per  # super-node U holds the nodes U, U + n_c, ...
+    a = np.repeat(np.arange(n_c), size)
+    b = (a + 1 + rng.integers(0, min(n_c - 1, max(1, size // 2)), a.shape[0])) % n_c
+    x = a + n_c * rng.integers(0, per, a.shape[0])
+    y = b + n_c * rng.integers(0, per, a.shape[0])
+    lo, hi = np.minimum(x, y).astype(np.int64), np.maximum(x, y)
+    key = np.unique(lo * n + hi)
+    eu, ev = key // n, key % n
+    w = rng.integers(1, 9, eu.shape[0]) if dtype == np.int32 else rng.random(eu.shape[0]) + 0.1
+    g = I.csr_from_edges(n, eu, ev, w.astype(dtype))
+    lift = (np.arange(n) % n_c).astype(np.int32)
+    c = O.contract(g, lift, n_c)
+    lv = ctx.contract(api.CSR.from_graph(g), torch.from_numpy(lift).cuda(), n_c)
+    assert np.array_equal(lv.emap.cpu().numpy(), c.emap)
+    inter = np.flatnonzero(c.emap >= 0)
+    perm = inter[np.argsort(c.emap[inter], kind="stable")]
+    assert np.array_equal(lv.perm.cpu().numpy()[:perm.size], perm)
+    assert np.array_equal(lv.seg.cpu().numpy(), np.searchsorted(c.emap[perm], np.arange(lv.m_c + 1)))
+    assert np.array_equal(_bits(lv.a_und.cpu().numpy()), _bits(c.a_und))
+    assert np.array_equal(lv.rowptr_c.cpu().numpy(), c.graph.rowptr)
+    assert np.array_equal(lv.col_c.cpu().numpy(), c.graph.col)
+    assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(c.graph.w))
