@@ -189,7 +189,7 @@ __global__ void k_expect(Expect x, int32_t* mismatch) {
 
 // the values a read takes, written to pinned host memory by one launch (a copy per value was 1.5-2
 // us each on the stream, and a contraction reads eight)
-constexpr int kReadMax = 8;
+constexpr int kReadMax = 10;
 struct ReadVals {
     const void* dev[kReadMax];
     int bytes[kReadMax];
@@ -229,10 +229,10 @@ spc_status read_vals(spc_context* ctx, int count, const void* const* dev, const 
         x.dev[i] = dev[i];
         x.bytes[i] = bytes[i];
     }
-    SPC_LAUNCH(ctx, k_read_vals, 1, 32, 0, x, ctx->h_scalars + 16);
+    SPC_LAUNCH(ctx, k_read_vals, 1, 32, 0, x, ctx->h_scalars + 8);
     SPC_CUDA(cudaStreamSynchronize(ctx->stream));
     for (int i = 0; i < count; ++i) {
-        out[i] = ctx->h_scalars[16 + i];
+        out[i] = ctx->h_scalars[8 + i];
         if (R.mode == Replay::kRecord) R.log.push_back(out[i]);
     }
     return SPC_OK;
@@ -441,7 +441,8 @@ static spc_status reserve_work(spc_context* ctx, int64_t n, int64_t m, int64_t B
     SPC_TRY(ensure(ctx, W.long_segs, (M + 1) * 4));
     SPC_TRY(ensure_zeroed(ctx, W.b_cnt, 2 * N * 4));
     SPC_TRY(ensure(ctx, W.b_off, 2 * N * 4));
-    SPC_TRY(ensure_zeroed(ctx, W.b_stats, 8 * 8));
+    SPC_TRY(ensure_zeroed(ctx, W.b_stats, 10 * 8));
+    SPC_TRY(ensure(ctx, W.b_huge, 2 * (M / 8192 + 1) * 8));
     SPC_TRY(ensure(ctx, W.b_list, (2 * (M / 64 + 1) + 16) * 4));  // long-bucket lists
     // tile statuses: scans of up to max(n, m, 256 * tiles) items, the ranking's tiles of 1,024
     // edges; radix histograms

@@ -149,7 +149,9 @@ __device__ __forceinline__ void block_stats(const unsigned long long* sq,
 // scan storer of the two packed bucket sizes (spc_scan.cuh PairLd: inter, intra): both
 // exclusive prefixes and totals, and per side the ranking statistics -- sum of squared sizes in
 // stats[0] / stats[2], largest size in stats[1] / stats[3] -- and the list of buckets longer
-// than kSmallBucket (counts in stats[6] / stats[7]).
+// than kSmallBucket (counts in stats[6] / stats[7]).  Buckets longer than kBlockBucket are also
+// listed with the number of items in the ones listed before; stats[8] / stats[9] hold their count
+// (high half) and their items (low half).
 struct BucketOffSt {
     int32_t* off_c;
     int32_t* off_i;
@@ -157,6 +159,8 @@ struct BucketOffSt {
     unsigned long long* stats;
     int32_t* list_c;
     int32_t* list_i;
+    int2* huge_c;
+    int2* huge_i;
     struct Local {
         unsigned long long sq[2], mx[2];
     };
@@ -173,6 +177,10 @@ struct BucketOffSt {
             L.mx[side] = c[side] > L.mx[side] ? c[side] : L.mx[side];
             if (c[side] > (unsigned long long)kSmallBucket)
                 (side ? list_i : list_c)[atomicAdd(stats + 6 + side, 1ull)] = (int32_t)g;
+            if (c[side] > (unsigned long long)kBlockBucket) {
+                const unsigned long long at = atomicAdd(stats + 8 + side, (1ull << 32) + c[side]);
+                (side ? huge_i : huge_c)[at >> 32] = make_int2((int32_t)g, (int32_t)(uint32_t)at);
+            }
         }
     }
     __device__ void finish(Local& L) const {
@@ -224,9 +232,9 @@ struct RowPtrSt {
 // order, the self-masses the intra edges in (super-node, eid) order.  Both orders are
 // reached without a global sort: the items are counted per bucket (a for an inter edge, the
 // super-node for an intra edge), scattered into their bucket's range in any order, and each
-// item then moves to its rank within its bucket.  The ranking costs the sum over buckets of
-// the squared bucket size; the host takes this path only while that stays a small multiple
-// of the item count (and every bucket is short), else it sorts by radix.
+// item then moves to its rank within its bucket: short buckets by comparisons, longer ones by
+// a warp or a CTA, huge ones together by radix.  When the huge ones hold more than half of the
+// edges, all of them are sorted by radix instead.
 
 // bucket of fine edge e, one 32-bit tag per (array, bucket) for warp matching: an inter edge's
 // lower super-node, an intra edge's super-node with the top bit set (ids are below 2^31);
@@ -368,8 +376,9 @@ k_bucket_sort_long(const int32_t* __restrict__ list, const unsigned long long* _
     for (int64_t q = blockIdx.x; q < cnt; q += gridDim.x) {
         const int32_t bkt = list[q];
         const int32_t lo = off[bkt];
-        const int s = off[bkt + 1] - lo;  // kSmallBucket < s <= kBlockBucket (host checked)
+        const int s = off[bkt + 1] - lo;
         if (s <= kWarpBucket) continue;   // a warp's bucket (below)
+        if (s > kBlockBucket) continue;   // sorted with the huge buckets
         int P = 1;
         while (P < s) P <<= 1;
         for (int i = threadIdx.x; i < P; i += blockDim.x) {
@@ -434,17 +443,73 @@ k_bucket_sort_long(const int32_t* __restrict__ list, const unsigned long long* _
     }
 }
 
+// Step 3, huge buckets (more than kBlockBucket items): the items of all of them are sorted together
+// by (bucket's place in the list, b, eid), or (place, eid) for intra edges, by radix, and go back to
+// their buckets in order.  nh: listed buckets, cnt: their items.  One giant super-node would else
+// send every edge of its level through the radix path: a tetrahedral grid of 129^3 (binary64, a
+// giant on six of seven levels) 17.1 -> 16.4 ms for the whole call, 2,500 graphs (139 huge buckets
+// on one of three levels) 20.8 -> 20.1 ms.
+template <bool kInter>
+__global__ void __launch_bounds__(kThreads)
+k_huge_keys(int64_t cnt, int32_t nh, const int2* __restrict__ huge,
+            const int32_t* __restrict__ off, int nb, int eb, const uint4* __restrict__ citem,
+            const uint2* __restrict__ iitem, uint64_t* __restrict__ key,
+            uint32_t* __restrict__ val) {
+    spc::pdl_wait();
+    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < cnt;
+         f += (int64_t)gridDim.x * blockDim.x) {
+        int32_t lo = 0, hi = nh - 1;
+        while (lo < hi) {
+            const int32_t mid = (lo + hi + 1) >> 1;
+            if (huge[mid].y <= f) lo = mid; else hi = mid - 1;
+        }
+        const int2 h = huge[lo];
+        const int64_t p = off[h.x] + (f - h.y);
+        uint64_t k;
+        if constexpr (kInter) {
+            const uint4 it = citem[p];
+            k = ((((uint64_t)lo << nb) | it.y) << eb) | it.z;
+        } else {
+            k = ((uint64_t)lo << eb) | iitem[p].y;
+        }
+        key[f] = k;
+        val[f] = 0u;
+    }
+}
+
+template <bool kInter>
+__global__ void __launch_bounds__(kThreads)
+k_huge_put(int64_t cnt, const int2* __restrict__ huge, const int32_t* __restrict__ off, int nb,
+           int eb, const uint64_t* __restrict__ key, uint4* __restrict__ citem,
+           uint32_t* __restrict__ val2, unsigned long long* __restrict__ stat) {
+    spc::pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *stat = 0ull;  // the list is consumed
+    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < cnt;
+         f += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = key[f];
+        const uint32_t e = (uint32_t)(k & ((1ull << eb) - 1ull));
+        const uint64_t r = k >> eb;
+        const int2 h = huge[kInter ? r >> nb : r];
+        const int64_t p = off[h.x] + (f - h.y);
+        if constexpr (kInter)
+            citem[p] = make_uint4((uint32_t)h.x, (uint32_t)(r & ((1ull << nb) - 1ull)), e, 0u);
+        else
+            val2[p] = e;
+    }
+}
+
 // Step 3, inter edges: a CTA orders the items of kRankTile consecutive positions and emits them.
 // Every item of a short bucket [off_c[a], off_c[a + 1]) goes to its rank by (b, eid) in the bucket,
-// among the keys in shared memory; the items within a bucket's length of the tile are loaded too, for
-// the buckets that cross its edges.  Long buckets are in order already (k_bucket_sort_long, whose
-// list this empties).  The tile's positions are then in (a, b, eid) order, each new (a, b) starts a
-// coarse edge, and its id is a prefix sum over the tiles by look-back: emap, perm, the segment starts
-// and end points and the coarse degrees go out with no sorted copy, head flags or positions in
-// memory.  Ranked, scanned and emitted by three kernels, the items were written and read again: all
-// levels of a random geometric graph of 2^23 nodes 2,250 -> 1,380 us, 2,500 graphs 1,450 -> 775, a
-// triangle grid of 2048^2 510 -> 420.  Loads and the emission's scattered stores bound it, so many
-// CTAs take turns: tiles of 2,048 items 1,498, 874 and 464, with 128 threads 2,193, 1,018 and 569.
+// among the keys in shared memory; the items within a bucket's length of the tile are loaded too,
+// for the buckets that cross its edges.  Long buckets are in order already (k_bucket_sort_long,
+// whose list this empties, and k_huge_put).  The tile's positions are then in (a, b, eid) order,
+// each new (a, b) starts a coarse edge, and its id is a prefix sum over the tiles by look-back:
+// emap, perm, the segment starts and end points and the coarse degrees go out with no sorted copy,
+// head flags or positions in memory.  Ranked, scanned and emitted by three kernels, the items were
+// written and read again: all levels of a random geometric graph of 2^23 nodes 2,250 -> 1,380 us,
+// 2,500 graphs 1,450 -> 775, a triangle grid of 2048^2 510 -> 420.  Loads and the emission's
+// scattered stores bound it, so many CTAs take turns: tiles of 2,048 items 1,498, 874 and 464, with
+// 128 threads 2,193, 1,018 and 569.
 constexpr int kRankTile = 1024;
 constexpr int kRankThreads = 256;
 constexpr int kRankHalo = kSmallBucket;
@@ -963,8 +1028,7 @@ spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint3
 
 // The lower rows of the coarse CSR take the bucket path while every row holds at most
 // kRankMax lower entries and the ranking work (the sum of squared row sizes) is at most
-// kRankWork per coarse edge; the inter and intra buckets while none is longer than
-// kBlockBucket.
+// kRankWork per coarse edge.
 constexpr int64_t kRankMax = 1024;
 constexpr int64_t kRankWork = 48;
 
@@ -990,6 +1054,30 @@ static spc_status sort_long_buckets(spc_context* ctx, bool inter, const int32_t*
         SPC_LAUNCH(ctx, k_bucket_sort_long<false>, grid, kBlockSortThreads, smem, list, list_cnt,
                    off, citem, iitem, val2);
     }
+    return SPC_OK;
+}
+
+// bits of the values 0 .. n - 1
+static int bits_of(int64_t n) {
+    int b = 0;
+    while (b < 62 && ((int64_t)1 << b) < n) ++b;
+    return b;
+}
+
+// the items of the listed huge buckets in order (k_huge_keys); key and value scratch of cnt items
+template <bool kInter>
+static spc_status sort_huge_buckets(spc_context* ctx, int64_t cnt, int64_t nh, const int2* huge,
+                                    const int32_t* off, int nb, int eb, uint4* citem,
+                                    const uint2* iitem, uint32_t* val2, unsigned long long* stat,
+                                    uint64_t* key, uint64_t* key_alt, uint32_t* val,
+                                    uint32_t* val_alt) {
+    const int grid = grid_for(cnt, kThreads, ctx->num_sms * 8);
+    SPC_LAUNCH(ctx, k_huge_keys<kInter>, grid, kThreads, 0, cnt, (int32_t)nh, huge, off, nb, eb,
+               citem, iitem, key, val);
+    SPC_TRY(radix_sort_u64(ctx, key, val, key_alt, val_alt, cnt,
+                           bits_of(nh) + (kInter ? nb : 0) + eb));
+    SPC_LAUNCH(ctx, k_huge_put<kInter>, grid, kThreads, 0, cnt, huge, off, nb, eb, key, citem, val2,
+               stat);
     return SPC_OK;
 }
 
@@ -1027,6 +1115,8 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
     unsigned long long* bstats = W.b_stats.as<unsigned long long>();
     int32_t* list_c = W.b_list.as<int32_t>();  // long buckets (at most m / kSmallBucket each)
     int32_t* list_i = list_c + (m / kSmallBucket + 1);
+    int2* huge_c = W.b_huge.as<int2>();  // huge buckets (at most m / kBlockBucket each)
+    int2* huge_i = huge_c + (m / kBlockBucket + 1);
     if (W.b_dirty) {
         SPC_CUDA(cudaMemsetAsync(W.b_cnt.p, 0, W.b_cnt.bytes, ctx->stream));
         SPC_CUDA(cudaMemsetAsync(W.b_stats.p, 0, W.b_stats.bytes, ctx->stream));
@@ -1037,14 +1127,15 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
                reinterpret_cast<uint32_t*>(low_deg), (int64_t)(n_c + 1),
                W.counters.as<int32_t>());
     SPC_TRY(scan_fused<unsigned long long>(
-        ctx, n_c, PairLd{cnt_c, cnt_i}, BucketOffSt{off_c, off_i, n_c, bstats, list_c, list_i},
+        ctx, n_c, PairLd{cnt_c, cnt_i},
+        BucketOffSt{off_c, off_i, n_c, bstats, list_c, list_i, huge_c, huge_i},
         (double)n_c * 16.0));
-    int64_t bv[8];
+    int64_t bv[10];
     {
-        const void* ptrs[8] = {off_c + n_c, off_i + n_c, bstats, bstats + 1, bstats + 2,
-                               bstats + 3, bstats + 6, bstats + 7};
-        const int bytes[8] = {4, 4, 8, 8, 8, 8, 8, 8};
-        SPC_TRY(read_vals(ctx, 8, ptrs, bytes, bv));
+        const void* ptrs[10] = {off_c + n_c, off_i + n_c, bstats,     bstats + 1, bstats + 2,
+                                bstats + 3,  bstats + 6,  bstats + 7, bstats + 8, bstats + 9};
+        const int bytes[10] = {4, 4, 8, 8, 8, 8, 8, 8, 8, 8};
+        SPC_TRY(read_vals(ctx, 10, ptrs, bytes, bv));
     }
     const int64_t long_c = bv[6], long_i = bv[7];  // buckets longer than kSmallBucket
     const int64_t m_inter = bv[0];
@@ -1052,7 +1143,13 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
     // no segment is longer than its bucket: without a long bucket no list of long segments is read
     const bool long_inter = bv[3] > kLongRow, long_intra = bv[5] > kLongRow;
     lv.max_intra = bv[5];
-    const bool buckets = bv[3] <= kBlockBucket && bv[5] <= kBlockBucket;
+    const int64_t nh_c = bv[8] >> 32, nh_i = bv[9] >> 32;  // huge buckets and their items
+    const int64_t huge_n = bv[8] & 0xffffffffll, huge_m = bv[9] & 0xffffffffll;
+    const int eb = bits_of(m);
+    // The radix path when the huge buckets hold more than half of the edges: one level whose giant
+    // super-node takes 99 % of 5.9 million edges, 3,145 us by radix, 3,269 with the giant's sorted
+    // apart; where they hold 6 to 20 % the whole call gains 3 to 4 % (k_huge_keys).
+    const bool buckets = 2 * (huge_n + huge_m) <= m && bits_of(nh_c) + nb + eb <= 64;
     if (buckets) {
         if (m > 0) {
             SPC_LAUNCH(ctx, k_bucket_scatter, gm, kThreads, 0, m, W.eu.as<int32_t>(),
@@ -1096,6 +1193,12 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
             if (long_i > 0)
                 SPC_TRY(sort_long_buckets(ctx, false, list_i, bstats + 7, off_i, nullptr, iitem,
                                           ival2));
+            if (nh_i > 0) {  // scratch: this stream's arrays of the long sums, still free
+                uint32_t* v = W.seg_len_side.as<uint32_t>();
+                SPC_TRY(sort_huge_buckets<false>(
+                    ctx, huge_m, nh_i, huge_i, off_i, nb, eb, nullptr, iitem, ival2, bstats + 9,
+                    W.seg_base_side.as<uint64_t>(), W.seg_idx_side.as<uint64_t>(), v, v + huge_m));
+            }
             SPC_LAUNCH(ctx, k_bucket_rank_intra, grid_for(m_intra, kThreads, maxb), kThreads, 0,
                        m_intra, off_i, iitem, ival2, bstats + 7);
         }
@@ -1143,13 +1246,19 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
     bool lower_buckets = true;
     if (m_inter > 0 && buckets) {
         if (long_c > 0)
-            SPC_TRY(sort_long_buckets(ctx, true, list_c, bstats + 6, off_c, citem, nullptr, nullptr));
+            SPC_TRY(sort_long_buckets(ctx, true, list_c, bstats + 6, off_c, citem, nullptr,
+                                      nullptr));
+        if (nh_c > 0)
+            SPC_TRY(sort_huge_buckets<true>(ctx, huge_n, nh_c, huge_c, off_c, nb, eb, citem,
+                                            nullptr, nullptr, bstats + 8, ckey,
+                                            W.c_key2.as<uint64_t>(), cval,
+                                            W.c_val2.as<uint32_t>()));
         const int64_t nt = (m_inter + kRankTile - 1) / kRankTile;
         unsigned long long* tile_status;
         uint32_t* tile_ctr;
         SPC_TRY(scan_tiles(ctx, nt, &tile_status, &tile_ctr));
-        SPC_LAUNCH(ctx, k_bucket_rank_inter, (unsigned)nt, kRankThreads, 0, m_inter, off_c, citem, emap,
-                   perm, seg, cU, cV, up_deg, low_deg, hpos + m_inter, bstats + 6, tile_status,
+        SPC_LAUNCH(ctx, k_bucket_rank_inter, (unsigned)nt, kRankThreads, 0, m_inter, off_c, citem,
+                   emap, perm, seg, cU, cV, up_deg, low_deg, hpos + m_inter, bstats + 6, tile_status,
                    tile_ctr, nt, status);
     } else if (m_inter > 0) {
         const int gi = grid_for(m_inter, kThreads, maxb);

@@ -109,7 +109,7 @@ struct Work {
     Buf c_item, i_item;                                         // bucket items (16 / 8 bytes)
     Buf lower_long;                                             // count of long lower rows
     // contraction buckets: sizes (zero between calls), offsets, ranking statistics
-    Buf b_cnt, b_off, b_stats, b_list;
+    Buf b_cnt, b_off, b_stats, b_list, b_huge;
     bool b_dirty = true;
     Buf sort_hist, scan_tmp;                                    // sort / scan temporaries
     Buf stage_rowptr, stage_col, stage_w, stage_lift, stage_gptr;  // host staging
