@@ -442,7 +442,7 @@ static spc_status reserve_work(spc_context* ctx, int64_t n, int64_t m, int64_t B
     SPC_TRY(ensure_zeroed(ctx, W.b_cnt, 2 * N * 4));
     SPC_TRY(ensure(ctx, W.b_off, 2 * N * 4));
     SPC_TRY(ensure_zeroed(ctx, W.b_stats, 10 * 8));
-    SPC_TRY(ensure(ctx, W.b_huge, 2 * (M / 8192 + 1) * 8));
+    SPC_TRY(ensure(ctx, W.b_huge, 2 * (M / 2048 + 1) * 8));
     SPC_TRY(ensure(ctx, W.b_list, (2 * (M / 64 + 1) + 16) * 4));  // long-bucket lists
     // tile statuses: scans of up to max(n, m, 256 * tiles) items, the ranking's tiles of 1,024
     // edges; radix histograms

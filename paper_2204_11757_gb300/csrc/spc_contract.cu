@@ -98,12 +98,16 @@ __device__ __forceinline__ void warp_count(int32_t* cnt, int32_t key, bool act) 
 // Buckets of at most kSmallBucket items: each item is ranked by one thread (at most
 // kSmallBucket comparisons per item).  Longer ones are listed by the scan of the bucket sizes:
 // up to kWarpBucket items, one warp ranks the bucket's items by comparison in shared memory;
-// up to kBlockBucket items, one CTA sorts the bucket in shared memory (bitonic network).
+// up to kBlockBucket items, one CTA sorts the bucket in shared memory (bitonic network); longer ones
+// are sorted together by radix, which costs less per item from there on (2,500 graphs with 500
+// buckets of 1,025 to 8,192 items on two of three levels, whole call: 19.9 ms with the network up to
+// 8,192 items, 19.7 up to 2,048 or 1,024).
 constexpr int kSmallBucket = 64;
 constexpr int kWarpBucket = 256;
-constexpr int kBlockBucket = 8192;
+constexpr int kBlockBucket = 2048;
 constexpr int kBlockSortThreads = 512;
-static_assert((kBlockSortThreads / 32) * kWarpBucket <= kBlockBucket,
+constexpr int kStageKeys = 4096;
+static_assert(kBlockBucket <= kStageKeys && (kBlockSortThreads / 32) * kWarpBucket <= kStageKeys,
               "the warps' stages share the CTA's");
 
 // Statistics of a block's scanned values, K sides of (sum of squares, maximum), added into
@@ -371,7 +375,7 @@ k_bucket_sort_long(const int32_t* __restrict__ list, const unsigned long long* _
                    const int32_t* __restrict__ off, uint4* citem,
                    const uint2* __restrict__ iitem, uint32_t* __restrict__ val2) {
     spc::pdl_wait();
-    extern __shared__ unsigned long long sk[];  // kBlockBucket keys
+    extern __shared__ unsigned long long sk[];  // kStageKeys keys
     const int64_t cnt = (int64_t)*list_cnt;
     for (int64_t q = blockIdx.x; q < cnt; q += gridDim.x) {
         const int32_t bkt = list[q];
@@ -1032,11 +1036,11 @@ spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint3
 constexpr int64_t kRankMax = 1024;
 constexpr int64_t kRankWork = 48;
 
-// one CTA per long bucket, each with kBlockBucket keys of shared memory
+// one CTA per long bucket, each with kStageKeys keys of shared memory
 static spc_status sort_long_buckets(spc_context* ctx, bool inter, const int32_t* list,
                                     const unsigned long long* list_cnt, const int32_t* off,
                                     uint4* citem, const uint2* iitem, uint32_t* val2) {
-    constexpr int smem = kBlockBucket * 8;
+    constexpr int smem = kStageKeys * 8;
     static std::atomic<unsigned long long> attr_devs{0};  // devices already set up
     const unsigned long long bit = 1ull << (ctx->device & 63);
     if (!(attr_devs.load() & bit)) {

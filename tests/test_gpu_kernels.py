@@ -275,30 +275,31 @@ def test_buckets_across_the_ranking_tiles(ctx, dtype, size):
 
 
 @pytest.mark.parametrize("dtype", [np.int32, np.float32, np.float64])
-@pytest.mark.parametrize("blocks,extra,clique", [(1, 0, 10), (1, 1, 129), (1, 0, 140), (3, 1, 10),
-                                                 (5, 1, 140)])
+@pytest.mark.parametrize("blocks,extra,clique", [(1, 0, 10), (1, 1, 64), (1, 0, 65), (3, 1, 10),
+                                                 (5, 1, 140), (90, 1, 10)])
 def test_huge_buckets_among_short_ones(ctx, dtype, blocks, extra, clique):
-    """Buckets of 8,192 and 8,193 inter edges and intra buckets on both sides of 8,192 (a clique of
-    129 has 8,256 edges), fewer than half of the edges: sorted apart from the ranked ones."""
+    """Buckets of 2,048 and 2,049 inter edges and intra buckets on both sides of 2,048 (cliques of 64
+    and 65 have 2,016 and 2,080 edges), fewer than half of the edges: sorted apart from the ranked
+    ones."""
     from paper_2204_11757_gb300 import api
     rng = np.random.default_rng(blocks + extra)
     eu, ev, lift, n, U = [], [], [], 0, 0
     for q in range(blocks):  # a complete bipartite block: one bucket, one or two coarse edges
-        A, B = n + np.arange(64), n + 64 + np.arange(128)
-        eu.append(np.repeat(A, 128))
-        ev.append(np.tile(B, 64))
+        A, B = n + np.arange(32), n + 32 + np.arange(64)
+        eu.append(np.repeat(A, 64))
+        ev.append(np.tile(B, 32))
         if extra:
             eu.append(A[:1])
             ev.append(B[-1:] + 1)  # into whatever comes next
-        lift += [U] * 64 + [U + 1] * 128
-        n, U = n + 192, U + 2
+        lift += [U] * 32 + [U + 1] * 64
+        n, U = n + 96, U + 2
     for _ in range(2):
         iu, iv = np.triu_indices(clique, 1)
         eu.append(n + iu)
         ev.append(n + iv)
         lift += [U] * clique
         n, U = n + clique, U + 1
-    k = 30000 * blocks
+    k = 30000 + 3000 * blocks
     C = n + np.arange(k)
     eu.append(C)
     ev.append(np.roll(C, -1))
@@ -306,9 +307,8 @@ def test_huge_buckets_among_short_ones(ctx, dtype, blocks, extra, clique):
     n, U = n + k, U + k // 2
     perm = rng.permutation(n)  # node numbers in any order
     eu, ev = perm[np.concatenate(eu)], perm[np.concatenate(ev)]
-    nl = np.empty(n, dtype=np.int64)
-    nl[perm] = lift
-    lift = rng.permutation(U)[nl].astype(np.int32)
+    lift, old = np.empty(n, dtype=np.int32), lift
+    lift[perm] = old
     w = rng.integers(1, 99, eu.shape[0]) if dtype == np.int32 else rng.random(eu.shape[0]) + 0.1
     g = I.csr_from_edges(n, eu, ev, w.astype(dtype))
     c = O.contract(g, lift, U)
@@ -318,7 +318,7 @@ def test_huge_buckets_among_short_ones(ctx, dtype, blocks, extra, clique):
         prof = ctx.kernel_profile()
     finally:
         ctx.time_kernel(None)
-    assert any("k_huge_put" in k for k in prof) == bool(extra or clique > 128)
+    assert any("k_huge_put" in k for k in prof) == bool(extra or clique > 64)
     assert not any("k_classify" in k for k in prof)
     assert np.array_equal(lv.emap.cpu().numpy(), c.emap)
     assert np.array_equal(_bits(lv.a_und.cpu().numpy()), _bits(c.a_und))
