@@ -22,6 +22,8 @@
 //      first n_b - target_b of each graph are united.
 //   3. Relabel: root = smallest member; flag roots, exclusive scan, id = scan[root] (Definition
 //      1's super-nodes, numbered by smallest member).
+// Small graphs -- one, or a batch of which every graph fits -- take these steps in one CTA each, in
+// shared memory (k_select_small).
 // Every retry loop is bounded (spin_limit: kSpinLimit unless the context lowered it); giving up
 // sets DEV_TIMEOUT in the status word.
 #include <atomic>
@@ -617,10 +619,10 @@ template <> struct GpShift<unsigned long long> { static constexpr int s1 = 52, s
 // count before it.  Every thread of the block calls it.
 __device__ void cta_find_bin(const uint32_t* hist, int64_t need, int* bin_out,
                              int64_t* before_out) {
-    __shared__ unsigned long long s_part[kGpThreads / 32];
+    __shared__ unsigned long long s_part[32];
     __shared__ int s_bin;
     __shared__ long long s_before;
-    constexpr int kPer = kGpBins / kGpThreads;
+    const int kPer = kGpBins / (int)blockDim.x;  // blocks of 256, 512 or 1024 threads
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     unsigned long long loc = 0;
     for (int j = 0; j < kPer; ++j) loc += hist[t * kPer + j];
@@ -632,8 +634,8 @@ __device__ void cta_find_bin(const uint32_t* hist, int64_t need, int* bin_out,
     if (lane == 31) s_part[w] = incl;
     if (t == 0) s_bin = kGpBins - 1;
     __syncthreads();
-    unsigned long long base = 0;
-    for (int i = 0; i < w; ++i) base += s_part[i];
+    // (the counts of one graph's edges: below 2^31)
+    const unsigned base = __reduce_add_sync(0xffffffffu, lane < w ? (unsigned)s_part[lane] : 0u);
     unsigned long long run = base + incl - loc;  // count before this thread's bins
     if (run < (unsigned long long)need && run + loc >= (unsigned long long)need) {
         for (int j = 0; j < kPer; ++j) {
@@ -653,10 +655,11 @@ __device__ void cta_find_bin(const uint32_t* hist, int64_t need, int* bin_out,
 }
 
 // the smallest threshold t (its low s2 bits all set) with at least `need` keys of key[e0, e1)
-// at or below it; 1 <= need <= e1 - e0.  Every thread of the block calls it.
+// at or below it, and (unless null) their number; 1 <= need <= e1 - e0.  Every thread of the block
+// calls it.
 template <class KT>
 __device__ KT cta_select_key(const KT* __restrict__ key, int64_t e0, int64_t e1, int64_t need,
-                             uint32_t* hist) {
+                             uint32_t* hist, int64_t* below = nullptr) {
     constexpr int S1 = GpShift<KT>::s1, S2 = GpShift<KT>::s2;
     constexpr int kB = 8;  // keys per thread in flight (one CTA may walk a large graph)
     const int64_t step = (int64_t)blockDim.x * kB;
@@ -696,6 +699,7 @@ __device__ KT cta_select_key(const KT* __restrict__ key, int64_t e0, int64_t e1,
     int c2;
     int64_t before2;
     cta_find_bin(hist, need - before, &c2, &before2);
+    if (below) *below = before + before2 + hist[c2];
     return ((KT)c1 << S1) | ((KT)c2 << S2) | (((KT)1 << S2) - 1);
 }
 
@@ -827,6 +831,545 @@ __device__ __forceinline__ uint32_t sel_digit(KT hi, uint32_t lo, int r) {
     const int top = 32 - kSelBits * q;
     const int lowb = top - kSelBits > 0 ? top - kSelBits : 0;
     return (lo >> lowb) & ((1u << (top - lowb)) - 1u);
+}
+
+// ---- the merge selection of small graphs, one CTA per graph --------------------------------------
+// The whole selection of one graph -- score slabs, spanning-forest rounds, the k lightest forest
+// edges, the second union-find and the numbering inside the graph -- with the union-find and the
+// components' best edges in shared memory.  A graph of a few thousand nodes has too little work per
+// round for the whole GPU: every grid barrier or launch costs more than the round's work, while a
+// batch keeps an SM per graph busy.  Shared memory bounds it (random 8-byte slots, compare-and-swap
+// on them, walks).  2,500 graphs of 20 to 19,881 nodes, binary32, a call of three levels: 19.7 ms
+// with the launches of select_batch over all graphs at once, 17.0 so; one graph of 4,096 nodes and
+// 12,033 edges down to a half (a sixteenth): 129 (144) us in k_select_coop, 52 (91) here.
+template <class KT>
+struct SmallArgs {
+    int64_t n, m, target;         // one graph: graph_ptr null
+    const int64_t* graph_ptr;     // a batch: block b takes graph b when n_min < its nodes <= n_max
+    const int64_t* targets;
+    const int32_t* up_ptr;
+    int32_t n_min, n_max;
+    int32_t bytes;                // dynamic shared memory
+    const int32_t* eu;
+    const int32_t* ev;
+    const KT* key;
+    unsigned long long* lk;       // scratch for live edges that do not fit into shared memory: keys
+    int32_t* le;                  // (32-bit ones with the edge's place below), places (64-bit keys)
+    uint32_t* lp;                 // and two 16-bit ends
+    KT* fk;                       // scratch: the forest edges' keys and ids
+    uint32_t* fe;
+    int32_t* lift;                // super-node of every node, counted from 0 in its graph
+    uint8_t* merged;
+    int32_t* n_c;                 // super-nodes of every graph
+    uint32_t* status;
+};
+
+// One CTA's limits: edges that one SM reads in a few tens of us, and nodes that fit into 203 KB of
+// shared memory (the rest is L1's); 1,024 threads on an SM whatever the class: four CTAs of 256,
+// two of 512, one of 1,024.  What the nodes leave of a CTA's shared memory holds the live edges.
+// One graph alone comes here up to kSmallOne nodes: 9,216 nodes and 27,265 edges take 91 us (to a
+// half) and 174 (to a sixteenth) here, 155 and 170 in k_select_coop; 13,806 nodes 127 and 244
+// against 162 and 177.
+constexpr int64_t kSmallOne = 8192;
+constexpr int kSmallEdgeBits = 17;
+constexpr int64_t kSmallEdges = int64_t{1} << kSmallEdgeBits;
+constexpr int kSmallBytes[3] = {54 * 1024, 110 * 1024, 203 * 1024};
+template <class KT>
+struct SmallMem {
+    // best slot, 16-bit parent and (64-bit scores) best edge of every node
+    static constexpr int kNode = 8 + 2 + (MinKey<KT>::two_phase ? 4 : 0);
+    static constexpr int kItem = 8 + 4 + (MinKey<KT>::two_phase ? 4 : 0);  // of a live edge
+    static constexpr int kFixed = kGpBins * 4;
+    static constexpr int nodes(int bytes) { return (bytes - kFixed) / kNode / 4 * 4; }
+    static constexpr int kMaxNodes = nodes(kSmallBytes[2]);
+};
+static_assert(SmallMem<unsigned int>::kMaxNodes < 65536 &&
+                  SmallMem<unsigned long long>::kMaxNodes >= kSmallOne,
+              "16-bit ends and parents; one graph fits");
+
+// union-find in shared memory, as uf_find_n and uf_unite above (bounded; giving up returns a node
+// of the set)
+template <int N>
+__device__ __forceinline__ void sm_find_n(volatile uint16_t* par, int32_t (&x)[N], unsigned live,
+                                          uint32_t lim, uint32_t* status) {
+    for (uint32_t it = 0; it < lim; ++it) {
+        int32_t p[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) p[i] = (live >> i & 1u) ? (int32_t)par[x[i]] : x[i];
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (p[i] == x[i]) live &= ~(1u << i);
+        if (!live) return;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            if (!(live >> i & 1u)) continue;
+            const int32_t gp = par[p[i]];
+            if (gp == p[i]) live &= ~(1u << i);
+            else par[x[i]] = (uint16_t)gp;
+            x[i] = gp;
+        }
+        if (!live) return;
+    }
+    atomicOr(status, DEV_TIMEOUT);
+}
+
+__device__ __forceinline__ bool sm_unite(uint16_t* par, int32_t a, int32_t b, uint32_t lim,
+                                         uint32_t* status) {
+    int32_t x[2] = {a, b};
+    for (uint32_t it = 0; it < lim; ++it) {
+        sm_find_n<2>(par, x, 3u, lim, status);
+        if (x[0] == x[1]) return false;
+        if (x[0] > x[1]) {
+            const int32_t t = x[0];
+            x[0] = x[1];
+            x[1] = t;
+        }
+        if (atomicCAS(par + x[1], (uint16_t)x[1], (uint16_t)x[0]) == x[1]) return true;
+    }
+    atomicOr(status, DEV_TIMEOUT);
+    return false;
+}
+
+// atomicMin that first looks (the slot of a component with many edges is rarely lowered)
+__device__ __forceinline__ void sm_min(unsigned long long* a, unsigned long long v) {
+    if (v < *reinterpret_cast<volatile unsigned long long*>(a)) atomicMin(a, v);
+}
+
+constexpr int kSmallFlight = 4;  // live edges of a thread in flight
+
+template <class KT, int T>
+__global__ void __launch_bounds__(T, 1024 / T) k_select_small(SmallArgs<KT> a) {
+    spc::pdl_wait();
+    constexpr bool two = MinKey<KT>::two_phase;
+    constexpr int H = SelBits<KT>::kHiRounds, P = kSmallFlight;
+    extern __shared__ unsigned long long sm_raw[];
+    __shared__ int32_t s_forest, s_live;
+    __shared__ int32_t s_max[2];
+    __shared__ int32_t s_sum[T / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lim = spin_limit(a.status);
+    const int64_t b = blockIdx.x;
+    const int64_t n0 = a.graph_ptr ? a.graph_ptr[b] : 0;
+    const int64_t n1 = a.graph_ptr ? a.graph_ptr[b + 1] : a.n;
+    const int32_t nb = (int32_t)(n1 - n0), first = (int32_t)n0;
+    if (nb <= a.n_min || nb > a.n_max) return;  // another class's graph
+    const int64_t e0 = a.graph_ptr ? a.up_ptr[n0] : 0, e1 = a.graph_ptr ? a.up_ptr[n1] : a.m;
+    const int32_t mb = (int32_t)(e1 - e0);
+    const int64_t k_b = nb - (a.graph_ptr ? a.targets[b] : a.target);
+    const int32_t k = k_b > 0 ? (int32_t)k_b : 0;
+    const int32_t nm = (nb + 3) / 4 * 4;
+    const int32_t cap = (a.bytes - SmallMem<KT>::kFixed - nm * SmallMem<KT>::kNode) /
+                        SmallMem<KT>::kItem;
+    unsigned long long* best = sm_raw;                               // [nm] best slots
+    unsigned long long* sk = best + nm;                              // [cap] live edges: lk, lp, le
+    uint32_t* hist = reinterpret_cast<uint32_t*>(sk + cap);          // [kGpBins]
+    uint32_t* sp = hist + kGpBins;                                   // [cap]
+    int32_t* se = reinterpret_cast<int32_t*>(sp + cap);              // [cap] when two
+    int32_t* beste = se + (two ? cap : 0);                           // [nm] when two
+    uint16_t* par = reinterpret_cast<uint16_t*>(beste + (two ? nm : 0));  // [nm]
+    const KT* __restrict__ key = a.key + e0;
+    const int32_t* __restrict__ eu = a.eu + e0;
+    const int32_t* __restrict__ ev = a.ev + e0;
+    KT* fk = a.fk + e0;
+    uint32_t* fe = a.fe + e0;
+    for (int32_t x = tid; x < nb; x += T) {
+        par[x] = (uint16_t)x;
+        best[x] = ~0ull;
+        if (two) beste[x] = INT32_MAX;
+    }
+    if (a.merged)
+        for (int32_t e = tid; e < mb; e += T) a.merged[e0 + e] = 0;
+    if (tid == 0) {
+        s_forest = 0;
+        s_live = 0;
+        s_max[0] = 0;
+        s_max[1] = 0;
+    }
+    __syncthreads();
+    // ---- forest: slabs of 1.5 k keys, then twice as many, until the forest holds k edges
+    int32_t forest = 0;
+    int64_t need = (int64_t)k + k / 2, taken = 0;  // taken: keys at or below lo
+    KT lo = 0;
+    bool above = false;  // the slab starts above lo
+    // 32-bit keys: every round's entries of the best slots lie below the earlier rounds', so the
+    // slots need no reset (16 bits of round, 31 of key, 17 of the edge's place in its graph)
+    unsigned tag = 0xffffu;
+    while (k > 0) {
+        const bool all = need >= mb;
+        int64_t upto = mb;
+        const KT tau = all ? ~KT(0) : cta_select_key<KT>(key, 0, mb, need, hist, &upto);
+        // the slab's edges, listed densely: thread t takes the places t, t + T, ...
+        bool shared = upto - taken <= cap;
+        unsigned long long* lk = shared ? sk : a.lk + e0;
+        uint32_t* lp = shared ? sp : a.lp + e0;
+        int32_t* le = shared ? se : a.le + e0;
+        for (int32_t w0 = warp * 32; w0 < mb; w0 += 2 * P * T) {  // warp-uniform
+            KT kk[2 * P];
+            unsigned in = 0;
+#pragma unroll
+            for (int q = 0; q < 2 * P; ++q) {
+                const int32_t e = w0 + q * T + lane;
+                kk[q] = e < mb ? key[e] : KT(0);
+                if (e < mb && kk[q] <= tau && (!above || kk[q] > lo)) in |= 1u << q;
+            }
+            // the ends of every taken edge in flight: no branch between the loads
+            int32_t u[2 * P], v[2 * P];
+#pragma unroll
+            for (int q = 0; q < 2 * P; ++q) {
+                const int32_t e = in >> q & 1u ? w0 + q * T + lane : 0;
+                u[q] = eu[e];
+                v[q] = ev[e];
+            }
+            const int32_t mine = __reduce_add_sync(0xffffffffu, __popc(in));
+            int32_t at = 0;
+            if (lane == 0 && mine > 0) at = atomicAdd(&s_live, mine);
+            at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+            for (int q = 0; q < 2 * P; ++q) {
+                const bool take = in >> q & 1u;
+                const unsigned lanes = __ballot_sync(0xffffffffu, take);
+                const int32_t to = at + __popc(lanes & ((1u << lane) - 1u));
+                at += __popc(lanes);
+                if (!take) continue;
+                const int32_t e = w0 + q * T + lane;
+                if constexpr (two) {
+                    lk[to] = kk[q];
+                    le[to] = e;
+                } else {
+                    lk[to] = ((unsigned long long)kk[q] << kSmallEdgeBits) | (uint32_t)e;
+                }
+                lp[to] = (uint32_t)(u[q] - first) | ((uint32_t)(v[q] - first) << 16);
+            }
+        }
+        __syncthreads();
+        const int32_t live0 = s_live;
+        int32_t cnt = (live0 - tid + T - 1) / T;
+        int32_t most = (live0 + T - 1) / T;  // the longest column
+        for (int round = 0;; ++round) {
+            // the live edges between components lower both components' best slots
+            --tag;
+            const bool move = !shared && (int64_t)most * T <= cap;  // into shared memory
+            unsigned long long* dk = move ? sk : lk;
+            uint32_t* dp = move ? sp : lp;
+            int32_t* de = move ? se : le;
+            int32_t keep = 0;
+            for (int32_t j0 = 0; j0 < cnt; j0 += P) {
+                unsigned long long pk[P];
+                int32_t e[P], x[2 * P];
+                unsigned live = 0;
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const int32_t at = (j0 + q) * T + tid;
+                    const bool in = j0 + q < cnt;
+                    pk[q] = in ? lk[at] : 0ull;
+                    e[q] = two && in ? le[at] : 0;
+                    const uint32_t uv = in ? lp[at] : 0u;
+                    x[2 * q] = (int32_t)(uv & 0xffffu);
+                    x[2 * q + 1] = (int32_t)(uv >> 16);
+                    if (in) live |= 3u << (2 * q);
+                }
+                // round 0 of the first slab: every node is its own component
+                if (round > 0 || above) sm_find_n<2 * P>(par, x, live, lim, a.status);
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const int32_t u = x[2 * q], v = x[2 * q + 1];
+                    if (u == v) continue;  // (both 0 past the end)
+                    const unsigned long long t =
+                        two ? pk[q] : pk[q] | (unsigned long long)tag << 48;
+                    sm_min(best + u, t);
+                    sm_min(best + v, t);
+                    const int32_t to = keep * T + tid;
+                    dk[to] = pk[q];
+                    if (two) de[to] = e[q];
+                    dp[to] = (uint32_t)u | ((uint32_t)v << 16);
+                    ++keep;
+                }
+            }
+            cnt = keep;
+            if (move) {
+                shared = true;
+                lk = sk;
+                lp = sp;
+                le = se;
+            }
+            const int32_t wmax = __reduce_max_sync(0xffffffffu, cnt);
+            if (lane == 0 && wmax > 0) atomicMax(&s_max[round & 1], wmax);
+            __syncthreads();
+            most = s_max[round & 1];
+            if (tid == 0) s_max[(round & 1) ^ 1] = 0;
+            if (most == 0) break;
+            if (round > 64) {  // every round at least halves the components that still have edges
+                if (tid == 0) atomicOr(a.status, DEV_TIMEOUT);
+                break;
+            }
+            if constexpr (two) {  // the smallest edge id among the ties
+                for (int32_t j = 0; j < cnt; ++j) {
+                    const int32_t at = j * T + tid;
+                    const uint32_t uv = lp[at];
+                    const int32_t e = le[at], u = (int32_t)(uv & 0xffffu), v = (int32_t)(uv >> 16);
+                    const unsigned long long pk = lk[at];
+                    if (best[u] == pk) atomicMin(beste + u, e);
+                    if (best[v] == pk) atomicMin(beste + v, e);
+                }
+                __syncthreads();
+            }
+            // the chosen edges are forest edges
+            for (int32_t j0 = 0; j0 < cnt; j0 += P) {
+                unsigned long long pk[P];
+                int32_t e[P];
+                uint32_t uv[P];
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const int32_t at = (j0 + q) * T + tid;
+                    const bool in = j0 + q < cnt;
+                    pk[q] = in ? lk[at] : 0ull;
+                    e[q] = two && in ? le[at] : (int32_t)(pk[q] & (kSmallEdges - 1));
+                    uv[q] = in ? lp[at] : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    if (uv[q] == 0u) continue;  // two components: not both 0
+                    const int32_t u = (int32_t)(uv[q] & 0xffffu), v = (int32_t)(uv[q] >> 16);
+                    bool pick;
+                    if constexpr (two) {
+                        pick = (best[u] == pk[q] && beste[u] == e[q]) ||
+                               (best[v] == pk[q] && beste[v] == e[q]);
+                    } else {
+                        const unsigned long long t = pk[q] | (unsigned long long)tag << 48;
+                        pick = best[u] == t || best[v] == t;
+                    }
+                    if (pick && sm_unite(par, u, v, lim, a.status)) {
+                        const int32_t at_f = atomicAdd(&s_forest, 1);
+                        fk[at_f] = two ? (KT)pk[q] : (KT)(pk[q] >> kSmallEdgeBits);
+                        fe[at_f] = (uint32_t)e[q];
+                    }
+                }
+            }
+            __syncthreads();
+            if constexpr (two) {
+                for (int32_t j = 0; j < cnt; ++j) {
+                    const uint32_t uv = lp[j * T + tid];
+                    const int32_t u = (int32_t)(uv & 0xffffu), v = (int32_t)(uv >> 16);
+                    best[u] = ~0ull;
+                    best[v] = ~0ull;
+                    beste[u] = INT32_MAX;
+                    beste[v] = INT32_MAX;
+                }
+                __syncthreads();
+            }
+        }
+        forest = s_forest;
+        if (forest >= k || all) break;
+        lo = tau;
+        taken = upto;
+        above = true;
+        need *= 2;
+        __syncthreads();  // every thread has read s_forest and s_max
+        if (tid == 0) {
+            s_live = 0;
+            s_max[0] = 0;
+            s_max[1] = 0;
+        }
+        __syncthreads();
+    }
+    __syncthreads();
+    if (forest > k) {
+        // ---- the k lightest: the key digits of the k-th, most significant first, until all items
+        // that share them are wanted
+        KT hi = 0;
+        uint32_t low = 0;
+        int64_t rest = k;
+        int r = 0;
+        for (;; ++r) {
+            for (int i = tid; i < kSelBins; i += T) hist[i] = 0u;
+            __syncthreads();
+            const int top = r < H ? SelBits<KT>::kKeyBits - kSelBits * r : 32 - kSelBits * (r - H);
+            const int lowb = top - kSelBits > 0 ? top - kSelBits : 0;
+#pragma unroll 4
+            for (int32_t i = tid; i < forest; i += T) {
+                const KT x = fk[i];
+                const uint32_t y = fe[i];
+                const bool same = r < H ? (r == 0 || (x >> top) == hi)
+                                        : x == hi && (r == H || (y >> top) == low);
+                if (same) atomicAdd(hist + sel_digit<KT>(x, y, r), 1u);
+            }
+            __syncthreads();
+            int bin;
+            int64_t before;
+            cta_find_bin(hist, rest, &bin, &before);
+            rest -= before;
+            const bool whole = (int64_t)hist[bin] == rest;
+            if (r < H) hi = (KT)((hi << (top - lowb)) | (KT)bin);
+            else low = (low << (top - lowb)) | (uint32_t)bin;
+            __syncthreads();
+            if (whole || r == SelBits<KT>::kRounds - 1) break;
+        }
+        for (int32_t x = tid; x < nb; x += T) par[x] = (uint16_t)x;
+        __syncthreads();
+        const int top = r < H ? SelBits<KT>::kKeyBits - kSelBits * r : 32 - kSelBits * (r - H);
+        const int lowb = top - kSelBits > 0 ? top - kSelBits : 0;
+        for (int32_t i0 = tid; i0 < forest; i0 += P * T) {
+            KT x[P];
+            uint32_t y[P];
+            int32_t u[P], v[P];
+            bool in[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int32_t i = i0 + q * T < forest ? i0 + q * T : 0;
+                x[q] = fk[i];
+                y[q] = fe[i];
+            }
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                in[q] = i0 + q * T < forest &&
+                        (r < H ? (x[q] >> lowb) <= hi
+                               : x[q] < hi || (x[q] == hi && (y[q] >> lowb) <= low));
+                u[q] = eu[y[q]];
+                v[q] = ev[y[q]];
+                if (in[q] && a.merged) a.merged[e0 + y[q]] = 1;
+            }
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+                if (in[q]) sm_unite(par, u[q] - first, v[q] - first, lim, a.status);
+        }
+    } else if (a.merged) {
+        for (int32_t i = tid; i < forest; i += T) a.merged[e0 + fe[i]] = 1;
+    }
+    __syncthreads();
+    // ---- numbering by smallest member: roots are their sets' smallest nodes
+    int32_t* ids = reinterpret_cast<int32_t*>(best);  // [nb]
+    const int32_t per = (nb + T - 1) / T;
+    const int32_t x0 = tid * per < nb ? tid * per : nb, x1 = x0 + per < nb ? x0 + per : nb;
+    int32_t roots = 0;
+    for (int32_t x = x0; x < x1; ++x) roots += par[x] == x ? 1 : 0;
+    const int32_t incl = scanf::warp_incl_scan(roots);
+    if (lane == 31) s_sum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const int32_t t = scanf::warp_incl_scan(lane < T / 32 ? s_sum[lane] : 0);
+        if (lane < T / 32) s_sum[lane] = t;
+    }
+    __syncthreads();
+    int32_t id = (warp > 0 ? s_sum[warp - 1] : 0) + incl - roots;
+    for (int32_t x = x0; x < x1; ++x) {
+        const bool root = par[x] == x;
+        ids[x] = root ? id : 0;
+        id += root ? 1 : 0;
+    }
+    __syncthreads();
+    for (int32_t y0 = tid; y0 < nb; y0 += P * T) {
+        int32_t x[P];
+        unsigned live = 0;
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const bool in = y0 + q * T < nb;
+            x[q] = in ? y0 + q * T : 0;
+            if (in) live |= 1u << q;
+        }
+        sm_find_n<P>(par, x, live, lim, a.status);
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+            if (y0 + q * T < nb) a.lift[n0 + y0 + q * T] = ids[x[q]];
+    }
+    if (tid == 0) a.n_c[b] = s_sum[T / 32 - 1];
+}
+
+// a batch's numbering: every graph's super-nodes after those of the graphs before it
+__global__ void __launch_bounds__(kThreads)
+k_small_shift(int64_t B, const int64_t* __restrict__ graph_ptr, const int32_t* __restrict__ off,
+              const int64_t* __restrict__ targets, int32_t* __restrict__ lift,
+              int64_t* __restrict__ graph_ptr_c, int32_t* __restrict__ warn) {
+    spc::pdl_wait();
+    for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
+        const int32_t o = off[b];
+        for (int64_t x = graph_ptr[b] + threadIdx.x; x < graph_ptr[b + 1]; x += blockDim.x)
+            lift[x] += o;
+        if (threadIdx.x == 0) {
+            graph_ptr_c[b] = o;
+            if (b == B - 1) graph_ptr_c[B] = off[B];
+            if ((int64_t)off[b + 1] - o > targets[b]) atomicOr(warn, 1);
+        }
+    }
+}
+
+// the largest graph of a batch: out[0] nodes, out[1] edges; out[2] = 0 (the warn flag)
+__global__ void __launch_bounds__(1024)
+k_largest_graph(int64_t B, const int64_t* __restrict__ graph_ptr,
+                const int32_t* __restrict__ up_ptr, int32_t* __restrict__ out) {
+    spc::pdl_wait();
+    __shared__ int32_t s_n[32], s_m[32];
+    int32_t n = 0, m = 0;
+    for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
+        const int64_t n0 = graph_ptr[b], n1 = graph_ptr[b + 1];
+        n = max(n, (int32_t)(n1 - n0));
+        m = max(m, up_ptr[n1] - up_ptr[n0]);
+    }
+    n = __reduce_max_sync(0xffffffffu, n);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) {
+        s_n[threadIdx.x >> 5] = n;
+        s_m[threadIdx.x >> 5] = m;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        n = __reduce_max_sync(0xffffffffu, s_n[threadIdx.x]);
+        m = __reduce_max_sync(0xffffffffu, s_m[threadIdx.x]);
+        if (threadIdx.x == 0) {
+            out[0] = n;
+            out[1] = m;
+            out[2] = 0;
+        }
+    }
+}
+
+// k_select_small over B graphs of at most n_max nodes, by classes of sizes
+template <class KT, int T>
+spc_status launch_small_class(spc_context* ctx, SmallArgs<KT>& a, int64_t B, int bytes) {
+    a.n_max = SmallMem<KT>::nodes(bytes);
+    a.bytes = bytes;
+    static std::atomic<unsigned long long> attr_devs{0};  // devices already set up
+    const unsigned long long bit = 1ull << (ctx->device & 63);
+    if (!(attr_devs.load() & bit)) {
+        SPC_CUDA(cudaFuncSetAttribute(k_select_small<KT, T>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        attr_devs.fetch_or(bit);
+    }
+    SPC_LAUNCH(ctx, (k_select_small<KT, T>), (unsigned)B, T, bytes, a);
+    a.n_min = a.n_max;
+    return SPC_OK;
+}
+
+template <class KT>
+spc_status launch_small(spc_context* ctx, const GraphView& g, const KT* key, const SelectArgs& sa,
+                        int64_t B, int64_t n_max, int32_t* lift, uint8_t* merged, int32_t* n_c) {
+    Work& W = ctx->work;
+    SmallArgs<KT> a{};
+    a.n = g.n;
+    a.m = g.m;
+    a.target = sa.target;
+    a.graph_ptr = sa.d_graph_ptr;
+    a.targets = sa.d_targets;
+    a.up_ptr = W.up_ptr.as<int32_t>();
+    a.n_min = -1;
+    a.eu = W.eu.as<int32_t>();
+    a.ev = W.ev.as<int32_t>();
+    a.key = key;
+    a.lk = W.sel_key2.as<unsigned long long>();
+    a.le = W.wl_e[0].as<int32_t>();
+    a.lp = W.wl_u[0].as<uint32_t>();
+    a.fk = W.sel_key.as<KT>();
+    a.fe = W.sel_val.as<uint32_t>();
+    a.lift = lift;
+    a.merged = merged;
+    a.n_c = n_c;
+    a.status = ctx->d_status;
+    if (B > ctx->num_sms) {  // a graph per SM or less takes the most threads
+        SPC_TRY((launch_small_class<KT, 256>(ctx, a, B, kSmallBytes[0])));
+        if (n_max > a.n_max)
+            SPC_TRY((launch_small_class<KT, 512>(ctx, a, B, kSmallBytes[1])));
+        if (n_max <= a.n_max) return SPC_OK;
+    }
+    return launch_small_class<KT, 1024>(ctx, a, B, kSmallBytes[2]);
 }
 
 // root flags (a root is its set's smallest member and its own parent)
@@ -1582,6 +2125,21 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
                          int32_t* lift, uint8_t* merged, int64_t* n_c_out, int32_t* status_out) {
     Work& W = ctx->work;
     const int64_t n = g.n, m = g.m;
+    if (n <= kSmallOne && m <= kSmallEdges) {
+        SelectArgs sa;
+        sa.target = target;
+        int32_t* nc = W.counters.as<int32_t>() + 4;
+        SPC_TRY(launch_small<KT>(ctx, g, key, sa, 1, n, lift, merged, nc));
+        int64_t vals[2];
+        const void* ptrs[2] = {nc, ctx->d_status};
+        const int bytes[2] = {4, 4};
+        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, vals));
+        const spc_status st = status_from_bits((uint32_t)vals[1]);
+        if (st < 0) return st;
+        *n_c_out = vals[0];
+        *status_out = vals[0] > target ? SPC_WARN_TARGET_NOT_REACHED : SPC_OK;
+        return SPC_OK;
+    }
     CoopArgs<KT> a{};
     a.n = n;
     a.m = m;
@@ -1668,6 +2226,33 @@ spc_status select_batch(spc_context* ctx, const GraphView& g, const KT* key, con
     int32_t* parent = W.parent.as<int32_t>();
     int32_t* counters = W.counters.as<int32_t>();  // [0..1] work-list counts, [2] warn flag
     constexpr bool two = MinKey<KT>::two_phase;
+    // every graph small: one CTA each, and no slabs or sorts over all of them
+    {
+        int32_t* largest = counters + 4;
+        SPC_LAUNCH(ctx, k_largest_graph, 1, 1024, 0, sa.B, sa.d_graph_ptr, W.up_ptr.as<int32_t>(),
+                   largest);
+        int64_t big[2];
+        const void* ptrs[2] = {largest, largest + 1};
+        const int bytes[2] = {4, 4};
+        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, big));
+        if (big[0] <= SmallMem<KT>::kMaxNodes && big[1] <= kSmallEdges) {
+            int32_t* n_c = W.k_graph.as<int32_t>();
+            int32_t* off = W.seg_start.as<int32_t>();
+            SPC_TRY(launch_small<KT>(ctx, g, key, sa, sa.B, big[0], lift, merged, n_c));
+            SPC_TRY(scan_i32(ctx, n_c, off, sa.B));
+            SPC_LAUNCH(ctx, k_small_shift, grid_for(sa.B, 1, maxb), kThreads, 0, sa.B,
+                       sa.d_graph_ptr, off, sa.d_targets, lift, graph_ptr_c, largest + 2);
+            int64_t vals[3];
+            const void* vp[3] = {off + sa.B, largest + 2, status};
+            const int vb[3] = {4, 4, 4};
+            SPC_TRY(read_vals(ctx, 3, vp, vb, vals));
+            const spc_status st = status_from_bits((uint32_t)vals[2]);
+            if (st < 0) return st;
+            *n_c_out = vals[0];
+            *status_out = vals[1] != 0 ? SPC_WARN_TARGET_NOT_REACHED : SPC_OK;
+            return SPC_OK;
+        }
+    }
     int32_t* pos = W.c_pos.as<int32_t>();
     int64_t n_msf = 0;
     int32_t* node_graph = W.node_graph.as<int32_t>();

@@ -326,3 +326,62 @@ def test_huge_buckets_among_short_ones(ctx, dtype, blocks, extra, clique):
     assert np.array_equal(lv.rowptr_c.cpu().numpy(), c.graph.rowptr)
     assert np.array_equal(lv.col_c.cpu().numpy(), c.graph.col)
     assert np.array_equal(_bits(lv.w_c.cpu().numpy()), _bits(c.graph.w))
+
+
+def _sparse(n, dtype, connected=True):
+    """About 3 n random edges, and a path through all nodes in random order when connected."""
+    rng = np.random.default_rng(n)
+    e = rng.integers(0, n, (2, 3 * n))
+    if connected:
+        q = rng.permutation(n)
+        e = np.concatenate([e, [q[:-1], q[1:]]], axis=1)
+    lo, hi = e.min(axis=0), e.max(axis=0)
+    key = np.unique((lo * n + hi)[lo != hi])
+    w = np.ones(key.size) if dtype == np.int32 else rng.uniform(0.1, 2.0, key.size)
+    return I.csr_from_edges(n, key // n, key % n, w.astype(dtype))
+
+
+def _batch_checked(ctx, graphs, ratio, schedule, levels):
+    from paper_2204_11757_gb300 import api
+    b = I.batch_of(graphs)
+    res = O.coarsen_batch(b, ratio, schedule)
+    gp = torch.from_numpy(b.graph_ptr).cuda()
+    lift, gpc, _ = ctx.coarsen_batched(api.CSR.from_graph(b.graph), gp, ratio, levels=levels)
+    lift, gpc = lift.cpu().numpy(), gpc.cpu().numpy()
+    for i, (levels_ref, total) in enumerate(res):
+        n0, n1 = b.graph_ptr[i], b.graph_ptr[i + 1]
+        assert gpc[i + 1] - gpc[i] == levels_ref[-1].n_c
+        assert np.array_equal(lift[n0:n1] - gpc[i], total)
+
+
+# one CTA per graph: the node counts at which the classes of shared memory end (4,708, 10,444 and
+# 19,968 nodes with 32-bit scores, 3,364, 7,460 and 14,260 with 64-bit ones; past the last the batch
+# goes through the launches over all graphs), more graphs than SMs and fewer, tiny ones among them
+@pytest.mark.parametrize("dtype,sizes", [
+    (np.float32, [4708, 4709, 10444, 10445, 19968]), (np.float32, [4708]), (np.float32, [19969]),
+    (np.float64, [3364, 3365, 7460, 7461, 14260]), (np.float64, [14261]), (np.int32, [3364, 3365])])
+@pytest.mark.parametrize("many", [False, True])
+def test_small_graphs_at_the_classes_of_shared_memory(ctx, dtype, sizes, many):
+    rng = np.random.default_rng(len(sizes))
+    graphs = [_sparse(n, dtype, connected=bool(n & 1)) for n in sizes]
+    tiny = [_sparse(int(n), dtype) for n in rng.integers(2, 60, 400 if many else 5)]
+    for ratio, levels in ((2, 1), (16, 1), (8, 3)):
+        _batch_checked(ctx, tiny[:3] + graphs + tiny[3:], ratio, "halving" if levels > 1 else "one",
+                       levels)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n,p", [(8192, 0), (8193, 0), (700, 0.5), (700, 0.57)])
+def test_one_small_graph_at_its_limits(ctx, dtype, n, p):
+    """8,192 nodes, 131,072 edges (p = 0.5: 122,325, p = 0.57: 139,450), few distinct scores."""
+    from paper_2204_11757_gb300 import api
+    g = (I.random_graph(n, p, seed=n, weight="float", dtype=dtype, connected=True) if p
+         else _sparse(n, dtype))
+    csr = api.CSR.from_graph(g)
+    rng = np.random.default_rng(n)
+    for f in (O.score(g), (rng.integers(1, 4, g.m) * 0.25).astype(O.score(g).dtype)):
+        for target in (1, n // 3, n - 5):
+            lift, merged, n_c, _ = ctx.select_merges(csr, torch.from_numpy(f).cuda(), target)
+            ref, ref_n = O.relabel(O.greedy_merge(g, O.sort_fitness(f), target)[0])
+            assert n_c == ref_n and int(merged.sum()) == n - n_c
+            assert np.array_equal(lift.cpu().numpy(), ref)
