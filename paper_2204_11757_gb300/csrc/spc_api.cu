@@ -653,7 +653,8 @@ static spc_status run_levels(spc_context* ctx, const GraphView& g0, const Schedu
             // mass(U) = members' masses + this level's self-mass (the merged node of the proof
             // of Theorem 2 keeps the weight inside it)
             SPC_TRY(run_carry_mass(ctx, cur.n, lv.lift.as<int32_t>(), n_c, mass, lv.self_mass.p,
-                                   cur.wtype, lv.max_intra, lv.mass, &lv.mass_ptr));
+                                   cur.wtype, lv.max_intra, lv.member_work, lv.mass,
+                                   &lv.mass_ptr));
             mass = lv.mass_ptr;
         }
         lv.status = st;

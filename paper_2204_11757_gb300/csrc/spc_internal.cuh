@@ -72,6 +72,7 @@ struct LevelBufs {
     const void* mass_ptr = nullptr;
     int64_t n = 0, m = 0, n_c = 0, m_c = 0, m_inter = 0;
     int64_t max_intra = 0;  // the most fine edges inside one super-node
+    int64_t member_work = 0;  // a bound of the sum of the super-nodes' squared member counts
     int32_t status = 0;
     spc_dtype wtype = SPC_F64;
     float ms = -1.f;
@@ -508,10 +509,12 @@ spc_status run_contract_forward(spc_context* ctx, const int32_t* perm, const int
 // mass_out[U] = (the members' masses prev_mass[x], ascending x, summed left to right from 0)
 // + self_mass[U]; prev_mass null means all zero (then mass_out is self_mass itself and nothing
 // runs: *mass_ptr = self_mass).  Types: int64 for SPC_I32, else the weight type.  max_intra: the
-// most fine edges inside one super-node (each is connected, so it has at most one member more).
+// most fine edges inside one super-node (each is connected, so it has at most one member more);
+// member_work: a bound of the sum of the squared member counts.
 spc_status run_carry_mass(spc_context* ctx, int64_t n, const int32_t* lift, int64_t n_c,
                           const void* prev_mass, const void* self_mass, spc_dtype wt,
-                          int64_t max_intra, Buf& mass_out, const void** mass_ptr);
+                          int64_t max_intra, int64_t member_work, Buf& mass_out,
+                          const void** mass_ptr);
 // The graph g with entry (x, x) = 2 mass[x] in its ascending-column place for every x with
 // mass[x] != 0 (edge ids unchanged); written into the context's dg_* buffers, described by out.
 spc_status run_diag_graph(spc_context* ctx, const GraphView& g, const void* mass,

@@ -385,3 +385,25 @@ def test_one_small_graph_at_its_limits(ctx, dtype, n, p):
             ref, ref_n = O.relabel(O.greedy_merge(g, O.sort_fitness(f), target)[0])
             assert n_c == ref_n and int(merged.sum()) == n - n_c
             assert np.array_equal(lift.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("leaves", [3, 40, 126, 127, 128, 129, 200])
+def test_masses_carried_by_buckets_and_by_sort(ctx, dtype, leaves):
+    """Members of super-nodes listed by buckets up to 64 squared members a node, else sorted: fans of
+    leaves that merge into their hubs, beside a path as long."""
+    from paper_2204_11757_gb300 import api
+    rng = np.random.default_rng(leaves)
+    hubs, s = 6, leaves + 1
+    eu = [np.repeat(np.arange(hubs) * s, leaves), hubs * s + np.arange(hubs * s - 1),
+          np.arange(hubs) * s]
+    ev = [np.repeat(np.arange(hubs) * s, leaves) + np.tile(1 + np.arange(leaves), hubs),
+          hubs * s + 1 + np.arange(hubs * s - 1), hubs * s + np.arange(hubs)]
+    eu, ev = np.concatenate(eu), np.concatenate(ev)
+    g = I.csr_from_edges(2 * hubs * s, eu, ev, rng.uniform(0.5, 2, eu.shape[0]).astype(dtype))
+    ref, total = O.coarsen(g, 16, "halving")
+    lift, _, _ = ctx.coarsen(api.CSR.from_graph(g), ref[-1].target, levels=len(ref))
+    assert np.array_equal(lift.cpu().numpy(), total)
+    for lv, r in zip(ctx.levels(), ref):
+        assert np.array_equal(_bits(lv.self_mass.cpu().numpy()), _bits(r.coarse.self_mass))
+        assert np.array_equal(_bits(lv.score.cpu().numpy()), _bits(r.f))
