@@ -248,6 +248,13 @@ __device__ __forceinline__ uint32_t bucket_tag(int32_t U, int32_t V, bool act) {
     return U != V ? (uint32_t)(U < V ? U : V) : (0x80000000u | (uint32_t)U);
 }
 
+// Edges of a thread in flight (the walk eu -> lift -> atomic -> offset -> store is latency): the
+// count at one / two / four, all levels of 2,500 graphs 372 / 364 / 330 us, a triangle grid of
+// 2048^2 154 / 148 / 137; the scatter 537 / 440 / 571 and 238 / 212 / 264, one contraction of a
+// tetrahedral grid of 97^3 42 / 36 / 46.
+constexpr int kCountItems = 4;
+constexpr int kScatterItems = 2;
+
 // Step 1: the bucket sizes, one atomic (without a result) per group of equal buckets in a
 // warp.  Also zeroes what the contraction adds into later: the coarse degree counts and the
 // long-segment list counts of both streams.
@@ -260,18 +267,29 @@ k_bucket_count(int64_t m, const int32_t* __restrict__ eu, const int32_t* __restr
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x; e0 < m; e0 += stride) {  // warp-uniform
-        const int64_t e = e0 + threadIdx.x;
-        const bool act = e < m;
-        int32_t U = 0, V = 0;
-        if (act) {
-            U = lift[eu[e]];
-            V = lift[ev[e]];
+    for (int64_t e0 = (int64_t)blockIdx.x * kThreads * kCountItems; e0 < m;
+         e0 += stride * kCountItems) {  // warp-uniform
+        int32_t U[kCountItems], V[kCountItems];
+#pragma unroll
+        for (int k = 0; k < kCountItems; ++k) {
+            const int64_t e = e0 + k * kThreads + threadIdx.x;
+            U[k] = e < m ? eu[e] : -1;
+            V[k] = e < m ? ev[e] : 0;
         }
-        const uint32_t tag = bucket_tag(U, V, act);
-        const unsigned peers = __match_any_sync(0xffffffffu, tag);
-        if (act && lane == __ffs(peers) - 1)
-            atomicAdd((U != V ? cnt_c : cnt_i) + (tag & 0x7fffffffu), __popc(peers));
+#pragma unroll
+        for (int k = 0; k < kCountItems; ++k) {
+            if (U[k] < 0) continue;
+            U[k] = lift[U[k]];
+            V[k] = lift[V[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < kCountItems; ++k) {
+            const bool act = U[k] >= 0;
+            const uint32_t tag = bucket_tag(U[k], V[k], act);
+            const unsigned peers = __match_any_sync(0xffffffffu, tag);
+            if (act && lane == __ffs(peers) - 1)
+                atomicAdd((U[k] != V[k] ? cnt_c : cnt_i) + (tag & 0x7fffffffu), __popc(peers));
+        }
     }
     for (int64_t i = t0; i < words_bc; i += stride) {
         zero_b[i] = 0u;
@@ -300,30 +318,48 @@ k_bucket_scatter(int64_t m, const int32_t* __restrict__ eu, const int32_t* __res
     if (blockIdx.x == 0 && threadIdx.x < 4) stats[threadIdx.x] = 0ull;
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x; e0 < m; e0 += stride) {  // warp-uniform
-        const int64_t e = e0 + threadIdx.x;
-        const bool act = e < m;
-        int32_t U = 0, V = 0;
-        if (act) {
-            U = lift[eu[e]];
-            V = lift[ev[e]];
+    for (int64_t e0 = (int64_t)blockIdx.x * kThreads * kScatterItems; e0 < m;
+         e0 += stride * kScatterItems) {  // warp-uniform
+        int32_t U[kScatterItems], V[kScatterItems];
+        int32_t old[kScatterItems], at[kScatterItems], lead[kScatterItems];
+#pragma unroll
+        for (int k = 0; k < kScatterItems; ++k) {
+            const int64_t e = e0 + k * kThreads + threadIdx.x;
+            U[k] = e < m ? eu[e] : -1;
+            V[k] = e < m ? ev[e] : 0;
         }
-        const uint32_t tag = bucket_tag(U, V, act);
-        const unsigned peers = __match_any_sync(0xffffffffu, tag);
-        const int leader = __ffs(peers) - 1;
-        const bool inter = U != V;
-        const int32_t b = (int32_t)(tag & 0x7fffffffu);
-        int32_t old = 0;
-        if (act && lane == leader) old = atomicSub((inter ? cnt_c : cnt_i) + b, __popc(peers));
-        old = __shfl_sync(0xffffffffu, old, leader);
-        if (!act) continue;
-        const int below = __popc(peers & ((1u << lane) - 1u));
-        const int32_t q = (inter ? off_c : off_i)[b] + old - 1 - below;
-        if (inter) {
-            citem[q] = make_uint4((uint32_t)b, (uint32_t)(U < V ? V : U), (uint32_t)e, 0u);
-        } else {
-            iitem[q] = make_uint2((uint32_t)U, (uint32_t)e);
-            emap[e] = -1;
+#pragma unroll
+        for (int k = 0; k < kScatterItems; ++k) {
+            if (U[k] < 0) continue;
+            U[k] = lift[U[k]];
+            V[k] = lift[V[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < kScatterItems; ++k) {
+            const bool act = U[k] >= 0, inter = U[k] != V[k];
+            const int32_t b = inter && V[k] < U[k] ? V[k] : U[k];
+            const unsigned peers = __match_any_sync(0xffffffffu, bucket_tag(U[k], V[k], act));
+            const int leader = __ffs(peers) - 1;
+            at[k] = 0;
+            old[k] = 0;
+            if (act) at[k] = (inter ? off_c : off_i)[b] - 1 - __popc(peers & ((1u << lane) - 1u));
+            if (act && lane == leader)
+                old[k] = atomicSub((inter ? cnt_c : cnt_i) + b, __popc(peers));
+            lead[k] = leader;
+        }
+#pragma unroll
+        for (int k = 0; k < kScatterItems; ++k) {
+            const int64_t e = e0 + k * kThreads + threadIdx.x;
+            const int32_t q = at[k] + __shfl_sync(0xffffffffu, old[k], lead[k]);
+            if (U[k] < 0) continue;
+            if (U[k] != V[k]) {
+                const bool up = U[k] < V[k];
+                citem[q] = make_uint4((uint32_t)(up ? U[k] : V[k]),
+                                      (uint32_t)(up ? V[k] : U[k]), (uint32_t)e, 0u);
+            } else {
+                iitem[q] = make_uint2((uint32_t)U[k], (uint32_t)e);
+                emap[e] = -1;
+            }
         }
     }
 }
