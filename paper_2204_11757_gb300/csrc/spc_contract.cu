@@ -641,7 +641,10 @@ k_bucket_rank_inter(int64_t cnt, const int32_t* __restrict__ off_c,
             s_cnt[lane * kRankGroups + g] = run;
             run += c[g];
         }
-        if (lane == 0 && tile == nt - 1) *total = before + tot;
+        if (lane == 0 && tile == nt - 1) {
+            *total = before + tot;
+            seg[before + tot] = (int32_t)cnt;  // the end of the last segment
+        }
     }
     __syncthreads();
 #pragma unroll
@@ -735,6 +738,7 @@ k_emit_segments(int64_t cnt, int nb, const uint64_t* __restrict__ key,
                 cU[ce] = U;
                 cV[ce] = V;
             }
+            if (i == cnt - 1) seg[ce + 1] = (int32_t)cnt;  // the end of the last segment
         }
         warp_count(up_deg, U, h);
         warp_count(low_deg, V, h);
@@ -756,7 +760,7 @@ k_run_starts(int64_t cnt, const uint8_t* __restrict__ head, const int32_t* __res
 // Segment sums: out[slot(r)] = sum of w_und[idx[j]] for j in [start[r], start[r+1]), left to
 // right.  slot(r) = r, or key[start[r]] when `key` is given (self-mass by super-node).  Short
 // segments: one thread each; segments longer than kLongRow go to a list (long_segment_sums), the
-// largest length to *longest (may be null).
+// largest length to *longest (may be null).  plus (may be null): added to every sum at its end.
 // terms in flight; device time over all launches of a call at 4 / 6 / 8 (before): 2048^2 mesh 690 /
 // 699 / 707 us (802), 129^3 mesh 1051 / 847 / 832 (1089), 2^23 points 932 / 971 / 1121 (1003), 2,500
 // meshes 868 / 850 / 1240 (975)
@@ -767,7 +771,7 @@ __global__ void __launch_bounds__(kThreads)
 k_segsum_short(int64_t nseg, const int32_t* __restrict__ start, const uint32_t* __restrict__ idx,
                const uint32_t* __restrict__ key, const WT* __restrict__ w_und, Out* __restrict__ out,
                int32_t* __restrict__ long_list, int32_t* long_count, int32_t* longest,
-               uint32_t* status) {
+               uint32_t* status, const WT* __restrict__ plus) {
     spc::pdl_wait();
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nseg;
          r += (int64_t)gridDim.x * blockDim.x) {
@@ -796,6 +800,7 @@ k_segsum_short(int64_t nseg, const int32_t* __restrict__ start, const uint32_t* 
         if constexpr (std::is_same<WT, int32_t>::value && sizeof(Out) == 4) {
             if (s > 2147483647ll) atomicOr(status, DEV_OVERFLOW);
         }
+        if (plus) s = CT<WT>::add(s, plus[r]);
         out[key ? (int64_t)key[j0] : r] = (Out)s;
     }
 }
@@ -878,8 +883,9 @@ k_transpose_keys(int64_t m_c, const int32_t* __restrict__ cV, uint32_t* __restri
 // low_deg[V] down (zero afterwards)
 __global__ void __launch_bounds__(kThreads)
 k_lower_scatter(int64_t m_c, const int32_t* __restrict__ cV, const int32_t* __restrict__ lstart,
-                int32_t* low_deg, uint32_t* __restrict__ slot) {
+                int32_t* low_deg, uint32_t* __restrict__ slot, int32_t* __restrict__ long_count) {
     spc::pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *long_count = 0;  // of k_fill_lower_rows
     const int lane = threadIdx.x & 31;
     for (int64_t k0 = (int64_t)blockIdx.x * blockDim.x; k0 < m_c;
          k0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
@@ -1246,7 +1252,8 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         }
         SPC_LAUNCH(ctx, (k_segsum_short<WT, Acc>), grid_for(n_c, kThreads, maxb), kThreads, 0,
                    n_c, off_i, ival2, nullptr, W.w_und.as<WT>(), self_mass,
-                   W.long_segs_side.as<int32_t>(), W.counters.as<int32_t>() + 11, nullptr, status);
+                   W.long_segs_side.as<int32_t>(), W.counters.as<int32_t>() + 11, nullptr, status,
+                   nullptr);
         if (long_intra)
             SPC_TRY((long_segment_sums<WT, Acc>(ctx, off_i, ival2, nullptr, W.w_und.as<WT>(),
                                                  self_mass, bv[5])));
@@ -1268,7 +1275,7 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
             SPC_TRY(read_i32(ctx, ihpos + m_intra, &n_runs));
             SPC_LAUNCH(ctx, (k_segsum_short<WT, Acc>), grid_for(n_runs, kThreads, maxb),
                        kThreads, 0, n_runs, istart, ival, ikey, W.w_und.as<WT>(), self_mass,
-                       long_list, long_cnt, nullptr, status);
+                       long_list, long_cnt, nullptr, status, nullptr);
             if (long_intra)
                 SPC_TRY((long_segment_sums<WT, Acc>(ctx, istart, ival, ikey, W.w_und.as<WT>(),
                                                      self_mass, bv[5])));
@@ -1286,6 +1293,7 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
     int32_t* cV = W.cV.as<int32_t>();
     int64_t m_c = 0;
     bool lower_buckets = true;
+    int64_t max_lower = 0;  // the longest lower row
     if (m_inter > 0 && buckets) {
         if (long_c > 0)
             SPC_TRY(sort_long_buckets(ctx, true, list_c, bstats + 6, off_c, citem, nullptr,
@@ -1325,14 +1333,15 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         const int bytes[3] = {4, 8, 8};
         SPC_TRY(read_vals(ctx, 3, ptrs, bytes, ev));
         m_c = ev[0];
+        max_lower = ev[2];
         lower_buckets = ev[2] <= kRankMax && ev[1] <= kRankWork * m_c;
     }
-    SPC_LAUNCH(ctx, k_set_i32, 1, 32, 0, seg + m_c, (int32_t)m_inter);
+    if (m_inter == 0) SPC_LAUNCH(ctx, k_set_i32, 1, 32, 0, seg, 0);
     WT* a_und = lv.a_und.as<WT>();
     if (m_c > 0) {
         SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(m_c, kThreads, maxb), kThreads, 0,
                    m_c, seg, reinterpret_cast<const uint32_t*>(perm), nullptr, W.w_und.as<WT>(),
-                   a_und, long_list, long_cnt, nullptr, status);
+                   a_und, long_list, long_cnt, nullptr, status, nullptr);
         if (long_inter)
             SPC_TRY((long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm),
                                                 nullptr, W.w_und.as<WT>(), a_und, bv[3])));
@@ -1342,14 +1351,15 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         uint32_t* tkey = W.t_key.as<uint32_t>();
         uint32_t* tval = W.t_val.as<uint32_t>();
         if (lower_buckets) {
-            SPC_LAUNCH(ctx, k_lower_scatter, gc, kThreads, 0, m_c, cV, lstart, low_deg, tval);
             int32_t* lrows = W.t_key.as<int32_t>();  // free on the bucket path
             int32_t* lcount = W.lower_long.as<int32_t>();
-            SPC_CUDA(cudaMemsetAsync(lcount, 0, sizeof(int32_t), ctx->stream));
+            SPC_LAUNCH(ctx, k_lower_scatter, gc, kThreads, 0, m_c, cV, lstart, low_deg, tval,
+                       lcount);
             SPC_LAUNCH(ctx, k_fill_lower_rows<WT>, grid_for(n_c, kThreads, maxb), kThreads, 0,
                        n_c, tval, lstart, rowptr_c, cU, a_und, lv.col_c.as<int32_t>(),
                        lv.w_c.as<WT>(), lrows, lcount);
-            SPC_LAUNCH(ctx, k_fill_lower_long<WT>, ctx->num_sms * 2, kThreads, 0, lrows, lcount,
+            if (max_lower > kLowerRowThread)
+                SPC_LAUNCH(ctx, k_fill_lower_long<WT>, ctx->num_sms * 2, kThreads, 0, lrows, lcount,
                        tval, lstart, rowptr_c, cU, a_und, lv.col_c.as<int32_t>(),
                        lv.w_c.as<WT>());
         } else {
@@ -1385,7 +1395,7 @@ spc_status forward_typed(spc_context* ctx, const int32_t* perm, const int32_t* s
     SPC_CUDA(cudaMemsetAsync(long_cnt, 0, 2 * sizeof(int32_t), ctx->stream));
     SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(m_c, kThreads, ctx->num_sms * 8), kThreads,
                0, m_c, seg, reinterpret_cast<const uint32_t*>(perm), nullptr, w_und, a_und,
-               long_list, long_cnt, longest, ctx->d_status);
+               long_list, long_cnt, longest, ctx->d_status, nullptr);
     int64_t vals[3];
     {
         const void* ptrs[3] = {long_cnt, ctx->d_status, longest};
@@ -1413,8 +1423,10 @@ spc_status forward_typed(spc_context* ctx, const int32_t* perm, const int32_t* s
 // rank there.  The ranking reads the sum of the squared member counts, which the host bounds from
 // the contraction's intra edges (kMemberWork); past that bound, a stable sort of (lift[x], x).
 __global__ void __launch_bounds__(kThreads)
-k_member_count(int64_t n, const int32_t* __restrict__ lift, int32_t* cnt) {
+k_member_count(int64_t n, const int32_t* __restrict__ lift, int32_t* cnt,
+               int32_t* __restrict__ long_count) {
     spc::pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *long_count = 0;  // of the sums' list
     for (int64_t x0 = (int64_t)blockIdx.x * blockDim.x; x0 < n;
          x0 += (int64_t)gridDim.x * blockDim.x) {  // warp-uniform
         const int64_t x = x0 + threadIdx.x;
@@ -1459,8 +1471,9 @@ k_member_rank(int64_t n, const int32_t* __restrict__ lift, const int32_t* __rest
 // members of every super-node in ascending id: a stable sort of (lift[x], x) by lift
 __global__ void __launch_bounds__(kThreads)
 k_member_keys(int64_t n, const int32_t* __restrict__ lift, uint32_t* __restrict__ key,
-              uint32_t* __restrict__ val) {
+              uint32_t* __restrict__ val, int32_t* __restrict__ long_count) {
     spc::pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *long_count = 0;  // of the sums' list
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
         key[x] = (uint32_t)lift[x];
@@ -1652,31 +1665,33 @@ spc_status carry_mass_typed(spc_context* ctx, int64_t n, const int32_t* lift, in
         uint32_t* val = W.ms_val.as<uint32_t>();
         int32_t* start = W.ms_start.as<int32_t>();
         const int gn = grid_for(n, kThreads, maxb);
+        int32_t* long_list = W.long_segs.as<int32_t>();
+        int32_t* long_cnt = W.counters.as<int32_t>() + 9;
         if (max_intra < kMemberMax && member_work <= kMemberWork * n) {
             int32_t* cnt = W.b_cnt.as<int32_t>();
             W.b_dirty = true;  // the counts are zero again after k_member_place
-            SPC_LAUNCH(ctx, k_member_count, gn, kThreads, 0, n, lift, cnt);
+            SPC_LAUNCH(ctx, k_member_count, gn, kThreads, 0, n, lift, cnt, long_cnt);
             SPC_TRY(scan_i32(ctx, cnt, start, n_c));
             SPC_LAUNCH(ctx, k_member_place, gn, kThreads, 0, n, lift, start, cnt, key);
             SPC_LAUNCH(ctx, k_member_rank, gn, kThreads, 0, n, lift, start, key, val);
             W.b_dirty = false;
         } else {
-            SPC_LAUNCH(ctx, k_member_keys, gn, kThreads, 0, n, lift, key, val);
+            SPC_LAUNCH(ctx, k_member_keys, gn, kThreads, 0, n, lift, key, val, long_cnt);
             SPC_TRY(radix_sort_u32(ctx, key, val, W.ms_key2.as<uint32_t>(),
                                    W.ms_val2.as<uint32_t>(), n, nb));
             SPC_LAUNCH(ctx, k_member_starts, gn, kThreads, 0, n, n_c, key, start);
         }
-        int32_t* long_list = W.long_segs.as<int32_t>();
-        int32_t* long_cnt = W.counters.as<int32_t>() + 9;
-        SPC_LAUNCH(ctx, k_set_i32, 1, 32, 0, long_cnt, 0);
-        SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(n_c, kThreads, maxb), kThreads, 0,
-                   n_c, start, val, nullptr, prev, out, long_list, long_cnt, nullptr, ctx->d_status);
         // a super-node is connected by its intra edges: at most max_intra + 1 members
-        if (max_intra >= kLongRow)
+        const bool longs = max_intra >= kLongRow;
+        SPC_LAUNCH(ctx, (k_segsum_short<WT, WT>), grid_for(n_c, kThreads, maxb), kThreads, 0,
+                   n_c, start, val, nullptr, prev, out, long_list, long_cnt, nullptr,
+                   ctx->d_status, longs ? nullptr : self);
+        if (longs) {
             SPC_TRY((long_segment_sums<WT, WT>(ctx, start, val, nullptr, prev, out,
                                                max_intra + 1)));
-        SPC_LAUNCH(ctx, k_mass_add_self<WT>, grid_for(n_c, kThreads, maxb), kThreads, 0, n_c,
-                   self, out);
+            SPC_LAUNCH(ctx, k_mass_add_self<WT>, grid_for(n_c, kThreads, maxb), kThreads, 0, n_c,
+                       self, out);
+        }
         return SPC_OK;
     }
 }
