@@ -1363,6 +1363,8 @@ spc_status launch_small(spc_context* ctx, const GraphView& g, const KT* key, con
     a.merged = merged;
     a.n_c = n_c;
     a.status = ctx->d_status;
+    // every key read, the lift written (on the first class's launch for all of them)
+    note_bytes(ctx, (double)g.m * sizeof(KT) + 4.0 * g.n);
     if (B > ctx->num_sms) {  // a graph per SM or less takes the most threads
         SPC_TRY((launch_small_class<KT, 256>(ctx, a, B, kSmallBytes[0])));
         if (n_max > a.n_max)
@@ -2197,6 +2199,8 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
         SPC_LAUNCH(ctx, k_key_hist<KT>, ctx->num_sms, 1024, kTauBins * 4, m, key, a.hist_samp,
                    W.key_hist.as<uint32_t>());
     }
+    // every key read, the first slab's ends read, parents and lift written
+    note_bytes(ctx, (double)m * sizeof(KT) + 8.0 * (double)(a.need < m ? a.need : m) + 8.0 * n);
     SPC_LAUNCH_COOP(ctx, k_select_coop<KT>, grid, kCoopThreads, a);
     int64_t vals[2];
     {
