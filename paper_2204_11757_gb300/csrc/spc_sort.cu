@@ -1,11 +1,12 @@
 // Stable LSD radix sort of (key, uint32 value) pairs, 8-bit digits.
 //
-// Per digit: an upsweep builds one 256-bin histogram per 4096-item tile (digit-major), a
-// device-wide exclusive scan turns the histograms into output offsets, and a downsweep ranks
-// every item inside its tile (warp __match_any_sync ranks, per-warp counters, cross-warp
-// prefix), stages the tile in shared memory in digit order and writes it out so that items of
-// one digit leave the tile as one contiguous run.  Tiles keep input order and ranks are stable,
-// so equal keys keep their input order.  No inter-block waits.
+// The context's sorts are one-sweep: one histogram pass for all digits (k_os_hist), then one pass
+// per digit (k_os_pass) in which a tile of 4,096 items ranks its items (masks per digit in shared
+// memory, per-warp counters, cross-warp prefix), finds its offsets by a bounded look-back over the
+// tiles before it, stages its items in digit order and writes every digit's run contiguously.  The
+// allocation-free entry point sorts by an upsweep of histograms, a device-wide scan and a downsweep,
+// with no waits between blocks.  Tiles keep input order and ranks are stable, so equal keys keep
+// their input order.
 #include <atomic>
 
 #include "spc_internal.cuh"
