@@ -27,6 +27,7 @@
 // Every retry loop is bounded (spin_limit: kSpinLimit unless the context lowered it); giving up
 // sets DEV_TIMEOUT in the status word.
 #include <atomic>
+#include <memory>
 
 #include "spc_scan.cuh"
 
@@ -839,7 +840,7 @@ __device__ __forceinline__ uint32_t sel_digit(KT hi, uint32_t lo, int r) {
 // components' best edges in shared memory.  A graph of a few thousand nodes has too little work per
 // round for the whole GPU: every grid barrier or launch costs more than the round's work, while a
 // batch keeps an SM per graph busy.  Shared memory bounds it (random 8-byte slots, compare-and-swap
-// on them, walks).  2,500 graphs of 20 to 19,881 nodes, binary32, a call of three levels: 19.7 ms
+// on them, walks).  2,500 graphs of 200 to 19,881 nodes, binary32, a call of three levels: 19.7 ms
 // with the launches of select_batch over all graphs at once, 17.0 so; one graph of 4,096 nodes and
 // 12,033 edges down to a half (a sixteenth): 129 (144) us in k_select_coop, 52 (91) here.
 template <class KT>
@@ -1365,13 +1366,23 @@ spc_status launch_small(spc_context* ctx, const GraphView& g, const KT* key, con
     a.status = ctx->d_status;
     // every key read, the lift written (on the first class's launch for all of them)
     note_bytes(ctx, (double)g.m * sizeof(KT) + 4.0 * g.n);
-    if (B > ctx->num_sms) {  // a graph per SM or less takes the most threads
-        SPC_TRY((launch_small_class<KT, 256>(ctx, a, B, kSmallBytes[0])));
-        if (n_max > a.n_max)
-            SPC_TRY((launch_small_class<KT, 512>(ctx, a, B, kSmallBytes[1])));
-        if (n_max <= a.n_max) return SPC_OK;
-    }
-    return launch_small_class<KT, 1024>(ctx, a, B, kSmallBytes[2]);
+    if (B <= ctx->num_sms)  // a graph per SM or less takes the most threads
+        return launch_small_class<KT, 1024>(ctx, a, B, kSmallBytes[2]);
+    if (n_max <= SmallMem<KT>::nodes(kSmallBytes[0]))
+        return launch_small_class<KT, 256>(ctx, a, B, kSmallBytes[0]);
+    // The smaller classes on the second stream: their CTAs fill the SMs that the largest leaves at
+    // its end (2,500 graphs, the whole call: 16.77 ms one class after the other, 16.22 so).  A
+    // graph's lists lie in its own edges' range, so the classes share no scratch.
+    std::unique_ptr<SideBranch> side(new SideBranch(ctx));
+    SPC_TRY(side->status());
+    const bool three = n_max > SmallMem<KT>::nodes(kSmallBytes[1]);
+    SmallArgs<KT> last = a;
+    SPC_TRY((launch_small_class<KT, 256>(ctx, a, B, kSmallBytes[0])));
+    if (three) SPC_TRY((launch_small_class<KT, 512>(ctx, a, B, kSmallBytes[1])));
+    side->leave();
+    last.n_min = a.n_min;
+    if (three) return launch_small_class<KT, 1024>(ctx, last, B, kSmallBytes[2]);
+    return launch_small_class<KT, 512>(ctx, last, B, kSmallBytes[1]);
 }
 
 // root flags (a root is its set's smallest member and its own parent)
