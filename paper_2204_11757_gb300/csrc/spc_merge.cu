@@ -993,8 +993,9 @@ __global__ void __launch_bounds__(T, 1024 / T) k_select_small(SmallArgs<KT> a) {
     KT lo = 0;
     bool above = false;  // the slab starts above lo
     // 32-bit keys: every round's entries of the best slots lie below the earlier rounds', so the
-    // slots need no reset (16 bits of round, 31 of key, 17 of the edge's place in its graph)
-    unsigned tag = 0xffffu;
+    // slots need no reset (15 bits of round, 32 of key, 17 of the edge's place in its graph)
+    constexpr int kTagShift = 32 + kSmallEdgeBits;
+    unsigned tag = 0x7fffu;
     while (k > 0) {
         const bool all = need >= mb;
         int64_t upto = mb;
@@ -1076,7 +1077,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_select_small(SmallArgs<KT> a) {
                     const int32_t u = x[2 * q], v = x[2 * q + 1];
                     if (u == v) continue;  // (both 0 past the end)
                     const unsigned long long t =
-                        two ? pk[q] : pk[q] | (unsigned long long)tag << 48;
+                        two ? pk[q] : pk[q] | (unsigned long long)tag << kTagShift;
                     sm_min(best + u, t);
                     sm_min(best + v, t);
                     const int32_t to = keep * T + tid;
@@ -1136,7 +1137,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_select_small(SmallArgs<KT> a) {
                         pick = (best[u] == pk[q] && beste[u] == e[q]) ||
                                (best[v] == pk[q] && beste[v] == e[q]);
                     } else {
-                        const unsigned long long t = pk[q] | (unsigned long long)tag << 48;
+                        const unsigned long long t = pk[q] | (unsigned long long)tag << kTagShift;
                         pick = best[u] == t || best[v] == t;
                     }
                     if (pick && sm_unite(par, u, v, lim, a.status)) {
@@ -1293,33 +1294,33 @@ k_small_shift(int64_t B, const int64_t* __restrict__ graph_ptr, const int32_t* _
     }
 }
 
-// the largest graph of a batch: out[0] nodes, out[1] edges; out[2] = 0 (the warn flag)
-__global__ void __launch_bounds__(1024)
-k_largest_graph(int64_t B, const int64_t* __restrict__ graph_ptr,
-                const int32_t* __restrict__ up_ptr, int32_t* __restrict__ out) {
+// The shape of a batch (out zeroed before): out[0] = the most nodes, out[1] = the most edges of a
+// graph, out[2] != 0 when the graphs do not take the nodes in turn or an edge leaves its graph (such
+// a batch is merged by the general path, which indexes by the whole batch's nodes).
+__global__ void __launch_bounds__(kThreads)
+k_batch_shape(int64_t B, int64_t n, const int64_t* __restrict__ graph_ptr,
+              const int32_t* __restrict__ up_ptr, const int32_t* __restrict__ ev,
+              int32_t* __restrict__ out) {
     spc::pdl_wait();
-    __shared__ int32_t s_n[32], s_m[32];
-    int32_t n = 0, m = 0;
-    for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
+    for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
         const int64_t n0 = graph_ptr[b], n1 = graph_ptr[b + 1];
-        n = max(n, (int32_t)(n1 - n0));
-        m = max(m, up_ptr[n1] - up_ptr[n0]);
-    }
-    n = __reduce_max_sync(0xffffffffu, n);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) {
-        s_n[threadIdx.x >> 5] = n;
-        s_m[threadIdx.x >> 5] = m;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        n = __reduce_max_sync(0xffffffffu, s_n[threadIdx.x]);
-        m = __reduce_max_sync(0xffffffffu, s_m[threadIdx.x]);
-        if (threadIdx.x == 0) {
-            out[0] = n;
-            out[1] = m;
-            out[2] = 0;
+        bool bad = n0 < 0 || n1 < n0 || n1 > n || (b == 0 && n0 != 0) || (b == B - 1 && n1 != n);
+        if (!bad) {
+            const int32_t e0 = up_ptr[n0], e1 = up_ptr[n1];
+            for (int64_t i0 = (int64_t)e0 + threadIdx.x; i0 < e1; i0 += 4 * kThreads) {
+                int32_t v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    v[q] = i0 + q * kThreads < e1 ? ev[i0 + q * kThreads] : (int32_t)n0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) bad = bad || v[q] < n0 || v[q] >= n1;
+            }
+            if (threadIdx.x == 0) {
+                atomicMax(out, (int32_t)(n1 - n0));
+                atomicMax(out + 1, e1 - e0);
+            }
         }
+        if (bad) out[2] = 1;
     }
 }
 
@@ -2246,22 +2247,23 @@ spc_status select_batch(spc_context* ctx, const GraphView& g, const KT* key, con
     // 4.39 / 4.00 (5.18 / 4.64), 400 to a sixteenth at once 2.86 / 2.69 (2.93 / 2.83), two random
     // geometric graphs of 12,000 nodes 1.56 / 0.96 (1.76 / 1.11).
     {
-        int32_t* largest = counters + 4;
-        SPC_LAUNCH(ctx, k_largest_graph, 1, 1024, 0, sa.B, sa.d_graph_ptr, W.up_ptr.as<int32_t>(),
-                   largest);
-        int64_t big[2];
-        const void* ptrs[2] = {largest, largest + 1};
-        const int bytes[2] = {4, 4};
-        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, big));
-        if (big[0] <= SmallMem<KT>::kMaxNodes && big[1] <= kSmallEdges) {
+        int32_t* shape = counters + 4;  // [4]: k_batch_shape's three, the warn flag
+        SPC_CUDA(cudaMemsetAsync(shape, 0, 4 * sizeof(int32_t), ctx->stream));
+        SPC_LAUNCH(ctx, k_batch_shape, grid_for(sa.B, 1, maxb), kThreads, 0, sa.B, n,
+                   sa.d_graph_ptr, W.up_ptr.as<int32_t>(), W.ev.as<int32_t>(), shape);
+        int64_t big[3];
+        const void* ptrs[3] = {shape, shape + 1, shape + 2};
+        const int bytes[3] = {4, 4, 4};
+        SPC_TRY(read_vals(ctx, 3, ptrs, bytes, big));
+        if (big[0] <= SmallMem<KT>::kMaxNodes && big[1] <= kSmallEdges && big[2] == 0) {
             int32_t* n_c = W.k_graph.as<int32_t>();
             int32_t* off = W.seg_start.as<int32_t>();
             SPC_TRY(launch_small<KT>(ctx, g, key, sa, sa.B, big[0], lift, merged, n_c));
             SPC_TRY(scan_i32(ctx, n_c, off, sa.B));
             SPC_LAUNCH(ctx, k_small_shift, grid_for(sa.B, 1, maxb), kThreads, 0, sa.B,
-                       sa.d_graph_ptr, off, sa.d_targets, lift, graph_ptr_c, largest + 2);
+                       sa.d_graph_ptr, off, sa.d_targets, lift, graph_ptr_c, shape + 3);
             int64_t vals[3];
-            const void* vp[3] = {off + sa.B, largest + 2, status};
+            const void* vp[3] = {off + sa.B, shape + 3, status};
             const int vb[3] = {4, 4, 4};
             SPC_TRY(read_vals(ctx, 3, vp, vb, vals));
             const spc_status st = status_from_bits((uint32_t)vals[2]);

@@ -407,3 +407,24 @@ def test_masses_carried_by_buckets_and_by_sort(ctx, dtype, leaves):
     for lv, r in zip(ctx.levels(), ref):
         assert np.array_equal(_bits(lv.self_mass.cpu().numpy()), _bits(r.coarse.self_mass))
         assert np.array_equal(_bits(lv.score.cpu().numpy()), _bits(r.f))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_batches_that_are_not_block_diagonal(ctx, dtype):
+    """Edges between two graphs of a batch merge across them: such a batch takes the launches over
+    all graphs, as one with a graph too large for shared memory does (an added path of 20,001
+    nodes), with the same partition."""
+    from paper_2204_11757_gb300 import api
+    a, c = _sparse(3000, dtype), _sparse(5000, dtype)
+    eu = np.concatenate([a.eu, 3000 + c.eu, [17, 2999]])
+    ev = np.concatenate([a.ev, 3000 + c.ev, [3001, 7000]])
+    w = np.concatenate([a.w_und, c.w_und, np.full(2, 1.5, dtype)]).astype(dtype)
+    path = np.arange(20000)
+    wide_u, wide_v = np.concatenate([eu, 8000 + path]), np.concatenate([ev, 8001 + path])
+    ww = np.concatenate([w, np.ones(20000, dtype)])
+    g, wide = I.csr_from_edges(8000, eu, ev, w), I.csr_from_edges(28001, wide_u, wide_v, ww)
+    lift, _, _ = ctx.coarsen_batched(api.CSR.from_graph(g),
+                                     torch.tensor([0, 3000, 8000]).cuda(), 4, levels=2)
+    ref, _, _ = ctx.coarsen_batched(api.CSR.from_graph(wide),
+                                    torch.tensor([0, 3000, 8000, 28001]).cuda(), 4, levels=2)
+    assert np.array_equal(lift.cpu().numpy(), ref.cpu().numpy()[:8000])
