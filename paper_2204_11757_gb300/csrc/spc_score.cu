@@ -392,8 +392,9 @@ k_rows_edges_flat(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
         const int64_t r_lo = s_next;
         __syncthreads();  // every thread has read s_next
         tile_rows(rowptr, n, base, end, r_lo, kLongRow, s_row, &s_next,
-                  [&](int64_t x, int32_t rel, int64_t, int64_t r1) {
-                      if (rel < kFlatRows)
+                  [&](int64_t x, int32_t rel, int64_t r0, int64_t r1) {
+                      // (the second stream is writing the degrees of the long rows meanwhile)
+                      if (rel < kFlatRows && r1 - r0 <= kLongRow)
                           s_data[rel] = flat_row<WT>(x, rowptr, deg, nlow, up_ptr);
                       if constexpr (kF32)  // the row's end marker, by the tile of its last entry
                           if (pk && r1 <= end) pk[r1 + x] = make_uint2(0x7fffffffu, 0u);

@@ -114,3 +114,19 @@ def test_every_kernel_waits_for_its_predecessor_first():
                 continue
             assert re.fullmatch(r"(spc::)?pdl_wait\(\)", st), (f, name, st[:80])
             break
+
+
+def test_flat_normalise_reads_no_degree_of_a_long_row():
+    """While the flat normalise kernel runs, the second stream writes the degrees of the rows of
+    more than kLongRow entries (stream_rows or the tables): every read of a row's degree
+    (flat_row) must come after a test that leaves those rows out."""
+    body = [b for f, name, b in _kernels() if name == "k_rows_edges_flat"]
+    assert len(body) == 1
+    body = body[0][:body[0].index("__global__")] if "__global__" in body[0] else body[0]
+    calls = [mm.start() for mm in re.finditer(r"\bflat_row<", body)]
+    assert len(calls) == 2
+    # in the march over a tile's rows: by the row's length
+    guard = body[body.rindex("if (", 0, calls[0]):calls[0]]
+    assert re.search(r"r1 - r0 <= kLongRow", guard), guard
+    # where an entry's row is not in shared memory: entries of long rows were passed over
+    assert "if (rel < 0) continue;" in body[calls[0]:calls[1]]
