@@ -59,6 +59,13 @@ static void raw_free(spc_context* ctx, void* p) {
     else cudaFree(p);
 }
 
+// the captured schedule and the record it came from; the next call like it runs host-driven
+static void drop_graph(Replay& R);
+static void forget_schedule(Replay& R) {
+    drop_graph(R);
+    R.recorded = false;
+}
+
 spc_status ensure(spc_context* ctx, Buf& b, size_t bytes) {
     bytes = (bytes + 255) & ~(size_t)255;
     if (bytes == 0) bytes = 256;
@@ -67,6 +74,8 @@ spc_status ensure(spc_context* ctx, Buf& b, size_t bytes) {
     if (b.p) {
         // the old block may still be read by queued work
         SPC_CUDA(cudaStreamSynchronize(ctx->stream));
+        // a captured schedule holds the block's address, its record the levels' masses
+        forget_schedule(ctx->replay);
         raw_free(ctx, b.p);
         b.p = nullptr;
         b.bytes = 0;
@@ -866,17 +875,13 @@ static spc_status drive(spc_context* ctx, const GraphView& v, const Schedule& S,
     if (again) SPC_CUDA(cudaStreamSynchronize(ctx->stream));
     if (again && R.hash == checksum_value(ctx)) {
         if (R.exec && R.timer_substr != tsub) drop_graph(R);
-        if (!R.exec && capture_graph(ctx, v, S, lift_int) != SPC_OK) {
-            drop_graph(R);
-            R.recorded = false;
-        }
+        if (!R.exec && capture_graph(ctx, v, S, lift_int) != SPC_OK) forget_schedule(R);
         if (R.exec) {
             bool mismatch = false;
             const spc_status st = replay_graph(ctx, &mismatch);
             if (st < 0) {
                 // a replay that stopped in between leaves counters that the graph takes as zero
-                drop_graph(R);
-                R.recorded = false;
+                forget_schedule(R);
                 ctx->work.sel_dirty = true;
                 ctx->work.b_dirty = true;
                 return st;
@@ -902,16 +907,14 @@ static spc_status drive(spc_context* ctx, const GraphView& v, const Schedule& S,
                 *warn = R.warn;
                 return SPC_OK;
             }
-            drop_graph(R);  // the device disagreed with the record: run host-driven again
-            R.recorded = false;
+            forget_schedule(R);  // the device disagreed with the record: run host-driven again
         }
     }
     R.mode = use_graph ? Replay::kRecord : Replay::kDirect;
     R.log.clear();
     const spc_status st = run_levels(ctx, v, S, lift_int, ncf, warn);
     R.mode = Replay::kDirect;
-    drop_graph(R);
-    R.recorded = false;
+    forget_schedule(R);
     if (st == SPC_OK && use_graph) {
         R.recorded = true;
         R.key = key;

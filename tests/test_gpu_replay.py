@@ -1,0 +1,89 @@
+"""The captured schedule of a repeated coarsening when other calls on the context come between:
+it is replayed only while everything it takes for granted still holds."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import oracle as O  # noqa: E402
+from paper_2204_11757_gb300 import inputs as I  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_2204_11757_gb300 import api as A
+    return A
+
+
+class Repeated:
+    """One coarsening call made again and again on one context."""
+
+    def __init__(self, api, ctx, graph, levels):
+        self.ctx, self.csr, self.levels = ctx, api.CSR.from_graph(graph), levels
+        self.ref, self.total = O.coarsen(graph, 1 << levels, "halving")
+
+    def run(self, replayed):
+        lift, n_c, _ = self.ctx.coarsen(self.csr, self.ref[-1].target, levels=self.levels)
+        assert self.ctx.last_call_replayed == replayed
+        assert n_c == self.ref[-1].n_c
+        assert np.array_equal(lift.cpu().numpy(), self.total)
+        for lv, r in zip(self.ctx.levels(), self.ref):
+            assert np.array_equal(lv.w_c.cpu().numpy().view(np.uint64),
+                                  r.coarse.graph.w.view(np.uint64))
+            assert np.array_equal(lv.emap.cpu().numpy(), r.coarse.emap)
+
+
+def _mesh(nx, ny, seed):
+    return I.tri_mesh_2d(nx, ny, seed, jitter=0.3, weight="inv_len", dtype=np.float64)
+
+
+def _other_call(api, ctx, op, g):
+    csr = api.CSR.from_graph(g)
+    if op == "contract":
+        lift = (np.arange(g.n) // 2).astype(np.int32)
+        lv = ctx.contract(csr, torch.from_numpy(lift).cuda(), int(lift[-1]) + 1)
+        assert np.array_equal(lv.emap.cpu().numpy(), O.contract(g, lift, int(lift[-1]) + 1).emap)
+    elif op == "score":
+        assert np.array_equal(ctx.score(csr).cpu().numpy().view(np.uint64),
+                              O.score(g).view(np.uint64))
+    elif op == "select":
+        f = O.score(g)
+        lift, _, _, _ = ctx.select_merges(csr, torch.from_numpy(f).cuda(), g.n // 2)
+        assert np.array_equal(lift.cpu().numpy(), O.coarsen_level(g, g.n // 2).lift)
+    else:
+        f = np.random.default_rng(1).random(g.m)
+        order = ctx.sort_fitness(torch.from_numpy(f).cuda()).cpu().numpy()
+        assert np.array_equal(order, np.argsort(f, kind="stable"))
+
+
+@pytest.mark.parametrize("op", ["contract", "score", "select", "sort"])
+def test_a_larger_call_between_drops_the_captured_schedule(api, op):
+    """The larger call grows workspace blocks, so the addresses inside the captured schedule are
+    no longer the context's: the next call runs host-driven and is captured anew."""
+    with api.Context() as c:
+        r = Repeated(api, c, _mesh(60, 51, 2), 3)
+        for replayed in (False, True, True):
+            r.run(replayed)
+        _other_call(api, c, op, _mesh(180, 170, 3))
+        for replayed in (False, True, True):
+            r.run(replayed)
+        _other_call(api, c, op, _mesh(181, 170, 4))
+        _other_call(api, c, op, _mesh(50, 40, 5))
+        for replayed in (False, True):
+            r.run(replayed)
+
+
+@pytest.mark.parametrize("op", ["contract", "score", "select", "sort"])
+def test_a_smaller_call_between_keeps_the_captured_schedule(api, op):
+    with api.Context() as c:
+        r = Repeated(api, c, _mesh(181, 170, 4), 4)
+        r.run(False)
+        r.run(True)
+        _other_call(api, c, op, _mesh(60, 51, 2))
+        r.run(True)
+        _other_call(api, c, op, _mesh(50, 40, 5))
+        r.run(True)
