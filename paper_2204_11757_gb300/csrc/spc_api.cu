@@ -875,16 +875,19 @@ static spc_status drive(spc_context* ctx, const GraphView& v, const Schedule& S,
     if (again) SPC_CUDA(cudaStreamSynchronize(ctx->stream));
     if (again && R.hash == checksum_value(ctx)) {
         if (R.exec && R.timer_substr != tsub) drop_graph(R);
+        // the schedule takes the counters as zero, whatever call came between
+        SPC_TRY(clean_selection(ctx));
+        SPC_TRY(clean_buckets(ctx));
         if (!R.exec && capture_graph(ctx, v, S, lift_int) != SPC_OK) forget_schedule(R);
         if (R.exec) {
             bool mismatch = false;
             const spc_status st = replay_graph(ctx, &mismatch);
-            if (st < 0) {
-                // a replay that stopped in between leaves counters that the graph takes as zero
+            if (st < 0 || mismatch) {
+                // a replay that stopped in between, or ran on sizes that were not its own
                 forget_schedule(R);
                 ctx->work.sel_dirty = true;
                 ctx->work.b_dirty = true;
-                return st;
+                if (st < 0) return st;
             }
             if (!mismatch) {
                 ctx->replayed_last = 1;
@@ -907,7 +910,7 @@ static spc_status drive(spc_context* ctx, const GraphView& v, const Schedule& S,
                 *warn = R.warn;
                 return SPC_OK;
             }
-            forget_schedule(R);  // the device disagreed with the record: run host-driven again
+            // the device disagreed with the record: run host-driven again
         }
     }
     R.mode = use_graph ? Replay::kRecord : Replay::kDirect;

@@ -1163,10 +1163,7 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
     int32_t* list_i = list_c + (m / kSmallBucket + 1);
     int2* huge_c = W.b_huge.as<int2>();  // huge buckets (at most m / kBlockBucket each)
     int2* huge_i = huge_c + (m / kBlockBucket + 1);
-    if (W.b_dirty) {
-        SPC_CUDA(cudaMemsetAsync(W.b_cnt.p, 0, W.b_cnt.bytes, ctx->stream));
-        SPC_CUDA(cudaMemsetAsync(W.b_stats.p, 0, W.b_stats.bytes, ctx->stream));
-    }
+    SPC_TRY(clean_buckets(ctx));
     W.b_dirty = true;
     SPC_LAUNCH(ctx, k_bucket_count, gm, kThreads, 0, m, W.eu.as<int32_t>(), W.ev.as<int32_t>(),
                lift, cnt_c, cnt_i, bstats, reinterpret_cast<uint32_t*>(up_deg),
@@ -1737,6 +1734,15 @@ spc_status diag_graph_typed(spc_context* ctx, const GraphView& g, const void* ma
 }
 
 }  // namespace
+
+spc_status clean_buckets(spc_context* ctx) {
+    Work& W = ctx->work;
+    if (!W.b_dirty || !W.b_cnt.p || !W.b_stats.p) return SPC_OK;
+    SPC_CUDA(cudaMemsetAsync(W.b_cnt.p, 0, W.b_cnt.bytes, ctx->stream));
+    SPC_CUDA(cudaMemsetAsync(W.b_stats.p, 0, W.b_stats.bytes, ctx->stream));
+    W.b_dirty = false;
+    return SPC_OK;
+}
 
 spc_status run_contract(spc_context* ctx, const GraphView& g, const int32_t* lift, int64_t n_c,
                         LevelBufs& lv) {

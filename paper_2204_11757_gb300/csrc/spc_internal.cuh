@@ -493,6 +493,12 @@ spc_status run_select(spc_context* ctx, const GraphView& g, const void* score,
                       const SelectArgs& sa, int32_t* lift, uint8_t* merged, int64_t* n_c,
                       int64_t* graph_ptr_c, int32_t* status);
 
+// State that the selection and the contraction take as zero and leave zero: the counters and score
+// histogram of one graph's selection, the bucket counts and statistics.  A call that stops in
+// between leaves Work::sel_dirty or b_dirty set; these zero what a set flag stands for.
+spc_status clean_selection(spc_context* ctx);
+spc_status clean_buckets(spc_context* ctx);
+
 // S7.  Writes into lv's buffers (allocated by the caller through ensure()).
 spc_status run_contract(spc_context* ctx, const GraphView& g, const int32_t* lift, int64_t n_c,
                         LevelBufs& lv);

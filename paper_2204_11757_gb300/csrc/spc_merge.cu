@@ -1488,6 +1488,7 @@ constexpr int kRestMax = 4096;           // candidates every CTA selects among b
 // histogram) for the next call, so no memset comes between the launches; kCtNc is the result
 enum { kCtList0 = 0, kCtList1 = 1, kCtForest = 2, kCtCand = 3, kCtBar = 4, kCtTau = 5,
        kCtDone = 6, kCtZeroed = 7, kCtNc = 7, kCtCount = 8 };
+constexpr int kCtFirst = 16;  // their place among the context's counters
 
 template <class KT>
 struct CoopArgs {
@@ -2181,7 +2182,7 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
     a.ids = W.ids.as<int32_t>();
     a.lift = lift;
     a.merged = merged;
-    a.ct = W.counters.as<int32_t>() + 16;
+    a.ct = W.counters.as<int32_t>() + kCtFirst;
     a.status = ctx->d_status;
     SPC_TRY(ensure_key_hist(ctx));
     a.rhist = W.key_hist.as<uint32_t>() + kTauBins;
@@ -2200,10 +2201,7 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
     const int grid = grid_for(big, kCoopThreads * 2, ctx->num_sms * bps);
     SPC_TRY(ensure(ctx, W.sel_blk, (size_t)(ctx->num_sms * bps) * 4));
     a.blk = W.sel_blk.as<int32_t>();
-    if (W.sel_dirty) {  // the first call, or one after a call that did not finish
-        SPC_CUDA(cudaMemsetAsync(a.ct, 0, kCtCount * 4, ctx->stream));
-        SPC_CUDA(cudaMemsetAsync(W.key_hist.p, 0, (size_t)kTauBins * 4, ctx->stream));
-    }
+    SPC_TRY(clean_selection(ctx));
     W.sel_dirty = true;
     if (m > 65536 && a.k_need > 0 && a.need < m) {
         a.hist = W.key_hist.as<uint32_t>();
@@ -2426,6 +2424,15 @@ spc_status select_batch(spc_context* ctx, const GraphView& g, const KT* key, con
 }
 
 }  // namespace
+
+spc_status clean_selection(spc_context* ctx) {
+    Work& W = ctx->work;
+    if (!W.sel_dirty || !W.counters.p || !W.key_hist.p) return SPC_OK;
+    SPC_CUDA(cudaMemsetAsync(W.counters.as<int32_t>() + kCtFirst, 0, kCtCount * 4, ctx->stream));
+    SPC_CUDA(cudaMemsetAsync(W.key_hist.p, 0, (size_t)kTauBins * 4, ctx->stream));
+    W.sel_dirty = false;
+    return SPC_OK;
+}
 
 template <class KT>
 static spc_status select_any(spc_context* ctx, const GraphView& g, const void* score,

@@ -87,3 +87,50 @@ def test_a_smaller_call_between_keeps_the_captured_schedule(api, op):
         r.run(True)
         _other_call(api, c, op, _mesh(50, 40, 5))
         r.run(True)
+
+
+def _selection_gives_up(ctx, csr, f, n_c):
+    """A stand-alone selection of one large graph whose grid barrier gives up: the wait limit is
+    raised from one poll until the selection's kernel is reached (at small limits the scans before
+    it give up first); a phase of it takes longer than a few polls."""
+    from paper_2204_11757_gb300 import native as N
+    stopped = 0
+    for limit in (1, 2, 4, 8, 12, 16, 24, 32) * 4:
+        ctx.set_wait_limit(limit)
+        ctx.time_kernel("k_select_coop")
+        try:
+            ctx.select_merges(csr, f, n_c)
+            code = 0
+        except N.SpcError as e:
+            code = e.status
+        finally:
+            ctx.set_wait_limit(0)
+        reached = ctx.kernel_time()[0] > 0
+        ctx.time_kernel(None)
+        assert code in (0, -7)  # SPC_ERR_TIMEOUT
+        stopped += 1 if reached and code == -7 else 0
+        if stopped == 3:
+            return
+    raise AssertionError("no selection reached its grid barrier and gave up")
+
+
+@pytest.mark.parametrize("recorded_only", [True, False])
+def test_a_selection_that_gave_up_leaves_a_repeated_call_right(api, recorded_only):
+    """A grid barrier that gives up leaves the selection's counters and its barrier word nonzero;
+    the next call clears them, whether it runs host-driven, is captured or is replayed."""
+    g = _mesh(181, 170, 4)
+    assert g.n > 8192  # past the one-CTA selection
+    with api.Context() as c:
+        r = Repeated(api, c, g, 4)
+        r.run(False)
+        if not recorded_only:
+            r.run(True)
+        f = torch.from_numpy(O.score(g)).cuda()
+        _selection_gives_up(c, r.csr, f, g.n // 3)
+        r.run(True)
+        r.run(True)
+        _selection_gives_up(c, r.csr, f, g.n // 3)
+        lift, _, n_c, _ = c.select_merges(r.csr, f, g.n // 2)
+        assert n_c == g.n // 2
+        assert np.array_equal(lift.cpu().numpy(), r.ref[0].lift)
+        r.run(True)
