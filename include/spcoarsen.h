@@ -173,10 +173,12 @@ SPC_API spc_status spc_context_create(spc_context** out, const spc_allocator* al
 SPC_API void spc_context_destroy(spc_context* ctx);
 
 /* Bound every device-side wait and retry loop of later calls on the context (the look-back
- * of the scans and sorts, the union-find walks of the merge selection) to `iterations`;
- * 0 restores the default of 2^22.  A wait that reaches the bound gives up and the call returns
- * SPC_ERR_TIMEOUT; every index stays in range when a wait gives up, so the context stays
- * usable.  Meant for exercising the timeout path: a small bound makes waits give up. */
+ * of the scans and sorts, the union-find walks and grid barriers of the merge selection) to
+ * `iterations`; 0 restores the default of 2^22.  A wait that reaches the bound gives up and the call
+ * returns SPC_ERR_TIMEOUT; every index stays in range when a wait gives up, so the context stays
+ * usable: while a bound is set, the calls read the status after every scan and sort, so nothing
+ * indexes with entries that a wait that gave up left unwritten, and no captured schedule is
+ * replayed.  Meant for exercising the timeout path: a small bound makes waits give up. */
 SPC_API spc_status spc_context_set_wait_limit(spc_context* ctx, uint32_t iterations);
 
 /* Change the stream later calls are issued on (captured graphs are re-captured). */

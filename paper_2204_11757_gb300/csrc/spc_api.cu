@@ -284,6 +284,10 @@ spc_status check_status(spc_context* ctx) {
     return sync_status(ctx);
 }
 
+spc_status check_waits(spc_context* ctx) {
+    return ctx->wait_limit == 0 ? SPC_OK : check_status(ctx);
+}
+
 spc_status sync_status(spc_context* ctx) {
     SPC_CUDA(cudaMemcpyAsync(ctx->h_status, ctx->d_status, sizeof(uint32_t),
                              cudaMemcpyDeviceToHost, ctx->stream));
@@ -869,6 +873,7 @@ static spc_status drive(spc_context* ctx, const GraphView& v, const Schedule& S,
     int32_t* lift_int = ctx->work.lift_final.as<int32_t>();
     const std::vector<int64_t> key = call_key(v, S);
     const std::string tsub = ctx->timer.on ? ctx->timer.substr : "";
+    if (ctx->wait_limit != 0) use_graph = false;  // a replay cannot stop after a wait (check_waits)
     if (use_graph) SPC_TRY(input_checksum(ctx, v, S));
     // waited for here only where the arguments repeat; else the run's own reads come after it
     const bool again = use_graph && R.recorded && R.key == key;
@@ -1043,6 +1048,7 @@ spc_status spc_context_set_wait_limit(spc_context* ctx, uint32_t iterations) {
     SPC_CUDA(cudaMemcpyAsync(ctx->d_status + 1, &iterations, sizeof(uint32_t),
                              cudaMemcpyHostToDevice, ctx->stream));
     SPC_CUDA(cudaStreamSynchronize(ctx->stream));
+    ctx->wait_limit = iterations;
     return SPC_OK;
 }
 

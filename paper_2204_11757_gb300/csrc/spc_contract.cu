@@ -1307,6 +1307,7 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         SPC_LAUNCH(ctx, k_bucket_rank_inter, (unsigned)nt, kRankThreads, 0, m_inter, off_c, citem,
                    emap, perm, seg, cU, cV, up_deg, low_deg, hpos + m_inter, bstats + 6, tile_status,
                    tile_ctr, nt, status);
+        SPC_TRY(check_waits(ctx));
     } else if (m_inter > 0) {
         const int gi = grid_for(m_inter, kThreads, maxb);
         SPC_TRY(radix_sort_u64(ctx, ckey, cval, W.c_key2.as<uint64_t>(), W.c_val2.as<uint32_t>(),

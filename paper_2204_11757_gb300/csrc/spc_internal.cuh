@@ -195,6 +195,7 @@ struct spc_context {
     uint32_t* d_status = nullptr;    // device status word
     uint32_t* h_status = nullptr;    // pinned mirror
     int64_t* h_scalars = nullptr;    // pinned readback area
+    uint32_t wait_limit = 0;         // spc_context_set_wait_limit (0: kSpinLimit)
     std::vector<spc::Block> blocks;  // everything allocated, for destroy
     spc::Work work;
     std::vector<spc::LevelBufs> levels;
@@ -558,6 +559,11 @@ spc_status read_i64(spc_context* ctx, const int64_t* dev, int64_t* out);
 // status is read after the replay).
 spc_status check_status(spc_context* ctx);
 inline bool capturing(const spc_context* ctx) { return ctx->replay.mode == Replay::kCapture; }
+// After a kernel whose waits may give up (scans, sorts, the ranking): its output then has entries
+// that nobody wrote, which later kernels would index with.  A caller who lowered the bound has the
+// status read here, and the call ends.  With the default bound a wait for a tile that has already
+// started does not give up, and nothing is read.
+spc_status check_waits(spc_context* ctx);
 // record an event (an external event node during a capture)
 cudaError_t record_event(spc_context* ctx, cudaEvent_t ev);
 

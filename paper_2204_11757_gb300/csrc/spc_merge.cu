@@ -1439,11 +1439,14 @@ spc_status finish_batch(spc_context* ctx, const GraphView& g, const SelectArgs& 
                status);
     SPC_LAUNCH(ctx, k_graph_ptr_c, grid_for(sa.B + 1, kThreads, maxb), kThreads, 0, sa.B,
                sa.d_graph_ptr, ids, sa.d_targets, graph_ptr_c, warn);
-    int64_t vals[2];
+    int64_t vals[3];
     {
-        const void* ptrs[2] = {ids + n, warn};
-        const int bytes[2] = {4, 4};
-        SPC_TRY(read_vals(ctx, 2, ptrs, bytes, vals));
+        // a walk that gave up can leave n_c in the lift: nothing may index with it
+        const void* ptrs[3] = {ids + n, warn, status};
+        const int bytes[3] = {4, 4, 4};
+        SPC_TRY(read_vals(ctx, 3, ptrs, bytes, vals));
+        const spc_status st = status_from_bits((uint32_t)vals[2]);
+        if (st < 0) return st;
     }
     const int64_t n_c = vals[0];
     const int32_t warn_b = (int32_t)vals[1];

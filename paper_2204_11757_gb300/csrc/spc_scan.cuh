@@ -254,7 +254,7 @@ spc_status scan_fused(spc_context* ctx, int64_t n, const Ld& ld, const St& st, d
     if (bytes > 0) note_bytes(ctx, bytes);
     SPC_LAUNCH(ctx, (k_scan_fused<T, Ld, St>), (unsigned)nt, ST, 0, ld, st, n, status, tile_ctr,
                nt, ctx->d_status);
-    return SPC_OK;
+    return check_waits(ctx);
 }
 
 // ---- plain array loader and storer ----------------------------------------------------------

@@ -436,7 +436,7 @@ spc_status radix_sort_impl(spc_context* ctx, K* keys, uint32_t* vals, K* keys_al
         SPC_CUDA(cudaMemcpyAsync(vals, va, (size_t)count * sizeof(uint32_t),
                                  cudaMemcpyDeviceToDevice, ctx->stream));
     }
-    return SPC_OK;
+    return check_waits(ctx);
 }
 
 }  // namespace
