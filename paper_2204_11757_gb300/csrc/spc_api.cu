@@ -1125,17 +1125,17 @@ spc_status spc_select_merges(spc_context* ctx, const spc_csr* g, const void* f, 
     GraphView v;
     SPC_TRY(stage_graph(ctx, g, v));
     SPC_TRY(reserve_work(ctx, v.n, v.nnz / 2, 1));
-    if (ctx->levels.empty()) ctx->levels.resize(1);
-    SPC_TRY(reserve_level(ctx, ctx->levels[0], v.n, v.nnz / 2, 1));
     SPC_TRY(run_score(ctx, v, true, nullptr, 1));  // edge list only
     const size_t fsz = score_is_f32(v.wtype) ? 4 : 8;
     const void* fd;
-    SPC_TRY(stage_in(ctx, f, (size_t)v.m * fsz, ctx->levels[0].score, &fd));
+    SPC_TRY(stage_in(ctx, f, (size_t)v.m * fsz, ctx->work.stage_score, &fd));
     SelectArgs sa;
     sa.target = n_c;
     const bool dev_lift = is_device_ptr(lift_out);
     const bool dev_merged = merged_out && is_device_ptr(merged_out);
-    int32_t* lift = dev_lift ? lift_out : ctx->levels[0].lift.as<int32_t>();
+    // (the levels keep the last coarsening's results)
+    if (!dev_lift) SPC_TRY(ensure(ctx, ctx->work.stage_lift, ((size_t)v.n + 1) * 4));
+    int32_t* lift = dev_lift ? lift_out : ctx->work.stage_lift.as<int32_t>();
     uint8_t* merged = merged_out ? (dev_merged ? merged_out : ctx->work.c_flag.as<uint8_t>()) : nullptr;
     int64_t nc = 0;
     int32_t st = 0;

@@ -113,7 +113,7 @@ struct Work {
     Buf b_cnt, b_off, b_stats, b_list, b_huge;
     bool b_dirty = true;
     Buf sort_hist, scan_tmp;                                    // sort / scan temporaries
-    Buf stage_rowptr, stage_col, stage_w, stage_lift, stage_gptr;  // host staging
+    Buf stage_rowptr, stage_col, stage_w, stage_lift, stage_gptr, stage_score;  // host staging
     Buf pool_key, pool_val, pool_key2, pool_val2, pool_cnt, pool_off;  // feature pooling
     Buf pool_nch, pool_choff, pool_owner, pool_part, pool_stats;
     // the same temporaries for work running on the second stream (SideBranch)

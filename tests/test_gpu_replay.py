@@ -134,3 +134,26 @@ def test_a_selection_that_gave_up_leaves_a_repeated_call_right(api, recorded_onl
         assert n_c == g.n // 2
         assert np.array_equal(lift.cpu().numpy(), r.ref[0].lift)
         r.run(True)
+
+
+@pytest.mark.parametrize("device", ["cuda", "cpu"])
+@pytest.mark.parametrize("levels", [1, 3])
+def test_a_selection_keeps_the_last_coarsening(api, levels, device):
+    """The retained levels, and a result taken from them, hold until the next coarsening call,
+    whatever graph a stand-alone selection runs on in between."""
+    g, big = _mesh(60, 51, 2), _mesh(181, 170, 4)
+    with api.Context() as c:
+        r = Repeated(api, c, g, levels)
+        r.run(False)
+        with_mass = c.take_result().tensors()
+        f = torch.from_numpy(O.score(big)).to(device)
+        lift, _, _, _ = c.select_merges(api.CSR.from_graph(big, device=device), f, big.n // 2)
+        assert np.array_equal(lift.cpu().numpy(), O.coarsen_level(big, big.n // 2).lift)
+        for lv, x in zip(c.levels(), r.ref):
+            assert np.array_equal(lv.lift.cpu().numpy(), x.lift)
+            assert np.array_equal(lv.score.cpu().numpy().view(np.uint64), x.f.view(np.uint64))
+            assert np.array_equal(lv.emap.cpu().numpy(), x.coarse.emap)
+        again = c.take_result().tensors()
+        assert with_mass.keys() == again.keys()
+        for name, t in with_mass.items():
+            assert (t is None and again[name] is None) or torch.equal(t, again[name]), name
