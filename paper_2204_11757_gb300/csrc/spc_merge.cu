@@ -1814,6 +1814,22 @@ __device__ __forceinline__ void coop_hook(const CoopArgs<KT>& a, int64_t cnt, in
     }
 }
 
+// Every node's parent its root, between phases.  On graphs without locality the trees of a round's
+// unions are deep, and all walks of the next phase run down them at once, before any has shortened
+// the way for the others; one walk per node first leaves the phase walks of one step.  Before a
+// further slab it costs no barrier (the slots are reset then); between the rounds of a slab one, so
+// there only while the round's edges outnumber half the nodes, and up to kFlattenNodes nodes (a
+// random graph of 10^6 nodes gains nothing).  The kernel, without / with, binary32: random graphs of
+// 10^5 nodes and 6 10^5 edges to n/2 752 -> 505 us, to n/16 1,546 -> 830, to n/256 1,561 -> 763; 3 10^4
+// nodes to n/16 450 -> 311; 10^5 points to n/16 754 -> 606; meshes and halved point sets unchanged.
+constexpr int64_t kFlattenNodes = int64_t{1} << 18;
+
+template <class KT>
+__device__ __forceinline__ void coop_flatten(const CoopArgs<KT>& a, int64_t t0, int64_t stride) {
+    for (int64_t i = t0; i < a.n; i += stride)
+        a.parent[i] = uf_find(a.parent, (int32_t)i, a.status);
+}
+
 // histogram of digit r over the items whose digits 0 .. r-1 are dig[0 .. r-1], into sh_h
 template <class KT>
 __device__ __forceinline__ void coop_digit_hist(int r, int64_t n, const KT* keys,
@@ -1961,6 +1977,10 @@ k_select_coop(const __grid_constant__ CoopArgs<KT> a) {
                     break;
                 }
                 if (!grid_sync(bar, a.status)) return;
+                if (a.n <= kFlattenNodes && cnt * 2 > a.n) {
+                    coop_flatten(a, t0, stride);
+                    if (!grid_sync(bar, a.status)) return;
+                }
                 in = out;
             }
             if (!grid_sync(bar, a.status)) return;
@@ -1981,6 +2001,7 @@ k_select_coop(const __grid_constant__ CoopArgs<KT> a) {
             if (need >= a.m) prefix = false;  // the last slab: every remaining score
             lo = top;
             for (int64_t i = t0; i < a.n; i += stride) {
+                a.parent[i] = uf_find(a.parent, (int32_t)i, a.status);  // (coop_flatten)
                 a.bk[0][i] = ~0ull;
                 a.bk[1][i] = ~0ull;
                 if (two) {

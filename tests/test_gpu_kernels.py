@@ -428,3 +428,18 @@ def test_batches_that_are_not_block_diagonal(ctx, dtype):
     ref, _, _ = ctx.coarsen_batched(api.CSR.from_graph(wide),
                                     torch.tensor([0, 3000, 8000, 28001]).cuda(), 4, levels=2)
     assert np.array_equal(lift.cpu().numpy(), ref.cpu().numpy()[:8000])
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n", [20011, 262144, 262145])
+def test_deep_trees_of_random_graphs(ctx, dtype, n):
+    """Graphs without locality, whose trees are flattened between rounds (up to 2^18 nodes) and before
+    every further slab (a target of n / 16 takes several)."""
+    from paper_2204_11757_gb300 import api
+    g = _sparse(n, dtype)
+    csr = api.CSR.from_graph(g)
+    for target in (n // 2, n // 16):
+        ref = O.coarsen_level(g, target)
+        lift, n_c, _ = ctx.coarsen(csr, target, levels=1)
+        assert n_c == ref.n_c
+        assert np.array_equal(lift.cpu().numpy(), ref.lift)
