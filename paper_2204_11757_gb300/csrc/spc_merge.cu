@@ -26,6 +26,7 @@
 // shared memory (k_select_small).
 // Every retry loop is bounded (spin_limit: kSpinLimit unless the context lowered it); giving up
 // sets DEV_TIMEOUT in the status word.
+#include <algorithm>
 #include <atomic>
 #include <memory>
 
@@ -868,10 +869,19 @@ struct SmallArgs {
 // One CTA's limits: edges that one SM reads in a few tens of us, and nodes that fit into 203 KB of
 // shared memory (the rest is L1's); 1,024 threads on an SM whatever the class: four CTAs of 256,
 // two of 512, one of 1,024.  What the nodes leave of a CTA's shared memory holds the live edges.
-// One graph alone comes here up to kSmallOne nodes: 9,216 nodes and 27,265 edges take 91 us (to a
-// half) and 174 (to a sixteenth) here, 155 and 170 in k_select_coop; 13,806 nodes 127 and 244
-// against 162 and 177.
+// One graph alone leaves the other SMs idle here, and comes only while its work is small: up to
+// kSmallOne nodes, and at most kSmallWork of nodes and edges, where an edge counts up to four times
+// for every merge wanted (the slabs stop there), or halved at best and at most kSmallHalved edges
+// (one slab of few rounds).  64-bit scores cost a pass more per round.  Whole replayed calls here /
+// in k_select_coop, binary32: 2,100 nodes and 6,300 edges to a sixteenth 258 / 306 us; 8,192 nodes
+// and 24,576 edges to a half 304 / 409, to a sixteenth 450 / 455; binary64, 8,192 nodes and 32,768
+// edges to a sixteenth 698 / 501.  Over 948 calls of 800 to 8,192 nodes, 4 to 60 entries a row, three
+// weight types, targets from a half to one super-node, this choice loses 1.1 % to the better way of
+// each; all of them here would lose 5.8 %, none of them 11.8 %.
 constexpr int64_t kSmallOne = 8192;
+template <class KT>
+constexpr int64_t kSmallWork = MinKey<KT>::two_phase ? 14000 : 20000;
+constexpr int64_t kSmallHalved = 30000;
 constexpr int kSmallEdgeBits = 17;
 constexpr int64_t kSmallEdges = int64_t{1} << kSmallEdgeBits;
 constexpr int kSmallBytes[3] = {54 * 1024, 110 * 1024, 203 * 1024};
@@ -2158,13 +2168,21 @@ k_select_coop(const __grid_constant__ CoopArgs<KT> a) {
         for (int i = 0; i < kCtZeroed; ++i) a.ct[i] = 0;  // every other CTA has left its barriers
 }
 
+// whether one graph of n nodes and m edges that wants k merges is selected in one CTA
+template <class KT>
+bool one_cta(int64_t n, int64_t m, int64_t k) {
+    if (n > kSmallOne || m > kSmallEdges) return false;
+    return std::min(m, 4 * k) + n <= kSmallWork<KT> || (2 * k <= n + 1 && m <= kSmallHalved);
+}
+
 // one cooperative grid that the device holds at once, at most one CTA per kCoopThreads * 2 items
 template <class KT>
 spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, int64_t target,
                          int32_t* lift, uint8_t* merged, int64_t* n_c_out, int32_t* status_out) {
     Work& W = ctx->work;
     const int64_t n = g.n, m = g.m;
-    if (n <= kSmallOne && m <= kSmallEdges) {
+    const int64_t k_need = n - target > 0 ? n - target : 0;
+    if (one_cta<KT>(n, m, k_need)) {
         SelectArgs sa;
         sa.target = target;
         int32_t* nc = W.counters.as<int32_t>() + 4;
@@ -2182,7 +2200,7 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
     CoopArgs<KT> a{};
     a.n = n;
     a.m = m;
-    a.k_need = n - target > 0 ? n - target : 0;
+    a.k_need = k_need;
     a.need = a.k_need + a.k_need / 2;
     a.eu = W.eu.as<int32_t>();
     a.ev = W.ev.as<int32_t>();

@@ -443,3 +443,45 @@ def test_deep_trees_of_random_graphs(ctx, dtype, n):
         lift, n_c, _ = ctx.coarsen(csr, target, levels=1)
         assert n_c == ref.n_c
         assert np.array_equal(lift.cpu().numpy(), ref.lift)
+
+
+@pytest.mark.parametrize("dtype,work", [(np.float32, 20000), (np.float64, 14000), (np.int32, 14000)])
+def test_one_graph_on_both_sides_of_its_rule(ctx, dtype, work):
+    """One graph is selected in one CTA while its nodes and edges are few (an edge counts up to four
+    times per merge wanted), or when it is halved at best and has at most 30,000 edges."""
+    from paper_2204_11757_gb300 import api
+
+    def check(g, target, one_cta):
+        csr = api.CSR.from_graph(g)
+        ref = O.coarsen_level(g, target)
+        ctx.time_kernel("*")
+        try:
+            lift, n_c, _ = ctx.coarsen(csr, target, levels=1)
+            prof = ctx.kernel_profile()
+        finally:
+            ctx.time_kernel(None)
+        assert any("k_select_small" in k for k in prof) == one_cta
+        assert any("k_select_coop" in k for k in prof) == (not one_cta)
+        assert n_c == ref.n_c
+        assert np.array_equal(lift.cpu().numpy(), ref.lift)
+
+    def graph(n, m):  # a path and the first edges of a denser one
+        rng = np.random.default_rng(m)
+        e = rng.integers(0, n, (2, 2 * m))
+        key = np.unique(np.minimum(e[0], e[1]) * n + np.maximum(e[0], e[1]))
+        key = key[(key // n + 1 < key % n)]  # no self-loop, no edge of the path
+        key = np.r_[np.arange(n - 1) * n + np.arange(n - 1) + 1,
+                    rng.permutation(key)[:m - (n - 1)]]
+        w = np.ones(m) if dtype == np.int32 else rng.uniform(0.1, 2.0, m)
+        return I.csr_from_edges(n, key // n, key % n, w.astype(dtype))
+
+    n = 5000
+    check(graph(n, work - n), 1, True)
+    check(graph(n, work - n + 1), 1, False)
+    k = (work - n) // 4  # four edges per merge
+    check(graph(n, 40000), n - k, True)
+    check(graph(n, 40000), n - k - 1, False)
+    check(graph(8192, 30000), 4096, True)
+    check(graph(8192, 30000), 4095, False)
+    check(graph(8192, 30001), 4096, False)
+    check(graph(8193, 9000), 8000, False)
