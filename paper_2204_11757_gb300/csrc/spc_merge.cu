@@ -885,6 +885,18 @@ constexpr int64_t kSmallHalved = 30000;
 constexpr int kSmallEdgeBits = 17;
 constexpr int64_t kSmallEdges = int64_t{1} << kSmallEdgeBits;
 constexpr int kSmallBytes[3] = {54 * 1024, 110 * 1024, 203 * 1024};
+// A batch's graphs of up to kTinyNodes nodes, when at least kTinyMin of them make up for the launch,
+// take CTAs of two warps, 16 on an SM (with four CTAs of 256 threads a graph of a few nodes held a
+// quarter of an SM for 8 us).  Whole replayed calls, the launches over all graphs at once / CTAs of 256 /
+// these: 10^5 graphs of 20 to 50 nodes, one level, binary32, 3.43 / 3.66 / 2.28 ms; 10^5 of 3 to 11
+// 1.53 / 2.02 / 1.14; up to 128 nodes here, 4 10^4 graphs of 50 to 119 2.80 / 2.64 / 3.34 (2.55 with 64).
+constexpr int kTinyNodes = 64;
+constexpr int kTinyBytes = 12 * 1024;
+constexpr int64_t kTinyMin = 1000;
+// Past this many graphs of fewer than kTraceNodes nodes on average, the launches over all graphs are
+// faster: 2 10^5 graphs of 2 to 4 nodes 1.45 ms, 1.63 with a CTA each.
+constexpr int64_t kTraceMin = int64_t{1} << 17;
+constexpr int64_t kTraceNodes = 5;
 template <class KT>
 struct SmallMem {
     // best slot, 16-bit parent and (64-bit scores) best edge of every node
@@ -947,6 +959,12 @@ __device__ __forceinline__ void sm_min(unsigned long long* a, unsigned long long
 }
 
 constexpr int kSmallFlight = 4;  // live edges of a thread in flight
+// Up to kSmallAll edges a graph's first slab is all of them (the two histogram passes of a threshold
+// cost more), and up to kSmallRank forest edges the k lightest are found by comparing each with all:
+// 2 10^4 graphs of 20 to 50 nodes, one level, binary32, replayed: 1,343 -> 875 us, 8,000 of 50 to 119
+// 855 -> 692.
+constexpr int kSmallAll = 512;
+constexpr int kSmallRank = 256;
 
 template <class KT, int T>
 __global__ void __launch_bounds__(T, 1024 / T) k_select_small(SmallArgs<KT> a) {
@@ -1007,7 +1025,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_select_small(SmallArgs<KT> a) {
     constexpr int kTagShift = 32 + kSmallEdgeBits;
     unsigned tag = 0x7fffu;
     while (k > 0) {
-        const bool all = need >= mb;
+        const bool all = need >= mb || mb <= kSmallAll;
         int64_t upto = mb;
         const KT tau = all ? ~KT(0) : cta_select_key<KT>(key, 0, mb, need, hist, &upto);
         // the slab's edges, listed densely: thread t takes the places t, t + T, ...
@@ -1185,7 +1203,29 @@ __global__ void __launch_bounds__(T, 1024 / T) k_select_small(SmallArgs<KT> a) {
         __syncthreads();
     }
     __syncthreads();
-    if (forest > k) {
+    if (forest > k && forest <= (T < kSmallRank ? T : kSmallRank)) {
+        // ---- the k lightest of few: every forest edge's rank by comparison
+        KT* rk = reinterpret_cast<KT*>(hist);
+        uint32_t* re = hist + kSmallRank * (sizeof(KT) / 4);
+        if (tid < forest) {
+            rk[tid] = fk[tid];
+            re[tid] = fe[tid];
+        }
+        for (int32_t x = tid; x < nb; x += T) par[x] = (uint16_t)x;
+        __syncthreads();
+        if (tid < forest) {
+            const KT x = rk[tid];
+            const uint32_t y = re[tid];
+            int32_t rank = 0;
+#pragma unroll 4
+            for (int32_t i = 0; i < forest; ++i)
+                rank += rk[i] < x || (rk[i] == x && re[i] < y) ? 1 : 0;
+            if (rank < k) {
+                sm_unite(par, eu[y] - first, ev[y] - first, lim, a.status);
+                if (a.merged) a.merged[e0 + y] = 1;
+            }
+        }
+    } else if (forest > k) {
         // ---- the k lightest: the key digits of the k-th, most significant first, until all items
         // that share them are wanted
         KT hi = 0;
@@ -1305,7 +1345,7 @@ k_small_shift(int64_t B, const int64_t* __restrict__ graph_ptr, const int32_t* _
 }
 
 // The shape of a batch (out zeroed before): out[0] = the most nodes, out[1] = the most edges of a
-// graph, out[2] != 0 when the graphs do not take the nodes in turn or an edge leaves its graph (such
+// graph, out[3] = the graphs of at most kTinyNodes nodes, out[2] != 0 when the graphs do not take the nodes in turn or an edge leaves its graph (such
 // a batch is merged by the general path, which indexes by the whole batch's nodes).
 __global__ void __launch_bounds__(kThreads)
 k_batch_shape(int64_t B, int64_t n, const int64_t* __restrict__ graph_ptr,
@@ -1328,16 +1368,17 @@ k_batch_shape(int64_t B, int64_t n, const int64_t* __restrict__ graph_ptr,
             if (threadIdx.x == 0) {
                 atomicMax(out, (int32_t)(n1 - n0));
                 atomicMax(out + 1, e1 - e0);
+                if (n1 - n0 <= kTinyNodes) atomicAdd(out + 3, 1);
             }
         }
         if (bad) out[2] = 1;
     }
 }
 
-// k_select_small over B graphs of at most n_max nodes, by classes of sizes
+// k_select_small over B graphs of at most n_max nodes (tiny: of at most kTinyNodes), by classes of sizes
 template <class KT, int T>
 spc_status launch_small_class(spc_context* ctx, SmallArgs<KT>& a, int64_t B, int bytes) {
-    a.n_max = SmallMem<KT>::nodes(bytes);
+    a.n_max = T == 64 ? kTinyNodes : SmallMem<KT>::nodes(bytes);
     a.bytes = bytes;
     static std::atomic<unsigned long long> attr_devs{0};  // devices already set up
     const unsigned long long bit = 1ull << (ctx->device & 63);
@@ -1353,7 +1394,8 @@ spc_status launch_small_class(spc_context* ctx, SmallArgs<KT>& a, int64_t B, int
 
 template <class KT>
 spc_status launch_small(spc_context* ctx, const GraphView& g, const KT* key, const SelectArgs& sa,
-                        int64_t B, int64_t n_max, int32_t* lift, uint8_t* merged, int32_t* n_c) {
+                        int64_t B, int64_t n_max, int64_t tiny, int32_t* lift, uint8_t* merged,
+                        int32_t* n_c) {
     Work& W = ctx->work;
     SmallArgs<KT> a{};
     a.n = g.n;
@@ -1379,6 +1421,10 @@ spc_status launch_small(spc_context* ctx, const GraphView& g, const KT* key, con
     note_bytes(ctx, (double)g.m * sizeof(KT) + 4.0 * g.n);
     if (B <= ctx->num_sms)  // a graph per SM or less takes the most threads
         return launch_small_class<KT, 1024>(ctx, a, B, kSmallBytes[2]);
+    const bool few = tiny < kTinyMin;  // too few tiny graphs for a launch of their own
+    if (n_max <= kTinyNodes && !few) return launch_small_class<KT, 64>(ctx, a, B, kTinyBytes);
+    if (!few && n_max <= SmallMem<KT>::nodes(kSmallBytes[0]))
+        SPC_TRY((launch_small_class<KT, 64>(ctx, a, B, kTinyBytes)));
     if (n_max <= SmallMem<KT>::nodes(kSmallBytes[0]))
         return launch_small_class<KT, 256>(ctx, a, B, kSmallBytes[0]);
     // The smaller classes on the second stream: their CTAs fill the SMs that the largest leaves at
@@ -1388,6 +1434,7 @@ spc_status launch_small(spc_context* ctx, const GraphView& g, const KT* key, con
     SPC_TRY(side->status());
     const bool three = n_max > SmallMem<KT>::nodes(kSmallBytes[1]);
     SmallArgs<KT> last = a;
+    if (!few) SPC_TRY((launch_small_class<KT, 64>(ctx, a, B, kTinyBytes)));
     SPC_TRY((launch_small_class<KT, 256>(ctx, a, B, kSmallBytes[0])));
     if (three) SPC_TRY((launch_small_class<KT, 512>(ctx, a, B, kSmallBytes[1])));
     side->leave();
@@ -2186,7 +2233,7 @@ spc_status select_single(spc_context* ctx, const GraphView& g, const KT* key, in
         SelectArgs sa;
         sa.target = target;
         int32_t* nc = W.counters.as<int32_t>() + 4;
-        SPC_TRY(launch_small<KT>(ctx, g, key, sa, 1, n, lift, merged, nc));
+        SPC_TRY(launch_small<KT>(ctx, g, key, sa, 1, n, 0, lift, merged, nc));
         int64_t vals[2];
         const void* ptrs[2] = {nc, ctx->d_status};
         const int bytes[2] = {4, 4};
@@ -2287,23 +2334,24 @@ spc_status select_batch(spc_context* ctx, const GraphView& g, const KT* key, con
     // 4.39 / 4.00 (5.18 / 4.64), 400 to a sixteenth at once 2.86 / 2.69 (2.93 / 2.83), two random
     // geometric graphs of 12,000 nodes 1.56 / 0.96 (1.76 / 1.11).
     {
-        int32_t* shape = counters + 4;  // [4]: k_batch_shape's three, the warn flag
-        SPC_CUDA(cudaMemsetAsync(shape, 0, 4 * sizeof(int32_t), ctx->stream));
+        int32_t* shape = counters + 24;  // [5]: k_batch_shape's four, the warn flag
+        SPC_CUDA(cudaMemsetAsync(shape, 0, 5 * sizeof(int32_t), ctx->stream));
         SPC_LAUNCH(ctx, k_batch_shape, grid_for(sa.B, 1, maxb), kThreads, 0, sa.B, n,
                    sa.d_graph_ptr, W.up_ptr.as<int32_t>(), W.ev.as<int32_t>(), shape);
-        int64_t big[3];
-        const void* ptrs[3] = {shape, shape + 1, shape + 2};
-        const int bytes[3] = {4, 4, 4};
-        SPC_TRY(read_vals(ctx, 3, ptrs, bytes, big));
-        if (big[0] <= SmallMem<KT>::kMaxNodes && big[1] <= kSmallEdges && big[2] == 0) {
+        int64_t big[4];
+        const void* ptrs[4] = {shape, shape + 1, shape + 2, shape + 3};
+        const int bytes[4] = {4, 4, 4, 4};
+        SPC_TRY(read_vals(ctx, 4, ptrs, bytes, big));
+        const bool trace = sa.B >= kTraceMin && n < kTraceNodes * sa.B;
+        if (!trace && big[0] <= SmallMem<KT>::kMaxNodes && big[1] <= kSmallEdges && big[2] == 0) {
             int32_t* n_c = W.k_graph.as<int32_t>();
             int32_t* off = W.seg_start.as<int32_t>();
-            SPC_TRY(launch_small<KT>(ctx, g, key, sa, sa.B, big[0], lift, merged, n_c));
+            SPC_TRY(launch_small<KT>(ctx, g, key, sa, sa.B, big[0], big[3], lift, merged, n_c));
             SPC_TRY(scan_i32(ctx, n_c, off, sa.B));
             SPC_LAUNCH(ctx, k_small_shift, grid_for(sa.B, 1, maxb), kThreads, 0, sa.B,
-                       sa.d_graph_ptr, off, sa.d_targets, lift, graph_ptr_c, shape + 3);
+                       sa.d_graph_ptr, off, sa.d_targets, lift, graph_ptr_c, shape + 4);
             int64_t vals[3];
-            const void* vp[3] = {off + sa.B, shape + 3, status};
+            const void* vp[3] = {off + sa.B, shape + 4, status};
             const int vb[3] = {4, 4, 4};
             SPC_TRY(read_vals(ctx, 3, vp, vb, vals));
             const spc_status st = status_from_bits((uint32_t)vals[2]);

@@ -485,3 +485,49 @@ def test_one_graph_on_both_sides_of_its_rule(ctx, dtype, work):
     check(graph(8192, 30000), 4095, False)
     check(graph(8192, 30001), 4096, False)
     check(graph(8193, 9000), 8000, False)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64, np.int32])
+@pytest.mark.parametrize("larger", [[], [300, 4000], [300, 4000, 9000, 12000]])
+def test_batches_of_tiny_graphs(ctx, dtype, larger):
+    """Graphs of up to 64 nodes in CTAs of their own (1,000 and more of them), on both sides of 512 edges
+    and of the 64 nodes, with few distinct scores, without edges, of one node."""
+    rng = np.random.default_rng(len(larger))
+    shapes = [_sparse(int(n), dtype, connected=bool(n & 1)) for n in (2, 3, 5, 17, 31, 63, 64, 65, 70)]
+    shapes += [I.complete_graph(n, dtype) for n in (32, 33, 64, 65)]  # 496, 528, 2,016, 2,080 edges
+    shapes += [I.random_graph(60, 0.3, 1, weight="int", dtype=dtype), I.path_graph(40, dtype)]
+    none = np.zeros(0, np.int64)
+    shapes += [I.csr_from_edges(n, none, none, none.astype(dtype)) for n in (1, 6)]
+    graphs = [shapes[i] for i in rng.integers(0, len(shapes), 1500)]
+    graphs += [_sparse(n, dtype) for n in larger]
+    for ratio, levels in ((2, 1), (8, 1), (4, 2)):
+        _batch_checked(ctx, graphs, ratio, "halving" if levels > 1 else "one", levels)
+
+
+def test_batch_of_a_hundred_thousand_traces(ctx):
+    """131,072 graphs of fewer than five nodes on average take the launches over all graphs: every one
+    is merged as the same graph in a small batch, which the oracle checks."""
+    from paper_2204_11757_gb300 import api
+    shapes = [_sparse(2 + i % 4, np.float32) for i in range(64)]
+    _batch_checked(ctx, shapes, 2, "one", 1)
+    small = I.batch_of(shapes)
+    lift, gpc, _ = ctx.coarsen_batched(api.CSR.from_graph(small.graph),
+                                       torch.from_numpy(small.graph_ptr).cuda(), 2, levels=1)
+    reps, n, nnz = 2048, small.graph.n, small.graph.col.shape[0]
+    g = small.graph
+    big = api.CSR.from_numpy(
+        np.r_[0, (g.rowptr[1:][None, :] + nnz * np.arange(reps)[:, None]).ravel()],
+        (g.col[None, :] + n * np.arange(reps)[:, None]).ravel().astype(np.int32),
+        np.tile(g.w, reps))
+    gp = np.r_[0, (small.graph_ptr[1:][None, :] + n * np.arange(reps)[:, None]).ravel()]
+    ctx.time_kernel("*")
+    try:
+        blift, bgpc, _ = ctx.coarsen_batched(big, torch.from_numpy(gp).cuda(), 2, levels=1)
+        prof = ctx.kernel_profile()
+    finally:
+        ctx.time_kernel(None)
+    assert not any("k_select_small" in k for k in prof)
+    n_c = int(gpc[-1])
+    want = (lift.cpu().numpy()[None, :] + n_c * np.arange(reps)[:, None]).ravel()
+    assert np.array_equal(blift.cpu().numpy(), want)
+    assert int(bgpc[-1]) == n_c * reps
