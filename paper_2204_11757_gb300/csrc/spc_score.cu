@@ -335,7 +335,10 @@ __device__ __forceinline__ bool has_mirror(const int32_t* __restrict__ col, cons
 // 0.67, 1.42, 1.52 (fewer CTAs); four entries in flight instead of two slowed the searching version by
 // a quarter on binary32.
 constexpr int64_t kFlatTile = 2048;
-constexpr int kFlatRows = 768;  // rows of a tile kept in shared memory (more: read where used)
+// rows of a tile kept in shared memory (more are read where they are used): paths have 1,024, and a
+// reciprocal per entry is dear (a path of 5 10^6 nodes, binary64, 193 -> 184 us)
+template <class P>
+constexpr int kFlatRows = sizeof(P) == 8 ? 1024 : 768;
 constexpr int kFlatItems = 2;   // entries of a thread in flight
 
 // what an entry needs of its row: the degree, its reciprocal (0: divide), and the edge id of
@@ -349,13 +352,13 @@ struct FlatRow {
 template <class WT>
 __device__ __forceinline__ FlatRow<typename Tr<WT>::P> flat_row(
     int64_t x, const int64_t* __restrict__ rowptr, const typename Tr<WT>::Acc* __restrict__ deg,
-    const int32_t* __restrict__ nlow, const int32_t* __restrict__ up_ptr) {
+    const int32_t* __restrict__ nlow, const int32_t* __restrict__ up_ptr, bool quotients) {
     using P = typename Tr<WT>::P;
     FlatRow<P> r;
     r.d = (P)deg[x];
     r.rcp = P(0);
     if constexpr (std::is_same<P, double>::value)
-        if (mid_range(r.d)) r.rcp = __drcp_rn(r.d);
+        if (quotients && mid_range(r.d)) r.rcp = __drcp_rn(r.d);
     r.ubase = (int64_t)up_ptr[x] - (rowptr[x] + nlow[x]);
     return r;
 }
@@ -375,7 +378,7 @@ k_rows_edges_flat(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
     constexpr bool kF32 = std::is_same<WT, float>::value;
     __shared__ int64_t s_next;            // the row of the next tile's first entry
     __shared__ int32_t s_row[kFlatTile];  // row of each entry of the tile minus the first row
-    __shared__ FlatRow<P> s_data[kFlatRows];
+    __shared__ FlatRow<P> s_data[kFlatRows<P>];
     uint64_t fp = 0;                      // this thread's fingerprint terms
     // a contiguous range of tiles per block
     const int64_t tiles = (nnz + kFlatTile - 1) / kFlatTile;
@@ -394,8 +397,8 @@ k_rows_edges_flat(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
         tile_rows(rowptr, n, base, end, r_lo, kLongRow, s_row, &s_next,
                   [&](int64_t x, int32_t rel, int64_t r0, int64_t r1) {
                       // (the second stream is writing the degrees of the long rows meanwhile)
-                      if (rel < kFlatRows && r1 - r0 <= kLongRow)
-                          s_data[rel] = flat_row<WT>(x, rowptr, deg, nlow, up_ptr);
+                      if (rel < kFlatRows<P> && r1 - r0 <= kLongRow)
+                          s_data[rel] = flat_row<WT>(x, rowptr, deg, nlow, up_ptr, p != nullptr);
                       if constexpr (kF32)  // the row's end marker, by the tile of its last entry
                           if (pk && r1 <= end) pk[r1 + x] = make_uint2(0x7fffffffu, 0u);
                   });
@@ -421,9 +424,9 @@ k_rows_edges_flat(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
                     if (sym && (int64_t)y[q] != x)
                         fp += sym_term(x, y[q], __float_as_uint(wj[q]), k0, k1);
                 if (rel < 0) continue;  // long row: k_long_rows_edges
-                const FlatRow<P> r = rel < kFlatRows
+                const FlatRow<P> r = rel < kFlatRows<P>
                                          ? s_data[rel]
-                                         : flat_row<WT>(x, rowptr, deg, nlow, up_ptr);
+                                         : flat_row<WT>(x, rowptr, deg, nlow, up_ptr, p != nullptr);
                 if constexpr (kF32) {
                     if (p || pk) {
                         const float pj = __fdiv_rn(wj[q], r.d);
@@ -431,7 +434,8 @@ k_rows_edges_flat(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
                         if (pk) pk[j + x] = make_uint2((uint32_t)y[q], __float_as_uint(pj));
                     }
                 } else {
-                    if (p) p[j] = div_row((double)wj[q], r.d, r.rcp, r.rcp != 0.0);
+                    // (the high word: a comparison of doubles takes the pipe that the division needs)
+                    if (p) p[j] = div_row((double)wj[q], r.d, r.rcp, __double2hiint(r.rcp) != 0);
                 }
                 if ((int64_t)y[q] > x) {
                     const int64_t e = r.ubase + j;
@@ -1531,7 +1535,13 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
             sym = W.sym.as<unsigned long long>();
             SPC_CUDA(cudaMemsetAsync(sym, 0, 8, ctx->stream));
         }
-        SPC_LAUNCH(ctx, k_rows_edges_flat<WT>, grid_for(nnz, (int)kFlatTile, maxb), kThreads, 0, n,
+        // Ranges of tiles, per SM: 24 with the divisions, whose CTAs (six at a time) differ in length
+        // and would leave a long last wave; else one wave.  Rows of four, 20 M entries, binary64: 8 /
+        // 6 / 12 / 24 ranges 253 / 194 / 206 / 199 us with scores, 164 / 118 / 127 / 128 without;
+        // binary32 (eight CTAs) 181 / 180 / 193 / 167 and 99 / 106 / 115 / 99.
+        const int ranges = score != nullptr ? 24 : f32 ? 8 : 6;
+        SPC_LAUNCH(ctx, k_rows_edges_flat<WT>, grid_for(nnz, (int)kFlatTile, ctx->num_sms * ranges),
+                   kThreads, 0, n,
                    nnz, g.rowptr, g.col, static_cast<const WT*>(g.w), W.deg.as<Acc>(),
                    W.first_up.as<int32_t>(), W.up_ptr.as<int32_t>(),
                    need_p ? W.p.as<P>() : nullptr,
