@@ -731,7 +731,10 @@ __global__ void k_fs_walk(int64_t nseq, const F* __restrict__ terms,
 // registers, their grid units in the running sum's binade prefix-summed by the block, the sum
 // taken up to the first term that crosses the binade or ties, that term added natively, and the rest
 // of the block summed again in the new binade.  After the first 32 terms (added natively) a
-// sum meets about one crossing and one tie per doubling, 1 us each.  The tables of a batch of
+// sum meets about one crossing per doubling, 1 us each.  A block with ties (a term half a grid unit off,
+// which rounds to the even sum) carries every prefix for an even and for an odd start (sum_pair): one
+// stop per tie made 65,536 binary32 terms of half precision 15.4 ms, 0.2 so (13.1 by tables).  After a
+// negative term the rest of the block is added natively (a caller's own weights have any sign).  The tables of a batch of
 // sequences take about 15 launches and two sizes read back, 60-150 us whatever the lengths; here
 // one launch reads its count on the device, so the caller need not know it.  Whole calls: 2,500
 // meshes, whose coarse levels have thousands of sums of 257 to 3,000 terms, 25.0 -> 22.3 ms; 129^3
@@ -769,6 +772,23 @@ struct GatherSeq {  // segment list[q]: terms w[idx[j]], j in [start[r], start[r
     }
 };
 
+// The units that a run of terms adds, for an even (0) and an odd (1) sum before it.
+struct SumPair {
+    unsigned long long d0, d1;
+};
+
+// a's terms, then b's: a sum's parity after a is its parity before plus a's units
+__device__ __forceinline__ SumPair sum_pair(const SumPair& a, const SumPair& b) {
+    return SumPair{sat_add(a.d0, a.d0 & 1ull ? b.d1 : b.d0),
+                   sat_add(a.d1, a.d1 & 1ull ? b.d0 : b.d1)};
+}
+
+// units of one term after a sum of the given parity: a tie goes to the even sum
+__device__ __forceinline__ unsigned long long tie_units(unsigned long long r, bool tie,
+                                                        unsigned long long sum) {
+    return tie ? r + ((sum + r) & 1ull) : r;
+}
+
 template <class F, class Seq>
 __global__ void __launch_bounds__(kStreamThreads)
 k_seq_stream(const int32_t* __restrict__ count, Seq seq) {
@@ -777,6 +797,8 @@ k_seq_stream(const int32_t* __restrict__ count, Seq seq) {
     constexpr int kNone = INT32_MAX;
     __shared__ F sh_s, sh_t;
     __shared__ unsigned long long sh_w[kStreamThreads / 32], sh_pre;
+    __shared__ SumPair sh_pair[kStreamThreads / 32];
+    __shared__ F sh_v[kStreamTerms];
     __shared__ int sh_first;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t nseq = *count;
@@ -808,11 +830,35 @@ k_seq_stream(const int32_t* __restrict__ count, Seq seq) {
             }
             const int n = L - k < kStreamTerms ? (int)(L - k) : kStreamTerms;
             int pos = 0;  // terms [k, k + pos) are in s
+            bool native = false;
             while (pos < n) {
                 const unsigned long long sb = FB<F>::bits(s);
                 const int eb = (int)(sb >> FB<F>::kMant);
-                if (eb == kInfE) break;  // infinite from here on
-                const bool zero = sb == 0ull, subnormal = eb == 0 && !zero;
+                const bool zero = sb == 0ull;
+                if (native || (!zero && (eb == 0 || eb >= kInfE))) {
+                    // after a negative term, or with a sum that is subnormal, infinite, NaN or (the
+                    // sign is eb's highest bit) negative: the rest of the block natively, in order
+                    bool finite = (eb & kInfE) == kInfE;  // finite terms change no such sum
+#pragma unroll
+                    for (int j = 0; j < kStreamItems; ++j)
+                        finite = finite && ((FB<F>::bits(v[j]) >> FB<F>::kMant) & kInfE) != kInfE;
+                    if (!__syncthreads_or(!finite)) {
+                        pos = n;
+                        continue;
+                    }
+#pragma unroll
+                    for (int j = 0; j < kStreamItems; ++j) sh_v[i0 + j] = v[j];
+                    __syncthreads();
+                    if (warp == 0) {
+#pragma unroll 8
+                        for (int i = pos; i < n; ++i) s = FB<F>::add(s, sh_v[i]);
+                        if (lane == 0) sh_s = s;
+                    }
+                    __syncthreads();
+                    s = sh_s;
+                    pos = n;
+                    continue;
+                }
                 const unsigned long long S =
                     (sb & ((1ull << FB<F>::kMant) - 1ull)) | (1ull << FB<F>::kMant);
                 const unsigned long long lim = (1ull << (FB<F>::kMant + 1)) - S;
@@ -833,32 +879,58 @@ k_seq_stream(const int32_t* __restrict__ count, Seq seq) {
                     if (lane >= o) incl = sat_add(incl, u);
                 }
                 if (lane == 31) sh_w[warp] = incl;
-                __syncthreads();
                 unsigned long long run = 0, total = 0;
-                for (int w = 0; w < kStreamThreads / 32; ++w) {
-                    if (w == warp) run = total;
-                    total = sat_add(total, sh_w[w]);
+                if (!__syncthreads_or(ties != 0u)) {
+                    for (int w = 0; w < kStreamThreads / 32; ++w) {
+                        if (w == warp) run = total;
+                        total = sat_add(total, sh_w[w]);
+                    }
+                    unsigned long long before = __shfl_up_sync(0xffffffffu, incl, 1);
+                    if (lane == 0) before = 0ull;
+                    run = sat_add(run, before);
+                } else {
+                    SumPair pr{0ull, 0ull};
+#pragma unroll
+                    for (int j = 0; j < kStreamItems; ++j) {
+                        const bool tie = ties >> j & 1u;
+                        pr = sum_pair(pr, SumPair{tie_units(r[j], tie, 0ull),
+                                                  tie_units(r[j], tie, 1ull)});
+                    }
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const SumPair u{__shfl_up_sync(0xffffffffu, pr.d0, o),
+                                        __shfl_up_sync(0xffffffffu, pr.d1, o)};
+                        if (lane >= o) pr = sum_pair(u, pr);
+                    }
+                    if (lane == 31) sh_pair[warp] = pr;
+                    __syncthreads();
+                    for (int w = 0; w < kStreamThreads / 32; ++w) {
+                        if (w == warp) run = total;
+                        const bool odd = (S + total) & 1ull;
+                        total = sat_add(total, odd ? sh_pair[w].d1 : sh_pair[w].d0);
+                    }
+                    SumPair before{__shfl_up_sync(0xffffffffu, pr.d0, 1),
+                                   __shfl_up_sync(0xffffffffu, pr.d1, 1)};
+                    if (lane == 0) before = SumPair{0ull, 0ull};
+                    run = sat_add(run, (S + run) & 1ull ? before.d1 : before.d0);
                 }
-                unsigned long long before = __shfl_up_sync(0xffffffffu, incl, 1);
-                if (lane == 0) before = 0ull;
-                run = sat_add(run, before);
                 // the first term that needs a native addition (a zero sum: the first nonzero term)
                 int first = kNone;
                 unsigned long long pre = 0;
                 F tv = F(0);
 #pragma unroll
                 for (int j = 0; j < kStreamItems; ++j) {
+                    const unsigned long long after =
+                        sat_add(run, tie_units(r[j], ties >> j & 1u, S + run));
                     if (first == kNone && i0 + j >= pos && i0 + j < n) {
-                        const bool stop = zero ? FB<F>::bits(v[j]) != 0ull
-                                               : subnormal || (ties >> j & 1u) ||
-                                                     sat_add(run, r[j]) > lim;
+                        const bool stop = zero ? FB<F>::bits(v[j]) != 0ull : after > lim;
                         if (stop) {
                             first = i0 + j;
                             pre = run;
                             tv = v[j];
                         }
                     }
-                    run = sat_add(run, r[j]);
+                    run = after;
                 }
                 if (first != kNone) atomicMin(&sh_first, first);
                 __syncthreads();
@@ -872,9 +944,10 @@ k_seq_stream(const int32_t* __restrict__ count, Seq seq) {
                     if (!zero) s = from_units<F>(S + total, eb);
                     pos = n;
                 } else {
-                    const F base = zero ? F(0) : subnormal ? s : from_units<F>(S + sh_pre, eb);
+                    const F base = zero ? F(0) : from_units<F>(S + sh_pre, eb);
                     s = FB<F>::add(base, sh_t);
                     pos = at + 1;
+                    native = (FB<F>::bits(sh_t) >> (8 * sizeof(F) - 1)) != 0ull;
                     __syncthreads();
                     if (threadIdx.x == 0) sh_first = kNone;
                 }

@@ -531,3 +531,34 @@ def test_batch_of_a_hundred_thousand_traces(ctx):
     want = (lift.cpu().numpy()[None, :] + n_c * np.arange(reps)[:, None]).ravel()
     assert np.array_equal(blift.cpu().numpy(), want)
     assert int(bgpc[-1]) == n_c * reps
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("L", [257, 1056, 1057, 5000, 65536])
+def test_long_sums_of_any_terms(ctx, dtype, L):
+    """A caller's own weights: of any sign, infinite, NaN, subnormal, and of few mantissa bits, whose
+    additions are ties; left to right, as numpy accumulates."""
+    rng = np.random.default_rng(L)
+    top, low = (1e306, 1e-310) if dtype == np.float64 else (1e36, 1e-41)
+    one_inf, opposite, nan = (np.ones(L) for _ in range(3))
+    one_inf[L // 2] = np.inf
+    opposite[[L // 3, L // 2]] = np.inf, -np.inf
+    nan[L // 2] = np.nan
+    late = rng.uniform(0.5, 2.0, L)
+    late[-3] = -3.0 * L
+    with np.errstate(all="ignore"):
+        data = [rng.standard_normal(L), -rng.uniform(0.5, 2.0, L), -np.zeros(L), late,
+                np.where(rng.random(L) < 0.01, -1, 1) * rng.uniform(0.5, 2.0, L),
+                rng.uniform(0, 1, L).astype(np.float16), rng.uniform(0, 1, L) * low,
+                rng.uniform(0.5, 1, L) * top, one_inf, opposite, nan,
+                np.resize([1.0, 2.0 ** -24, 3 * 2.0 ** -24, 2.0 ** -53, 3 * 2.0 ** -53], L),
+                rng.integers(0, 2, L) * 0.5 + rng.integers(0, 3, L) * 2.0 ** 30]
+        perm = torch.from_numpy(rng.permutation(L + 40).astype(np.int32)).cuda()
+        seg = torch.tensor([0, 40, L + 40], dtype=torch.int32).cuda()
+        for d in data:
+            w = np.empty(L + 40, dtype)
+            w[perm.cpu().numpy()] = np.r_[np.ones(40), d].astype(dtype)
+            ref = dtype(0) + np.add.accumulate(d.astype(dtype))[-1]
+            a = ctx.contract_forward(perm, seg, 2, torch.from_numpy(w).cuda()).cpu().numpy()
+            assert a[0] == 40
+            assert _bits(a[1:]) == _bits(np.array([ref])) or (np.isnan(a[1]) and np.isnan(ref))
