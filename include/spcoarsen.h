@@ -290,7 +290,8 @@ SPC_API spc_status spc_contract(spc_context* ctx, const spc_csr* g, const int32_
 
 /* S7 weights only, the assignment held fixed: a_und[k] = sum over perm[seg[k] .. seg[k+1]) of
  * w_und[e], summed in that (ascending eid) order.  w_und[m] and a_und[m_c] of type wtype
- * (SPC_F32 or SPC_F64), perm/seg as retained by a contraction.  Device pointers. */
+ * (SPC_F32 or SPC_F64), perm/seg as retained by a contraction; w_und may hold any values, of any
+ * sign.  Device pointers. */
 SPC_API spc_status spc_contract_forward(spc_context* ctx, const int32_t* perm, const int32_t* seg,
                                 int64_t m_c, const void* w_und, spc_dtype wtype, void* a_und);
 

@@ -816,8 +816,8 @@ k_segsum_long(const int32_t* __restrict__ start, const uint32_t* __restrict__ id
     for (int32_t q = blockIdx.x; q < cnt; q += gridDim.x) {
         const int64_t r = long_list[q];
         const int32_t j0 = start[r], j1 = start[r + 1];
-        // integer weights only (exact in any order); floating-point long segments go through
-        // the per-binade tables (long_segment_sums)
+        // integer weights only (exact in any order); floating-point long segments are streamed or
+        // summed by per-binade tables (long_segment_sums)
         static_assert(std::is_same<WT, int32_t>::value, "integer weights only");
         const long long s =
             cta_sum_i64(j1 - j0, [&](int64_t k) { return (long long)w_und[idx[j0 + k]]; });
@@ -845,16 +845,18 @@ __global__ void k_long_seg_prep(const int32_t* __restrict__ long_list,
     }
 }
 
-// the terms of all long segments, gathered contiguously (segment q at base[q])
+// the terms of all long segments, gathered contiguously (segment q at base[q]); *signed_terms (may be
+// null) = 1 when one of them is negative or NaN
 template <class WT>
 __global__ void __launch_bounds__(kThreads)
 k_gather_long_terms(const int32_t* __restrict__ long_list, const int32_t* __restrict__ long_count,
                     const int32_t* __restrict__ start, const uint32_t* __restrict__ idx,
                     const WT* __restrict__ w_und, const int64_t* __restrict__ base,
-                    WT* __restrict__ terms) {
+                    WT* __restrict__ terms, int32_t* signed_terms) {
     spc::pdl_wait();
     const int32_t cnt = *long_count;
     const int64_t total = base[cnt];
+    bool neg = false;
     for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < total;
          f += (int64_t)gridDim.x * blockDim.x) {
         int32_t lo = 0, hi = cnt - 1;
@@ -863,8 +865,11 @@ k_gather_long_terms(const int32_t* __restrict__ long_list, const int32_t* __rest
             if (base[mid] <= f) lo = mid; else hi = mid - 1;
         }
         const int32_t r = long_list[lo];
-        terms[f] = w_und[idx[start[r] + (f - base[lo])]];
+        const WT t = w_und[idx[start[r] + (f - base[lo])]];
+        terms[f] = t;
+        neg = neg || !(t >= WT(0));
     }
+    if (signed_terms && neg) *signed_terms = 1;
 }
 
 // lower rows by radix sort: key V, value the coarse edge id
@@ -1033,11 +1038,12 @@ k_backward(int64_t m, const int32_t* __restrict__ emap, const WT* __restrict__ g
 
 // Sums of the segments that k_segsum_short left to the long list, none longer than `bound`: integer
 // weights by CTA reductions, floating point exactly left to right, streamed or by per-binade tables.
-// nlong: their number when the host knows it.
+// nlong: their number when the host knows it.  any_sign: the terms are a caller's own, of any sign;
+// the tables hold sums of non-negative terms only, so others are streamed whatever their length.
 template <class WT, class Out>
 spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint32_t* idx,
                              const uint32_t* key, const WT* w_und, Out* out, int64_t bound,
-                             int64_t nlong = -1) {
+                             int64_t nlong = -1, bool any_sign = false) {
     Work& W = ctx->work;
     const bool side = on_side(ctx);
     int32_t* long_list = (side ? W.long_segs_side : W.long_segs).as<int32_t>();
@@ -1063,8 +1069,15 @@ spc_status long_segment_sums(spc_context* ctx, const int32_t* start, const uint3
         Buf& tbuf = side ? W.seg_terms_side : W.seg_terms;
         SPC_TRY(ensure(ctx, tbuf, (size_t)(total + 1) * sizeof(WT)));
         WT* terms = tbuf.as<WT>();
+        int32_t* neg = any_sign ? W.counters.as<int32_t>() + 12 : nullptr;
+        if (neg) SPC_CUDA(cudaMemsetAsync(neg, 0, sizeof(int32_t), ctx->stream));
         SPC_LAUNCH(ctx, k_gather_long_terms<WT>, grid_for(total, kThreads, ctx->num_sms * 8),
-                   kThreads, 0, long_list, long_cnt, start, idx, w_und, base, terms);
+                   kThreads, 0, long_list, long_cnt, start, idx, w_und, base, terms, neg);
+        int64_t has_neg = 0;
+        if (neg) SPC_TRY(read_i32(ctx, neg, &has_neg));
+        if (has_neg)
+            return stream_segments(ctx, std::is_same<WT, float>::value, long_cnt, long_list, start,
+                                   idx, key, w_und, out);
         const bool f32 = std::is_same<WT, float>::value;
         SeqTabBufs& tab = side ? W.tab_s_side : W.tab_s;
         SPC_TRY(seqtab_full(ctx, terms, f32, nlong, base, len, oidx, out, tab));
@@ -1403,7 +1416,7 @@ spc_status forward_typed(spc_context* ctx, const int32_t* perm, const int32_t* s
         if (st < 0 || vals[0] == 0) return st;
     }
     SPC_TRY((long_segment_sums<WT, WT>(ctx, seg, reinterpret_cast<const uint32_t*>(perm), nullptr,
-                                       w_und, a_und, vals[2], vals[0])));
+                                       w_und, a_und, vals[2], vals[0], true)));
     return sync_status(ctx);
 }
 

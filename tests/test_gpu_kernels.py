@@ -534,7 +534,7 @@ def test_batch_of_a_hundred_thousand_traces(ctx):
 
 
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
-@pytest.mark.parametrize("L", [257, 1056, 1057, 5000, 65536])
+@pytest.mark.parametrize("L", [257, 1056, 1057, 5000, 65536, 65537])
 def test_long_sums_of_any_terms(ctx, dtype, L):
     """A caller's own weights: of any sign, infinite, NaN, subnormal, and of few mantissa bits, whose
     additions are ties; left to right, as numpy accumulates."""
