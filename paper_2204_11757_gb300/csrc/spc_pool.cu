@@ -307,8 +307,19 @@ k_pool_mean(int64_t n_c, int64_t F, const int32_t* __restrict__ cnt,
 // flight (lift, count and gradient reads are dependent), 16-byte accesses where they are
 // aligned.  Bound by memory: 2^22 rows of 64 binary32 features write 1.07 GB and gather as much
 // from 134 MB of coarse gradients, 0.565 -> 0.297 ms (8 rows in flight 0.416; a multiplication
-// in the division's place 0.287).
+// in the division's place 0.287).  Binary64 quotients go by one reciprocal per row (div_row) where a
+// lane has two of a row or more: the IEEE divisions filled the FP64 pipe (2^18 rows of 256 features,
+// the call 1,039 us, 500 so).
 constexpr int kBackRows = 4;
+
+__device__ __forceinline__ float back_rcp(float, int32_t) { return 0.f; }
+__device__ __forceinline__ double back_rcp(double, int32_t c) { return __drcp_rn((double)c); }
+__device__ __forceinline__ float back_div(float g, int32_t c, float) {
+    return PoolOps<float>::div(g, c);
+}
+__device__ __forceinline__ double back_div(double g, int32_t c, double rcp) {
+    return div_row(g, (double)c, rcp, __double2hiint(rcp) != 0);
+}
 
 template <class T, int V>
 __global__ void __launch_bounds__(kThreads)
@@ -333,6 +344,10 @@ k_pool_backward(int64_t n, int64_t F, int lp, const int32_t* __restrict__ lift,
         }
 #pragma unroll
         for (int q = 0; q < kBackRows; ++q) c[q] = cnt[u[q]];
+        T rcp[kBackRows];
+#pragma unroll
+        for (int q = 0; q < kBackRows; ++q)
+            rcp[q] = V > 1 || units > lp ? back_rcp(T(0), c[q]) : T(0);
         for (int64_t k = k0; k < units; k += lp) {
             Vec t[kBackRows];
 #pragma unroll
@@ -342,7 +357,7 @@ k_pool_backward(int64_t n, int64_t F, int lp, const int32_t* __restrict__ lift,
                 const int64_t v = v0 + (int64_t)q * subs;
                 if (v < n) {
 #pragma unroll
-                    for (int i = 0; i < V; ++i) t[q].x[i] = PoolOps<T>::div(t[q].x[i], c[q]);
+                    for (int i = 0; i < V; ++i) t[q].x[i] = back_div(t[q].x[i], c[q], rcp[q]);
                     pool_st_once(out + v * units + k, t[q]);
                 }
             }

@@ -19,26 +19,6 @@
 
 namespace spc {
 
-// w / d for every entry of a row that shares the degree d, with y = RN(1/d) computed once per row:
-// Markstein's theorem (IBM J. Res. Dev. 34(1), 1990; also Muller et al., Handbook of
-// Floating-Point Arithmetic, ch. 4): if y is within half an ulp of 1/d and q0 within one ulp of
-// w/d, then r = w - d*q0 is exact (one FMA) and RN(q0 + r*y) = RN(w/d).  q0 = RN(w*y) is within
-// one ulp.  With w and d in [2^-400, 2^400) every intermediate is a normal number (q0 within
-// (2^-800, 2^800), the residual a multiple of about 2^-505 or 0); outside that range the IEEE
-// division is used directly.  The range tests read the exponent fields with integer
-// instructions: GB300's FP64 pipe is narrow, and the divisions of a level are bound by it.
-__device__ __forceinline__ bool mid_range(double v) {
-    const unsigned e = ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
-    return e - (1023u - 400u) < 800u;
-}
-
-__device__ __forceinline__ double div_row(double w, double d, double y, bool d_mid) {
-    if (!(d_mid && mid_range(w))) return __ddiv_rn(w, d);
-    const double q0 = __dmul_rn(w, y);
-    const double r = __fma_rn(-d, q0, w);
-    return __fma_rn(r, y, q0);
-}
-
 template <class WT> struct Tr;
 template <> struct Tr<int32_t> {
     using Acc = long long;

@@ -562,3 +562,16 @@ def test_long_sums_of_any_terms(ctx, dtype, L):
             a = ctx.contract_forward(perm, seg, 2, torch.from_numpy(w).cuda()).cpu().numpy()
             assert a[0] == 40
             assert _bits(a[1:]) == _bits(np.array([ref])) or (np.isnan(a[1]) and np.isnan(ref))
+
+
+@pytest.mark.parametrize("F", [1, 2, 3, 40, 130])
+def test_pooled_gradients_of_any_size(ctx, F):
+    """Binary64 gradients are divided by one reciprocal per row where a lane has several: the same
+    quotients as IEEE division, zeros, subnormals, huge and infinite values among them."""
+    rng = np.random.default_rng(F)
+    lift = rng.permutation(np.repeat(np.arange(40), np.arange(1, 41))).astype(np.int32)
+    g = rng.standard_normal((40, F)) * np.exp2(rng.integers(-1070, 1020, (40, F)))
+    g.ravel()[::7] = rng.choice([0.0, -0.0, np.inf, -np.inf, 5e-324, 1.7e308], g.ravel()[::7].shape)
+    gx = ctx.pool_features_backward(torch.from_numpy(lift).cuda(), 40, torch.from_numpy(g).cuda())
+    ref = g[lift] / np.arange(1, 41)[lift][:, None].astype(np.float64)
+    assert np.array_equal(_bits(gx.cpu().numpy()), _bits(ref))
