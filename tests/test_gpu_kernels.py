@@ -575,3 +575,44 @@ def test_pooled_gradients_of_any_size(ctx, F):
     gx = ctx.pool_features_backward(torch.from_numpy(lift).cuda(), 40, torch.from_numpy(g).cuda())
     ref = g[lift] / np.arange(1, 41)[lift][:, None].astype(np.float64)
     assert np.array_equal(_bits(gx.cpu().numpy()), _bits(ref))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_batches_that_are_not_block_diagonal_against_the_merge_loop(ctx, dtype):
+    """The launches over all graphs on a batch with edges between graphs: of the minimum spanning forest
+    of the whole batch, each graph's lightest edges (an edge belongs to its smaller end's graph) up
+    to its own merges, found here by the merge loop itself."""
+    from paper_2204_11757_gb300 import api
+    a, c = _sparse(3000, dtype), _sparse(5000, dtype)
+    eu = np.concatenate([a.eu, 3000 + c.eu, [17, 2999]])
+    ev = np.concatenate([a.ev, 3000 + c.ev, [3001, 7000]])
+    w = np.concatenate([a.w_und, c.w_und, np.full(2, 1.5, dtype)]).astype(dtype)
+    g, gp, ratio = I.csr_from_edges(8000, eu, ev, w), np.array([0, 3000, 8000]), 4
+    assert g.m <= 65536  # one slab: the whole batch's forest
+
+    def find(p, x):
+        while p[x] != x:
+            p[x] = p[p[x]]
+            x = p[x]
+        return x
+
+    forest, merged = list(range(g.n)), list(range(g.n))
+    left = [n - max(1, n // ratio) for n in np.diff(gp)]
+    for e in np.lexsort((np.arange(g.m), O.score(g))):
+        u, v = int(g.eu[e]), int(g.ev[e])
+        ru, rv = find(forest, u), find(forest, v)
+        if ru == rv:
+            continue
+        forest[max(ru, rv)] = min(ru, rv)
+        b = 0 if u < 3000 else 1
+        if left[b] > 0:
+            left[b] -= 1
+            ru, rv = find(merged, u), find(merged, v)
+            merged[max(ru, rv)] = min(ru, rv)
+    root = np.array([find(merged, x) for x in range(g.n)])
+    is_root = root == np.arange(g.n)
+    ids = np.r_[0, np.cumsum(is_root)]
+    lift, gpc, _ = ctx.coarsen_batched(api.CSR.from_graph(g), torch.from_numpy(gp).cuda(), ratio,
+                                       levels=1)
+    assert np.array_equal(lift.cpu().numpy(), ids[root])
+    assert np.array_equal(gpc.cpu().numpy(), ids[gp])
