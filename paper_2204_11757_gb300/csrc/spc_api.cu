@@ -197,8 +197,7 @@ __global__ void k_expect(Expect x, int32_t* mismatch) {
 }
 
 // the values a read takes, written to pinned host memory by one launch (a copy per value was 1.5-2
-// us each on the stream, and a contraction reads eight)
-constexpr int kReadMax = 10;
+// us each on the stream, and a contraction's bucket sizes are ten)
 struct ReadVals {
     const void* dev[kReadMax];
     int bytes[kReadMax];
@@ -1089,10 +1088,13 @@ spc_status spc_score(spc_context* ctx, const spc_csr* g, void* f_out, int64_t* m
     const bool dev_out = is_device_ptr(f_out);
     Buf& tmp = ctx->work.sel_key;  // sized >= m * 8
     // binary32 rows go through the packed pairs: 2^21-point random geometric graph, the score
-    // kernel 1.43 ms walking rows in place, 0.49 ms packed.  Binary64 and integer rows are walked
-    // in place (2048^2 mesh 0.70 ms, staged 1.42 ms; 129^3 mesh 1.44 and 2.25 ms; 2^21-point
-    // random geometric graph 2.66 and 3.07 ms), and so are binary32 rows of more than 48 entries
-    // on average, which do not fit the packed schedule's stage.
+    // kernel 1.43 ms walking rows in place, 0.49 ms packed.  The stage holds 32 rows b of 18 entries
+    // on average, and longer ones are walked as pairs where they lie, which still beats walking
+    // columns and quotients apart: random graphs of 20 M entries, the whole call, in place / packed,
+    // mean rows of 12 1.57 / 0.69 ms, 18 2.00 / 0.91, 24 2.43 / 1.20, 36 3.27 / 1.71, 48 4.08 / 2.19;
+    // rows of neighbouring numbers 0.81 / 0.56, 1.03 / 0.62, 1.25 / 0.73, 1.69 / 0.87, 2.21 / 1.69.
+    // Longer rows are walked in place, and so are binary64 and integer ones (2048^2 mesh 0.70 ms,
+    // staged 1.42 ms; 129^3 mesh 1.44 and 2.25 ms; 2^21-point random geometric graph 2.66 and 3.07).
     const int schedule = score_is_f32(v.wtype) && v.nnz <= 48 * v.n ? 3 : 1;
     SPC_TRY(run_score(ctx, v, true, dev_out ? f_out : tmp.p, schedule));
     if (!dev_out) SPC_TRY(copy_out(ctx, f_out, tmp.p, (size_t)v.m * fsz));

@@ -2,14 +2,15 @@
 // forward with the assignment held fixed.
 //
 // For every fine undirected edge e = (u, v): U = c(u), V = c(v).  U == V: the edge is inside a
-// super-node; emap[e] = -1 and its weight goes to self_mass[U].  Otherwise key(e) =
-// (min(U,V), max(U,V)).  A stable radix sort of (key, eid) -- input in eid order -- groups the
-// fine edges of every coarse edge with ascending eids; segment heads numbered by a scan give
-// the coarse edge ids in lexicographic (U, V) order, and each coarse weight is the sequential
-// sum of its segment (ascending eid, IEEE round-to-nearest), so the result is reproducible.
-// The coarse CSR: row U holds first the coarse edges (V', U) with V' < U (a stable sort by
-// the second end point, the "transpose") and then the edges (U, V) with V > U (contiguous in
-// coarse-edge order), which leaves every row sorted.
+// super-node; emap[e] = -1 and its weight goes to self_mass[U].  Otherwise e belongs to the coarse
+// edge (min(U,V), max(U,V)).  The edges are counted and scattered into a bucket per lower super-node
+// and each bucket is ordered by (upper super-node, eid) (one stable radix sort of all edges where
+// huge buckets hold more than half of them): the fine edges of every coarse edge lie together with
+// ascending eids, coarse edge ids run in lexicographic (U, V) order, and each coarse weight is the
+// sequential sum of its segment (ascending eid, IEEE round-to-nearest), so the result is
+// reproducible.  The coarse CSR: row U holds first the coarse edges (V', U) with V' < U (the
+// "transpose", by buckets or a stable sort of the second end point) and then the edges (U, V) with
+// V > U (contiguous in coarse-edge order), which leaves every row sorted.
 #include <type_traits>
 
 #include <atomic>
@@ -1191,6 +1192,7 @@ spc_status contract_typed(spc_context* ctx, const GraphView& g, const int32_t* l
         const void* ptrs[10] = {off_c + n_c, off_i + n_c, bstats,     bstats + 1, bstats + 2,
                                 bstats + 3,  bstats + 6,  bstats + 7, bstats + 8, bstats + 9};
         const int bytes[10] = {4, 4, 8, 8, 8, 8, 8, 8, 8, 8};
+        static_assert(sizeof(ptrs) / sizeof(ptrs[0]) <= kReadMax, "one read");
         SPC_TRY(read_vals(ctx, 10, ptrs, bytes, bv));
     }
     const int64_t long_c = bv[6], long_i = bv[7];  // buckets longer than kSmallBucket

@@ -565,6 +565,8 @@ spc_status run_contract_backward(spc_context* ctx, const int32_t* emap, int64_t 
 // read the status word (synchronises)
 spc_status sync_status(spc_context* ctx);
 
+// the most values of one read_vals
+constexpr int kReadMax = 10;
 // A device value the host driver needs (int32 or int64 at `dev`).  Direct and recording runs
 // copy it back (synchronising; a recording run logs it); a capture returns the logged value and
 // enqueues a check that flags a replay whose device value differs.

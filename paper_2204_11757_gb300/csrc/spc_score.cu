@@ -89,7 +89,7 @@ k_rows_degree(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
             nlow_out[x] = 0;
             continue;
         }
-        if (r1 - r0 > kLongRow) {  // long rows: k_long_rows_meta and the per-binade tables
+        if (r1 - r0 > kLongRow) {  // long rows: k_long_rows_meta and the sums of long rows
             long_rows[atomicAdd(long_count, 1)] = (int32_t)x;
             continue;
         }
@@ -116,8 +116,8 @@ k_rows_degree(int64_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
 }
 
 // S0 for rows longer than kLongRow, part 1: one warp per row records the row as a sequence
-// (base, length) for the exact degree sum (the per-binade tables of spc_seqtab.cu evaluate
-// it) and counts its entries at or below the diagonal by a 32-way search for x among the
+// (base, length) for the exact degree sum (streamed or by per-binade tables, spc_seqtab.cu)
+// and counts its entries at or below the diagonal by a 32-way search for x among the
 // sorted columns.  On an unsorted row the count is wrong but in range; part 2 reports the row.
 template <class WT>
 __global__ void __launch_bounds__(kThreads)
@@ -1488,8 +1488,8 @@ static spc_status score_typed(spc_context* ctx, GraphView& g, bool validate, voi
     constexpr bool f32 = std::is_same<WT, float>::value;
     const bool need_p = score != nullptr && (!f32 || n_long > 0 || schedule != 3);
     {
-        // long rows (exact degrees from per-binade tables, then p and their edges) on the
-        // second stream while the short rows run here
+        // long rows (exact degrees, streamed up to kStreamMax entries, else from per-binade tables;
+        // then p and their edges) on the second stream while the short rows run here
         std::unique_ptr<SideBranch> side;
         if (n_long > 0) {
             side.reset(new SideBranch(ctx));
