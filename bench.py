@@ -324,6 +324,11 @@ TRAFFIC = {
     ("c2_tri2048_f64", "(k_score_edges<P, Key, kScoreChains>)"): 2.226063e8,
     ("c3_tet129_f64", "(k_score_edges<P, Key, kScoreChains>)"): 3.163520e8,
     ("c5_batch10k_f32", "k_score_packed<Key>"): 3.893167e+09,
+    ("c4_rgg8m_f32", "k_select_coop<KT>"): 9.607736e+08,
+    ("c4_rgg8m_f32_one", "k_select_coop<KT>"): 1.398084e+10,
+    ("c4_rgg8m_f32_reordered", "k_select_coop<KT>"): 8.477027e+08,
+    ("c2_tri2048_f64", "k_select_coop<KT>"): 4.364679e+08,
+    ("c5_batch10k_f32", "(k_select_small<KT, T>)"): 1.0402e+09,
 }
 
 HEADLINE = "c4_rgg8m_f32"

@@ -310,10 +310,10 @@ __device__ __forceinline__ bool has_mirror(const int32_t* __restrict__ col, cons
 // than kLongRow are left to k_long_rows_edges.  With `sym` (input validation of binary32 rows), every
 // entry of every row, long ones included, also adds its symmetry fingerprint term into *sym.
 // Bound by the entries' traffic and, binary64, by that pipe (three operations an entry).  All
-// launches of a call, a thread per row or a search per tile before: 129^3 mesh 1.37 -> 0.67 ms, 2048^2
-// mesh 0.81 -> 0.66, 2^23 points 1.55 -> 1.22, 2,500 meshes 1.57 -> 1.30.  Tiles of 4,096 entries: 0.69,
-// 0.67, 1.42, 1.52 (fewer CTAs); four entries in flight instead of two slowed the searching version by
-// a quarter on binary32.
+// launches of a call, a thread per row or a search per tile before: 129^3 mesh 1.37 -> 0.49 ms, 2^23
+// points 1.55 -> 1.16, 2,500 meshes 1.57 -> 1.21.  Tiles of 4,096 entries were 3 % (binary64) to 17 %
+// slower than these with fewer CTAs; four entries in flight instead of two slowed the searching version
+// by a quarter on binary32.
 constexpr int64_t kFlatTile = 2048;
 // rows of a tile kept in shared memory (more are read where they are used): paths have 1,024, and a
 // reciprocal per entry is dear (a path of 5 10^6 nodes, binary64, 193 -> 184 us)
