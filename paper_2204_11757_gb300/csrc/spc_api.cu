@@ -75,7 +75,7 @@ spc_status ensure(spc_context* ctx, Buf& b, size_t bytes) {
         // the old block may still be read by queued work
         SPC_CUDA(cudaStreamSynchronize(ctx->stream));
         // a captured schedule holds the block's address, its record the levels' masses
-        forget_schedule(ctx->replay);
+        if (b.in_schedule) forget_schedule(ctx->replay);
         raw_free(ctx, b.p);
         b.p = nullptr;
         b.bytes = 0;

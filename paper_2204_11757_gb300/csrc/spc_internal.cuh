@@ -60,6 +60,7 @@ struct Context;
 struct Buf {
     void* p = nullptr;
     size_t bytes = 0;
+    bool in_schedule = true;  // a captured schedule may hold the block's address
     template <class T> T* as() const { return static_cast<T*>(p); }
 };
 
@@ -114,8 +115,11 @@ struct Work {
     bool b_dirty = true;
     Buf sort_hist, scan_tmp;                                    // sort / scan temporaries
     Buf stage_rowptr, stage_col, stage_w, stage_lift, stage_gptr, stage_score;  // host staging
-    Buf pool_key, pool_val, pool_key2, pool_val2, pool_cnt, pool_off;  // feature pooling
-    Buf pool_nch, pool_choff, pool_owner, pool_part, pool_stats;
+    // feature pooling (no part of a coarsening)
+    Buf pool_key{nullptr, 0, false}, pool_val{nullptr, 0, false}, pool_key2{nullptr, 0, false};
+    Buf pool_val2{nullptr, 0, false}, pool_cnt{nullptr, 0, false}, pool_off{nullptr, 0, false};
+    Buf pool_nch{nullptr, 0, false}, pool_choff{nullptr, 0, false}, pool_owner{nullptr, 0, false};
+    Buf pool_part{nullptr, 0, false}, pool_stats{nullptr, 0, false};
     // the same temporaries for work running on the second stream (SideBranch)
     Buf sort_hist_side, scan_tmp_side, long_segs_side;
     Buf seg_base_side, seg_len_side, seg_idx_side, seg_terms_side;

@@ -157,3 +157,18 @@ def test_a_selection_keeps_the_last_coarsening(api, levels, device):
         assert with_mass.keys() == again.keys()
         for name, t in with_mass.items():
             assert (t is None and again[name] is None) or torch.equal(t, again[name]), name
+
+
+def test_pooling_between_keeps_the_captured_schedule(api):
+    """A training step coarsens and pools: pooling on growing sizes, by both of its routes, touches no
+    block that a coarsening uses."""
+    with api.Context() as c:
+        r = Repeated(api, c, _mesh(181, 170, 4), 4)
+        r.run(False)
+        r.run(True)
+        for n, n_c in ((3000, 900), (90000, 20000), (300000, 3)):
+            lift = (np.arange(n) % n_c).astype(np.int32)
+            x = np.random.default_rng(n).standard_normal((n, 5))
+            xc = c.pool_features(torch.from_numpy(lift).cuda(), n_c, torch.from_numpy(x).cuda())
+            assert np.array_equal(xc.cpu().numpy(), O.pool_features(lift, n_c, x))
+            r.run(True)
