@@ -1345,8 +1345,9 @@ k_small_shift(int64_t B, const int64_t* __restrict__ graph_ptr, const int32_t* _
 }
 
 // The shape of a batch (out zeroed before): out[0] = the most nodes, out[1] = the most edges of a
-// graph, out[3] = the graphs of at most kTinyNodes nodes, out[2] != 0 when the graphs do not take the nodes in turn or an edge leaves its graph (such
-// a batch is merged by the general path, which indexes by the whole batch's nodes).
+// graph, out[3] = the graphs of at most kTinyNodes nodes, out[2] != 0 when the graphs do not take
+// the nodes in turn or an edge leaves its graph (such a batch is merged by the general path, which
+// indexes by the whole batch's nodes).
 __global__ void __launch_bounds__(kThreads)
 k_batch_shape(int64_t B, int64_t n, const int64_t* __restrict__ graph_ptr,
               const int32_t* __restrict__ up_ptr, const int32_t* __restrict__ ev,

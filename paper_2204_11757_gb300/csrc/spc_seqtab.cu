@@ -734,8 +734,8 @@ __global__ void k_fs_walk(int64_t nseq, const F* __restrict__ terms,
 // sum meets about one crossing per doubling, 1 us each.  A block with ties (a term half a grid unit off,
 // which rounds to the even sum) carries every prefix for an even and for an odd start (sum_pair): one
 // stop per tie made 65,536 binary32 terms of half precision 15.4 ms, 0.2 so (13.1 by tables).  After a
-// negative term the rest of the block is added natively (a caller's own weights have any sign).  The tables of a batch of
-// sequences take about 15 launches and two sizes read back, 60-150 us whatever the lengths; here
+// negative term the rest of the block is added natively (a caller's own weights have any sign).
+// The tables of a batch of sequences take about 15 launches and two sizes read back, 60-150 us whatever the lengths; here
 // one launch reads its count on the device, so the caller need not know it.  Whole calls: 2,500
 // meshes, whose coarse levels have thousands of sums of 257 to 3,000 terms, 25.0 -> 22.3 ms; 129^3
 // mesh 21.6 -> 19.9; 2^23 points 21.6 -> 20.1.  The launches at 8 terms a thread (4): 0.46 ms (0.34),
