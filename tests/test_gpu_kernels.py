@@ -504,33 +504,38 @@ def test_batches_of_tiny_graphs(ctx, dtype, larger):
         _batch_checked(ctx, graphs, ratio, "halving" if levels > 1 else "one", levels)
 
 
-def test_batch_of_a_hundred_thousand_traces(ctx):
-    """131,072 graphs of fewer than five nodes on average take the launches over all graphs: every one
-    is merged as the same graph in a small batch, which the oracle checks."""
+def test_batches_of_ten_thousand_graphs(ctx):
+    """Of very many graphs a block looks at eight together, a warp at each but the larger ones: every
+    graph is merged as the same graph in a small batch, which the oracle checks; an edge that leaves
+    its graph is seen wherever it is."""
     from paper_2204_11757_gb300 import api
-    shapes = [_sparse(2 + i % 4, np.float32) for i in range(64)]
+    shapes = [_sparse(2 + i % 4, np.float32) for i in range(96)]
+    shapes[17], shapes[40], shapes[41] = (_sparse(n, np.float32) for n in (1500, 300, 1100))
+    shapes[70] = _sparse(1023, np.float32)
     _batch_checked(ctx, shapes, 2, "one", 1)
     small = I.batch_of(shapes)
     lift, gpc, _ = ctx.coarsen_batched(api.CSR.from_graph(small.graph),
                                        torch.from_numpy(small.graph_ptr).cuda(), 2, levels=1)
-    reps, n, nnz = 2048, small.graph.n, small.graph.col.shape[0]
-    g = small.graph
-    big = api.CSR.from_numpy(
-        np.r_[0, (g.rowptr[1:][None, :] + nnz * np.arange(reps)[:, None]).ravel()],
-        (g.col[None, :] + n * np.arange(reps)[:, None]).ravel().astype(np.int32),
-        np.tile(g.w, reps))
-    gp = np.r_[0, (small.graph_ptr[1:][None, :] + n * np.arange(reps)[:, None]).ravel()]
-    ctx.time_kernel("*")
-    try:
-        blift, bgpc, _ = ctx.coarsen_batched(big, torch.from_numpy(gp).cuda(), 2, levels=1)
-        prof = ctx.kernel_profile()
-    finally:
-        ctx.time_kernel(None)
-    assert not any("k_select_small" in k for k in prof)
-    n_c = int(gpc[-1])
-    want = (lift.cpu().numpy()[None, :] + n_c * np.arange(reps)[:, None]).ravel()
-    assert np.array_equal(blift.cpu().numpy(), want)
-    assert int(bgpc[-1]) == n_c * reps
+    g, n, nnz, n_c = small.graph, small.graph.n, small.graph.col.shape[0], int(gpc[-1])
+    for reps in (100, 127):  # 9,600 and 12,192 graphs
+        big = api.CSR.from_numpy(
+            np.r_[0, (g.rowptr[1:][None, :] + nnz * np.arange(reps)[:, None]).ravel()],
+            (g.col[None, :] + n * np.arange(reps)[:, None]).ravel().astype(np.int32),
+            np.tile(g.w, reps))
+        gp = np.r_[0, (small.graph_ptr[1:][None, :] + n * np.arange(reps)[:, None]).ravel()]
+        want = (lift.cpu().numpy()[None, :] + n_c * np.arange(reps)[:, None]).ravel()
+        for split in (None, 17, 40 + 96 * (reps - 1)):  # the graph divided in two: its edges leave it
+            ptr = gp if split is None else np.r_[gp[:split + 1], gp[split] + 200, gp[split + 1:]]
+            ctx.time_kernel("*")
+            try:
+                blift, bgpc, _ = ctx.coarsen_batched(big, torch.from_numpy(ptr).cuda(), 2, levels=1)
+                prof = ctx.kernel_profile()
+            finally:
+                ctx.time_kernel(None)
+            assert any("k_select_small" in k for k in prof) == (split is None)
+            if split is None:
+                assert np.array_equal(blift.cpu().numpy(), want)
+                assert int(bgpc[-1]) == n_c * reps
 
 
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
